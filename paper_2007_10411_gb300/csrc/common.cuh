@@ -36,6 +36,8 @@ struct Geo {
     double dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
     // float32 derivative weights with 1/h folded in: D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
     float fx1, fx2, fz1, fz2;
+    double wx1, wx2, wy1, wy2, wz1, wz2;   // the same weights in float64 (and along y)
+    double gth;                       // g / theta0
     double inv_Pr;
     double two_over_dt;
     double scale[5], inv_scale[5];
@@ -117,6 +119,25 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 
 enum CounterSlot { CNT_STENCIL = 0, CNT_UPDATE, CNT_RESTART, CNT_PC, CNT_EDDY, CNT_MISC };
+
+// Square root for kernels bound by the FP64 pipe (64 cycles per warp
+// instruction): Goldschmidt's iteration (Markstein, "IA-64 and Elementary
+// Functions", 2000) from the hardware's 20-bit reciprocal square root estimate,
+// seven FP64 operations: one coupled step takes g ~ sqrt(x), h ~ 1/(2 sqrt(x))
+// to ~39 bits, the residual step g + h (x - g^2) rounds the result (within one
+// unit in the last place).  Zero, subnormal, negative and non-finite operands go to sqrt().
+__device__ __forceinline__ double root(double x) {
+    const int hi = __double2hiint(x);
+    if (hi < 0x00100000 || hi >= 0x7ff00000) return sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = __dmul_rn(x, y), h = __dmul_rn(0.5, y);
+    const double r = __fma_rn(-g, h, 0.5);
+    g = __fma_rn(g, r, g);
+    h = __fma_rn(h, r, h);
+    return __fma_rn(__fma_rn(-g, g, x), h, g);
+}
+__device__ __forceinline__ float root(float x) { return sqrtf(x); }
 
 // ---------------------------------------------------------------- reductions
 // Sum NV thread-local values over the block and store them, as float64, at

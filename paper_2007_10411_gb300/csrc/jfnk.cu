@@ -353,6 +353,13 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     G.fx2 = (float)(-1.0 / 12.0 / dx);
     G.fz1 = (float)(2.0 / 3.0 / dz);
     G.fz2 = (float)(-1.0 / 12.0 / dz);
+    G.wx1 = 2.0 / 3.0 / dx;
+    G.wx2 = -1.0 / 12.0 / dx;
+    G.wy1 = 2.0 / 3.0 / dy;
+    G.wy2 = -1.0 / 12.0 / dy;
+    G.wz1 = 2.0 / 3.0 / dz;
+    G.wz2 = -1.0 / 12.0 / dz;
+    G.gth = strat->g / strat->theta0;
     G.theta0 = strat->theta0;
     G.beta = strat->beta;
     G.pbar = strat->pbar;
@@ -555,7 +562,7 @@ static jfnk_status autotune_impl(jfnk_handle* h, const double* u, int* tiles) {
         G.tile_pc = c;
         for (int pass = 0; pass < 4; ++pass) {          // pass 0 warms up (and sets shared-memory limits)
             CK(cudaEventRecord(e0, s));
-            for (int r = 0; r < reps; ++r) CK(launch_jv_diff<T>(G, uT, dir, (T*)h->w, h->part, h->ctl, 0, s));
+            for (int r = 0; r < reps; ++r) CK(launch_jv_diff(G, uT, dir, (T*)h->w, h->part, h->ctl, 0, s));
             CK(cudaEventRecord(e1, s));
             CK(cudaEventSynchronize(e1));
             float ms = 0.f;
@@ -662,7 +669,7 @@ static jfnk_status jv_impl(jfnk_handle* h, const double* u, const double* F_u, c
     T* wh = (T*)h->tB;
     CK((launch_rescale<double, T>(G, v, vh, h->n, 0, s)));
     h->launches += 4;
-    if (sizeof(T) == sizeof(double)) {
+    if constexpr (sizeof(T) == sizeof(double)) {
         const double* Fu = F_u;
         if (!Fu) {
             CK(launch_stencil<double>(MODE_F, G, u, nullptr, nullptr, nullptr, h->tmp64, nullptr,
@@ -675,7 +682,7 @@ static jfnk_status jv_impl(jfnk_handle* h, const double* u, const double* F_u, c
     } else {
         T* uT = (T*)h->uT;
         CK((launch_convert<double, T>(u, uT, h->n, s)));
-        CK(launch_jv_diff<T>(G, uT, vh, wh, h->part, h->ctl, 0, s));
+        CK(launch_jv_diff(G, uT, vh, wh, h->part, h->ctl, 0, s));
         h->launches += 1;
     }
     CK((launch_rescale<T, double>(G, wh, Jv, h->n, 1, s)));
@@ -762,11 +769,11 @@ static jfnk_status read_ctl(jfnk_handle* h) {
 template <typename T>
 static jfnk_status apply_jv(jfnk_handle* h, const T* uT, const T* z, T* w, int check_done) {
     kt_begin(h, JFNK_KF_JV);
-    if (sizeof(T) == sizeof(double)) {
+    if constexpr (sizeof(T) == sizeof(double)) {
         CK(launch_stencil<double>(MODE_JV, h->G, (const double*)uT, (const double*)z, h->Fu64,
                                   nullptr, (double*)w, nullptr, h->part, h->ctl, check_done, h->stream));
     } else {
-        CK(launch_jv_diff<T>(h->G, uT, z, w, h->part, h->ctl, check_done, h->stream));
+        CK(launch_jv_diff(h->G, uT, z, w, h->part, h->ctl, check_done, h->stream));
     }
     kt_end(h, JFNK_KF_JV, (double)h->n * (h->mixed ? 3.0 * 4.0 : 4.0 * 8.0));
     h->launches += 1;

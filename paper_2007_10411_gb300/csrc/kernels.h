@@ -8,9 +8,6 @@ namespace jfnk {
 enum StencilMode { MODE_F = 0, MODE_RHS = 1, MODE_RES = 2, MODE_JV = 3,
                    MODE_RHSRES = 4 };   // f = 2u/dt + F(u) into out and R(u) = -2 F(u) into out2, with norms
 
-// Number of blocks of the 2-D stencil grid for element type T.
-template <typename T> int stencil_blocks(const Geo& G);
-
 // F / 2u/dt + F / residual / plain forward-difference Jv (see stencil.cu).
 template <typename T>
 cudaError_t launch_stencil(int mode, const Geo& G, const T* u, const T* v, const T* Fu,
@@ -18,8 +15,7 @@ cudaError_t launch_stencil(int mode, const Geo& G, const T* u, const T* v, const
                            int check_done, cudaStream_t s);
 
 // Mixed-path Jv: difference F(u + eps V) - F(u) formed without cancellation.
-template <typename T>
-cudaError_t launch_jv_diff(const Geo& G, const T* u, const T* v, T* out, double* part, Ctl* ctl,
+cudaError_t launch_jv_diff(const Geo& G, const float* u, const float* v, float* out, double* part, Ctl* ctl,
                            int check_done, cudaStream_t s);
 
 // Smagorinsky nu at every point of u, and its maximum into ctl->kmax.
@@ -45,8 +41,7 @@ size_t stencil3d_scratch_bytes(const Geo& G);
 template <typename T>
 cudaError_t launch_stencil3d(int mode, const Geo& G, const T* u, const T* v, const T* Fu, const double* f,
                              T* out, T* out2, double* part, Ctl* ctl, int check_done, cudaStream_t s);
-template <typename T>
-cudaError_t launch_jv_diff3d(const Geo& G, const T* u, const T* v, T* out, Ctl* ctl, int check_done,
+cudaError_t launch_jv_diff3d(const Geo& G, const float* u, const float* v, float* out, Ctl* ctl, int check_done,
                              cudaStream_t s);
 template <typename T>
 cudaError_t launch_eddy3d(const Geo& G, const T* u, T* nu, double* part, Ctl* ctl, cudaStream_t s);

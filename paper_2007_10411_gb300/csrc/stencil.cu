@@ -14,14 +14,12 @@
 //   * x periodic, z cell-centred with mirror ghosts (w odd, theta and p even,
 //     u even for free slip / odd for no slip); the eddy field is mirrored even.
 //
-// Tiling: one CTA computes a TX x TZ tile of output points.  Stage 1 stages
-// the four fields with a halo of 2r = 4 points in shared memory (periodic /
-// mirror index mapping, coalesced along x); stage 2 forms the first
-// derivatives of u, w, theta (and nu) on the tile plus a halo of r = 2;
-// stage 3 assembles the fluxes, the second application of D and the
-// point-wise terms, and writes coalesced rows.  Nothing but the inputs and
-// the outputs touches HBM: the eddy viscosity and the derivatives live only
-// in shared memory.
+// Tiling: one CTA computes a TX x TZ tile of output points.  The fields are
+// staged with a halo of 2r = 4 points in shared memory (periodic / mirror
+// index mapping, coalesced along x); every flux that D differentiates is
+// formed once at the points and on the arms it is read from, and then
+// differentiated.  Nothing but the inputs and the outputs touches HBM: the
+// eddy viscosity and the derivatives live only on the chip.
 #include <math.h>
 
 #include <algorithm>
@@ -35,15 +33,9 @@ namespace jfnk {
 constexpr int R = 2;          // derivative radius for p = 2
 constexpr int HALO = 2 * R;   // input halo (derivative applied twice)
 
-template <typename T> struct Tile;
-template <> struct Tile<double> { static constexpr int TX = 32, TZ = 16; };
-template <> struct Tile<float>  { static constexpr int TX = 64, TZ = 16; };
 // Candidate tiles of the Jacobian-product and preconditioner kernels (float32
 // path); jfnk_autotune times each on the handle's workload and keeps the
 // fastest (Geo::tile_jv, Geo::tile_pc).  The float64 path uses the first entry.
-template <int I> struct JvTile;          // float64 Jacobian product (jv_diff2d): entry 1
-template <> struct JvTile<0> { static constexpr int TX = 32, TZ = 16; };
-template <> struct JvTile<1> { static constexpr int TX = 32, TZ = 8; };
 template <int I> struct JvcTile;         // float32 Jacobian product (jvc2d): tile and staging buffers
 template <> struct JvcTile<0> { static constexpr int TX = 32, TZ = 16, NBUF = 1; };
 template <> struct JvcTile<1> { static constexpr int TX = 32, TZ = 16, NBUF = 2; };
@@ -68,21 +60,6 @@ __device__ __forceinline__ T dd(const T* s, int i, int st, T inv_h) {
     return rmul(rfma(T(2.0 / 3.0), d1, rmul(T(-1.0 / 12.0), d2)), inv_h);
 }
 
-// derivative of the point-wise product a*b
-template <typename T>
-__device__ __forceinline__ T ddp(const T* a, const T* b, int i, int st, T inv_h) {
-    const T d1 = rfma(a[i + st], b[i + st], -rmul(a[i - st], b[i - st]));
-    const T d2 = rfma(a[i + 2 * st], b[i + 2 * st], -rmul(a[i - 2 * st], b[i - 2 * st]));
-    return rmul(rfma(T(2.0 / 3.0), d1, rmul(T(-1.0 / 12.0), d2)), inv_h);
-}
-
-// derivative of the flux K*g where K may be a constant (Kc) or an array
-template <typename T, bool KARR>
-__device__ __forceinline__ T ddk(const T* K, T Kc, const T* g, int i, int st, T inv_h) {
-    if (KARR) return ddp(K, g, i, st, inv_h);
-    return Kc * dd(g, i, st, inv_h);
-}
-
 // Source row / sign of a ghost-extended z index.  side: 0 interior, 1 bottom, 2 top.
 __device__ __forceinline__ int mirror_z(int gz, int nz, int& side) {
     side = 0;
@@ -97,6 +74,16 @@ __device__ __forceinline__ int wrap_x(int gx, int nx) {
     return r < 0 ? r + nx : r;
 }
 
+// -x by the sign bit (an FP64 multiplication by -1, predicated off or not, costs the FP64 pipe)
+__device__ __forceinline__ float flip(float x) { return __int_as_float(__float_as_int(x) ^ 0x80000000); }
+__device__ __forceinline__ double flip(double x) {
+    return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
+}
+// Ghost row (side 1 bottom, 2 top) of a field that is odd at that wall.
+__device__ __forceinline__ bool odd_ghost(const Geo& G, int f, int side) {
+    return (side == 1 && G.pb[f] < 0) || (side == 2 && G.pt[f] < 0);
+}
+
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
     using type = float4;
@@ -106,6 +93,7 @@ template <> struct Vec16<float> {
         return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
     }
     __device__ static float4 mul(float a, float4 x) { return make_float4(a * x.x, a * x.y, a * x.z, a * x.w); }
+    __device__ static float4 neg(float4 x) { return make_float4(flip(x.x), flip(x.y), flip(x.z), flip(x.w)); }
 };
 template <> struct Vec16<double> {
     using type = double2;
@@ -115,6 +103,7 @@ template <> struct Vec16<double> {
         return make_double2(::fma(a, x.x, y.x), ::fma(a, x.y, y.y));
     }
     __device__ static double2 mul(double a, double2 x) { return make_double2(a * x.x, a * x.y); }
+    __device__ static double2 neg(double2 x) { return make_double2(flip(x.x), flip(x.y)); }
 };
 
 // True when the whole x-range [x0 - HALO, x0 - HALO + SX) of a tile is inside the
@@ -153,8 +142,7 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
                         val = Vec16<T>::fma(ev[f], *reinterpret_cast<const VT*>(v + o),
                                             *reinterpret_cast<const VT*>(u + o));
                     else val = Vec16<T>::mul(ev[f], *reinterpret_cast<const VT*>(v + o));
-                    if (side == 1) val = Vec16<T>::mul(T(G.pb[f]), val);
-                    else if (side == 2) val = Vec16<T>::mul(T(G.pt[f]), val);
+                    if (odd_ghost(G, f, side)) val = Vec16<T>::neg(val);
                 }
                 *reinterpret_cast<VT*>(s + (q * SZ + iz) * SX + c * VW) = val;
             }
@@ -179,56 +167,11 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
                 if (LOADMODE == 0) val = u[o];
                 else if (LOADMODE == 1) val = u[o] + ev[f] * v[o];
                 else val = ev[f] * v[o];
-                if (side == 1) val *= T(G.pb[f]);
-                else if (side == 2) val *= T(G.pt[f]);
+                if (odd_ghost(G, f, side)) val = flip(val);
             }
             s[(q * SZ + iz) * SX + ix] = val;
         }
     }
-}
-
-// Work item w of a QZ x QX halo region -> (qz, qx): the first 32 * (QX / 32)
-// columns of every row in 32-wide blocks (a warp stays inside one row, so its
-// shared-memory taps are consecutive words and free of bank conflicts), then
-// the remaining QX % 32 columns of all rows.
-__device__ __forceinline__ void halo_item(int w, int QX, int QZ, int& qz, int& qx) {
-    const int wide = QX & ~31, main = QZ * wide;
-    if (w < main) {
-        qz = w / wide;
-        qx = w - qz * wide;
-    } else {
-        const int rem = QX - wide, r = w - main;
-        qz = r / rem;
-        qx = wide + (r - qz * rem);
-    }
-}
-
-// Stage 2: first derivatives of u, w, theta on the halo-r region.
-template <typename T>
-__device__ __forceinline__ void first_derivs(const T* s1, T* d, int SX, int SZ, int QX, int QZ,
-                                             T idx_, T idz_) {
-    const int total = QX * QZ;
-    for (int w = threadIdx.x; w < total; w += blockDim.x) {
-        int qz, qx;
-        halo_item(w, QX, QZ, qz, qx);
-        const int idx = qz * QX + qx;
-        const int i1 = (qz + R) * SX + qx + R;
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            const T* sf = s1 + f * SZ * SX;
-            d[(2 * f) * total + idx] = dd(sf, i1, 1, idx_);
-            d[(2 * f + 1) * total + idx] = dd(sf, i1, SX, idz_);
-        }
-    }
-}
-
-// Row of the halo-r region whose eddy value a ghost row takes (even mirror); -1 if unused.
-__device__ __forceinline__ int eddy_row(int qz, int z0, int nz, int QZ) {
-    const int gz = z0 + qz - R;
-    int iq = qz;
-    if (gz < 0) iq = (-1 - gz) - z0 + R;
-    else if (gz >= nz) iq = (gz < nz + R) ? (2 * nz - 1 - gz) - z0 + R : -1;
-    return (iq >= 0 && iq < QZ) ? iq : -1;
 }
 
 // Deardorff heat factor s (1 + a l(s)), l = min(Delta, c_l s) (c_l < 0: l = Delta).
@@ -248,30 +191,180 @@ __device__ __forceinline__ T smag_nu(T ux, T uz, T wx, T wz, T cs2) {
 
 // ============================================================================
 // F, 2u/dt + F, residual and plain forward-difference Jv
+//
+// Compute-once tiles.  Every term of F that is differentiated along an axis
+// is one flux, formed once per point,
+//   X_phi = K D_x phi - 1/2 u phi,   Z_phi = K D_z phi - 1/2 w phi   (K = 0 for p),
+// so that F_phi = D_x X_phi + D_z Z_phi + S_phi with the point-wise part
+//   S_phi = -1/2 (u D_x phi + w D_z phi) + pressure gradient, buoyancy, ...
+// Phase 1 stages the four fields of a TX x TZ tile with a halo of 4; phase 2
+// forms both fluxes and S at the tile's points, X alone on two columns either
+// side and Z alone on two rows above and below (the arms); phase 3, one item
+// per point and field, differentiates the fluxes and writes the mode's output.
+//
+// Bound (float64): the FP64 pipe, 2 FMA per clock and SM, that is 64 cycles
+// per warp instruction and sub-partition, so only the number of FP64
+// operations counts: about 130 a point (32 first derivatives, 17 eddy
+// coefficient, 14 fluxes, 18 point-wise, 32 flux derivatives, 16 output and
+// norms) and 45 per arm point, against about 255 for the form that rebuilt
+// the products at every tap and formed all derivatives on the whole halo.
+// One F(u) at 1024 x 512, Smagorinsky: 236 -> 142 us; at 128 x 64: 31 -> 6 us.
 // ============================================================================
-template <typename T, int MODE, int SMAG>
-__global__ void __launch_bounds__(NTHREADS)
-stencil2d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
-          const double* __restrict__ f, T* __restrict__ out, T* __restrict__ out2,
-          double* __restrict__ part, Ctl* ctl, int check_done) {
-    constexpr int TX = Tile<T>::TX, TZ = Tile<T>::TZ;
-    constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO;
-    constexpr int QX = TX + 2 * R, QZ = TZ + 2 * R;
-    constexpr int QN = QX * QZ;
-    if (MODE == MODE_JV && check_done && ctl->done) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* s1 = reinterpret_cast<T*>(smem_raw);
-    T* d = s1 + 4 * SZ * SX;
-    T* nu = d + 6 * QN;                  // Smagorinsky nu, or the strain s (Deardorff)
-    T* gh = nu + QN;                     // Deardorff: s (1 + a_h l) and s (1 + a_z l)
-    T* gH = gh + QN;
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
+// The strain magnitude sqrt(2 S:S) from the velocity gradients.
+template <typename T>
+__device__ __forceinline__ T flux_strain(T ux, T uz, T wx, T wz) {
+    const T a = uz + wx;                            // 2 S:S = 2 (ux^2 + wz^2) + (uz + wx)^2
+    const T d = rfma(ux, ux, rmul(wz, wz));
+    return root(rfma(a, a, d + d));
+}
 
+// D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
+template <typename T>
+__device__ __forceinline__ T wd(const T* s, int i, int st, T w1, T w2) {
+    return rfma(w1, s[i + st] - s[i - st], rmul(w2, s[i + 2 * st] - s[i - 2 * st]));
+}
+
+struct FluxShape {
+    int lx, lz;                                     // TX = 1 << lx, TZ = 1 << lz
+    __host__ __device__ int tx() const { return 1 << lx; }
+    __host__ __device__ int tz() const { return 1 << lz; }
+    __host__ __device__ int cn() const { return 1 << (lx + lz); }
+    __host__ __device__ int sx() const { return tx() + 2 * HALO; }
+    __host__ __device__ int plane() const { return sx() * (tz() + 2 * HALO); }
+    __host__ __device__ int xn() const { return (tx() + 2 * R) * tz(); }       // X flux of one field
+    __host__ __device__ int zn() const { return tx() * (tz() + 2 * R); }       // Z flux of one field
+    __host__ __device__ int ppt() const { return cn() / NTHREADS; }            // 0: phase 3 per point and field
+    __host__ __device__ int elems() const { return 4 * (plane() + xn() + zn() + (ppt() ? 0 : cn())); }
+};
+
+// Tile row whose eddy value a flux point in tile row iz takes: its mirror
+// image in the two ghost rows next to a wall (K is mirrored even), else itself.
+__device__ __forceinline__ int flux_eddy_row(int iz, int z0, int nz) {
+    const int gz = z0 + iz;
+    if (gz < 0) return (-1 - gz) - z0;
+    if (gz >= nz) return (2 * nz - 1 - gz) - z0;
+    return iz;
+}
+
+// Phase 2 at one point.  i: staged index; is: staged index of the point whose
+// eddy coefficient it takes.  XF / ZF: form the X / Z fluxes; both: a tile
+// point, which also gets its point-wise part.
+template <typename T, int SMAG, bool XF, bool ZF>
+__device__ __forceinline__ void flux_point(const Geo& G, const FluxShape& sh, const T* __restrict__ s, int i, int is,
+                                           T* __restrict__ X, T* __restrict__ Z, T (&S)[4]) {
+    const int PL = sh.plane(), SX = sh.sx(), XN = sh.xn(), ZN = sh.zn();
+    const T wx1 = T(G.wx1), wx2 = T(G.wx2), wz1 = T(G.wz1), wz2 = T(G.wz2);
+    const T *U = s, *W = s + PL, *H = s + 2 * PL, *P = s + 3 * PL;
+    T ux = T(0), uz = T(0), wx = T(0), wz = T(0), tx = T(0), tz = T(0);
+    if (XF || SMAG) { ux = wd(U, i, 1, wx1, wx2); wx = wd(W, i, 1, wx1, wx2); }
+    if (ZF || SMAG) { uz = wd(U, i, SX, wz1, wz2); wz = wd(W, i, SX, wz1, wz2); }
+    if (XF) tx = wd(H, i, 1, wx1, wx2);
+    if (ZF) tz = wd(H, i, SX, wz1, wz2);
+    T kx = T(G.K_M), kz = T(G.K_M), kxh = T(G.K_H), kzh = T(G.K_H);
+    if (SMAG) {
+        const T st = is == i ? flux_strain(ux, uz, wx, wz)
+                             : flux_strain(wd(U, is, 1, wx1, wx2), wd(U, is, SX, wz1, wz2),
+                                           wd(W, is, 1, wx1, wx2), wd(W, is, SX, wz1, wz2));
+        if (SMAG == 2) {       // Deardorff: K_m along x, K_M along z, heat with its own factors
+            kx = rmul(T(G.dd_cm), st);
+            kz = rmul(T(G.dd_cM), st);
+            if (XF) kxh = rmul(T(G.dd_cm), dd_heat(st, T(G.dd_ah), G));
+            if (ZF) kzh = rmul(T(G.dd_cM), dd_heat(st, T(G.dd_az), G));
+        } else {
+            kx = kz = rmul(T(G.cs2), st);
+            kxh = kzh = rmul(kx, T(G.inv_Pr));
+        }
+    }
+    const T hu = rmul(T(0.5), U[i]), hw = rmul(T(0.5), W[i]);
+    if (XF) {
+        X[0] = rfma(kx, ux, -rmul(hu, U[i]));
+        X[XN] = rfma(kx, wx, -rmul(hu, W[i]));
+        X[2 * XN] = rfma(kxh, tx, -rmul(hu, H[i]));
+        X[3 * XN] = -rmul(hu, P[i]);
+    }
+    if (ZF) {
+        Z[0] = rfma(kz, uz, -rmul(hw, U[i]));
+        Z[ZN] = rfma(kz, wz, -rmul(hw, W[i]));
+        Z[2 * ZN] = rfma(kzh, tz, -rmul(hw, H[i]));
+        Z[3 * ZN] = -rmul(hw, P[i]);
+    }
+    if (XF && ZF) {
+        const T px = wd(P, i, 1, wx1, wx2), pz = wd(P, i, SX, wz1, wz2);
+        const T th0 = T(G.theta0);
+        S[0] = rfma(-hu, ux, rfma(-hw, uz, -rmul(th0, px)));
+        S[1] = rfma(-hu, wx, rfma(-hw, wz, rfma(T(G.gth), H[i], -rmul(th0, pz))));
+        S[2] = rfma(-hu, tx, rfma(-hw, tz, -rmul(T(G.beta), W[i])));
+        S[3] = rfma(-hu, px, rfma(-hw, pz, -rmul(rmul(T(G.gamma_p), T(G.pbar) + P[i]), ux + wz)));
+    }
+}
+
+// Derivative of the fluxes of field fl at tile point (tx, tz) plus S.
+template <typename T>
+__device__ __forceinline__ T flux_div(const Geo& G, const FluxShape& sh, const T* X, const T* Z, int fl, int tz, int tx,
+                                      T S) {
+    const int PXW = sh.tx() + 2 * R, TX = sh.tx();
+    const T* x = X + fl * sh.xn() + tz * PXW + tx + R;
+    const T* z = Z + fl * sh.zn() + (tz + R) * TX + tx;
+    return rfma(T(G.wx1), x[1] - x[-1],
+                rfma(T(G.wx2), x[2] - x[-2],
+                     rfma(T(G.wz1), z[TX] - z[-TX], rfma(T(G.wz2), z[2 * TX] - z[-2 * TX], S))));
+}
+
+// The mode's output at point o of field fl from F (ar, au: sums of R^2 and u^2
+// of the field in its own units).
+template <typename T>
+__device__ __forceinline__ void flux_out(const Geo& G, int mode, int fl, T Fv, double uo, size_t o,
+                                         const T* __restrict__ v, const T* __restrict__ Fu,
+                                         const double* __restrict__ f, T* __restrict__ out, T* __restrict__ out2,
+                                         double cf, double& ar, double& au) {
+    const double Fd = (double)Fv;
+    if (mode == MODE_F) {
+        out[o] = Fv;
+    } else if (mode == MODE_JV) {   // w_hat = 2 v_hat/dt - (F(u + eps V) - F(u)) / (eps scale)
+        const double diff = Fd - (double)Fu[o];
+        out[o] = T(G.two_over_dt * (double)v[o] - diff * cf);
+    } else if (mode == MODE_RHS) {
+        out[o] = T(G.two_over_dt * uo + Fd);
+    } else {
+        double Rv;
+        if (mode == MODE_RHSRES) {
+            // at u = u^n the residual 2u/dt - F(u) - f with f = 2u/dt + F(u) is -2 F(u)
+            out[o] = T(G.two_over_dt * uo + Fd);
+            Rv = -2.0 * Fd;
+            out2[o] = T(Rv);
+        } else {
+            Rv = G.two_over_dt * uo - Fd - f[o];
+            out[o] = T(Rv);
+            if (out2 != nullptr) out2[o] = Fv;
+        }
+        ar = fma(Rv, Rv, ar);
+        au = fma(uo, uo, au);
+    }
+}
+
+// PPT > 0: TX * TZ = PPT * NTHREADS; a thread keeps the point-wise parts of its
+// PPT points in registers and finishes them itself.  PPT = 0 (tiles of fewer
+// points than threads): the point-wise parts go through shared memory and phase
+// 3 runs one item per point and field, which spreads a small tile over the
+// sub-partitions' FP64 pipes.
+template <typename T, int SMAG, int PPT>
+__global__ void __launch_bounds__(NTHREADS)
+flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
+       const double* __restrict__ f, T* __restrict__ out, T* __restrict__ out2, double* __restrict__ part, Ctl* ctl,
+       int check_done) {
+    pdl_wait();
+    if (mode == MODE_JV && check_done && ctl->done) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int TX = sh.tx(), TZ = sh.tz(), CN = sh.cn(), SX = sh.sx(), PXW = TX + 2 * R;
+    T* s1 = reinterpret_cast<T*>(smem_raw);         // [4][SZ][SX]
+    T* X = s1 + 4 * sh.plane();                     // [4][TZ][TX + 4]
+    T* Z = X + 4 * sh.xn();                         // [4][TZ + 4][TX]
+    T* Ss = Z + 4 * sh.zn();                        // [4][TZ][TX] (PPT = 0)
+    const int x0 = blockIdx.x << sh.lx, z0 = blockIdx.y << sh.lz;
     T ev[4] = {T(0), T(0), T(0), T(0)};
-    __shared__ double cfs[4];            // 1 / (eps scale_f), computed once per block
-    __shared__ T evs[4];                 // eps scale_f
-    if (MODE == MODE_JV) {
+    __shared__ double cfs[4];                       // 1 / (eps scale_f), computed once per block
+    __shared__ T evs[4];                            // eps scale_f
+    if (mode == MODE_JV) {
         if (threadIdx.x < 4) {
             const double e = ctl->eps_jv * G.scale[threadIdx.x];
             evs[threadIdx.x] = T(e);
@@ -280,123 +373,74 @@ stencil2d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __re
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < 4; ++q) ev[q] = evs[q];
-        load_fields<T, 1>(s1, u, v, ev, G, x0, z0, SX, SZ);
+        load_fields<T, 1>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
     } else {
-        load_fields<T, 0>(s1, u, v, ev, G, x0, z0, SX, SZ);
+        load_fields<T, 0>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
     }
     __syncthreads();
-    first_derivs(s1, d, SX, SZ, QX, QZ, idx_, idz_);
-    __syncthreads();
-    if (SMAG) {
-        const T cs2 = SMAG == 2 ? T(1) : T(G.cs2);     // Deardorff: the strain s = sqrt(2 S:S) itself
-        for (int w = threadIdx.x; w < QN; w += blockDim.x) {
-            int qz, qx;
-            halo_item(w, QX, QZ, qz, qx);
-            const int idx = qz * QX + qx;
-            const int iq = eddy_row(qz, z0, G.nz, QZ);
-            T val = T(0);
-            if (iq >= 0) {
-                const int q = iq * QX + qx;
-                val = smag_nu(d[q], d[QN + q], d[2 * QN + q], d[3 * QN + q], cs2);
-            }
-            nu[idx] = val;
-            if (SMAG == 2) {
-                gh[idx] = dd_heat(val, T(G.dd_ah), G);
-                gH[idx] = dd_heat(val, T(G.dd_az), G);
-            }
-        }
-        __syncthreads();
+    T S[PPT > 0 ? PPT : 1][4];
+    auto point = [&](int w, T (&Sw)[4]) {           // a tile point
+        const int iz = w >> sh.lx, ix = w & (TX - 1);
+        if (z0 + iz > G.nz + 1 || x0 + ix > G.nx + 1) return;        // feeds no output
+        const int i = (iz + HALO) * SX + ix + HALO;
+        const int is = SMAG ? (flux_eddy_row(iz, z0, G.nz) + HALO) * SX + ix + HALO : i;
+        flux_point<T, SMAG, true, true>(G, sh, s1, i, is, X + iz * PXW + ix + R, Z + (iz + R) * TX + ix, Sw);
+    };
+    if (PPT > 0) {
+#pragma unroll
+        for (int k = 0; k < PPT; ++k) point(threadIdx.x + k * NTHREADS, S[k]);
+    } else if (threadIdx.x < CN) {
+        point(threadIdx.x, S[0]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) Ss[q * CN + threadIdx.x] = S[0][q];
     }
-
-    const T* su = s1;
-    const T* sw = s1 + SZ * SX;
-    const T* st = s1 + 2 * SZ * SX;
-    const T* sp = s1 + 3 * SZ * SX;
-    const T* dux = d;
-    const T* duz = d + QN;
-    const T* dwx = d + 2 * QN;
-    const T* dwz = d + 3 * QN;
-    const T* dtx = d + 4 * QN;
-    const T* dtz = d + 5 * QN;
-    const T KMc = T(G.K_M), KHc = T(G.K_H), iPr = T(G.inv_Pr);
-    const T th0 = T(G.theta0);
-
+    // the arms; a small tile gives them to the warps that have no tile point
+    for (int a = PPT > 0 ? threadIdx.x : (threadIdx.x + NTHREADS - CN) % NTHREADS; a < 4 * (TX + TZ); a += NTHREADS) {
+        const bool zarm = a < 4 * TX;
+        const int b = a - 4 * TX, r = zarm ? a >> sh.lx : b & 3;
+        const int ix = zarm ? a & (TX - 1) : (r < 2 ? r - 2 : TX + r - 2);
+        const int iz = zarm ? (r < 2 ? r - 2 : TZ + r - 2) : b >> 2;
+        if (z0 + iz > G.nz + 1 || x0 + ix > G.nx + 1) continue;
+        const int i = (iz + HALO) * SX + ix + HALO;
+        const int is = SMAG ? (flux_eddy_row(iz, z0, G.nz) + HALO) * SX + ix + HALO : i;
+        T none[4];
+        if (zarm) flux_point<T, SMAG, false, true>(G, sh, s1, i, is, X, Z + (iz + R) * TX + ix, none);
+        else flux_point<T, SMAG, true, false>(G, sh, s1, i, is, X + iz * PXW + ix + R, Z, none);
+    }
+    __syncthreads();
     double acc[2] = {0.0, 0.0};
-    for (int idx = threadIdx.x; idx < TX * TZ; idx += blockDim.x) {
-        const int tz = idx / TX, tx = idx - tz * TX;
+    auto finish = [&](int fl, int pt, T Sv, double& ar, double& au) {
+        const int tz = pt >> sh.lx, tx = pt & (TX - 1);
         const int gz = z0 + tz, gx = x0 + tx;
-        if (gz >= G.nz || gx >= G.nx) continue;
-        const int i1 = (tz + HALO) * SX + tx + HALO;
-        const int q = (tz + R) * QX + tx + R;
-        const T uc = su[i1], wc = sw[i1], tc = st[i1], pc = sp[i1];
-        const T px = dd(sp, i1, 1, idx_), pz = dd(sp, i1, SX, idz_);
-        // skew-symmetric convection of every field
-        const T cu = T(0.5) * (ddp(su, su, i1, 1, idx_) + ddp(sw, su, i1, SX, idz_)) +
-                     T(0.5) * (uc * dux[q] + wc * duz[q]);
-        const T cw = T(0.5) * (ddp(su, sw, i1, 1, idx_) + ddp(sw, sw, i1, SX, idz_)) +
-                     T(0.5) * (uc * dwx[q] + wc * dwz[q]);
-        const T ct = T(0.5) * (ddp(su, st, i1, 1, idx_) + ddp(sw, st, i1, SX, idz_)) +
-                     T(0.5) * (uc * dtx[q] + wc * dtz[q]);
-        const T cp = T(0.5) * (ddp(su, sp, i1, 1, idx_) + ddp(sw, sp, i1, SX, idz_)) +
-                     T(0.5) * (uc * px + wc * pz);
-        // eddy diffusion sum_j D_j(K D_j phi)
-        T du, dw, dt_;
-        if (SMAG == 2) {
-            // anisotropic: D_x(K_m D_x phi) + D_z(K_M D_z phi), heat with K_h, K_H
-            const T cm = T(G.dd_cm), cM = T(G.dd_cM);
-            du = cm * ddp(nu, dux, q, 1, idx_) + cM * ddp(nu, duz, q, QX, idz_);
-            dw = cm * ddp(nu, dwx, q, 1, idx_) + cM * ddp(nu, dwz, q, QX, idz_);
-            dt_ = cm * ddp(gh, dtx, q, 1, idx_) + cM * ddp(gH, dtz, q, QX, idz_);
-        } else if (SMAG) {
-            du = ddp(nu, dux, q, 1, idx_) + ddp(nu, duz, q, QX, idz_);
-            dw = ddp(nu, dwx, q, 1, idx_) + ddp(nu, dwz, q, QX, idz_);
-            dt_ = iPr * (ddp(nu, dtx, q, 1, idx_) + ddp(nu, dtz, q, QX, idz_));
-        } else {
-            du = KMc * (dd(dux, q, 1, idx_) + dd(duz, q, QX, idz_));
-            dw = KMc * (dd(dwx, q, 1, idx_) + dd(dwz, q, QX, idz_));
-            dt_ = KHc * (dd(dtx, q, 1, idx_) + dd(dtz, q, QX, idz_));
-        }
-        T Fv[4];
-        Fv[0] = -cu - th0 * px + du;
-        Fv[1] = -cw - th0 * pz + dw + T(G.g) * tc / th0;
-        Fv[2] = -ct - T(G.beta) * wc + dt_;
-        if (G.heat != nullptr && gz == 0) Fv[2] += T(G.heat[gx] * G.heat_coef);
-        Fv[3] = -cp - T(G.gamma_p) * (T(G.pbar) + pc) * (dux[q] + dwz[q]);
-
-        const size_t off = (size_t)gz * G.nx + gx;
+        if (gz >= G.nz || gx >= G.nx) return;
+        T Fv = flux_div(G, sh, X, Z, fl, tz, tx, Sv);
+        if (fl == 2 && gz == 0 && G.heat != nullptr) Fv += T(G.heat[gx] * G.heat_coef);
+        const double uo = (double)s1[fl * sh.plane() + (tz + HALO) * SX + tx + HALO];
+        flux_out(G, mode, fl, Fv, uo, (size_t)fl * G.npt + (size_t)gz * G.nx + gx, v, Fu, f, out, out2,
+                 mode == MODE_JV ? cfs[fl] : 0.0, ar, au);
+    };
+    if (PPT > 0) {
 #pragma unroll
         for (int fl = 0; fl < 4; ++fl) {
-            const size_t o = (size_t)fl * G.npt + off;
-            if (MODE == MODE_F) {
-                out[o] = Fv[fl];
-            } else if (MODE == MODE_RHS) {
-                out[o] = T(G.two_over_dt * (double)u[o] + (double)Fv[fl]);
-            } else if (MODE == MODE_RHSRES) {
-                // at u = u^n the residual 2u/dt - F(u) - f with f = 2u/dt + F(u) is -2 F(u)
-                const double uo = (double)u[o];
-                const double Fd = (double)Fv[fl];
-                out[o] = T(G.two_over_dt * uo + Fd);
-                const double Rv = -2.0 * Fd;
-                out2[o] = T(Rv);
-                const double rs = Rv * G.inv_scale[fl], us = uo * G.inv_scale[fl];
-                acc[0] += rs * rs;
-                acc[1] += us * us;
-            } else if (MODE == MODE_RES) {
-                const double uo = (double)u[o];
-                const double Rv = G.two_over_dt * uo - (double)Fv[fl] - f[o];
-                out[o] = T(Rv);
-                if (out2 != nullptr) out2[o] = Fv[fl];
-                const double rs = Rv * G.inv_scale[fl], us = uo * G.inv_scale[fl];
-                acc[0] += rs * rs;
-                acc[1] += us * us;
-            } else {  // MODE_JV: w_hat = 2 v_hat/dt - (F(u + eps V) - F(u)) / (eps scale)
-                const double vh = (double)v[o];
-                const double diff = (double)Fv[fl] - (double)Fu[o];
-                out[o] = T(G.two_over_dt * vh - diff * cfs[fl]);
-            }
+            double ar = 0.0, au = 0.0;
+#pragma unroll
+            for (int k = 0; k < PPT; ++k) finish(fl, threadIdx.x + k * NTHREADS, S[k][fl], ar, au);
+            const double i2 = G.inv_scale[fl] * G.inv_scale[fl];
+            acc[0] = fma(ar, i2, acc[0]);
+            acc[1] = fma(au, i2, acc[1]);
+        }
+    } else {
+        for (int w = threadIdx.x; w < 4 * CN; w += NTHREADS) {
+            const int fl = w >> (sh.lx + sh.lz), pt = w & (CN - 1);
+            double ar = 0.0, au = 0.0;
+            finish(fl, pt, Ss[w], ar, au);
+            const double i2 = G.inv_scale[fl] * G.inv_scale[fl];
+            acc[0] = fma(ar, i2, acc[0]);
+            acc[1] = fma(au, i2, acc[1]);
         }
     }
-    if (MODE == MODE_RES || MODE == MODE_RHSRES) {
+    pdl_trigger();
+    if (mode == MODE_RES || mode == MODE_RHSRES) {
         const int nblk = gridDim.x * gridDim.y;
         const int blk = blockIdx.y * gridDim.x + blockIdx.x;
         block_partials<2>(acc, 2, part, nblk, blk);
@@ -473,246 +517,6 @@ __device__ __forceinline__ void jv_stage_issue(T* s, const T* __restrict__ u, co
             cpa_elem<sizeof(T)>(d + f * plane, u + (size_t)f * G.npt + off, ok ? (int)sizeof(T) : 0);
             cpa_elem<sizeof(T)>(d + (4 + f) * plane, v + (size_t)f * G.npt + off, ok ? (int)sizeof(T) : 0);
         }
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void jv_stage_fix(T* s, const T (&ev)[4], const Geo& G, int x0, int z0, int SX,
-                                             int SZ) {
-    using VT = typename Vec16<T>::type;
-    constexpr int VW = Vec16<T>::W;
-    const int plane = SZ * SX;
-    const bool vec = rows_vectorisable<T>(G, x0, SX);
-    const int per = vec ? SX / VW : SX;
-    const int total = per * SZ;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int iz = idx / per, c = idx - iz * per;
-        int side;
-        const int sz = mirror_z(z0 + iz - HALO, G.nz, side);
-        if (sz < 0 || sz >= G.nz) continue;       // zero-filled row
-        T* d = s + iz * SX + (vec ? c * VW : c);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            const T sg = side == 1 ? T(G.pb[f]) : side == 2 ? T(G.pt[f]) : T(1);
-            if (vec) {
-                VT* pu = reinterpret_cast<VT*>(d + f * plane);
-                VT* pv = reinterpret_cast<VT*>(d + (4 + f) * plane);
-                if (side) *pu = Vec16<T>::mul(sg, *pu);
-                VT b = Vec16<T>::mul(ev[f], *pv);
-                if (side) b = Vec16<T>::mul(sg, b);
-                *pv = b;
-            } else {
-                if (side) d[f * plane] *= sg;
-                T b = ev[f] * d[(4 + f) * plane];
-                if (side) b *= sg;
-                d[(4 + f) * plane] = b;
-            }
-        }
-    }
-}
-
-// ============================================================================
-// Mixed-path Jv: the forward difference F(u + eps V) - F(u) with every term
-// expanded as a difference (a = u, b = eps V, a' = a + b), e.g.
-//   a'_j phi' - a_j phi = a_j b_phi + b_j phi',
-//   (pbar + p') div a' - (pbar + p) div a = (pbar + p') div b + b_p div a,
-//   nu(a') - nu(a) = (Cs Delta)^2 2 (S':S' - S:S) / (sqrt(2 S':S') + sqrt(2 S:S)),
-// so the float32 result carries float32 relative accuracy on the difference
-// itself instead of on F.  Same quantity as the forward difference of Eq. fd.
-// ============================================================================
-//
-// Persistent and pipelined (NBUF = 2): a CTA walks the tiles t = blockIdx.x,
-// blockIdx.x + gridDim.x, ...; the cp.async copies of tile t + gridDim.x go
-// into the second staging buffer while tile t is computed, so the staging
-// latency hides behind the derivative and flux stages.  NBUF = 1 stages each
-// tile before computing it (one tile per CTA, the float64 path).
-template <typename T, int SMAG, int TX, int TZ, int NBUF>
-__global__ void __launch_bounds__(NTHREADS)
-jv_diff2d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict__ out,
-          const double* part, Ctl* ctl, int check_done) {
-    constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO;
-    constexpr int QX = TX + 2 * R, QZ = TZ + 2 * R;
-    constexpr int QN = QX * QZ;
-    constexpr int STG = 8 * SZ * SX;
-    pdl_wait();
-    if (check_done && ctl->done) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* stg = reinterpret_cast<T*>(smem_raw);
-    T* da = stg + NBUF * STG;
-    T* db = da + 6 * QN;
-    T* Ka = db + 6 * QN;
-    T* dK = Ka + QN;
-    const int ntx = (G.nx + TX - 1) / TX;
-    const int ntiles = ntx * ((G.nz + TZ - 1) / TZ);
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
-    int t = blockIdx.x;
-    if (t < ntiles) jv_stage_issue(stg, u, v, G, (t % ntx) * TX, (t / ntx) * TZ, SX, SZ);
-    cpa_commit();
-    // the step, while the first tile's copies are in flight
-    const double eps = pending_eps(ctl, part);
-    __shared__ T cfs[4];                 // 1 / (eps scale_f), computed once per block
-    __shared__ T evs[4];                 // eps scale_f
-    if (threadIdx.x < 4) {
-        const double e = eps * G.scale[threadIdx.x];
-        evs[threadIdx.x] = T(e);
-        cfs[threadIdx.x] = T(e != 0.0 ? 1.0 / e : 0.0);
-    }
-    __syncthreads();
-    T ev[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) ev[q] = evs[q];
-    for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
-    const int x0 = (t % ntx) * TX, z0 = (t / ntx) * TZ;
-    T* sa = stg + (NBUF == 2 ? (it & 1) * STG : 0);
-    T* sb = sa + 4 * SZ * SX;
-    // the direction at this thread's outputs (consumed at the end of the tile)
-    constexpr int NOUT = (TX * TZ + NTHREADS - 1) / NTHREADS;
-    T vout[NOUT][4];
-#pragma unroll
-    for (int q = 0; q < NOUT; ++q) {
-        const int idx = threadIdx.x + q * NTHREADS;
-        const int tz = idx / TX, tx = idx - tz * TX;
-        const int gz = z0 + tz, gx = x0 + tx;
-        const bool ok = idx < TX * TZ && gz < G.nz && gx < G.nx;
-#pragma unroll
-        for (int fl = 0; fl < 4; ++fl)
-            vout[q][fl] = ok ? v[(size_t)fl * G.npt + (size_t)gz * G.nx + gx] : T(0);
-    }
-    if (NBUF == 2) {
-        const int tn = t + gridDim.x;
-        if (tn < ntiles)
-            jv_stage_issue(stg + ((it + 1) & 1) * STG, u, v, G, (tn % ntx) * TX, (tn / ntx) * TZ, SX, SZ);
-        cpa_commit();
-        cpa_wait<1>();
-    } else {
-        cpa_wait<0>();
-    }
-    jv_stage_fix(sa, ev, G, x0, z0, SX, SZ);
-    __syncthreads();
-    first_derivs(sa, da, SX, SZ, QX, QZ, idx_, idz_);
-    first_derivs(sb, db, SX, SZ, QX, QZ, idx_, idz_);
-    __syncthreads();
-    if (SMAG) {
-        const T cs2 = T(G.cs2);
-        for (int w = threadIdx.x; w < QN; w += blockDim.x) {
-            int qz, qx;
-            halo_item(w, QX, QZ, qz, qx);
-            const int idx = qz * QX + qx;
-            const int iq = eddy_row(qz, z0, G.nz, QZ);
-            T ka = T(0), dk = T(0);
-            if (iq >= 0) {
-                const int q = iq * QX + qx;
-                const T aux = da[q], auz = da[QN + q], awx = da[2 * QN + q], awz = da[3 * QN + q];
-                const T bux = db[q], buz = db[QN + q], bwx = db[2 * QN + q], bwz = db[3 * QN + q];
-                const T a13 = T(0.5) * (auz + awx), b13 = T(0.5) * (buz + bwx);
-                const T ssa = aux * aux + awz * awz + T(2) * a13 * a13;
-                // S':S' - S:S = (2 S + S_b) : S_b
-                const T dss = (T(2) * aux + bux) * bux + (T(2) * awz + bwz) * bwz +
-                              T(2) * (T(2) * a13 + b13) * b13;
-                const T na = sqrt(T(2) * ssa);
-                const T np = sqrt(T(2) * (ssa + dss) > T(0) ? T(2) * (ssa + dss) : T(0));
-                ka = cs2 * na;
-                const T den = na + np;
-                dk = den > T(0) ? cs2 * T(2) * dss / den : T(0);
-            }
-            Ka[idx] = ka;
-            dK[idx] = dk;
-        }
-        __syncthreads();
-    }
-    const T* au = sa; const T* aw = sa + SZ * SX; const T* at = sa + 2 * SZ * SX; const T* ap = sa + 3 * SZ * SX;
-    const T* bu = sb; const T* bw = sb + SZ * SX; const T* bt = sb + 2 * SZ * SX; const T* bp = sb + 3 * SZ * SX;
-    const T KMc = T(G.K_M), KHc = T(G.K_H), iPr = T(G.inv_Pr), th0 = T(G.theta0);
-
-#pragma unroll
-    for (int qo = 0; qo < NOUT; ++qo) {
-        const int idx = threadIdx.x + qo * NTHREADS;
-        if (idx >= TX * TZ) break;
-        const int tz = idx / TX, tx = idx - tz * TX;
-        const int gz = z0 + tz, gx = x0 + tx;
-        if (gz >= G.nz || gx >= G.nx) continue;
-        const int i1 = (tz + HALO) * SX + tx + HALO;
-        const int q = (tz + R) * QX + tx + R;
-        const T auc = au[i1], awc = aw[i1], apc = ap[i1];
-        const T buc = bu[i1], bwc = bw[i1], btc = bt[i1], bpc = bp[i1];
-        const T apx = dd(ap, i1, 1, idx_), apz = dd(ap, i1, SX, idz_);
-        const T bpx = dd(bp, i1, 1, idx_), bpz = dd(bp, i1, SX, idz_);
-        T dF[4];
-        // convection differences: 1/2 D_j(a_j b_phi + b_j phi') + 1/2 (a_j D b_phi + b_j D phi')
-        const T* as[4] = {au, aw, at, ap};
-        const T* bs[4] = {bu, bw, bt, bp};
-#pragma unroll
-        for (int fl = 0; fl < 4; ++fl) {
-            const T* A = as[fl];
-            const T* B = bs[fl];
-            T fx = T(0), fz = T(0);
-#pragma unroll
-            for (int l = 1; l <= 2; ++l) {
-                const T c = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                const int ip = i1 + l, im = i1 - l;
-                const int kp = i1 + l * SX, km = i1 - l * SX;
-                fx += c * ((au[ip] * B[ip] + bu[ip] * (A[ip] + B[ip])) -
-                           (au[im] * B[im] + bu[im] * (A[im] + B[im])));
-                fz += c * ((aw[kp] * B[kp] + bw[kp] * (A[kp] + B[kp])) -
-                           (aw[km] * B[km] + bw[km] * (A[km] + B[km])));
-            }
-            T dax, daz, dbx, dbz;
-            if (fl < 3) {
-                dax = da[(2 * fl) * QN + q]; daz = da[(2 * fl + 1) * QN + q];
-                dbx = db[(2 * fl) * QN + q]; dbz = db[(2 * fl + 1) * QN + q];
-            } else {
-                dax = apx; daz = apz; dbx = bpx; dbz = bpz;
-            }
-            const T adv = auc * dbx + awc * dbz + buc * (dax + dbx) + bwc * (daz + dbz);
-            dF[fl] = -(T(0.5) * (fx * idx_ + fz * idz_) + T(0.5) * adv);
-        }
-        // diffusion differences: D_j(K_a D_j b_phi + dK D_j phi')
-#pragma unroll
-        for (int fl = 0; fl < 3; ++fl) {
-            const T* dax = da + (2 * fl) * QN; const T* daz = da + (2 * fl + 1) * QN;
-            const T* dbx = db + (2 * fl) * QN; const T* dbz = db + (2 * fl + 1) * QN;
-            T sx = T(0), sz = T(0);
-            const T kc = fl == 2 ? KHc : KMc;
-#pragma unroll
-            for (int l = 1; l <= 2; ++l) {
-                const T c = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                const int xp = q + l, xm = q - l, zp = q + l * QX, zm = q - l * QX;
-                if (SMAG) {
-                    sx += c * ((Ka[xp] * dbx[xp] + dK[xp] * (dax[xp] + dbx[xp])) -
-                               (Ka[xm] * dbx[xm] + dK[xm] * (dax[xm] + dbx[xm])));
-                    sz += c * ((Ka[zp] * dbz[zp] + dK[zp] * (daz[zp] + dbz[zp])) -
-                               (Ka[zm] * dbz[zm] + dK[zm] * (daz[zm] + dbz[zm])));
-                } else {
-                    sx += c * (dbx[xp] - dbx[xm]);
-                    sz += c * (dbz[zp] - dbz[zm]);
-                }
-            }
-            T dif = sx * idx_ + sz * idz_;
-            if (SMAG) { if (fl == 2) dif *= iPr; } else dif *= kc;
-            dF[fl] += dif;
-        }
-        dF[0] += -th0 * bpx;
-        dF[1] += -th0 * bpz + T(G.g) * btc / th0;
-        dF[2] += -T(G.beta) * bwc;
-        const T diva = da[q] + da[3 * QN + q];
-        const T divb = db[q] + db[3 * QN + q];
-        dF[3] += -T(G.gamma_p) * ((T(G.pbar) + apc + bpc) * divb + bpc * diva);
-
-        const size_t off = (size_t)gz * G.nx + gx;
-#pragma unroll
-        for (int fl = 0; fl < 4; ++fl) {
-            const size_t o = (size_t)fl * G.npt + off;
-            // the difference dF is already free of cancellation: the quotient
-            // and the 2 v/dt term need no wider type than the result
-            out[o] = T(G.two_over_dt) * vout[qo][fl] - dF[fl] * cfs[fl];
-        }
-    }
-    __syncthreads();     // staging buffer and derivative arrays are reused by the next tile
-    if (NBUF == 1) {
-        const int tn = t + gridDim.x;
-        if (tn < ntiles) jv_stage_issue(stg, u, v, G, (tn % ntx) * TX, (tn / ntx) * TZ, SX, SZ);
-        cpa_commit();
-    }
     }
 }
 
@@ -1704,43 +1508,66 @@ budgets2d(Geo G, const double* __restrict__ u, double dV, double dz, double lz, 
 // ============================================================================
 // launchers
 // ============================================================================
-template <typename T> int stencil_blocks(const Geo& G) {
-    return ((G.nx + Tile<T>::TX - 1) / Tile<T>::TX) * ((G.nz + Tile<T>::TZ - 1) / Tile<T>::TZ);
-}
-template int stencil_blocks<float>(const Geo&);
-template int stencil_blocks<double>(const Geo&);
-
-template <typename T, int SMAG>
-static size_t stencil_smem() {
-    constexpr int TX = Tile<T>::TX, TZ = Tile<T>::TZ;
-    constexpr int NQ = SMAG == 2 ? 9 : 7;        // derivatives (6) + eddy field(s)
-    return sizeof(T) * (4 * (TZ + 2 * HALO) * (TX + 2 * HALO) + NQ * (TX + 2 * R) * (TZ + 2 * R));
-}
-
-template <typename T, int TX, int TZ, int NBUF>
-static size_t jvd_smem() {
-    return sizeof(T) * (NBUF * 8 * (TZ + 2 * HALO) * (TX + 2 * HALO) + 14 * (TX + 2 * R) * (TZ + 2 * R));
-}
-
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <typename T, int MODE, int SMAG>
-static cudaError_t launch_stencil_t(const Geo& G, const T* u, const T* v, const T* Fu,
-                                    const double* f, T* out, T* out2, double* part, Ctl* ctl,
-                                    int check_done, cudaStream_t s) {
+// Tile of flux2d for a grid: the shape with the least FP64 time, counted in
+// operations per sub-partition: phase 2 (81 a tile point, 45 an arm point, no
+// less than one warp's 81) and phase 3 (12 a point and field), times the
+// rounds of tiles over the SMs.  Large grids take 32 x 16 (arms 14 % of the
+// work); where 32 x 16 leaves SMs idle (128 x 64: 16 tiles for 152 SMs) the
+// smallest tile that still fits one round spreads the points over all of them.
+// F(u) per tile 8x8 / 16x8 / 16x16 / 32x16: 8 / 12 / 16 / 27 us at 128 x 64,
+// 18 / 16 / 16 / 27 at 250 x 119, - / - / 152 / 142 at 1024 x 512.
+static FluxShape flux_shape(const Geo& G) {
+    constexpr int SMS = 152;
+    constexpr FluxShape cand[] = {{3, 3}, {4, 3}, {4, 4}, {5, 4}};
+    FluxShape best = cand[3];
+    double least = 1e300;
+    for (const FluxShape& c : cand) {
+        const long long tiles = (long long)((G.nx + c.tx() - 1) >> c.lx) * ((G.nz + c.tz() - 1) >> c.lz);
+        const double cw = c.cn() / 32.0, aw = 4.0 * (c.tx() + c.tz()) / 32.0;
+        const double cost = (double)((tiles + SMS - 1) / SMS) *
+                            (std::max(81.0, (81.0 * cw + 45.0 * aw) / 4.0) + std::max(12.0, 12.0 * cw));
+        if (cost <= least) {      // on a tie the larger tile: fewer arm points
+            if (cost < least || tiles > 2 * SMS) best = c;
+            least = cost;
+        }
+    }
+    return best;
+}
+
+template <typename T, int SMAG, int PPT>
+static cudaError_t launch_flux_t(const FluxShape& sh, int mode, const Geo& G, const T* u, const T* v, const T* Fu,
+                                 const double* f, T* out, T* out2, double* part, Ctl* ctl, int check_done,
+                                 cudaStream_t s) {
     static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
-    const size_t sm = stencil_smem<T, SMAG>();
     if (!configured) {
-        cudaError_t e = set_smem(stencil2d<T, MODE, SMAG>, sm);
+        const FluxShape big{5, 4};
+        cudaError_t e = set_smem(flux2d<T, SMAG, PPT>, big.elems() * sizeof(T));
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    dim3 grid((G.nx + Tile<T>::TX - 1) / Tile<T>::TX, (G.nz + Tile<T>::TZ - 1) / Tile<T>::TZ);
-    stencil2d<T, MODE, SMAG><<<grid, NTHREADS, sm, s>>>(G, u, v, Fu, f, out, out2, part, ctl, check_done);
+    const size_t sm = sh.elems() * sizeof(T);
+    dim3 grid((G.nx + sh.tx() - 1) >> sh.lx, (G.nz + sh.tz() - 1) >> sh.lz);
+    if (mode == MODE_JV)
+        return launch_pdl(flux2d<T, SMAG, PPT>, grid, NTHREADS, sm, s, G, mode, sh, u, v, Fu, f, out, out2, part, ctl,
+                          check_done);
+    flux2d<T, SMAG, PPT><<<grid, NTHREADS, sm, s>>>(G, mode, sh, u, v, Fu, f, out, out2, part, ctl, check_done);
     return cudaGetLastError();
+}
+
+template <typename T, int SMAG>
+static cudaError_t launch_flux(int mode, const Geo& G, const T* u, const T* v, const T* Fu, const double* f, T* out,
+                               T* out2, double* part, Ctl* ctl, int check_done, cudaStream_t s) {
+    const FluxShape sh = flux_shape(G);
+    switch (sh.ppt()) {
+        case 2: return launch_flux_t<T, SMAG, 2>(sh, mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+        case 1: return launch_flux_t<T, SMAG, 1>(sh, mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+        default: return launch_flux_t<T, SMAG, 0>(sh, mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+    }
 }
 
 template <typename T>
@@ -1748,50 +1575,15 @@ cudaError_t launch_stencil(int mode, const Geo& G, const T* u, const T* v, const
                            const double* f, T* out, T* out2, double* part, Ctl* ctl,
                            int check_done, cudaStream_t s) {
     if (G.dim == 3) return launch_stencil3d<T>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-#define JF_CASE(M)                                                                           \
-    case M:                                                                                  \
-        return G.sgs == 2 ? launch_stencil_t<T, M, 2>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s) \
-             : G.smag     ? launch_stencil_t<T, M, 1>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s) \
-                          : launch_stencil_t<T, M, 0>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-    switch (mode) {
-        JF_CASE(MODE_F)
-        JF_CASE(MODE_RHS)
-        JF_CASE(MODE_RES)
-        JF_CASE(MODE_JV)
-        JF_CASE(MODE_RHSRES)
-        default: return cudaErrorInvalidValue;
-    }
-#undef JF_CASE
+    if (mode < MODE_F || mode > MODE_RHSRES) return cudaErrorInvalidValue;
+    return G.sgs == 2 ? launch_flux<T, 2>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s)
+         : G.smag     ? launch_flux<T, 1>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s)
+                      : launch_flux<T, 0>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
 }
 template cudaError_t launch_stencil<float>(int, const Geo&, const float*, const float*, const float*,
                                            const double*, float*, float*, double*, Ctl*, int, cudaStream_t);
 template cudaError_t launch_stencil<double>(int, const Geo&, const double*, const double*, const double*,
                                             const double*, double*, double*, double*, Ctl*, int, cudaStream_t);
-
-// float32: persistent, double-buffered (one CTA per resident slot, capped at
-// the tile count); float64: one tile per CTA.
-template <typename T, int SMAG, int TX, int TZ>
-static cudaError_t launch_jvd_t(const Geo& G, const T* u, const T* v, T* out, const double* part, Ctl* ctl,
-                                int check_done, cudaStream_t s) {
-    constexpr int NBUF = sizeof(T) == sizeof(float) ? 2 : 1;
-    static std::atomic<int> slots{0};   // resident CTAs on the device; set once (races are benign)
-    const size_t sm = jvd_smem<T, TX, TZ, NBUF>();
-    if (slots.load() == 0) {
-        cudaError_t e = set_smem(jv_diff2d<T, SMAG, TX, TZ, NBUF>, sm);
-        if (e != cudaSuccess) return e;
-        int dev = 0, nsm = 0, per = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-            (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jv_diff2d<T, SMAG, TX, TZ, NBUF>, NTHREADS,
-                                                               sm)) != cudaSuccess)
-            return e;
-        slots = std::max(1, nsm * per);
-    }
-    const int ntiles = ((G.nx + TX - 1) / TX) * ((G.nz + TZ - 1) / TZ);
-    const int grid = NBUF == 2 ? std::min(ntiles, slots.load()) : ntiles;
-    return launch_pdl(jv_diff2d<T, SMAG, TX, TZ, NBUF>, dim3(grid), NTHREADS, sm, s, G, u, v, out,
-                      (const double*)part, ctl, check_done);
-}
 
 // float32: the compute-once kernel jvc2d, persistent (one CTA per resident
 // slot, capped at the tile count), double-buffered staging.
@@ -1830,34 +1622,13 @@ static cudaError_t launch_jvc_tile(const Geo& G, const float* u, const float* v,
 #undef JF_JVC
 }
 
-template <typename T, int SMAG>
-static cudaError_t launch_jvd_tile(const Geo& G, const T* u, const T* v, T* out, const double* part, Ctl* ctl,
-                                   int check_done, cudaStream_t s) {
-    if constexpr (sizeof(T) == sizeof(double)) {
-        return launch_jvd_t<T, SMAG, JvTile<1>::TX, JvTile<1>::TZ>(G, u, v, out, part, ctl, check_done, s);
-    } else {
-        return launch_jvc_tile<SMAG>(G, u, v, out, part, ctl, check_done, s);
-    }
-}
-
-template <typename T>
-cudaError_t launch_jv_diff(const Geo& G, const T* u, const T* v, T* out, double* part, Ctl* ctl,
+cudaError_t launch_jv_diff(const Geo& G, const float* u, const float* v, float* out, double* part, Ctl* ctl,
                            int check_done, cudaStream_t s) {
-    if (G.dim == 3) return launch_jv_diff3d<T>(G, u, v, out, ctl, check_done, s);
-    if (G.sgs == 2) {
-        // Deardorff: the float32 compute-once kernel only (float64 handles take the
-        // plain forward difference of stencil2d)
-        if constexpr (sizeof(T) == sizeof(float)) {
-            return launch_jvc_tile<2>(G, u, v, out, part, ctl, check_done, s);
-        } else {
-            return cudaErrorNotSupported;
-        }
-    }
-    return G.smag ? launch_jvd_tile<T, 1>(G, u, v, out, part, ctl, check_done, s)
-                  : launch_jvd_tile<T, 0>(G, u, v, out, part, ctl, check_done, s);
+    if (G.dim == 3) return launch_jv_diff3d(G, u, v, out, ctl, check_done, s);
+    if (G.sgs == 2) return launch_jvc_tile<2>(G, u, v, out, part, ctl, check_done, s);
+    return G.smag ? launch_jvc_tile<1>(G, u, v, out, part, ctl, check_done, s)
+                  : launch_jvc_tile<0>(G, u, v, out, part, ctl, check_done, s);
 }
-template cudaError_t launch_jv_diff<float>(const Geo&, const float*, const float*, float*, double*, Ctl*, int, cudaStream_t);
-template cudaError_t launch_jv_diff<double>(const Geo&, const double*, const double*, double*, double*, Ctl*, int, cudaStream_t);
 
 static int stream_blocks(size_t n) {
     size_t b = (n + NTHREADS - 1) / NTHREADS;

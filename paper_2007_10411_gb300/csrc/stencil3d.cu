@@ -1206,14 +1206,11 @@ template cudaError_t launch_stencil3d<float>(int, const Geo&, const float*, cons
 template cudaError_t launch_stencil3d<double>(int, const Geo&, const double*, const double*, const double*,
                                               const double*, double*, double*, double*, Ctl*, int, cudaStream_t);
 
-template <typename T>
-cudaError_t launch_jv_diff3d(const Geo& G, const T* u, const T* v, T* out, Ctl* ctl, int check_done,
+cudaError_t launch_jv_diff3d(const Geo& G, const float* u, const float* v, float* out, Ctl* ctl, int check_done,
                              cudaStream_t s) {
     using namespace d3;
-    return launch_split_m<T, d3::MODE_DJV>(G, u, v, nullptr, nullptr, out, nullptr, nullptr, ctl, check_done, s);
+    return launch_split_m<float, d3::MODE_DJV>(G, u, v, nullptr, nullptr, out, nullptr, nullptr, ctl, check_done, s);
 }
-template cudaError_t launch_jv_diff3d<float>(const Geo&, const float*, const float*, float*, Ctl*, int, cudaStream_t);
-template cudaError_t launch_jv_diff3d<double>(const Geo&, const double*, const double*, double*, Ctl*, int, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_eddy3d(const Geo& G, const T* u, T* nu, double* part, Ctl* ctl, cudaStream_t s) {

@@ -20,8 +20,21 @@ constexpr int MAX_DOT_BLOCKS = 3 * 152;     // Arnoldi passes A and C: three CTA
 constexpr int MAX_REDUCE_BLOCKS = 8192;     // multi-dot grids grow so a thread sums <= 64 vectors' worth
 constexpr int MAX_PC_SWEEPS = 64;
 
+// The float32 kernels' copies of the constants of Geo.  A float64 -> float32
+// conversion in a kernel runs at the FP64 pipe's rate (64 cycles per warp
+// instruction and sub-partition): a dozen per thread cost several microseconds
+// of a 20 us launch.
+struct GeoF {
+    float inv_dx, inv_dy, inv_dz, wx1, wx2, wy1, wy2, wz1, wz2;
+    float theta0, beta, pbar, gth, gamma_p, K_M, K_H, cs2, inv_Pr;
+    float dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
+    float two_over_dt, helm_a, schur_cdiv, schur_cgrad, half_dt;
+    float scale[5];
+};
+
 // Geometry and physics constants, passed by value to the stencil kernels.
 struct Geo {
+    GeoF f32;
     int dim, nx, ny, nz, npt, nf;     // 2-D: ny = 1, nf = 4 (u, w, theta, p); 3-D: nf = 5 (u, v, w, theta, p)
     double inv_dy;
     int pb[5], pt[5];                 // mirror parity per field at bottom / top (+1 / -1)
@@ -34,9 +47,8 @@ struct Geo {
     // K_h = K_m (1 + dd_ah l), K_H = K_M (1 + dd_az l), l = min(dd_delta, dd_cl s)
     // (dd_cl < 0: l = dd_delta)
     double dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
-    // float32 derivative weights with 1/h folded in: D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
-    float fx1, fx2, fz1, fz2;
-    double wx1, wx2, wy1, wy2, wz1, wz2;   // the same weights in float64 (and along y)
+    // derivative weights with 1/h folded in: D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
+    double wx1, wx2, wy1, wy2, wz1, wz2;
     double gth;                       // g / theta0
     double inv_Pr;
     double two_over_dt;
@@ -50,6 +62,14 @@ struct Geo {
     double helm_a, schur_cdiv, schur_cgrad, half_dt;
     void* s3;                         // 3-D: scratch of the split stencil passes (stencil3d_scratch_bytes)
 };
+
+// Constant `name` of Geo in the kernel's type T.
+template <typename T>
+__device__ __forceinline__ T geo_const(double d, float f) {
+    if constexpr (sizeof(T) == sizeof(double)) return d;
+    else return f;
+}
+#define GC(name) geo_const<T>(G.name, G.f32.name)
 
 constexpr int NUM_TILE_SHAPES = 4;
 
@@ -74,7 +94,7 @@ struct Ctl {
     double res2;         // ||W R||^2 of the last residual evaluation
     double unorm2;       // ||W u||^2 of the same state
     double eps_mach;     // unit roundoff of the stencil precision
-    double eps_jv;       // finite-difference step of the next Jacobian-vector product
+    double eps_jv;       // finite-difference step of the next Jacobian-vector product (put_eps)
     double kmax;         // max eddy coefficient K_M (preconditioner bounds)
     double gstart;       // ||r|| at the start of the current GMRES cycle
     double gres;         // rotated residual |g_{j+1}| after the latest Arnoldi step
@@ -89,8 +109,31 @@ struct Ctl {
                               // (1 unless the lagged second projection normalised w_k on the fly)
     // Chebyshev coefficients per field block and sweep: 1/theta_c, rho_k rho_{k-1}, 2 rho_k / delta
     double cheb[6][MAX_PC_SWEEPS][3];   // slot 5: pressure Helmholtz of the Schur complement
+    float chebf[6][MAX_PC_SWEEPS][3];   // the same in float32
     unsigned int counter[8];         // last-block counters, one per kernel family
+    double scale[5];                 // field scales (Geo::scale), set once
+    // eps_jv scale_f and its reciprocal rounded to float32, for the float32 3-D passes: formed
+    // once in float64 with the step instead of by every block
+    float evf[5], cff[5];
 };
+
+// The one writer of a finite-difference step that is not pending (eps_part).
+__device__ __forceinline__ void put_eps(Ctl* ctl, double e) {
+    ctl->eps_jv = e;
+    ctl->eps_part = 0;
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+        const double s = ctl->scale[f], es = e * s;
+        ctl->evf[f] = (float)es;
+        ctl->cff[f] = (float)(es != 0.0 ? 1.0 / es : 0.0);
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ T cheb_coef(const Ctl* ctl, int f, int k, int i) {
+    if constexpr (sizeof(T) == sizeof(double)) return ctl->cheb[f][k][i];
+    else return ctl->chebf[f][k][i];
+}
 
 // Programmatic dependent launch.  Kernels of the Arnoldi step are launched
 // with launch_pdl: the next kernel may be scheduled before this one has
@@ -119,6 +162,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 
 enum CounterSlot { CNT_STENCIL = 0, CNT_UPDATE, CNT_RESTART, CNT_PC, CNT_EDDY, CNT_MISC };
+
+// -x by the sign bit (an FP64 multiplication by -1, predicated off or not, costs the FP64 pipe)
+__device__ __forceinline__ float flip(float x) { return __int_as_float(__float_as_int(x) ^ 0x80000000); }
+__device__ __forceinline__ double flip(double x) {
+    return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
+}
 
 // Square root for kernels bound by the FP64 pipe (64 cycles per warp
 // instruction): Goldschmidt's iteration (Markstein, "IA-64 and Elementary

@@ -349,10 +349,6 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     G.inv_dx = 1.0 / dx;
     G.inv_dy = 1.0 / dy;
     G.inv_dz = 1.0 / dz;
-    G.fx1 = (float)(2.0 / 3.0 / dx);
-    G.fx2 = (float)(-1.0 / 12.0 / dx);
-    G.fz1 = (float)(2.0 / 3.0 / dz);
-    G.fz2 = (float)(-1.0 / 12.0 / dz);
     G.wx1 = 2.0 / 3.0 / dx;
     G.wx2 = -1.0 / 12.0 / dx;
     G.wy1 = 2.0 / 3.0 / dy;
@@ -400,6 +396,37 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     G.helm_a = strat->gamma_p * strat->pbar * strat->theta0 * G.half_dt;
     G.schur_cdiv = strat->gamma_p * strat->pbar * G.half_dt * G.scale[0] * G.inv_scale[nf - 1];
     G.schur_cgrad = strat->theta0 * G.scale[nf - 1] * G.inv_scale[0];
+    GeoF& F = G.f32;
+    F.inv_dx = (float)G.inv_dx;
+    F.inv_dy = (float)G.inv_dy;
+    F.inv_dz = (float)G.inv_dz;
+    F.wx1 = (float)G.wx1;
+    F.wx2 = (float)G.wx2;
+    F.wy1 = (float)G.wy1;
+    F.wy2 = (float)G.wy2;
+    F.wz1 = (float)G.wz1;
+    F.wz2 = (float)G.wz2;
+    F.theta0 = (float)G.theta0;
+    F.beta = (float)G.beta;
+    F.pbar = (float)G.pbar;
+    F.gth = (float)G.gth;
+    F.gamma_p = (float)G.gamma_p;
+    F.K_M = (float)G.K_M;
+    F.K_H = (float)G.K_H;
+    F.cs2 = (float)G.cs2;
+    F.inv_Pr = (float)G.inv_Pr;
+    F.dd_cm = (float)G.dd_cm;
+    F.dd_cM = (float)G.dd_cM;
+    F.dd_cl = (float)G.dd_cl;
+    F.dd_delta = (float)G.dd_delta;
+    F.dd_ah = (float)G.dd_ah;
+    F.dd_az = (float)G.dd_az;
+    F.two_over_dt = (float)G.two_over_dt;
+    F.helm_a = (float)G.helm_a;
+    F.schur_cdiv = (float)G.schur_cdiv;
+    F.schur_cgrad = (float)G.schur_cgrad;
+    F.half_dt = (float)G.half_dt;
+    for (int f = 0; f < nf; ++f) F.scale[f] = (float)G.scale[f];
 
     const size_t eT = h->mixed ? sizeof(float) : sizeof(double);
     const size_t nb8 = h->ld * sizeof(double);
@@ -477,6 +504,7 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     // so its step need not grow with the float32 roundoff.
     init.eps_mach = ldexp(1.0, -52);
     init.m = m;
+    for (int f = 0; f < nf; ++f) init.scale[f] = G.scale[f];
     if (cudaMemcpy(h->ctl, &init, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(h->part, 0, part_len * sizeof(double)) != cudaSuccess ||
         cudaMemset(h->x, 0, nb8) != cudaSuccess) {

@@ -786,8 +786,7 @@ update_x(const T* __restrict__ Z, size_t ldz, double* __restrict__ x, T* __restr
         if (threadIdx.x == 0) {
             ctl->scratch[0] = tot[0];
             const double xn = sqrt(tot[0]);
-            ctl->eps_jv = xn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / xn : 0.0;
-            ctl->eps_part = 0;
+            put_eps(ctl, xn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / xn : 0.0);
         }
     }
 }
@@ -820,8 +819,7 @@ cycle_init(Geo G, const double* __restrict__ R, T* __restrict__ V0, double* __re
         ctl->m = m;
         for (int k = 0; k < KMAX; ++k) ctl->zscale[k] = 1.0;
         if (pc_none) {
-            ctl->eps_jv = sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2)));
-            ctl->eps_part = 0;
+            put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
         }
     }
 }
@@ -864,8 +862,7 @@ restart_scale(T* __restrict__ V0, size_t n, int pc_none, Ctl* ctl) {
         ctl->k = 0;
         for (int k = 0; k < KMAX; ++k) ctl->zscale[k] = 1.0;
         if (pc_none) {
-            ctl->eps_jv = sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2)));
-            ctl->eps_part = 0;
+            put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
         }
     }
 }
@@ -899,16 +896,14 @@ left_scale(const T* __restrict__ z, T* __restrict__ V0, size_t n, int first, Ctl
         ctl->done = 0;
         ctl->breakdown = 0;
         ctl->k = 0;
-        ctl->eps_jv = sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2)));
-        ctl->eps_part = 0;
+        put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
     }
 }
 
 // The finite-difference step of a Jacobian product on a unit vector (left
 // preconditioning: restores it after a preconditioner apply left its own).
 __global__ void unit_eps_k(Ctl* ctl) {
-    ctl->eps_jv = sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2)));
-    ctl->eps_part = 0;
+    put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
 }
 
 // u += W^{-1} x (float64), uT = u rounded to T.
@@ -960,13 +955,12 @@ norm2_k(Geo G, const T* __restrict__ a, size_t n, int weighted, int slot, double
 }
 
 __global__ void set_eps_k(double eps, int su, int sv, Ctl* ctl) {
-    ctl->eps_part = 0;
-    if (eps > 0.0) {
-        ctl->eps_jv = eps;
-    } else {
+    double e = eps;
+    if (!(eps > 0.0)) {
         const double vn = sqrt(ctl->scratch[sv]);
-        ctl->eps_jv = vn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->scratch[su]))) / vn : 0.0;
+        e = vn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->scratch[su]))) / vn : 0.0;
     }
+    put_eps(ctl, e);
 }
 
 // ------------------------------------------------- learned preconditioner
@@ -1051,8 +1045,7 @@ pc_eps_k(const float* __restrict__ z, size_t n, double* part, Ctl* ctl) {
         final_sums(part, gridDim.x, 1, tot);
         if (threadIdx.x == 0) {
             const double zn = sqrt(tot[0]);
-            ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-            ctl->eps_part = 0;
+            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
         }
     }
 }

@@ -74,11 +74,6 @@ __device__ __forceinline__ int wrap_x(int gx, int nx) {
     return r < 0 ? r + nx : r;
 }
 
-// -x by the sign bit (an FP64 multiplication by -1, predicated off or not, costs the FP64 pipe)
-__device__ __forceinline__ float flip(float x) { return __int_as_float(__float_as_int(x) ^ 0x80000000); }
-__device__ __forceinline__ double flip(double x) {
-    return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
-}
 // Ghost row (side 1 bottom, 2 top) of a field that is odd at that wall.
 __device__ __forceinline__ bool odd_ghost(const Geo& G, int f, int side) {
     return (side == 1 && G.pb[f] < 0) || (side == 2 && G.pt[f] < 0);
@@ -177,8 +172,8 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
 // Deardorff heat factor s (1 + a l(s)), l = min(Delta, c_l s) (c_l < 0: l = Delta).
 template <typename T>
 __device__ __forceinline__ T dd_heat(T s, T a, const Geo& G) {
-    const T cls = rmul(T(G.dd_cl), s);
-    const T l = G.dd_cl < 0.0 ? T(G.dd_delta) : (cls < T(G.dd_delta) ? cls : T(G.dd_delta));
+    const T cls = rmul(GC(dd_cl), s);
+    const T l = GC(dd_cl) < T(0) ? GC(dd_delta) : (cls < GC(dd_delta) ? cls : GC(dd_delta));
     return rmul(s, rfma(a, l, T(1)));
 }
 
@@ -253,26 +248,26 @@ template <typename T, int SMAG, bool XF, bool ZF>
 __device__ __forceinline__ void flux_point(const Geo& G, const FluxShape& sh, const T* __restrict__ s, int i, int is,
                                            T* __restrict__ X, T* __restrict__ Z, T (&S)[4]) {
     const int PL = sh.plane(), SX = sh.sx(), XN = sh.xn(), ZN = sh.zn();
-    const T wx1 = T(G.wx1), wx2 = T(G.wx2), wz1 = T(G.wz1), wz2 = T(G.wz2);
+    const T wx1 = GC(wx1), wx2 = GC(wx2), wz1 = GC(wz1), wz2 = GC(wz2);
     const T *U = s, *W = s + PL, *H = s + 2 * PL, *P = s + 3 * PL;
     T ux = T(0), uz = T(0), wx = T(0), wz = T(0), tx = T(0), tz = T(0);
     if (XF || SMAG) { ux = wd(U, i, 1, wx1, wx2); wx = wd(W, i, 1, wx1, wx2); }
     if (ZF || SMAG) { uz = wd(U, i, SX, wz1, wz2); wz = wd(W, i, SX, wz1, wz2); }
     if (XF) tx = wd(H, i, 1, wx1, wx2);
     if (ZF) tz = wd(H, i, SX, wz1, wz2);
-    T kx = T(G.K_M), kz = T(G.K_M), kxh = T(G.K_H), kzh = T(G.K_H);
+    T kx = GC(K_M), kz = GC(K_M), kxh = GC(K_H), kzh = GC(K_H);
     if (SMAG) {
         const T st = is == i ? flux_strain(ux, uz, wx, wz)
                              : flux_strain(wd(U, is, 1, wx1, wx2), wd(U, is, SX, wz1, wz2),
                                            wd(W, is, 1, wx1, wx2), wd(W, is, SX, wz1, wz2));
         if (SMAG == 2) {       // Deardorff: K_m along x, K_M along z, heat with its own factors
-            kx = rmul(T(G.dd_cm), st);
-            kz = rmul(T(G.dd_cM), st);
-            if (XF) kxh = rmul(T(G.dd_cm), dd_heat(st, T(G.dd_ah), G));
-            if (ZF) kzh = rmul(T(G.dd_cM), dd_heat(st, T(G.dd_az), G));
+            kx = rmul(GC(dd_cm), st);
+            kz = rmul(GC(dd_cM), st);
+            if (XF) kxh = rmul(GC(dd_cm), dd_heat(st, GC(dd_ah), G));
+            if (ZF) kzh = rmul(GC(dd_cM), dd_heat(st, GC(dd_az), G));
         } else {
-            kx = kz = rmul(T(G.cs2), st);
-            kxh = kzh = rmul(kx, T(G.inv_Pr));
+            kx = kz = rmul(GC(cs2), st);
+            kxh = kzh = rmul(kx, GC(inv_Pr));
         }
     }
     const T hu = rmul(T(0.5), U[i]), hw = rmul(T(0.5), W[i]);
@@ -290,11 +285,11 @@ __device__ __forceinline__ void flux_point(const Geo& G, const FluxShape& sh, co
     }
     if (XF && ZF) {
         const T px = wd(P, i, 1, wx1, wx2), pz = wd(P, i, SX, wz1, wz2);
-        const T th0 = T(G.theta0);
+        const T th0 = GC(theta0);
         S[0] = rfma(-hu, ux, rfma(-hw, uz, -rmul(th0, px)));
-        S[1] = rfma(-hu, wx, rfma(-hw, wz, rfma(T(G.gth), H[i], -rmul(th0, pz))));
-        S[2] = rfma(-hu, tx, rfma(-hw, tz, -rmul(T(G.beta), W[i])));
-        S[3] = rfma(-hu, px, rfma(-hw, pz, -rmul(rmul(T(G.gamma_p), T(G.pbar) + P[i]), ux + wz)));
+        S[1] = rfma(-hu, wx, rfma(-hw, wz, rfma(GC(gth), H[i], -rmul(th0, pz))));
+        S[2] = rfma(-hu, tx, rfma(-hw, tz, -rmul(GC(beta), W[i])));
+        S[3] = rfma(-hu, px, rfma(-hw, pz, -rmul(rmul(GC(gamma_p), GC(pbar) + P[i]), ux + wz)));
     }
 }
 
@@ -305,9 +300,9 @@ __device__ __forceinline__ T flux_div(const Geo& G, const FluxShape& sh, const T
     const int PXW = sh.tx() + 2 * R, TX = sh.tx();
     const T* x = X + fl * sh.xn() + tz * PXW + tx + R;
     const T* z = Z + fl * sh.zn() + (tz + R) * TX + tx;
-    return rfma(T(G.wx1), x[1] - x[-1],
-                rfma(T(G.wx2), x[2] - x[-2],
-                     rfma(T(G.wz1), z[TX] - z[-TX], rfma(T(G.wz2), z[2 * TX] - z[-2 * TX], S))));
+    return rfma(GC(wx1), x[1] - x[-1],
+                rfma(GC(wx2), x[2] - x[-2],
+                     rfma(GC(wz1), z[TX] - z[-TX], rfma(GC(wz2), z[2 * TX] - z[-2 * TX], S))));
 }
 
 // The mode's output at point o of field fl from F (ar, au: sums of R^2 and u^2
@@ -663,12 +658,12 @@ __device__ __forceinline__ void jvc_point(const float* __restrict__ st, int i, i
         const bool wx = f < 2 ? DXUW : (f == 2 ? DXT : CEN);
         const bool wz = f < 2 ? DZUW : (f == 2 ? DZT : CEN);
         if (wx) {
-            dax[f] = ddf(A + f * PLANE, i, 1, G.fx1, G.fx2);
-            dbx[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, 1, G.fx1, G.fx2));
+            dax[f] = ddf(A + f * PLANE, i, 1, G.f32.wx1, G.f32.wx2);
+            dbx[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, 1, G.f32.wx1, G.f32.wx2));
         }
         if (wz) {
-            daz[f] = ddf(A + f * PLANE, i, SX, G.fz1, G.fz2);
-            dbz[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, SX, G.fz1, G.fz2));
+            daz[f] = ddf(A + f * PLANE, i, SX, G.f32.wz1, G.f32.wz2);
+            dbz[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, SX, G.f32.wz1, G.f32.wz2));
         }
     }
     // exchange coefficients along x and z, momentum [0] and heat [1], and their differences
@@ -678,11 +673,11 @@ __device__ __forceinline__ void jvc_point(const float* __restrict__ st, int i, i
         if (is == i) {
             jvc_strain(dax[0], daz[0], dax[1], daz[1], dbx[0], dbz[0], dbx[1], dbz[1], sa, sp, ds);
         } else {
-            jvc_strain(ddf(A, is, 1, G.fx1, G.fx2), ddf(A, is, SX, G.fz1, G.fz2), ddf(A + PLANE, is, 1, G.fx1, G.fx2),
-                       ddf(A + PLANE, is, SX, G.fz1, G.fz2), __fmul_rn(k.ev[0], ddf(V, is, 1, G.fx1, G.fx2)),
-                       __fmul_rn(k.ev[0], ddf(V, is, SX, G.fz1, G.fz2)),
-                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, 1, G.fx1, G.fx2)),
-                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, SX, G.fz1, G.fz2)), sa, sp, ds);
+            jvc_strain(ddf(A, is, 1, G.f32.wx1, G.f32.wx2), ddf(A, is, SX, G.f32.wz1, G.f32.wz2), ddf(A + PLANE, is, 1, G.f32.wx1, G.f32.wx2),
+                       ddf(A + PLANE, is, SX, G.f32.wz1, G.f32.wz2), __fmul_rn(k.ev[0], ddf(V, is, 1, G.f32.wx1, G.f32.wx2)),
+                       __fmul_rn(k.ev[0], ddf(V, is, SX, G.f32.wz1, G.f32.wz2)),
+                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, 1, G.f32.wx1, G.f32.wx2)),
+                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, SX, G.f32.wz1, G.f32.wz2)), sa, sp, ds);
         }
         if (SMAG == 2) {
             kx[0] = __fmul_rn(k.cm, sa); dkx[0] = __fmul_rn(k.cm, ds);
@@ -720,7 +715,7 @@ __device__ __forceinline__ void jvc_point(const float* __restrict__ st, int i, i
         }
     }
     if (CEN) {
-        const float th0 = (float)G.theta0;
+        const float th0 = G.f32.theta0;
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
             // a_u D_x b + a_w D_z b + b_u D_x phi' + b_w D_z phi'
@@ -728,13 +723,13 @@ __device__ __forceinline__ void jvc_point(const float* __restrict__ st, int i, i
                               __fmaf_rn(b[0], __fadd_rn(dax[f], dbx[f]), __fmul_rn(b[1], __fadd_rn(daz[f], dbz[f])))));
             S[f] = __fmul_rn(-0.5f, adv);
         }
-        const float gth = (float)(G.g / G.theta0);
+        const float gth = G.f32.gth;
         S[0] = __fmaf_rn(-th0, dbx[3], S[0]);
         S[1] = __fmaf_rn(-th0, dbz[3], __fmaf_rn(gth, b[2], S[1]));
-        S[2] = __fmaf_rn(-(float)G.beta, b[1], S[2]);
+        S[2] = __fmaf_rn(-G.f32.beta, b[1], S[2]);
         const float diva = __fadd_rn(dax[0], daz[1]), divb = __fadd_rn(dbx[0], dbz[1]);
-        const float pp = __fadd_rn(__fadd_rn((float)G.pbar, a[3]), b[3]);
-        S[3] = __fmaf_rn(-(float)G.gamma_p, __fmaf_rn(pp, divb, __fmul_rn(b[3], diva)), S[3]);
+        const float pp = __fadd_rn(__fadd_rn(G.f32.pbar, a[3]), b[3]);
+        S[3] = __fmaf_rn(-G.f32.gamma_p, __fmaf_rn(pp, divb, __fmul_rn(b[3], diva)), S[3]);
     }
 }
 
@@ -769,19 +764,19 @@ jvc2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __
     JvcConst k;
 #pragma unroll
     for (int f = 0; f < 4; ++f) k.ev[f] = evs[f];
-    k.idx = (float)G.inv_dx;
-    k.idz = (float)G.inv_dz;
-    k.cs2 = (float)G.cs2;
-    k.iPr = (float)G.inv_Pr;
-    k.KM = (float)G.K_M;
-    k.KH = (float)G.K_H;
-    k.cm = (float)G.dd_cm;
-    k.cM = (float)G.dd_cM;
-    k.cl = (float)G.dd_cl;
-    k.dlt = (float)G.dd_delta;
-    k.ah = (float)G.dd_ah;
-    k.az = (float)G.dd_az;
-    const float tdt = (float)G.two_over_dt;
+    k.idx = G.f32.inv_dx;
+    k.idz = G.f32.inv_dz;
+    k.cs2 = G.f32.cs2;
+    k.iPr = G.f32.inv_Pr;
+    k.KM = G.f32.K_M;
+    k.KH = G.f32.K_H;
+    k.cm = G.f32.dd_cm;
+    k.cM = G.f32.dd_cM;
+    k.cl = G.f32.dd_cl;
+    k.dlt = G.f32.dd_delta;
+    k.ah = G.f32.dd_ah;
+    k.az = G.f32.dd_az;
+    const float tdt = G.f32.two_over_dt;
     const int col = threadIdx.x % TX, r0 = (threadIdx.x / TX) * PPT;
     for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
         const int x0 = (t % ntx) * TX, z0 = (t / ntx) * TZ;
@@ -877,12 +872,12 @@ jvc2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __
             const size_t o = (size_t)gz * G.nx + gx;
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
-                const float conv = __fadd_rn(ddf(PX + f * PXN, ip, 1, G.fx1, G.fx2),
-                                             ddf(QZ + f * QZN, iq, TX, G.fz1, G.fz2));
+                const float conv = __fadd_rn(ddf(PX + f * PXN, ip, 1, G.f32.wx1, G.f32.wx2),
+                                             ddf(QZ + f * QZN, iq, TX, G.f32.wz1, G.f32.wz2));
                 float dF = __fmaf_rn(-0.5f, conv, Sv[q][f]);
                 if (f < 3)
-                    dF = __fadd_rn(dF, __fadd_rn(ddf(FX + f * PXN, ip, 1, G.fx1, G.fx2),
-                                                 ddf(FZ + f * QZN, iq, TX, G.fz1, G.fz2)));
+                    dF = __fadd_rn(dF, __fadd_rn(ddf(FX + f * PXN, ip, 1, G.f32.wx1, G.f32.wx2),
+                                                 ddf(FZ + f * QZN, iq, TX, G.f32.wz1, G.f32.wz2)));
                 out[(size_t)f * G.npt + o] = __fmaf_rn(tdt, Vc[q][f], __fmul_rn(-cfs[f], dF));
             }
         }
@@ -897,8 +892,8 @@ template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 eddy2d(Geo G, const T* __restrict__ u, T* __restrict__ nu, double* part, Ctl* ctl) {
     T mxT = T(0);
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
-    const T cs2 = G.sgs == 2 ? T(1) : T(G.cs2);     // Deardorff: the strain s (coefficients follow from it)
+    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
+    const T cs2 = G.sgs == 2 ? T(1) : GC(cs2);     // Deardorff: the strain s (coefficients follow from it)
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < G.npt; p += gridDim.x * blockDim.x) {
         const int z = p / G.nx, x = p - z * G.nx;
         T ux = T(0), uz = T(0), wx = T(0), wz = T(0);
@@ -940,63 +935,52 @@ eddy2d(Geo G, const T* __restrict__ u, T* __restrict__ nu, double* part, Ctl* ct
 //   x_{k+1} = x_k + d_k,   with x_1 = d_0 = r / theta_c.
 // ============================================================================
 // Coefficients of every sweep of every block, computed once per Newton
-// iteration from the (frozen) eddy maximum by one thread: 1/theta_c,
-// rho_k rho_{k-1} and 2 rho_k / delta, with rho_0 = 1/sigma, sigma = theta_c/delta.
+// iteration from the (frozen) eddy maximum: 1/theta_c, rho_k rho_{k-1} and
+// 2 rho_k / delta, with rho_0 = 1/sigma, sigma = theta_c/delta.  One thread per
+// block (slot 5: the pressure Helmholtz operator of the acoustic Schur
+// complement, H = (2/dt) I - a sum_j D_j D_j, a = gamma_p pbar theta0 dt / 2);
+// the recurrence is a serial chain of one division a sweep.  One thread doing
+// all slots with three divisions a sweep took 85 us at 32 sweeps.
 __global__ void pc_setup(Geo G, int sweeps, Ctl* ctl) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    const int f = threadIdx.x;
+    if (f > 5 || (f >= G.nf && f != 5)) return;
     const int fth = G.nf - 2, fp = G.nf - 1;         // theta and p
     const double h2 = G.inv_dx * G.inv_dx + G.inv_dz * G.inv_dz + (G.dim == 3 ? G.inv_dy * G.inv_dy : 0.0);
     // Deardorff: ctl->kmax is the largest strain s; every coefficient grows with s
     const double smax = ctl->kmax;
     const double lmax = G.dd_cl < 0.0 ? G.dd_delta : fmin(G.dd_delta, G.dd_cl * smax);
     const double hh2 = G.inv_dx * G.inv_dx + (G.dim == 3 ? G.inv_dy * G.inv_dy : 0.0);
-    for (int f = 0; f < G.nf; ++f) {
-        const double lo = G.two_over_dt;
-        double kh2 = 0.0;        // sum_j max K_j / h_j^2
-        if (f != fp) {
-            if (G.sgs == 2) {
-                const double fh = f == fth ? 1.0 + G.dd_ah * lmax : 1.0;
-                const double fz = f == fth ? 1.0 + G.dd_az * lmax : 1.0;
-                kh2 = G.dd_cm * smax * fh * hh2 + G.dd_cM * smax * fz * G.inv_dz * G.inv_dz;
-            } else {
-                kh2 = (G.smag ? ctl->kmax * (f == fth ? G.inv_Pr : 1.0) : (f == fth ? G.K_H : G.K_M)) * h2;
-            }
-        }
-        const double hi = lo + 2.25 * kh2;
-        const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo);
-        const bool degenerate = delta <= 1e-14 * theta;
-        const double sigma = degenerate ? 1.0 : theta / delta;
-        double rho = 1.0 / sigma;
-        ctl->cheb[f][0][0] = 1.0 / theta;
-        ctl->cheb[f][0][1] = 0.0;
-        ctl->cheb[f][0][2] = 0.0;
-        for (int k = 1; k < sweeps && k < MAX_PC_SWEEPS; ++k) {
-            const double rho_new = 1.0 / (2.0 * sigma - rho);
-            ctl->cheb[f][k][0] = 1.0 / theta;
-            ctl->cheb[f][k][1] = degenerate ? 0.0 : rho_new * rho;
-            ctl->cheb[f][k][2] = degenerate ? 0.0 : 2.0 * rho_new / delta;
-            rho = rho_new;
+    double kh2 = 0.0;        // sum_j max K_j / h_j^2
+    if (f == 5) {
+        kh2 = G.helm_a * h2;
+    } else if (f != fp) {
+        if (G.sgs == 2) {
+            const double fh = f == fth ? 1.0 + G.dd_ah * lmax : 1.0;
+            const double fz = f == fth ? 1.0 + G.dd_az * lmax : 1.0;
+            kh2 = G.dd_cm * smax * fh * hh2 + G.dd_cM * smax * fz * G.inv_dz * G.inv_dz;
+        } else {
+            kh2 = (G.smag ? ctl->kmax * (f == fth ? G.inv_Pr : 1.0) : (f == fth ? G.K_H : G.K_M)) * h2;
         }
     }
-    {
-        // slot 5 holds the pressure Helmholtz operator of the acoustic Schur
-        // complement, H = (2/dt) I - a sum_j D_j D_j, a = gamma_p pbar theta0 dt / 2
-        const double a = G.helm_a;
-        const double lo = G.two_over_dt, hi = lo + 2.25 * a * h2;
-        const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo);
-        const bool degenerate = delta <= 1e-14 * theta;
-        const double sigma = degenerate ? 1.0 : theta / delta;
-        double rho = 1.0 / sigma;
-        ctl->cheb[5][0][0] = 1.0 / theta;
-        ctl->cheb[5][0][1] = 0.0;
-        ctl->cheb[5][0][2] = 0.0;
-        for (int k = 1; k < sweeps && k < MAX_PC_SWEEPS; ++k) {
-            const double rho_new = 1.0 / (2.0 * sigma - rho);
-            ctl->cheb[5][k][0] = 1.0 / theta;
-            ctl->cheb[5][k][1] = degenerate ? 0.0 : rho_new * rho;
-            ctl->cheb[5][k][2] = degenerate ? 0.0 : 2.0 * rho_new / delta;
-            rho = rho_new;
-        }
+    const double lo = G.two_over_dt, hi = lo + 2.25 * kh2;
+    const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo);
+    const bool degenerate = delta <= 1e-14 * theta;
+    const double sigma = degenerate ? 1.0 : theta / delta, ith = 1.0 / theta;
+    const double two_over_delta = degenerate ? 0.0 : 2.0 / delta;
+    auto put = [&](int k, double c1, double c2) {
+        ctl->cheb[f][k][0] = ith;
+        ctl->cheb[f][k][1] = c1;
+        ctl->cheb[f][k][2] = c2;
+        ctl->chebf[f][k][0] = (float)ith;
+        ctl->chebf[f][k][1] = (float)c1;
+        ctl->chebf[f][k][2] = (float)c2;
+    };
+    double rho = 1.0 / sigma;
+    put(0, 0.0, 0.0);
+    for (int k = 1; k < sweeps && k < MAX_PC_SWEEPS; ++k) {
+        const double rho_new = 1.0 / (2.0 * sigma - rho);
+        put(k, degenerate ? 0.0 : rho_new * rho, rho_new * two_over_delta);
+        rho = rho_new;
     }
 }
 
@@ -1024,9 +1008,9 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const int fld = blockIdx.z;                     // 0 u, 1 w, 2 theta, 3 p (last sweep only)
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T ith = T(ctl->cheb[fld][k][0]);
-    const T a1 = T(ctl->cheb[fld][k][1]);
-    const T a2 = T(ctl->cheb[fld][k][2]);
+    const T ith = cheb_coef<T>(ctl, fld, k, 0);
+    const T a1 = cheb_coef<T>(ctl, fld, k, 1);
+    const T a2 = cheb_coef<T>(ctl, fld, k, 2);
     const T* rf = r + (size_t)fld * G.npt;
     T* zf = zout + (size_t)fld * G.npt;
     const int gxx = x0 + tx;
@@ -1067,7 +1051,7 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
         if (SMAG == 2) {
             // Deardorff: nu holds the strain s; K_m = c_m s along x, K_M = c_M s along z,
             // heat K_h = c_m s (1 + a_h l), K_H = c_M s (1 + a_z l)
-            const T cm = T(G.dd_cm), cM = T(G.dd_cM);
+            const T cm = GC(dd_cm), cM = GC(dd_cM);
             for (int qz = ty; qz < QZ; qz += TY) {
                 int side;
                 const int szr = mirror_z(z0 + qz - R, G.nz, side);
@@ -1075,12 +1059,12 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
                 const T* nrow = nu + szr * G.nx;
                 for (int qx = tx; qx < QX; qx += TX) {
                     const T sv = ok ? nrow[wrap_x(x0 + qx - R, G.nx)] : T(0);
-                    kk_[qz * QX + qx] = rmul(cm, fld == 2 ? dd_heat(sv, T(G.dd_ah), G) : sv);
-                    kz_[qz * QX + qx] = rmul(cM, fld == 2 ? dd_heat(sv, T(G.dd_az), G) : sv);
+                    kk_[qz * QX + qx] = rmul(cm, fld == 2 ? dd_heat(sv, GC(dd_ah), G) : sv);
+                    kz_[qz * QX + qx] = rmul(cM, fld == 2 ? dd_heat(sv, GC(dd_az), G) : sv);
                 }
             }
         } else if (SMAG) {
-            const T kscale = fld == 2 ? T(G.inv_Pr) : T(1);
+            const T kscale = fld == 2 ? GC(inv_Pr) : T(1);
             for (int qz = ty; qz < QZ; qz += TY) {
                 int side;
                 const int szr = mirror_z(z0 + qz - R, G.nz, side);
@@ -1091,7 +1075,7 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
             }
         }
         __syncthreads();
-        const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
+        const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
         for (int tz = ty; tz < TZ; tz += TY)              // D_x on tile rows, x-halo r
             for (int qx = tx; qx < QX; qx += TX)
                 gxs[tz * QX + qx] = dd(zs, (tz + HALO) * SX + qx + R, 1, idx_);
@@ -1099,7 +1083,7 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
             gzs[qz * TX + tx] = dd(zs, (qz + R) * SX + tx + HALO, SX, idz_);
         __syncthreads();
         const T Kc = T(fld == 2 ? G.K_H : G.K_M);
-        const T tdt = T(G.two_over_dt);
+        const T tdt = GC(two_over_dt);
         T* dof = LAST ? nullptr : dout + (size_t)fld * G.npt;
         if (colok) {
 #pragma unroll
@@ -1154,8 +1138,7 @@ cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
                 final_sums(part, nblk, 1, tot);
                 if (threadIdx.x == 0) {
                     const double zn = sqrt(tot[0]);
-                    ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-                    ctl->eps_part = 0;
+                    put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
                 }
             }
         }
@@ -1170,7 +1153,7 @@ pc_diag(Geo G, const T* __restrict__ r, T* __restrict__ z, size_t n, double* par
     if (check_done && ctl->done) return;
     T acc[1] = {T(0)};
     T inv_th[5];
-    for (int f = 0; f < G.nf; ++f) inv_th[f] = T(ctl->cheb[f][0][0]);
+    for (int f = 0; f < G.nf; ++f) inv_th[f] = cheb_coef<T>(ctl, f, 0, 0);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const int f = (int)(i / G.npt);
         const T zv = r[i] * inv_th[f];
@@ -1183,8 +1166,7 @@ pc_diag(Geo G, const T* __restrict__ r, T* __restrict__ z, size_t n, double* par
         final_sums(part, gridDim.x, 1, tot);
         if (threadIdx.x == 0) {
             const double zn = sqrt(tot[0]);
-            ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-            ctl->eps_part = 0;
+            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
         }
     }
 }
@@ -1228,8 +1210,8 @@ template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 schur_rhs2d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int check_done) {
     if (check_done && ctl->done) return;
-    const T cdiv = T(G.schur_cdiv);
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
+    const T cdiv = GC(schur_cdiv);
+    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < G.npt; p += gridDim.x * blockDim.x) {
         const int gz = p / G.nx, gx = p - gz * G.nx;
         const T du = plane_dx(r, G, gz, gx, idx_);
@@ -1256,9 +1238,9 @@ helm2d(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, const
     T* gzs = gxs + TZ * QX;                         // [QZ][TX]
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T ith = T(ctl->cheb[5][k][0]);
-    const T a1 = T(ctl->cheb[5][k][1]);
-    const T a2 = T(ctl->cheb[5][k][2]);
+    const T ith = cheb_coef<T>(ctl, 5, k, 0);
+    const T a1 = cheb_coef<T>(ctl, 5, k, 1);
+    const T a2 = cheb_coef<T>(ctl, 5, k, 2);
     const int gxx = x0 + tx;
     const bool colok = gxx < G.nx;
     constexpr int NR = TZ / TY;
@@ -1288,13 +1270,13 @@ helm2d(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, const
         zs[idx] = val;
     }
     __syncthreads();
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
+    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
     for (int tz = ty; tz < TZ; tz += TY)
         for (int qx = tx; qx < QX; qx += TX) gxs[tz * QX + qx] = dd(zs, (tz + HALO) * SX + qx + R, 1, idx_);
     for (int qz = ty; qz < QZ; qz += TY) gzs[qz * TX + tx] = dd(zs, (qz + R) * SX + tx + HALO, SX, idz_);
     __syncthreads();
-    const T ah = T(G.helm_a);
-    const T tdt = T(G.two_over_dt);
+    const T ah = GC(helm_a);
+    const T tdt = GC(two_over_dt);
     if (colok) {
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
@@ -1338,9 +1320,9 @@ helm2d_x2(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, co
     T* gx = x1 + EZ * EX;                        // [EZ][EX + 2R]  D_x rows (reused by sweep k+1)
     T* gz = gx + EZ * (EX + 2 * R);              // [EZ + 2R][EX]  D_z columns (reused)
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T ith = T(ctl->cheb[5][k][0]);
-    const T a1 = T(ctl->cheb[5][k][1]), a2 = T(ctl->cheb[5][k][2]);
-    const T b1 = T(ctl->cheb[5][k + 1][1]), b2 = T(ctl->cheb[5][k + 1][2]);
+    const T ith = cheb_coef<T>(ctl, 5, k, 0);
+    const T a1 = cheb_coef<T>(ctl, 5, k, 1), a2 = cheb_coef<T>(ctl, 5, k, 2);
+    const T b1 = cheb_coef<T>(ctl, 5, k + 1, 1), b2 = cheb_coef<T>(ctl, 5, k + 1, 2);
     const T pb = T(G.pb[3]), pt = T(G.pt[3]);
     // staging: x_k (halo 2 HALO), rhs and d_{k-1} (halo HALO); p parity in z, periodic x
     for (int idx = threadIdx.x; idx < SX * SZ; idx += blockDim.x) {
@@ -1362,8 +1344,8 @@ helm2d_x2(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, co
         }
     }
     __syncthreads();
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
-    const T ah = T(G.helm_a), tdt = T(G.two_over_dt);
+    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
+    const T ah = GC(helm_a), tdt = GC(two_over_dt);
     // sweep k on the first-sweep region
     for (int i = threadIdx.x; i < EZ * (EX + 2 * R); i += blockDim.x) {
         const int ez = i / (EX + 2 * R), c = i - ez * (EX + 2 * R);
@@ -1427,10 +1409,10 @@ template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 schur_back2d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ctl* ctl, int check_done) {
     if (check_done && ctl->done) return;
-    const T cgrad = T(G.schur_cgrad);
-    const T hdt = T(G.half_dt);
-    const T ith_t = T(ctl->cheb[2][0][0]);
-    const T idx_ = T(G.inv_dx), idz_ = T(G.inv_dz);
+    const T cgrad = GC(schur_cgrad);
+    const T hdt = GC(half_dt);
+    const T ith_t = cheb_coef<T>(ctl, 2, 0, 0);
+    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
     const size_t np = (size_t)G.npt;
     const T* dp = z + 3 * np;
     T acc[1] = {T(0)};
@@ -1451,8 +1433,7 @@ schur_back2d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ct
         final_sums(part, gridDim.x, 1, tot);
         if (threadIdx.x == 0) {
             const double zn = sqrt(tot[0]);
-            ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-            ctl->eps_part = 0;
+            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
         }
     }
 }

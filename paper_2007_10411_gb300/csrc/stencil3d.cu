@@ -18,28 +18,25 @@
 // needs:
 //   strain  |S| (and, for the difference-form Jacobian product, |S(a+b)| - |S(a)|
 //           without cancellation) at every point: a plane tile with a halo of
-//           r = 2 in x, y in shared memory, z neighbours read directly;
-//   plane   the x and y terms and the point-wise ones for a TX x TY tile of one
-//           plane: the fields with a halo of 2r = 4 in x and y, the first
-//           derivatives on the x / y arms (tile + r) computed once, the eddy
-//           coefficients on the arms from the strain pass; writes the partial sum;
-//   slab    the z terms for a TX x TZ slab of one y row: the fields with a halo
-//           of 4 in z (mirror ghosts), z derivatives on the z arms, then the
-//           partial sum of the plane pass is added and the mode's output
-//           (F, 2u/dt + F, the residual with its norms, or the Jacobian product)
-//           written.
+//           r = 2 in x, y in shared memory, z neighbours in registers;
+//   plane   the x and y terms and the point-wise ones for a tile of one plane:
+//           every flux formed once, then differentiated; writes the partial sum;
+//   column  the z terms, one column per thread marching in z with its values and
+//           fluxes in registers, then the partial sum of the plane pass is added
+//           and the mode's output (F, 2u/dt + F, the residual with its norms, or
+//           the Jacobian product) written.
 // Loads are coalesced along x in every pass; the halos are re-read from L2.
 //
 // Difference form (float32 Jacobian product): with a = u and b = eps v every
-// term of F(a + b) - F(a) is written as a difference (products a_j b_phi +
-// b_j (a_phi + b_phi), K(a) D b + (K(a + b) - K(a)) D(a + b)), so no O(1)
-// quantity is cancelled in float32.  The other modes evaluate F(b) with
-// a = 0 (b = u, or b = u + eps v for the plain forward difference), for
-// which the same formulas reduce to F term by term.
+// term of F(a + b) - F(a) is written as a difference about the midpoint
+// m = a + b/2 (products m_j b_phi + b_j m_phi, Km D b + dK D m), so no O(1)
+// quantity is cancelled in float32.  The other modes evaluate F(b) for
+// b = u, or b = u + eps v for the plain forward difference.
 #include <math.h>
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -49,10 +46,7 @@ namespace d3 {
 
 constexpr int R = 2;
 constexpr int HALO = 2 * R;
-constexpr int MODE_F = 0, MODE_RHS = 1, MODE_RES = 2, MODE_JV = 3, MODE_RHSRES = 4, MODE_DJV = 5;
-
-template <int MODE>
-struct Two { static constexpr bool v = MODE == MODE_DJV; };   // two states a, b (else a = 0)
+constexpr int MODE_F = 0, MODE_RHS = 1, MODE_RES = 2, MODE_JV = 3, MODE_RHSRES = 4;
 
 template <typename T>
 __device__ __forceinline__ T dd(const T* s, int i, int st, T ih) {
@@ -89,8 +83,8 @@ template <typename T>
 __device__ __forceinline__ T dd3_coef(T s, bool zarm, bool heat, const Geo& G) {
     const T c = T(zarm ? G.dd_cM : G.dd_cm);
     if (!heat) return c * s;
-    const T cls = T(G.dd_cl) * s;
-    const T l = G.dd_cl < 0.0 ? T(G.dd_delta) : (cls < T(G.dd_delta) ? cls : T(G.dd_delta));
+    const T cls = GC(dd_cl) * s;
+    const T l = GC(dd_cl) < T(0) ? GC(dd_delta) : (cls < GC(dd_delta) ? cls : GC(dd_delta));
     return c * (s * (T(1) + T(zarm ? G.dd_az : G.dd_ah) * l));
 }
 
@@ -102,7 +96,7 @@ __device__ __forceinline__ T dd3_coef(T s, bool zarm, bool heat, const Geo& G) {
 template <typename T, int SMAG>
 __device__ __forceinline__ void kpair(const Geo& G, T na, T ds, bool zarm, bool heat, T& k, T& dk) {
     if (SMAG == 1) {
-        const T c = T(G.cs2);
+        const T c = GC(cs2);
         k = c * na;
         dk = c * ds;
         return;
@@ -116,49 +110,115 @@ __device__ __forceinline__ void kpair(const Geo& G, T na, T ds, bool zarm, bool 
     // heat: g(s) = c s (1 + a l(s)); g(s') - g(s) = ds (1 + a l') + a s (l' - l),
     // l' - l = c_l ds while both are below the cap
     const T a = T(zarm ? G.dd_az : G.dd_ah);
-    const T dl_cap = T(G.dd_delta);
+    const T dl_cap = GC(dd_delta);
     T la = dl_cap, lp = dl_cap, dl = T(0);
-    if (G.dd_cl >= 0.0) {
-        const T ta = T(G.dd_cl) * na, tq = T(G.dd_cl) * (na + ds);
+    if (GC(dd_cl) >= T(0)) {
+        const T ta = GC(dd_cl) * na, tq = GC(dd_cl) * (na + ds);
         la = ta < dl_cap ? ta : dl_cap;
         lp = tq < dl_cap ? tq : dl_cap;
-        if (ta < dl_cap && tq < dl_cap) dl = T(G.dd_cl) * ds;
+        if (ta < dl_cap && tq < dl_cap) dl = GC(dd_cl) * ds;
         else if (ta < dl_cap || tq < dl_cap) dl = lp - la;
     }
     k = c * (na * (T(1) + a * la));
     dk = c * (ds * (T(1) + a * lp) + a * na * dl);
 }
 
-// The two states of field f at flat index o: DJV a = u, b = eps_f v;
-// JV a = 0, b = u + eps_f v; other modes a = 0, b = u.
-template <typename T, int MODE>
-__device__ __forceinline__ void load_ab(const T* __restrict__ u, const T* __restrict__ v, T ev, size_t o, T& a,
-                                        T& b) {
-    if constexpr (MODE == MODE_DJV) {
-        a = u[o];
+// ------------------------------------------------------------------ states
+// KIND of a pass: one state b = u (ONE) or b = u + eps v (SHIFT, the float64
+// forward difference), or the difference F(a + b) - F(a) with a = u, b = eps v
+// (PAIR).  PAIR works with the midpoint m = a + b/2, for which every
+// product of the two states is
+//   a'_j phi' - a_j phi = m_j b_phi + b_j m_phi,   K' D phi' - K D phi = Km D b + dK D m
+// (Km = (K + K')/2, dK = K' - K): exact, free of cancellation, and two
+// multiplications each.
+constexpr int ONE = 0, SHIFT = 1, PAIR = 2;
+
+template <typename T, int KIND>
+__device__ __forceinline__ void load_mb(const T* __restrict__ u, const T* __restrict__ v, T ev, size_t o, T& m, T& b) {
+    if constexpr (KIND == PAIR) {
         b = ev * v[o];
-    } else if constexpr (MODE == MODE_JV) {
-        a = T(0);
+        m = u[o] + T(0.5) * b;
+    } else if constexpr (KIND == SHIFT) {
         b = u[o] + ev * v[o];
     } else {
-        a = T(0);
         b = u[o];
     }
 }
 
-// eps_f = eps_jv * scale_f (Jacobian-product modes)
+// Exchange coefficients of an arm, momentum and heat: K(b) in dk (one state) or
+// (Km, dK) from na = |S(a)|, ds = |S(a + b)| - |S(a)|.
+template <typename T, int KIND, int SMAG>
+__device__ __forceinline__ void coefs(const Geo& G, T na, T ds, bool zarm, T (&km)[2], T (&dk)[2]) {
+    if constexpr (SMAG == 0) {
+        km[0] = dk[0] = GC(K_M);
+        km[1] = dk[1] = GC(K_H);
+    } else if constexpr (SMAG == 1) {
+        km[0] = KIND == PAIR ? GC(cs2) * (na + T(0.5) * ds) : T(0);
+        dk[0] = GC(cs2) * ds;
+        km[1] = KIND == PAIR ? km[0] * GC(inv_Pr) : T(0);
+        dk[1] = dk[0] * GC(inv_Pr);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            kpair<T, SMAG>(G, na, ds, zarm, h == 1, km[h], dk[h]);
+            if (KIND == PAIR) km[h] += T(0.5) * dk[h];
+        }
+    }
+}
+
+// Flux along one axis of a diffused field (heat: h = 1), K D phi - 1/2 u_j phi:
+// mj, bj half the velocity along the axis, m, b the field, dm, db its derivative.
+template <typename T, int KIND, int SMAG>
+__device__ __forceinline__ T flux_of(T km, T dk, T mj, T bj, T m, T b, T dm, T db) {
+    if constexpr (KIND == PAIR) {
+        T x = -(mj * b) - bj * m;
+        x += km * db;
+        return SMAG ? x + dk * dm : x;
+    } else {
+        return dk * db - bj * b;
+    }
+}
+// The same for p, which is not diffused.
+template <typename T, int KIND>
+__device__ __forceinline__ T flux_p(T mj, T bj, T m, T b) {
+    return KIND == PAIR ? -(mj * b) - bj * m : -(bj * b);
+}
+// The advective form -1/2 u_j D_j phi, added to s.
+template <typename T, int KIND>
+__device__ __forceinline__ T advect(T s, T mj, T bj, T dm, T db) {
+    return KIND == PAIR ? s - mj * db - bj * dm : s - bj * db;
+}
+
+// Asynchronous copy of one element into shared memory.
+template <typename T>
+__device__ __forceinline__ void cpa1(T* dst, const T* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"((int)sizeof(T)) : "memory");
+}
+
+// eps_f = eps_jv * scale_f and 1 / eps_f (Jacobian-product modes)
 template <typename T>
 __device__ __forceinline__ T eps_field(const Ctl* ctl, const Geo& G, int f) {
-    return T(ctl->eps_jv * G.scale[f]);
+    if constexpr (sizeof(T) == sizeof(float)) return ctl->evf[f];
+    else return ctl->eps_jv * G.scale[f];
+}
+template <typename T>
+__device__ __forceinline__ T inv_eps_field(const Ctl* ctl, const Geo& G, int f) {
+    if constexpr (sizeof(T) == sizeof(float)) return ctl->cff[f];
+    const T e = T(ctl->eps_jv * G.scale[f]);
+    return e != T(0) ? T(1) / e : T(0);
 }
 
 // ------------------------------------------------------------------ tiles
-constexpr int PX = 32, PY = 8;                 // plane tile (one output per thread)
 constexpr int KX = 32, KY = 8;                 // strain tile
-template <typename T> struct SlabT;            // slab tile TX x TZ
-template <> struct SlabT<float>  { static constexpr int TX = 32, TZ = 16; };
-template <> struct SlabT<double> { static constexpr int TX = 32, TZ = 8; };
-static_assert(PX * PY == NTHREADS && KX * KY == NTHREADS, "one output per thread");
+static_assert(KX * KY == NTHREADS, "one output per thread");
+
+// The strain pass's states: a = u, b = eps v (PAIR), else b alone.
+template <typename T, int KIND>
+__device__ __forceinline__ void load_ab(const T* __restrict__ u, const T* __restrict__ v, T ev, size_t o, T& a, T& b) {
+    a = KIND == PAIR ? u[o] : T(0);
+    b = KIND == PAIR ? ev * v[o] : (KIND == SHIFT ? u[o] + ev * v[o] : u[o]);
+}
 
 // ============================================================================
 // Strain pass: s = sqrt(2 S:S) of b (one-state modes) or, for the difference
@@ -171,21 +231,20 @@ static_assert(PX * PY == NTHREADS && KX * KY == NTHREADS, "one output per thread
 // ============================================================================
 constexpr int SZB = 16;      // planes per CTA of the strain pass
 
-template <typename T, int MODE, int EDDY>
+template <typename T, int KIND, int EDDY>
 __global__ void __launch_bounds__(NTHREADS)
 strain3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict__ s0, T* __restrict__ s1,
          double* part, Ctl* ctl, int check_done) {
-    constexpr bool TWO = Two<MODE>::v;
+    constexpr bool TWO = KIND == PAIR;            // a = u, b = eps v
     constexpr int SX = KX + 2 * R, SY = KY + 2 * R, SP = SX * SY;
     constexpr int NA = TWO ? 6 : 3;               // (b u, b v, b w) [, (a u, a v, a w)]
     constexpr int XS = (SP + NTHREADS - 1) / NTHREADS;
-    if ((MODE == MODE_JV || MODE == MODE_DJV) && check_done && ctl->done) return;
+    if (KIND != ONE && check_done && ctl->done) return;
     __shared__ T st[NA][SP];
     const int x0 = blockIdx.x * KX, y0 = blockIdx.y * KY;
     const int z0 = blockIdx.z * SZB, z1 = min(z0 + SZB, G.nz);
-    const T ix = T(G.inv_dx), iy = T(G.inv_dy), iz = T(G.inv_dz);
     T ev[3] = {T(0), T(0), T(0)};
-    if (MODE == MODE_JV || MODE == MODE_DJV) {
+    if (KIND != ONE) {
 #pragma unroll
         for (int f = 0; f < 3; ++f) ev[f] = eps_field<T>(ctl, G, f);
     }
@@ -205,93 +264,109 @@ strain3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict_
     auto col = [&](int z, int f, T& a, T& b) {
         int side;
         const int sz = mirror(z, G.nz, side);
-        load_ab<T, MODE>(u, v, ev[f], (size_t)f * G.npt + (size_t)sz * nxy + own, a, b);
-        const T sg = side == 1 ? T(G.pb[f]) : (side == 2 ? T(G.pt[f]) : T(1));
-        a *= sg;
-        b *= sg;
+        load_ab<T, KIND>(u, v, ev[f], (size_t)f * G.npt + (size_t)sz * nxy + own, a, b);
+        if ((side == 1 && G.pb[f] < 0) || (side == 2 && G.pt[f] < 0)) {
+            a = flip(a);
+            b = flip(b);
+        }
     };
-    if (inside) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int f = 0; f < 3; ++f) col(z0 - 2 + q, f, wa[f][q], wb[f][q]);
-    }
+        for (int f = 0; f < 3; ++f) col(z0 - 2 + q, f, wa[f][q], wb[f][q]);
+    // the next plane's staged values and the column's plane above them are loaded
+    // one step ahead, so that their latency overlaps the current plane
+    T na[XS][3], nb[XS][3], ca[3], cb[3];
+    auto fetch = [&](int z) {
+#pragma unroll
+        for (int q = 0; q < XS; ++q)
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+                if (xoff[q] >= 0)
+                    load_ab<T, KIND>(u, v, ev[f], (size_t)f * G.npt + (size_t)z * nxy + xoff[q], na[q][f], nb[q][f]);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) col(z + 2, f, ca[f], cb[f]);
+    };
+    fetch(z0);
     T mx = T(0);
     for (int z = z0; z < z1; ++z) {
         const size_t pz = (size_t)z * nxy;
 #pragma unroll
         for (int q = 0; q < XS; ++q) {
             if (xoff[q] < 0) continue;
-            const size_t o = pz + xoff[q];
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
-                T a, b;
-                load_ab<T, MODE>(u, v, ev[f], (size_t)f * G.npt + o, a, b);
-                st[f][threadIdx.x + q * NTHREADS] = b;
-                if (TWO) st[3 + f][threadIdx.x + q * NTHREADS] = a;
+                st[f][threadIdx.x + q * NTHREADS] = nb[q][f];
+                if (TWO) st[3 + f][threadIdx.x + q * NTHREADS] = na[q][f];
             }
         }
-        __syncthreads();
-        if (inside) {
 #pragma unroll
-            for (int f = 0; f < 3; ++f) col(z + 2, f, wa[f][4], wb[f][4]);
+        for (int f = 0; f < 3; ++f) {
+            wa[f][4] = ca[f];
+            wb[f][4] = cb[f];
+        }
+        __syncthreads();
+        if (z + 1 < z1) fetch(z + 1);
+        if (inside) {
             const int c = (ty + R) * SX + tx + R;
+            auto D = [&](const T* s, int st_, T w1, T w2) {
+                return w1 * (s[c + st_] - s[c - st_]) + w2 * (s[c + 2 * st_] - s[c - 2 * st_]);
+            };
             T gB[3][3], gA[3][3];
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
-                gB[f][0] = dd(st[f], c, 1, ix);
-                gB[f][1] = dd(st[f], c, SX, iy);
-                gB[f][2] = d5(wb[f][0], wb[f][1], wb[f][3], wb[f][4], iz);
+                gB[f][0] = D(st[f], 1, GC(wx1), GC(wx2));
+                gB[f][1] = D(st[f], SX, GC(wy1), GC(wy2));
+                gB[f][2] = GC(wz1) * (wb[f][3] - wb[f][1]) + GC(wz2) * (wb[f][4] - wb[f][0]);
                 if (TWO) {
-                    gA[f][0] = dd(st[3 + f], c, 1, ix);
-                    gA[f][1] = dd(st[3 + f], c, SX, iy);
-                    gA[f][2] = d5(wa[f][0], wa[f][1], wa[f][3], wa[f][4], iz);
+                    gA[f][0] = D(st[3 + f], 1, GC(wx1), GC(wx2));
+                    gA[f][1] = D(st[3 + f], SX, GC(wy1), GC(wy2));
+                    gA[f][2] = GC(wz1) * (wa[f][3] - wa[f][1]) + GC(wz2) * (wa[f][4] - wa[f][0]);
                 }
+            }
+            // 2 S:S = 2 sum g_ii^2 + sum_{i<j} (g_ij + g_ji)^2
+            T sym[3], syma[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int j = (i + 1) % 3;
+                sym[i] = gB[i][j] + gB[j][i];
+                if (TWO) syma[i] = gA[i][j] + gA[j][i];
             }
             const size_t p = pz + own;
             if (TWO) {
-                T ssa = T(0), dss = T(0);
+                T dA = T(0), oA = T(0), dD = T(0), oD = T(0);     // diagonal and off-diagonal sums of S:S, S':S' - S:S
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const T sA = T(0.5) * (gA[i][j] + gA[j][i]);
-                        const T sB = T(0.5) * (gB[i][j] + gB[j][i]);
-                        ssa += sA * sA;
-                        dss += (T(2) * sA + sB) * sB;       // S':S' - S:S
-                    }
-                const T na = sqrt(T(2) * ssa);
-                const T tp = T(2) * (ssa + dss);
-                const T np = sqrt(tp > T(0) ? tp : T(0));
-                const T den = na + np;
-                s0[p] = na;
-                s1[p] = den > T(0) ? T(2) * dss / den : T(0);
+                for (int i = 0; i < 3; ++i) {
+                    dA += gA[i][i] * gA[i][i];
+                    dD += (T(2) * gA[i][i] + gB[i][i]) * gB[i][i];
+                    oA += syma[i] * syma[i];
+                    oD += (T(2) * syma[i] + sym[i]) * sym[i];
+                }
+                const T sa = T(2) * dA + oA, ds = T(2) * dD + oD;     // 2 S:S and its difference
+                const T na_ = root(sa);
+                const T tp = sa + ds;
+                const T den = na_ + root(tp > T(0) ? tp : T(0));
+                s0[p] = na_;
+                s1[p] = den > T(0) ? ds / den : T(0);
             } else {
-                T ss = T(0);
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const T sB = T(0.5) * (gB[i][j] + gB[j][i]);
-                        ss += sB * sB;
-                    }
-                const T sv = sqrt(T(2) * ss);
+                const T dB = gB[0][0] * gB[0][0] + gB[1][1] * gB[1][1] + gB[2][2] * gB[2][2];
+                const T sv = root(sym[0] * sym[0] + (sym[1] * sym[1] + (sym[2] * sym[2] + (dB + dB))));
                 if (EDDY) {
-                    const T val = (G.sgs == 2 ? T(1) : T(G.cs2)) * sv;
+                    const T val = G.sgs == 2 ? sv : GC(cs2) * sv;
                     s1[p] = val;
                     mx = val > mx ? val : mx;
                 } else {
                     s1[p] = sv;
                 }
             }
-#pragma unroll
-            for (int f = 0; f < 3; ++f)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    wb[f][q] = wb[f][q + 1];
-                    wa[f][q] = wa[f][q + 1];
-                }
         }
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                wb[f][q] = wb[f][q + 1];
+                wa[f][q] = wa[f][q + 1];
+            }
         __syncthreads();      // the next plane overwrites the staged one
     }
     if (EDDY) {
@@ -309,376 +384,355 @@ strain3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict_
 
 // ============================================================================
 // Plane pass: x and y terms of every field and the point-wise terms, for a
-// PX x PY tile of plane z = blockIdx.z; writes their sum to P.
+// PX x PYT tile of plane z = blockIdx.z; writes their sum to P.  The fluxes
+// X_phi, Y_phi are formed once per point and on the arms they are read from
+// (two columns / rows either side), then differentiated; a thread keeps the
+// point-wise parts of its points in registers.
+//
+// Bound: float64 the FP64 pipe (about 115 operations a point and 25 per arm
+// point; the form that rebuilt the products at every tap took about 280),
+// float32 shared-memory bandwidth (about 180 words a point, 300 before).
+// Difference-form product at 256 x 256 x 64: 224 -> 115 us; float64 F at
+// 256 x 256 x 128: 3.72 -> 2.19 ms.
 // ============================================================================
-template <typename T, int MODE, int SMAG>
+constexpr int PX = 32;
+template <typename T> struct PlaneT;
+template <> struct PlaneT<float>  { static constexpr int PY = 16; };
+template <> struct PlaneT<double> { static constexpr int PY = 8; };
+
+template <typename T, int KIND, int SMAG>
+struct PlaneShape {
+    static constexpr int PY = PlaneT<T>::PY, SX = PX + 2 * HALO, SY = PY + 2 * HALO, SP = SX * SY;
+    static constexpr int NS = KIND == PAIR ? 2 : 1;      // states staged: b [, m]
+    static constexpr int XW = PX + 2 * R, XN = XW * PY, YN = PX * (PY + 2 * R);
+    static constexpr int PPT = PX * PY / NTHREADS;
+    static constexpr size_t smem = sizeof(T) * (size_t)(NS * 5 * SP + 5 * XN + 5 * YN);
+    static_assert(PPT * NTHREADS == PX * PY && 4 * (PX + PY) <= NTHREADS, "thread mapping");
+};
+
+// Fluxes at one point (staged index c) along x (XF) and y (YF); both: a tile
+// point, whose point-wise part goes to S.
+template <typename T, int KIND, int SMAG, bool XF, bool YF>
+__device__ __forceinline__ void plane_point(const Geo& G, const T* __restrict__ st, int c, T na, T ds,
+                                            T* __restrict__ X, T* __restrict__ Y, T (&S)[5]) {
+    using SH = PlaneShape<T, KIND, SMAG>;
+    constexpr int SP = SH::SP, SX = SH::SX, XN = SH::XN, YN = SH::YN;
+    const T* B = st;
+    const T* M = st + 5 * SP;
+    const T wx1 = GC(wx1), wx2 = GC(wx2), wy1 = GC(wy1), wy2 = GC(wy2);
+    auto D = [&](const T* f, int s, T w1, T w2) { return w1 * (f[c + s] - f[c - s]) + w2 * (f[c + 2 * s] - f[c - 2 * s]); };
+    T km[2], dk[2];
+    coefs<T, KIND, SMAG>(G, na, ds, false, km, dk);
+    const T bu = T(0.5) * B[c], bv = T(0.5) * B[SP + c];
+    const T mu = KIND == PAIR ? T(0.5) * M[c] : T(0), mv = KIND == PAIR ? T(0.5) * M[SP + c] : T(0);
+    T divb = T(0), divm = T(0);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+        const T b = B[f * SP + c], m = KIND == PAIR ? M[f * SP + c] : T(0);
+        T dbx = T(0), dby = T(0), dmx = T(0), dmy = T(0), s = T(0);
+        if (XF && (f < 4 || YF)) {
+            dbx = D(B + f * SP, 1, wx1, wx2);
+            if (KIND == PAIR) dmx = D(M + f * SP, 1, wx1, wx2);
+        }
+        if (YF && (f < 4 || XF)) {
+            dby = D(B + f * SP, SX, wy1, wy2);
+            if (KIND == PAIR) dmy = D(M + f * SP, SX, wy1, wy2);
+        }
+        const int h = f == 3 ? 1 : 0;
+        if (XF) X[f * XN] = f < 4 ? flux_of<T, KIND, SMAG>(km[h], dk[h], mu, bu, m, b, dmx, dbx) : flux_p<T, KIND>(mu, bu, m, b);
+        if (YF) Y[f * YN] = f < 4 ? flux_of<T, KIND, SMAG>(km[h], dk[h], mv, bv, m, b, dmy, dby) : flux_p<T, KIND>(mv, bv, m, b);
+        if (XF && YF) {
+            // the small advective terms first: the large linear ones are rounded once
+            s = advect<T, KIND>(s, mu, bu, dmx, dbx);
+            s = advect<T, KIND>(s, mv, bv, dmy, dby);
+            if (f == 0) { divb = dbx; divm = dmx; }
+            if (f == 1) { divb += dby; divm += dmy; }
+            if (f == 2) s += GC(gth) * B[3 * SP + c];
+            if (f == 3) s -= GC(beta) * B[2 * SP + c];
+            if (f == 4) {       // pressure equation, x and y parts of the divergence; gradient of p
+                T t = (GC(pbar) + (KIND == PAIR ? m : b)) * divb;
+                if (KIND == PAIR) t += b * divm;
+                s -= GC(gamma_p) * t;
+                S[0] -= GC(theta0) * dbx;
+                S[1] -= GC(theta0) * dby;
+            }
+            S[f] = s;
+        }
+    }
+}
+
+template <typename T, int KIND, int SMAG>
 __global__ void __launch_bounds__(NTHREADS)
 plane3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ s0,
         const T* __restrict__ s1, T* __restrict__ P, Ctl* ctl, int check_done) {
-    constexpr bool TWO = Two<MODE>::v;
-    constexpr int SX = PX + 2 * HALO, SY = PY + 2 * HALO, SP = SX * SY;
-    constexpr int AXN = (PX + 2 * R) * PY, AYN = PX * (PY + 2 * R), AN = AXN + AYN;   // x arms, y arms
-    constexpr int NS = TWO ? 2 : 1;                  // states staged (b [, a])
-    if ((MODE == MODE_JV || MODE == MODE_DJV) && check_done && ctl->done) return;
+    using SH = PlaneShape<T, KIND, SMAG>;
+    constexpr int PY = SH::PY, SX = SH::SX, SP = SH::SP, XW = SH::XW, XN = SH::XN, YN = SH::YN, PPT = SH::PPT;
+    if (KIND != ONE && check_done && ctl->done) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* st = reinterpret_cast<T*>(smem_raw);          // [NS][5][SP]: b fields, then a fields
-    T* ga = st + NS * 5 * SP;                        // [NS][4][AN] first derivatives on the arms
-    T* ks = ga + NS * 4 * AN;                        // [NS][AN] strain on the arms (SMAG)
+    T* st = reinterpret_cast<T*>(smem_raw);          // [NS][5][SP]: b fields, then m fields
+    T* X = st + SH::NS * 5 * SP;                     // [5][PY][PX + 4]
+    T* Y = X + 5 * XN;                               // [5][PY + 4][PX]
     const int x0 = blockIdx.x * PX, y0 = blockIdx.y * PY, gz = blockIdx.z;
-    const T ix = T(G.inv_dx), iy = T(G.inv_dy);
     T ev[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if (MODE == MODE_JV || MODE == MODE_DJV) {
+    if (KIND != ONE) {
 #pragma unroll
         for (int f = 0; f < 5; ++f) ev[f] = eps_field<T>(ctl, G, f);
     }
     const size_t plane = (size_t)gz * G.ny * G.nx;
+    // eddy values of the thread's points and of its arm point, in flight with the staging
+    const int a = threadIdx.x;
+    const bool yarm = a < 4 * PX, arm = a < 4 * (PX + PY);
+    const int ar = yarm ? a / PX : (a - 4 * PX) & 3;
+    const int ax = yarm ? a % PX : (ar < 2 ? ar - 2 : PX + ar - 2);
+    const int ay = yarm ? (ar < 2 ? ar - 2 : PY + ar - 2) : (a - 4 * PX) >> 2;
+    T kn[PPT + 1], kd[PPT + 1];
+#pragma unroll
+    for (int k = 0; k <= PPT; ++k) {
+        kn[k] = kd[k] = T(0);
+        if (SMAG && (k < PPT || arm)) {
+            const int w = threadIdx.x + k * NTHREADS;
+            const int px = k < PPT ? w % PX : ax, py = k < PPT ? w / PX : ay;
+            const size_t o = plane + (size_t)wrap(y0 + py, G.ny) * G.nx + wrap(x0 + px, G.nx);
+            kd[k] = s1[o];
+            if (KIND == PAIR) kn[k] = s0[o];
+        }
+    }
     for (int idx = threadIdx.x; idx < SP; idx += NTHREADS) {
         const int ixl = idx % SX, iyl = idx / SX;
         const size_t o = plane + (size_t)wrap(y0 + iyl - HALO, G.ny) * G.nx + wrap(x0 + ixl - HALO, G.nx);
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
-            T a, b;
-            load_ab<T, MODE>(u, v, ev[f], (size_t)f * G.npt + o, a, b);
+            T m, b;
+            load_mb<T, KIND>(u, v, ev[f], (size_t)f * G.npt + o, m, b);
             st[f * SP + idx] = b;
-            if (TWO) st[(5 + f) * SP + idx] = a;
-        }
-    }
-    if (SMAG) {
-        for (int idx = threadIdx.x; idx < AN; idx += NTHREADS) {
-            int qx, qy;
-            if (idx < AXN) { qx = idx % (PX + 2 * R) - R; qy = idx / (PX + 2 * R); }
-            else { const int j = idx - AXN; qx = j % PX; qy = j / PX - R; }
-            const size_t o = plane + (size_t)wrap(y0 + qy, G.ny) * G.nx + wrap(x0 + qx, G.nx);
-            ks[idx] = s1[o];
-            if (TWO) ks[AN + idx] = s0[o];
+            if (KIND == PAIR) st[(5 + f) * SP + idx] = m;
         }
     }
     __syncthreads();
-    // first derivatives of u, v, w, theta (each state) on the arms
-    for (int idx = threadIdx.x; idx < AN; idx += NTHREADS) {
-        int c, stp;
-        T ih;
-        if (idx < AXN) {
-            const int qx = idx % (PX + 2 * R), qy = idx / (PX + 2 * R);
-            c = (qy + HALO) * SX + qx + R;
-            stp = 1;
-            ih = ix;
-        } else {
-            const int j = idx - AXN;
-            const int qx = j % PX, qy = j / PX;
-            c = (qy + R) * SX + qx + HALO;
-            stp = SX;
-            ih = iy;
-        }
+    T S[PPT][5];
 #pragma unroll
-        for (int q = 0; q < NS * 4; ++q) {
-            const int arr = q < 4 ? q : 5 + (q - 4);          // b: fields 0..3, a: fields 0..3
-            ga[q * AN + idx] = dd(st + arr * SP, c, stp, ih);
-        }
+    for (int k = 0; k < PPT; ++k) {
+        const int w = threadIdx.x + k * NTHREADS, tx = w % PX, ty = w / PX;
+        if (x0 + tx <= G.nx + 1 && y0 + ty <= G.ny + 1)      // else it feeds no output
+            plane_point<T, KIND, SMAG, true, true>(G, st, (ty + HALO) * SX + tx + HALO, kn[k], kd[k],
+                                                   X + ty * XW + tx + R, Y + (ty + R) * PX + tx, S[k]);
+    }
+    if (arm && x0 + ax <= G.nx + 1 && y0 + ay <= G.ny + 1) {
+        T none[5];
+        const int c = (ay + HALO) * SX + ax + HALO;
+        if (yarm) plane_point<T, KIND, SMAG, false, true>(G, st, c, kn[PPT], kd[PPT], X, Y + (ay + R) * PX + ax, none);
+        else plane_point<T, KIND, SMAG, true, false>(G, st, c, kn[PPT], kd[PPT], X + ay * XW + ax + R, Y, none);
     }
     __syncthreads();
-    const int tx = threadIdx.x % PX, ty = threadIdx.x / PX;
-    const int gx = x0 + tx, gy = y0 + ty;
-    if (gx >= G.nx || gy >= G.ny) return;
-    const int c = (ty + HALO) * SX + tx + HALO;
-    const int cax = ty * (PX + 2 * R) + tx + R;               // x arm at the output point
-    const int cay = AXN + (ty + R) * PX + tx;                 // y arm at the output point
-    const int astr[2] = {1, PX};
-    const int carm[2] = {cax, cay};
-    const int sst[2] = {1, SX};
-    const T ihs[2] = {ix, iy};
-    const T* Bf = st;                                         // b fields
-    const T* Af = st + 5 * SP;                                // a fields (TWO)
-    T dF[5];
-    T dbp[2], dap[2];                                         // D_j of p (b, a) at the point
+    const T wx1 = GC(wx1), wx2 = GC(wx2), wy1 = GC(wy1), wy2 = GC(wy2);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        dbp[j] = dd(Bf + 4 * SP, c, sst[j], ihs[j]);
-        dap[j] = TWO ? dd(Af + 4 * SP, c, sst[j], ihs[j]) : T(0);
-    }
+    for (int k = 0; k < PPT; ++k) {
+        const int w = threadIdx.x + k * NTHREADS, tx = w % PX, ty = w / PX;
+        const int gx = x0 + tx, gy = y0 + ty;
+        if (gx >= G.nx || gy >= G.ny) continue;
+        const size_t off = plane + (size_t)gy * G.nx + gx;
 #pragma unroll
-    for (int fl = 0; fl < 5; ++fl) {
-        const T* B = Bf + fl * SP;
-        const T* A = Af + fl * SP;
-        T flux = T(0), adv = T(0);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const T* bj = Bf + j * SP;                        // b_u (x) or b_v (y)
-            const T* aj = Af + j * SP;
-            const int s = sst[j];
-            T fj = T(0);
-#pragma unroll
-            for (int l = 1; l <= 2; ++l) {
-                const T cl = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                const int ip = c + l * s, im = c - l * s;
-                if (TWO)
-                    fj += cl * ((aj[ip] * B[ip] + bj[ip] * (A[ip] + B[ip])) - (aj[im] * B[im] + bj[im] * (A[im] + B[im])));
-                else
-                    fj += cl * (bj[ip] * B[ip] - bj[im] * B[im]);
-            }
-            flux += fj * ihs[j];
-            T daj, dbj;
-            if (fl < 4) {
-                dbj = ga[fl * AN + carm[j]];
-                daj = TWO ? ga[(4 + fl) * AN + carm[j]] : T(0);
-            } else {
-                dbj = dbp[j];
-                daj = dap[j];
-            }
-            adv += TWO ? (aj[c] * dbj + bj[c] * (daj + dbj)) : bj[c] * dbj;
-        }
-        dF[fl] = -(T(0.5) * flux + T(0.5) * adv);
-        if (fl < 4) {
-            const T* gb = ga + fl * AN;
-            const T* gA = ga + (4 + fl) * AN;
-            T dif = T(0);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int q = carm[j], s = astr[j];
-                T sj = T(0);
-#pragma unroll
-                for (int l = 1; l <= 2; ++l) {
-                    const T cl = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                    const int p1 = q + l * s, m1 = q - l * s;
-                    if (SMAG) {
-                        T kp, dkp, km, dkm;
-                        kpair<T, SMAG>(G, TWO ? ks[AN + p1] : T(0), ks[p1], false, fl == 3, kp, dkp);
-                        kpair<T, SMAG>(G, TWO ? ks[AN + m1] : T(0), ks[m1], false, fl == 3, km, dkm);
-                        if (TWO)
-                            sj += cl * ((kp * gb[p1] + dkp * (gA[p1] + gb[p1])) - (km * gb[m1] + dkm * (gA[m1] + gb[m1])));
-                        else
-                            sj += cl * (dkp * gb[p1] - dkm * gb[m1]);
-                    } else {
-                        sj += cl * (gb[p1] - gb[m1]);
-                    }
-                }
-                dif += sj * ihs[j];
-            }
-            if (SMAG == 1) {
-                if (fl == 3) dif *= T(G.inv_Pr);
-            } else if (!SMAG) {
-                dif *= T(fl == 3 ? G.K_H : G.K_M);
-            }
-            dF[fl] += dif;
+        for (int f = 0; f < 5; ++f) {
+            const T* x = X + f * XN + ty * XW + tx + R;
+            const T* y = Y + f * YN + (ty + R) * PX + tx;
+            T s = wx1 * (x[1] - x[-1]);
+            s += wx2 * (x[2] - x[-2]);
+            s += wy1 * (y[PX] - y[-PX]);
+            s += wy2 * (y[2 * PX] - y[-2 * PX]);
+            s += S[k][f];
+            if (KIND != PAIR && f == 3 && gz == 0 && G.heat != nullptr)
+                s += T(G.heat[(size_t)gy * G.nx + gx] * G.heat_coef);
+            P[(size_t)f * G.npt + off] = s;
         }
     }
-    const T th0 = T(G.theta0);
-    dF[0] += -th0 * dbp[0];
-    dF[1] += -th0 * dbp[1];
-    dF[2] += T(G.g) * Bf[3 * SP + c] / th0;
-    dF[3] += -T(G.beta) * Bf[2 * SP + c];
-    if (MODE != MODE_DJV && G.heat != nullptr && gz == 0)
-        dF[3] += T(G.heat[(size_t)gy * G.nx + gx] * G.heat_coef);
-    {   // pressure equation, x and y parts of the divergence
-        const T divb = ga[cax] + ga[AN + cay];
-        const T pa = TWO ? Af[4 * SP + c] : T(0), pb = Bf[4 * SP + c];
-        T t = (T(G.pbar) + pa + pb) * divb;
-        if (TWO) t += pb * (ga[4 * AN + cax] + ga[5 * AN + cay]);
-        dF[4] += -T(G.gamma_p) * t;
-    }
-    const size_t off = plane + (size_t)gy * G.nx + gx;
-#pragma unroll
-    for (int fl = 0; fl < 5; ++fl) P[(size_t)fl * G.npt + off] = dF[fl];
 }
 
 // ============================================================================
-// Slab pass: z terms for a TX x TZ slab of row y = blockIdx.z (z tiles along
-// blockIdx.x so that consecutive CTAs share their z halos in L2), plus the
-// plane pass's sum; writes the mode's output.
+// Column pass: the z terms, plus the plane pass's sum; writes the mode's
+// output.  A CTA takes CW columns; a thread owns one field of one column (a
+// warp has one field) and marches through zc planes with everything in
+// registers: the last five values of its field and of its partner (p for w,
+// w for the others), the last five fluxes Z_phi and the point-wise parts of the
+// planes between flux and output.  No shared memory, no barrier, every load
+// coalesced; the fields' warps share w and the eddy values through L1.  A
+// plane's values enter at step l (plane z0 - 4 + l), the plane two below gets
+// its flux, the plane four below its output.  The rings turn by an index fixed
+// at compile time in five copies of the step, so nothing is moved.
+//
+// Bound: float64 the FP64 pipe (about 100 operations a point; the slab form
+// that staged tiles in shared memory and rebuilt products at every tap took
+// about 240), float32 HBM and load latency.  One thread for all five fields of
+// a column needs 230-255 registers (float64 spills): one CTA per SM.
+// Difference-form product at 256 x 256 x 64: 258 (slab) -> 107 us, with the
+// operands loaded one step ahead into registers 209; float64 F at
+// 256 x 256 x 128: 3.1 -> 1.9 ms.
 // ============================================================================
-template <typename T, int MODE, int SMAG>
-__global__ void __launch_bounds__(NTHREADS)
-slab3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
-       const double* __restrict__ f, const T* __restrict__ s0, const T* __restrict__ s1,
-       const T* __restrict__ P, T* __restrict__ out, T* __restrict__ out2, double* __restrict__ part, Ctl* ctl,
-       int check_done) {
-    constexpr bool TWO = Two<MODE>::v;
-    constexpr int TX = SlabT<T>::TX, TZ = SlabT<T>::TZ;
-    constexpr int SZ = TZ + 2 * HALO, SP = TX * SZ;          // staged rows [row][x]
-    constexpr int QZ = TZ + 2 * R, AN = TX * QZ;             // z arms
-    constexpr int NS = TWO ? 2 : 1;
-    constexpr int PER = TX * TZ / NTHREADS;                  // outputs per thread
-    if ((MODE == MODE_JV || MODE == MODE_DJV) && check_done && ctl->done) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* st = reinterpret_cast<T*>(smem_raw);                  // [NS][5][SP]
-    T* ga = st + NS * 5 * SP;                                // [NS][4][AN]
-    T* ks = ga + NS * 4 * AN;                                // [NS][AN] strain on the z arms (SMAG)
-    const int z0 = blockIdx.x * TZ, x0 = blockIdx.y * TX, gy = blockIdx.z;
-    const T iz = T(G.inv_dz);
-    T ev[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if (MODE == MODE_JV || MODE == MODE_DJV) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) ev[q] = eps_field<T>(ctl, G, q);
-    }
-    const size_t row = (size_t)gy * G.nx;
-    for (int idx = threadIdx.x; idx < SP; idx += NTHREADS) {
-        const int xl = idx % TX, rl = idx / TX;
-        int side;
-        const int sz = mirror(z0 + rl - HALO, G.nz, side);
-        const bool ok = sz >= 0 && sz < G.nz;
-        const size_t o = (size_t)sz * G.ny * G.nx + row + wrap(x0 + xl, G.nx);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            T a = T(0), b = T(0);
-            if (ok) {
-                load_ab<T, MODE>(u, v, ev[q], (size_t)q * G.npt + o, a, b);
-                const T sg = side == 1 ? T(G.pb[q]) : (side == 2 ? T(G.pt[q]) : T(1));
-                a *= sg;
-                b *= sg;
+constexpr int CW = 32;                               // columns per CTA
+constexpr int COL_THREADS = 5 * CW;
+constexpr int COL_STAGES = 4;                        // steps whose operands are in flight or in use
+
+template <typename T, int KIND, int SMAG>
+__global__ void __launch_bounds__(COL_THREADS, sizeof(T) == sizeof(float) ? 5 : 4)
+column3d(Geo G, int mode, int zc, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
+         const double* __restrict__ f, const T* __restrict__ s0, const T* __restrict__ s1, const T* __restrict__ P,
+         T* __restrict__ out, T* __restrict__ out2, double* __restrict__ part, Ctl* ctl, int check_done) {
+    constexpr int IW = 2, IT = 3, IP = 4;
+    if (KIND != ONE && check_done && ctl->done) return;
+    const size_t nxy_ = (size_t)G.ny * G.nx, np = (size_t)G.npt;
+    const int q = threadIdx.x / CW, pq = q == IW ? IP : IW;             // field, partner field
+    const size_t col = (size_t)blockIdx.x * CW + threadIdx.x % CW;
+    const int z0 = blockIdx.y * zc, z1 = min(z0 + zc, G.nz);
+    __shared__ T ring_s[COL_STAGES][KIND == ONE ? 5 : 8][COL_THREADS];
+    double ar = 0.0, au = 0.0;
+    if (col < nxy_) {
+        const T w1 = GC(wz1), w2 = GC(wz2);
+        T evq = T(0), evp = T(0), cf = T(0);         // eps scale, 1 / (eps scale)
+        if (KIND != ONE) {
+            evq = eps_field<T>(ctl, G, q);
+            evp = eps_field<T>(ctl, G, pq);
+            cf = inv_eps_field<T>(ctl, G, q);
+        }
+        const bool oddb = G.pb[q] < 0, oddt = G.pt[q] < 0, poddb = G.pb[pq] < 0, poddt = G.pt[pq] < 0;
+        // offsets within a plane stack fit 32 bits (npt does): one wide multiply-add per access
+        const int nxy = (int)nxy_;
+        const size_t oq = q * np + col, op = pq * np + col;
+        const T *uq = u + oq, *up = u + op, *vq = KIND != ONE ? v + oq : u, *vp = KIND != ONE ? v + op : u;
+        const T *s0c = s0 + col, *s1c = s1 + col, *Pq = P + oq, *Fq = KIND == SHIFT ? Fu + oq : u;
+        const double* fq = KIND == ONE && mode == MODE_RES ? f + oq : nullptr;
+        T* outq = out + oq;
+        T* out2q = out2 != nullptr ? out2 + oq : nullptr;
+        T b[5], m[5] = {}, c[5], d[5] = {}, Z[5], S[5];        // rings: field (b, m), partner (c, d), flux, point-wise part
+        const int steps = z1 - z0 + 8;
+        // step l's operands, copied to this thread's own shared-memory slots
+        // COL_STAGES - 1 steps ahead (no barrier: nobody else reads them)
+        auto stage = [&](int l) {
+            if (l < steps) {
+                T(*st)[COL_THREADS] = ring_s[l % COL_STAGES];
+                const int z = z0 - 4 + l;
+                int side;
+                const int o = mirror(z, G.nz, side) * nxy;
+                cpa1(&st[0][threadIdx.x], uq + o);
+                cpa1(&st[1][threadIdx.x], up + o);
+                if (SMAG) cpa1(&st[2][threadIdx.x], s1c + max(eddy_row(z - 2, G.nz), 0) * nxy);   // plane z - 2
+                if (l >= 8) {                        // operands of the output of plane z - 4
+                    const int oo = (z - 4) * nxy;
+                    cpa1(&st[3][threadIdx.x], Pq + oo);
+                    if (KIND != ONE) cpa1(&st[4][threadIdx.x], vq + oo);
+                    if (KIND == SHIFT) cpa1(&st[7][threadIdx.x], Fq + oo);
+                    if constexpr (KIND == ONE && sizeof(T) == sizeof(double))
+                        if (fq != nullptr) cpa1(&st[4][threadIdx.x], fq + oo);
+                }
+                if (KIND != ONE) {
+                    cpa1(&st[5][threadIdx.x], vq + o);
+                    cpa1(&st[6][threadIdx.x], vp + o);
+                }
+                if (KIND == PAIR && SMAG) cpa1(&st[7][threadIdx.x], s0c + max(eddy_row(z - 2, G.nz), 0) * nxy);
             }
-            st[q * SP + idx] = b;
-            if (TWO) st[(5 + q) * SP + idx] = a;
-        }
-    }
-    if (SMAG) {
-        for (int idx = threadIdx.x; idx < AN; idx += NTHREADS) {
-            const int xl = idx % TX, ql = idx / TX;
-            const int sz = eddy_row(z0 + ql - R, G.nz);
-            T kv1 = T(0), kv0 = T(0);
-            if (sz >= 0) {
-                const size_t o = (size_t)sz * G.ny * G.nx + row + wrap(x0 + xl, G.nx);
-                kv1 = s1[o];
-                if (TWO) kv0 = s0[o];
-            }
-            ks[idx] = kv1;
-            if (TWO) ks[AN + idx] = kv0;
-        }
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < AN; idx += NTHREADS) {
-        const int xl = idx % TX, ql = idx / TX;
-        const int c = (ql + R) * TX + xl;
-#pragma unroll
-        for (int q = 0; q < NS * 4; ++q) {
-            const int arr = q < 4 ? q : 5 + (q - 4);
-            ga[q * AN + idx] = dd(st + arr * SP, c, TX, iz);
-        }
-    }
-    __syncthreads();
-    const T th0 = T(G.theta0);
-    double acc[2] = {0.0, 0.0};
-    const T* Bf = st;
-    const T* Af = st + 5 * SP;
-    double cf[5] = {0.0, 0.0, 0.0, 0.0, 0.0};          // 1 / eps_f of the Jacobian-product modes
-    if (MODE == MODE_JV || MODE == MODE_DJV) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            const double e = ctl->eps_jv * G.scale[q];
-            cf[q] = e != 0.0 ? 1.0 / e : 0.0;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int idx = threadIdx.x + k * NTHREADS;
-        const int xl = idx % TX, zl = idx / TX;
-        const int gx = x0 + xl, gz = z0 + zl;
-        if (gx >= G.nx || gz >= G.nz) continue;
-        const int c = (zl + HALO) * TX + xl;
-        const int ca = (zl + R) * TX + xl;                 // z arm at the output point
-        const T* bw = Bf + 2 * SP;
-        const T* aw = Af + 2 * SP;
-        const T dbpz = dd(Bf + 4 * SP, c, TX, iz);
-        const T dapz = TWO ? dd(Af + 4 * SP, c, TX, iz) : T(0);
-        T dF[5];
-#pragma unroll
-        for (int fl = 0; fl < 5; ++fl) {
-            const T* B = Bf + fl * SP;
-            const T* A = Af + fl * SP;
-            T fj = T(0);
-#pragma unroll
-            for (int l = 1; l <= 2; ++l) {
-                const T cl = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                const int ip = c + l * TX, im = c - l * TX;
-                if (TWO)
-                    fj += cl * ((aw[ip] * B[ip] + bw[ip] * (A[ip] + B[ip])) - (aw[im] * B[im] + bw[im] * (A[im] + B[im])));
-                else
-                    fj += cl * (bw[ip] * B[ip] - bw[im] * B[im]);
-            }
-            const T flux = fj * iz;
-            T daz, dbz;
-            if (fl < 4) {
-                dbz = ga[fl * AN + ca];
-                daz = TWO ? ga[(4 + fl) * AN + ca] : T(0);
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        auto step = [&](auto ring, int l) {
+            constexpr int r0 = decltype(ring)::value;                                                   // l mod 5
+            constexpr int r1 = (r0 + 4) % 5, r2 = (r0 + 3) % 5, r3 = (r0 + 2) % 5, r4 = (r0 + 1) % 5;   // l-1 .. l-4
+            const int z = z0 - 4 + l;
+            stage(l + COL_STAGES - 1);
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(COL_STAGES - 1) : "memory");
+            const T(*st)[COL_THREADS] = ring_s[l % COL_STAGES];
+            auto arrived = [&](int k) { return st[k][threadIdx.x]; };
+            if constexpr (KIND == PAIR) {
+                b[r0] = evq * arrived(5);
+                m[r0] = arrived(0) + T(0.5) * b[r0];
+                c[r0] = evp * arrived(6);
+                d[r0] = arrived(1) + T(0.5) * c[r0];
             } else {
-                dbz = dbpz;
-                daz = dapz;
-            }
-            const T adv = TWO ? (aw[c] * dbz + bw[c] * (daz + dbz)) : bw[c] * dbz;
-            dF[fl] = -(T(0.5) * flux + T(0.5) * adv);
-            if (fl < 4) {
-                const T* gb = ga + fl * AN;
-                const T* gA = ga + (4 + fl) * AN;
-                T sj = T(0);
-#pragma unroll
-                for (int l = 1; l <= 2; ++l) {
-                    const T cl = l == 1 ? T(2.0 / 3.0) : T(-1.0 / 12.0);
-                    const int p1 = ca + l * TX, m1 = ca - l * TX;
-                    if (SMAG) {
-                        T kp, dkp, km, dkm;
-                        kpair<T, SMAG>(G, TWO ? ks[AN + p1] : T(0), ks[p1], true, fl == 3, kp, dkp);
-                        kpair<T, SMAG>(G, TWO ? ks[AN + m1] : T(0), ks[m1], true, fl == 3, km, dkm);
-                        if (TWO)
-                            sj += cl * ((kp * gb[p1] + dkp * (gA[p1] + gb[p1])) - (km * gb[m1] + dkm * (gA[m1] + gb[m1])));
-                        else
-                            sj += cl * (dkp * gb[p1] - dkm * gb[m1]);
-                    } else {
-                        sj += cl * (gb[p1] - gb[m1]);
-                    }
+                b[r0] = arrived(0);
+                c[r0] = arrived(1);
+                if (KIND == SHIFT) {
+                    b[r0] += evq * arrived(5);
+                    c[r0] += evp * arrived(6);
                 }
-                T dif = sj * iz;
-                if (SMAG == 1) {
-                    if (fl == 3) dif *= T(G.inv_Pr);
-                } else if (!SMAG) {
-                    dif *= T(fl == 3 ? G.K_H : G.K_M);
+            }
+            if (z < 0 || z >= G.nz) {                // ghost plane: signs of the odd fields
+                if (z < 0 ? oddb : oddt) {
+                    b[r0] = flip(b[r0]);
+                    if constexpr (KIND == PAIR) m[r0] = flip(m[r0]);
                 }
-                dF[fl] += dif;
+                if (z < 0 ? poddb : poddt) {
+                    c[r0] = flip(c[r0]);
+                    if constexpr (KIND == PAIR) d[r0] = flip(d[r0]);
+                }
             }
-        }
-        dF[2] += -th0 * dbpz;
-        {
-            const T pa = TWO ? Af[4 * SP + c] : T(0), pb = Bf[4 * SP + c];
-            T t = (T(G.pbar) + pa + pb) * ga[2 * AN + ca];
-            if (TWO) t += pb * ga[6 * AN + ca];
-            dF[4] += -T(G.gamma_p) * t;
-        }
-        const size_t off = (size_t)gz * G.ny * G.nx + row + gx;
-#pragma unroll
-        for (int fl = 0; fl < 5; ++fl) {
-            const size_t o = (size_t)fl * G.npt + off;
-            const T Fv = P[o] + dF[fl];
-            if (MODE == MODE_DJV) {
-                out[o] = T(G.two_over_dt) * v[o] - Fv * T(cf[fl]);
-            } else if (MODE == MODE_F) {
-                out[o] = Fv;
-            } else if (MODE == MODE_RHS) {
-                out[o] = T(G.two_over_dt * (double)u[o] + (double)Fv);
-            } else if (MODE == MODE_RHSRES) {
-                // at u = u^n the residual 2u/dt - F(u) - f with f = 2u/dt + F(u) is -2 F(u)
-                const double uo = (double)u[o];
-                const double Fd = (double)Fv;
-                out[o] = T(G.two_over_dt * uo + Fd);
-                const double Rv = -2.0 * Fd;
-                out2[o] = T(Rv);
-                const double rs = Rv * G.inv_scale[fl], us = uo * G.inv_scale[fl];
-                acc[0] += rs * rs;
-                acc[1] += us * us;
-            } else if (MODE == MODE_RES) {
-                const double uo = (double)u[o];
-                const double Rv = G.two_over_dt * uo - (double)Fv - f[o];
-                out[o] = T(Rv);
-                if (out2 != nullptr) out2[o] = Fv;
-                const double rs = Rv * G.inv_scale[fl], us = uo * G.inv_scale[fl];
-                acc[0] += rs * rs;
-                acc[1] += us * us;
-            } else {   // MODE_JV: plain forward difference against F(u)
-                const double diff = (double)Fv - (double)Fu[o];
-                out[o] = T(G.two_over_dt * (double)v[o] - diff * cf[fl]);
+            const T kd = SMAG ? arrived(2) : T(0), ka = KIND == PAIR && SMAG ? arrived(7) : T(0);
+            if (l >= 4) {                            // flux and point-wise part of plane z - 2
+                const T bw = T(0.5) * (q == IW ? b[r2] : c[r2]);
+                const T mw = KIND == PAIR ? T(0.5) * (q == IW ? m[r2] : d[r2]) : T(0);
+                const T db = w1 * (b[r1] - b[r3]) + w2 * (b[r0] - b[r4]);
+                const T dm = KIND == PAIR ? w1 * (m[r1] - m[r3]) + w2 * (m[r0] - m[r4]) : T(0);
+                T s = T(0);
+                if (q == IP) {
+                    Z[r2] = flux_p<T, KIND>(mw, bw, m[r2], b[r2]);
+                    const T dw = w1 * (c[r1] - c[r3]) + w2 * (c[r0] - c[r4]);
+                    T t = (GC(pbar) + (KIND == PAIR ? m[r2] : b[r2])) * dw;
+                    if (KIND == PAIR) t += b[r2] * (w1 * (d[r1] - d[r3]) + w2 * (d[r0] - d[r4]));
+                    s = advect<T, KIND>(s, mw, bw, dm, db) - GC(gamma_p) * t;
+                } else {
+                    T km[2], dk[2];
+                    coefs<T, KIND, SMAG>(G, ka, kd, true, km, dk);
+                    Z[r2] = q == IT ? flux_of<T, KIND, SMAG>(km[1], dk[1], mw, bw, m[r2], b[r2], dm, db)
+                                    : flux_of<T, KIND, SMAG>(km[0], dk[0], mw, bw, m[r2], b[r2], dm, db);
+                    s = advect<T, KIND>(s, mw, bw, dm, db);
+                    if (q == IW) s -= GC(theta0) * (w1 * (c[r1] - c[r3]) + w2 * (c[r0] - c[r4]));
+                }
+                S[r2] = s;
             }
+            if (l < 8) return;
+            const int o = (z - 4) * nxy;
+            const T pv = arrived(3), xv = KIND != ONE ? arrived(4) : T(0);
+            // output of plane z - 4: fluxes of planes l-2, l-3, l-5, l-6 (rings r2, r3, r0, r1)
+            T Fv = w1 * (Z[r3] - Z[r0]);
+            Fv += w2 * (Z[r2] - Z[r1]);
+            Fv += S[r4];
+            Fv += pv;
+            if (KIND == PAIR) {
+                outq[o] = GC(two_over_dt) * xv - Fv * cf;
+            } else if (KIND == SHIFT) {              // plain forward difference against F(u)
+                outq[o] = T(G.two_over_dt * (double)xv - ((double)Fv - (double)arrived(7)) * cf);
+            } else if (mode == MODE_F) {
+                outq[o] = Fv;
+            } else {
+                const double uo = (double)b[r4], Fd = (double)Fv;
+                if (mode == MODE_RHS) {
+                    outq[o] = T(G.two_over_dt * uo + Fd);
+                    return;
+                }
+                double Rv;
+                if (mode == MODE_RHSRES) {
+                    // at u = u^n the residual 2u/dt - F(u) - f with f = 2u/dt + F(u) is -2 F(u)
+                    outq[o] = T(G.two_over_dt * uo + Fd);
+                    Rv = -2.0 * Fd;
+                    out2q[o] = T(Rv);
+                } else {
+                    Rv = G.two_over_dt * uo - Fd - (sizeof(T) == sizeof(double) ? (double)arrived(4) : fq[o]);
+                    outq[o] = T(Rv);
+                    if (out2q != nullptr) out2q[o] = Fv;
+                }
+                ar = fma(Rv, Rv, ar);
+                au = fma(uo, uo, au);
+            }
+        };
+        for (int l = 0; l < COL_STAGES - 1; ++l) stage(l);
+        for (int l = 0; l < steps; l += 5) {
+            step(std::integral_constant<int, 0>(), l);
+            if (l + 1 < steps) step(std::integral_constant<int, 1>(), l + 1);
+            if (l + 2 < steps) step(std::integral_constant<int, 2>(), l + 2);
+            if (l + 3 < steps) step(std::integral_constant<int, 3>(), l + 3);
+            if (l + 4 < steps) step(std::integral_constant<int, 4>(), l + 4);
         }
     }
-    if (MODE == MODE_RES || MODE == MODE_RHSRES) {
-        const int nblk = gridDim.x * gridDim.y * gridDim.z;
-        const int blk = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    if (KIND == ONE && (mode == MODE_RES || mode == MODE_RHSRES)) {
+        const double i2 = G.inv_scale[q] * G.inv_scale[q];
+        double acc[2] = {ar * i2, au * i2};
+        const int nblk = gridDim.x * gridDim.y;
+        const int blk = blockIdx.y * gridDim.x + blockIdx.x;
         block_partials<2>(acc, 2, part, nblk, blk);
         if (arrive_last(&ctl->counter[CNT_STENCIL], nblk)) {
             __shared__ double tot[2];
@@ -692,27 +746,341 @@ slab3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __restr
     }
 }
 
+// ------------------------------------------------------------------ vectors
+// The marching sweeps (field blocks, Helmholtz) give a thread W consecutive
+// points along x: 16 bytes where nx allows it, one point otherwise.
+template <typename T, int W> struct VecT;
+template <> struct VecT<float, 4> { using type = float4; };
+template <> struct VecT<double, 2> { using type = double2; };
+template <> struct VecT<float, 2> { using type = float2; };
+template <> struct VecT<float, 1> { using type = float; };
+template <> struct VecT<double, 1> { using type = double; };
+
+template <typename T, int W>
+__device__ __forceinline__ void vload(const T* p, T (&v)[W]) {
+    *reinterpret_cast<typename VecT<T, W>::type*>(v) = *reinterpret_cast<const typename VecT<T, W>::type*>(p);
+}
+template <typename T, int W>
+__device__ __forceinline__ void vstore(T* p, const T (&v)[W]) {
+    *reinterpret_cast<typename VecT<T, W>::type*>(p) = *reinterpret_cast<const typename VecT<T, W>::type*>(v);
+}
+
+template <typename T, int W> struct HelmTile;      // threads of a sweep's CTA along x, y
+template <> struct HelmTile<float, 4> { static constexpr int NXT = 16, NYT = 16; };
+template <> struct HelmTile<double, 2> { static constexpr int NXT = 32, NYT = 8; };
+template <> struct HelmTile<float, 2> { static constexpr int NXT = 32, NYT = 8; };
+template <typename T> struct HelmTile<T, 1> { static constexpr int NXT = 32, NYT = 8; };
+
+template <typename T, int W>
+__device__ __forceinline__ void cpa(T* dst, const T* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (W * sizeof(T) == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"(W * (int)sizeof(T)) : "memory");
+}
+
 // ============================================================================
 // Field-block Chebyshev sweep (same recurrence as the 2-D kernel, Section 2.5.2).
-// One CTA = one field of a PX x PY column of ZB planes: blockIdx.z = zblock * 5
-// + field.  The CTA marches up its planes; each thread owns one (x, y) column
-// and keeps, in registers, the iterate at z-4 .. z+4 and the vertical fluxes
-// K D_z x at z-2 .. z+2 (each computed once, when its plane enters the
-// window).  Per plane the iterate is staged with a halo of 4 in x and y and
-// the eddy field with a halo of 2; the horizontal fluxes K D_x x, K D_y x are
-// formed once per arm point in shared memory.  The staging offsets are
-// computed once per CTA.  p (field 4) is written by the last sweep.
+// One CTA = one field of a TX x TY column of zb planes: blockIdx.z = zblock * 5
+// + field; p (field 4) is written by the last sweep.  A thread owns W
+// consecutive points along x and marches in z with, in registers, the column's
+// iterate at z-4 .. z+4, its eddy values at z .. z+2 and its vertical fluxes
+// K D_z x at z-2 .. z+2 (each formed once, when its plane enters).  Per plane the
+// column's own iterate and eddy values go to shared memory and only the rings
+// around the tile (4 and 2 points) are fetched, by cp.async, one plane ahead
+// into the other of two buffers: one barrier per plane.  The horizontal fluxes
+// a point's D reads are formed by the point's own thread (8 for 4 points along
+// x, 4 rows along y): about twice the arithmetic of sharing them, but no
+// second exchange and no arm items.
+//
+// Bound: instruction issue and load latency (r and the eddy field read, z
+// written: 44 B a point over the five fields with two sweeps).  Against the
+// form with one point per thread, fluxes exchanged through shared memory and
+// two barriers a plane: 175 -> 87 us per apply (two
+// sweeps) at 256 x 256 x 64, float32.
 // ============================================================================
+template <typename T, int W, int SMAG, int FIRST, int LAST>
+__global__ void __launch_bounds__(NTHREADS, 2)
+cheb3d(Geo G, int k, int zb, const T* __restrict__ r, const T* __restrict__ zin, const T* __restrict__ din,
+       T* __restrict__ zout, T* __restrict__ dout, const T* __restrict__ nu, double* part, Ctl* ctl,
+       int check_done) {
+    constexpr int NXT = HelmTile<T, W>::NXT, NYT = HelmTile<T, W>::NYT;
+    constexpr int TX = NXT * W, TY = NYT, SX = TX + 2 * HALO, SY = TY + 2 * HALO;
+    // eddy plane: the iterate's row layout (vectors stay aligned), a ring of 2 rows and of HALO columns
+    constexpr int KY2 = TY + 2 * R;
+    constexpr int NH = (2 * HALO * TX + 2 * HALO * TY) / W, HS = (NH + NTHREADS - 1) / NTHREADS;
+    constexpr int KROWS = SMAG ? KY2 : 1;
+    __shared__ __align__(16) T pl[2][SX * SY];
+    __shared__ __align__(16) T kp[2][SX * KROWS];
+    pdl_wait();
+    const int done = check_done ? ctl->done : 0;
+    const int fld = blockIdx.z % 5;
+    const int z0 = (blockIdx.z / 5) * zb, nzb = min(zb, G.nz - z0);
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const T ith = cheb_coef<T>(ctl, fld, k, 0), a1 = cheb_coef<T>(ctl, fld, k, 1), a2 = cheb_coef<T>(ctl, fld, k, 2);
+    const size_t nxy = (size_t)G.ny * G.nx;
+    const T* fr = r + (size_t)fld * G.npt;
+    const T* src = (FIRST ? r : zin) + (size_t)fld * G.npt;
+    const T* fdin = FIRST ? nullptr : din + (size_t)fld * G.npt;
+    T* fzo = zout + (size_t)fld * G.npt;
+    T* fdo = LAST ? nullptr : dout + (size_t)fld * G.npt;
+    const int tx = threadIdx.x % NXT, ty = threadIdx.x / NXT;
+    const int gx = x0 + tx * W, gy = y0 + ty;
+    const bool inside = gx < G.nx && gy < G.ny;
+    const size_t own = (size_t)wrap(gy, G.ny) * G.nx + wrap(gx, G.nx);
+    T acc[1] = {T(0)};
+    if (done) return;
+    if (fld == 4) {
+        if (LAST && inside) {
+            for (int z = z0; z < z0 + nzb; ++z) {
+                const size_t o = (size_t)z * nxy + own;
+                T v[W];
+                vload<T, W>(fr + o, v);
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    v[i] *= ith;
+                    acc[0] += v[i] * v[i];
+                }
+                vstore<T, W>(fzo + o, v);
+            }
+        }
+    } else {
+        int hdst[HS], hsrc[HS], kdst[HS];
+#pragma unroll
+        for (int q = 0; q < HS; ++q) {
+            int h = threadIdx.x + q * NTHREADS;
+            hdst[q] = kdst[q] = -1;
+            hsrc[q] = 0;
+            if (h < NH) {
+                int ly, lx;                                  // staged row, column (relative to the tile origin)
+                if (h < 2 * HALO * NXT) {
+                    ly = h / NXT;
+                    ly = ly < HALO ? ly - HALO : TY + ly - HALO;
+                    lx = (h % NXT) * W;
+                } else {
+                    h -= 2 * HALO * NXT;
+                    constexpr int PER = 2 * HALO / W;        // vectors of the two sides of a row
+                    ly = h / PER;
+                    const int c = h % PER;
+                    lx = c < PER / 2 ? c * W - HALO : TX + (c - PER / 2) * W;
+                }
+                hdst[q] = (ly + HALO) * SX + lx + HALO;
+                hsrc[q] = wrap(y0 + ly, G.ny) * G.nx + wrap(x0 + lx, G.nx);
+                if (SMAG && ly >= -R && ly < TY + R) kdst[q] = (ly + R) * SX + lx + HALO;
+            }
+        }
+        const int me = (ty + HALO) * SX + tx * W + HALO, mk = (ty + R) * SX + tx * W + HALO;
+        const bool odd_b = G.pb[fld] < 0, odd_t = G.pt[fld] < 0, heat = fld == 3;
+        const T kscale = heat ? GC(inv_Pr) : T(1);
+        auto coef = [&](T nv, bool zarm) -> T {              // exchange coefficient from the eddy value
+            if constexpr (SMAG == 2) return dd3_coef(nv, zarm, heat, G);
+            else return nv * kscale;
+        };
+        auto column = [&](int z, T (&v)[W]) {                // iterate of the column at plane z (signed mirror)
+            int side;
+            vload<T, W>(src + (size_t)mirror(z, G.nz, side) * nxy + own, v);
+            if ((side == 1 && odd_b) || (side == 2 && odd_t)) {
+#pragma unroll
+                for (int i = 0; i < W; ++i) v[i] = flip(v[i]);
+            }
+        };
+        auto eddy = [&](int z, T (&v)[W]) {                  // eddy values of the column (even mirror)
+            if (SMAG) vload<T, W>(nu + (size_t)max(eddy_row(z, G.nz), 0) * nxy + own, v);
+        };
+        auto ring = [&](int t) {
+            const size_t pz = (size_t)(z0 + t) * nxy;
+#pragma unroll
+            for (int q = 0; q < HS; ++q) {
+                if (hdst[q] >= 0) cpa<T, W>(&pl[t & 1][hdst[q]], src + pz + hsrc[q]);
+                if (SMAG && kdst[q] >= 0) cpa<T, W>(&kp[t & 1][kdst[q]], nu + pz + hsrc[q]);
+            }
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        const T wz1 = GC(wz1), wz2 = GC(wz2);
+        T xw[9][W], kw[3][W], fw[5][W], xn[W], kn[W], rv[W], dv[W];
+        ring(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) column(z0 - 4 + q, xw[q]);
+        {
+            T ka[4][W];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) eddy(z0 - 2 + q, ka[q]);
+            column(z0 + 4, xn);
+            eddy(z0 + 2, kn);
+            if (!FIRST) {
+                vload<T, W>(fr + (size_t)z0 * nxy + own, rv);
+                vload<T, W>(fdin + (size_t)z0 * nxy + own, dv);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    const T dz = wz1 * (xw[q + 3][i] - xw[q + 1][i]) + wz2 * (xw[q + 4][i] - xw[q][i]);
+                    fw[q][i] = SMAG ? coef(ka[q][i], true) * dz : dz;
+                    if (SMAG && q >= 2) kw[q - 2][i] = ka[q][i];
+                }
+        }
+        for (int t = 0; t < nzb; ++t) {
+            T* p = pl[t & 1];
+            T* kq = kp[t & 1];
+            vstore<T, W>(p + me, xw[4]);
+            if (SMAG) vstore<T, W>(kq + mk, kw[0]);
+            asm volatile("cp.async.wait_all;\n" ::: "memory");
+            __syncthreads();
+            if (t + 1 < nzb) ring(t + 1);     // its buffers were last read before this plane's barrier
+            T rc[W], dc[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                xw[8][i] = xn[i];
+                if (SMAG) kw[2][i] = kn[i];
+                rc[i] = FIRST ? xw[4][i] : rv[i];
+                if (!FIRST) dc[i] = dv[i];
+                const T dz = wz1 * (xw[7][i] - xw[5][i]) + wz2 * (xn[i] - xw[4][i]);
+                fw[4][i] = SMAG ? coef(kn[i], true) * dz : dz;
+            }
+            if (t + 1 < nzb) {
+                column(z0 + t + 5, xn);
+                eddy(z0 + t + 3, kn);
+                if (!FIRST) {
+                    vload<T, W>(fr + (size_t)(z0 + t + 1) * nxy + own, rv);
+                    vload<T, W>(fdin + (size_t)(z0 + t + 1) * nxy + own, dv);
+                }
+            }
+            T dif[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) dif[i] = wz1 * (fw[3][i] - fw[1][i]) + wz2 * (fw[4][i] - fw[0][i]);
+            {   // x: row values at -4 .. W+4, fluxes at -2 .. W+2
+                T e[W + 8], kx[W + 8];
+#pragma unroll
+                for (int i = 0; i < 4; i += W) {
+                    T a[W], b[W];
+                    vload<T, W>(p + me - 4 + i, a);
+                    vload<T, W>(p + me + W + i, b);
+#pragma unroll
+                    for (int j = 0; j < W; ++j) {
+                        e[i + j] = a[j];
+                        e[W + 4 + i + j] = b[j];
+                    }
+                    if (SMAG) {
+                        vload<T, W>(kq + mk - 4 + i, a);
+                        vload<T, W>(kq + mk + W + i, b);
+#pragma unroll
+                        for (int j = 0; j < W; ++j) {
+                            kx[i + j] = a[j];
+                            kx[W + 4 + i + j] = b[j];
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    e[4 + i] = xw[4][i];
+                    if (SMAG) kx[4 + i] = kw[0][i];
+                }
+                T fx[W + 4];
+#pragma unroll
+                for (int i = 0; i < W + 4; ++i) {
+                    if (W == 1 && i == 2) continue;              // the centre flux is not read
+                    const T dx = GC(wx1) * (e[i + 3] - e[i + 1]) + GC(wx2) * (e[i + 4] - e[i]);
+                    fx[i] = SMAG ? coef(kx[i + 2], false) * dx : dx;
+                }
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    dif[i] += GC(wx1) * (fx[i + 3] - fx[i + 1]);
+                    dif[i] += GC(wx2) * (fx[i + 4] - fx[i]);
+                }
+            }
+            {   // y: rows -4 .. 4, fluxes at rows -2, -1, 1, 2
+                T e[9][W];
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    if (q != 4) vload<T, W>(p + me + (q - 4) * SX, e[q]);
+#pragma unroll
+                for (int i = 0; i < W; ++i) e[4][i] = xw[4][i];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    if (q == 2) continue;
+                    T ky[W];
+                    if (SMAG) vload<T, W>(kq + mk + (q - 2) * SX, ky);
+                    const T w = q == 0 ? -GC(wy2) : (q == 1 ? -GC(wy1) : (q == 3 ? GC(wy1) : GC(wy2)));
+#pragma unroll
+                    for (int i = 0; i < W; ++i) {
+                        const T dy = GC(wy1) * (e[q + 3][i] - e[q + 1][i]) + GC(wy2) * (e[q + 4][i] - e[q][i]);
+                        dif[i] += w * (SMAG ? coef(ky[i], false) * dy : dy);
+                    }
+                }
+            }
+            const T Kc = SMAG ? T(1) : (heat ? GC(K_H) : GC(K_M));
+            T xo[W], dk[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                const T xk = FIRST ? ith * xw[4][i] : xw[4][i];
+                const T df = (FIRST ? ith * Kc : Kc) * dif[i];
+                const T res = rc[i] - (GC(two_over_dt) * xk - df);
+                dk[i] = a1 * (FIRST ? xk : dc[i]) + a2 * res;
+                xo[i] = xk + dk[i];
+            }
+            if (inside) {
+                const size_t o = (size_t)(z0 + t) * nxy + own;
+                vstore<T, W>(fzo + o, xo);
+                if (!LAST) vstore<T, W>(fdo + o, dk);
+                if (LAST) {
+#pragma unroll
+                    for (int i = 0; i < W; ++i) acc[0] += xo[i] * xo[i];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) xw[q][i] = xw[q + 1][i];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) fw[q][i] = fw[q + 1][i];
+                if (SMAG) {
+                    kw[0][i] = kw[1][i];
+                    kw[1][i] = kw[2][i];
+                }
+            }
+        }
+    }
+    pdl_trigger();
+    if (LAST) {
+        const int nblk = gridDim.x * gridDim.y * gridDim.z;
+        const int blk = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        block_partials<1, T>(acc, 1, part, nblk, blk);
+        if (arrive_last(&ctl->counter[CNT_PC], nblk)) {
+            __shared__ double tot[1];
+            final_sums(part, nblk, 1, tot);
+            if (threadIdx.x == 0) {
+                const double zn = sqrt(tot[0]);
+                put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
+            }
+        }
+    }
+}
+
+// ============================================================================
+// Field-block Chebyshev sweep with the horizontal fluxes shared (float64).  One
+// CTA = one field of a CX x CY column of CZB planes: blockIdx.z = zblock * 5 +
+// field.  Each thread owns one (x, y) column and keeps, in registers, the
+// iterate at z-4 .. z+4 and the vertical fluxes K D_z x at z-2 .. z+2; per plane
+// the iterate is staged with a halo of 4 and the eddy field with a halo of 2, and
+// the fluxes K D_x x, K D_y x are formed once per arm point in shared memory.
+// Bound: the FP64 pipe (about 37 operations a point and field; the vector sweep
+// forms every flux in each thread that reads it, about 55, which float32 does
+// not feel and float64 does: 2.6 against 3.0 ms per apply at 256 x 256 x 64).
+// ============================================================================
+constexpr int CX = 32, CY = 8;
+static_assert(CX * CY == NTHREADS, "one output per thread");
 constexpr int CZB = 16;      // planes per CTA of the Chebyshev sweep
 
 template <typename T, int SMAG, int FIRST, int LAST>
 __global__ void __launch_bounds__(NTHREADS)
-cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T* __restrict__ din,
+cheb3d_shared(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T* __restrict__ din,
        T* __restrict__ zout, T* __restrict__ dout, const T* __restrict__ nu, double* part, Ctl* ctl,
        int check_done) {
-    constexpr int SX = PX + 2 * HALO, SY = PY + 2 * HALO, SP = SX * SY;      // iterate plane
-    constexpr int NX = PX + 2 * R, NY = PY + 2 * R, NP = NX * NY;            // eddy plane
-    constexpr int AXN = (PX + 2 * R) * PY, AYN = PX * (PY + 2 * R), AN = AXN + AYN;
+    constexpr int SX = CX + 2 * HALO, SY = CY + 2 * HALO, SP = SX * SY;      // iterate plane
+    constexpr int NX = CX + 2 * R, NY = CY + 2 * R, NP = NX * NY;            // eddy plane
+    constexpr int AXN = (CX + 2 * R) * CY, AYN = CX * (CY + 2 * R), AN = AXN + AYN;
     constexpr int XS = (SP + NTHREADS - 1) / NTHREADS;    // staging slots per thread
     constexpr int NS = (NP + NTHREADS - 1) / NTHREADS;
     constexpr int AS = (AN + NTHREADS - 1) / NTHREADS;
@@ -723,18 +1091,17 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
     const int fld = blockIdx.z % 5;
     const int z0 = (blockIdx.z / 5) * CZB;
     const int z1 = min(z0 + CZB, G.nz);
-    const int x0 = blockIdx.x * PX, y0 = blockIdx.y * PY;
-    const T ith = T(ctl->cheb[fld][k][0]);
-    const T a1 = T(ctl->cheb[fld][k][1]);
-    const T a2 = T(ctl->cheb[fld][k][2]);
+    const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CY;
+    const T ith = cheb_coef<T>(ctl, fld, k, 0);
+    const T a1 = cheb_coef<T>(ctl, fld, k, 1);
+    const T a2 = cheb_coef<T>(ctl, fld, k, 2);
     const size_t nxy = (size_t)G.ny * G.nx;
     const T* fr = r + (size_t)fld * G.npt;
     const T* fsrc = (FIRST ? r : zin) + (size_t)fld * G.npt;
     const T* fdin = FIRST ? nullptr : din + (size_t)fld * G.npt;
     T* fzo = zout + (size_t)fld * G.npt;
     T* fdo = dout + (size_t)fld * G.npt;
-    const T sc = FIRST ? ith : T(1);
-    const int tx = threadIdx.x % PX, ty = threadIdx.x / PX;
+    const int tx = threadIdx.x % CX, ty = threadIdx.x / CX;
     const int gx = x0 + tx, gy = y0 + ty;
     const bool inside = gx < G.nx && gy < G.ny;
     const size_t own = inside ? (size_t)gy * G.nx + gx : 0;       // in-plane offset of the thread's column
@@ -770,7 +1137,7 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
                 anu[q] = (qy + R) * NX + qx;
             } else if (idx < AN) {
                 const int j = idx - AXN;
-                const int qx = j % PX, qy = j / PX;               // y arm at tile (qx, qy - R)
+                const int qx = j % CX, qy = j / CX;               // y arm at tile (qx, qy - R)
                 acen[q] = -((qy + R) * SX + qx + HALO) - 1;       // negative: a y arm
                 anu[q] = qy * NX + qx + R;
             } else {
@@ -778,27 +1145,31 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
                 anu[q] = -1;
             }
         }
-        const T kscale = fld == 3 ? T(G.inv_Pr) : T(1);
-        const T ix = T(G.inv_dx), iy = T(G.inv_dy), iz = T(G.inv_dz);
-        const T Kc = T(fld == 3 ? G.K_H : G.K_M);
+        // what the fluxes leave out: 1/Pr of theta, the constant K, 1/theta_c of a first sweep
+        const T fscale = (SMAG == 2 ? T(1) : SMAG ? (fld == 3 ? GC(inv_Pr) : T(1)) : (fld == 3 ? GC(K_H) : GC(K_M))) * (FIRST ? ith : T(1));
+        // FIRST: x_1 = r / theta_c enters as r, the sum of the fluxes is scaled at the end
+        const T wz1 = GC(wz1), wz2 = GC(wz2);
+        auto D = [](const T* s, int i, int st, T w1, T w2) {
+            return w1 * (s[i + st] - s[i - st]) + w2 * (s[i + 2 * st] - s[i - 2 * st]);
+        };
         auto xval = [&](int z) -> T {          // iterate at row z of the column (mirror ghosts)
             int side;
             const int sz = mirror(z, G.nz, side);
-            const T sg = side == 1 ? T(G.pb[fld]) : (side == 2 ? T(G.pt[fld]) : T(1));
-            return sg * sc * fsrc[(size_t)sz * nxy + own];
+            const T v = fsrc[(size_t)sz * nxy + own];
+            return (side == 1 && G.pb[fld] < 0) || (side == 2 && G.pt[fld] < 0) ? flip(v) : v;
         };
         auto zflux = [&](T d, int z) -> T {    // K D_z x at row z (eddy field mirrored even)
             if (!SMAG) return d;
             const int sz = eddy_row(z, G.nz);
             const T nv = sz >= 0 ? nu[(size_t)sz * nxy + own] : T(0);
-            return (SMAG == 2 ? dd3_coef(nv, true, fld == 3, G) : nv * kscale) * d;
+            return (SMAG == 2 ? dd3_coef(nv, true, fld == 3, G) : nv) * d;
         };
         T xw[9], fw[5];
         if (inside) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) xw[q] = xval(z0 - 4 + q);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) fw[q] = zflux(d5(xw[q], xw[q + 1], xw[q + 3], xw[q + 4], iz), z0 - 2 + q);
+            for (int q = 0; q < 4; ++q) fw[q] = zflux(wz1 * (xw[q + 3] - xw[q + 1]) + wz2 * (xw[q + 4] - xw[q]), z0 - 2 + q);
         }
         // every global value a plane needs (its staged tile and eddy plane, the
         // point's r, d, the iterate at z+4 and the eddy field at z+2) is loaded one
@@ -827,7 +1198,7 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
             const size_t pz = (size_t)z * nxy;
 #pragma unroll
             for (int q = 0; q < XS; ++q)
-                if (xoff[q] >= 0) xs[threadIdx.x + q * NTHREADS] = sc * px[q];
+                if (xoff[q] >= 0) xs[threadIdx.x + q * NTHREADS] = px[q];
             if (SMAG) {
 #pragma unroll
                 for (int q = 0; q < NS; ++q)
@@ -839,11 +1210,11 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
                 if (anu[q] < 0) continue;
                 const bool xarm = acen[q] >= 0;
                 const int c = xarm ? acen[q] : -acen[q] - 1;
-                const T d = xarm ? dd(xs, c, 1, ix) : dd(xs, c, SX, iy);
+                const T d = xarm ? D(xs, c, 1, GC(wx1), GC(wx2)) : D(xs, c, SX, GC(wy1), GC(wy2));
                 T kv = T(1);
                 if (SMAG) {
                     const T nv = ns[anu[q]];
-                    kv = SMAG == 2 ? dd3_coef(nv, false, fld == 3, G) : nv * kscale;
+                    kv = SMAG == 2 ? dd3_coef(nv, false, fld == 3, G) : nv;
                 }
                 kg[threadIdx.x + q * NTHREADS] = SMAG ? kv * d : d;
             }
@@ -853,21 +1224,16 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
             if (z + 1 < z1) prefetch(z + 1);
             if (inside) {
                 {
-                    const T dz2 = d5(xw[4], xw[5], xw[7], xw[8], iz);
-                    fw[4] = SMAG ? (SMAG == 2 ? dd3_coef(nu2, true, fld == 3, G) : nu2 * kscale) * dz2 : dz2;
+                    const T dz2 = wz1 * (xw[7] - xw[5]) + wz2 * (xw[8] - xw[4]);
+                    fw[4] = SMAG ? (SMAG == 2 ? dd3_coef(nu2, true, fld == 3, G) : nu2) * dz2 : dz2;
                 }
                 const int cax = ty * NX + tx + R;
-                const int cay = AXN + (ty + R) * PX + tx;
-                T dif;
-                if (SMAG) {
-                    dif = dd(kg, cax, 1, ix) + dd(kg, cay, PX, iy) +
-                          (T(2.0 / 3.0) * (fw[3] - fw[1]) - T(1.0 / 12.0) * (fw[4] - fw[0])) * iz;
-                } else {
-                    dif = Kc * dd(kg, cax, 1, ix) + Kc * dd(kg, cay, PX, iy) + Kc * d5(fw[0], fw[1], fw[3], fw[4], iz);
-                }
-                const T xk = xw[4];
+                const int cay = AXN + (ty + R) * CX + tx;
+                const T dif = D(kg, cax, 1, GC(wx1), GC(wx2)) + D(kg, cay, CX, GC(wy1), GC(wy2)) +
+                              (wz1 * (fw[3] - fw[1]) + wz2 * (fw[4] - fw[0]));
+                const T xk = FIRST ? ith * xw[4] : xw[4];
                 const size_t o = pz + own;
-                const T res = rv - (T(G.two_over_dt) * xk - dif);
+                const T res = rv - (GC(two_over_dt) * xk - fscale * dif);
                 const T dprev = FIRST ? rv * ith : dv;
                 const T dk = a1 * dprev + a2 * res;
                 const T xn = xk + dk;
@@ -890,8 +1256,7 @@ cheb3d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T
             final_sums(part, nblk, 1, tot);
             if (threadIdx.x == 0) {
                 const double zn = sqrt(tot[0]);
-                ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-                ctl->eps_part = 0;
+                put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
             }
         }
     }
@@ -956,22 +1321,6 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <typename T, int MODE>
-constexpr size_t plane_smem(int smag) {
-    constexpr int SP = (PX + 2 * HALO) * (PY + 2 * HALO);
-    constexpr int AN = (PX + 2 * R) * PY + PX * (PY + 2 * R);
-    constexpr int NS = Two<MODE>::v ? 2 : 1;
-    return sizeof(T) * ((size_t)NS * 5 * SP + (size_t)NS * 4 * AN + (smag ? (size_t)NS * AN : 0));
-}
-
-template <typename T, int MODE>
-constexpr size_t slab_smem(int smag) {
-    constexpr int TX = SlabT<T>::TX, TZ = SlabT<T>::TZ;
-    constexpr int SP = TX * (TZ + 2 * HALO), AN = TX * (TZ + 2 * R);
-    constexpr int NS = Two<MODE>::v ? 2 : 1;
-    return sizeof(T) * ((size_t)NS * 5 * SP + (size_t)NS * 4 * AN + (smag ? (size_t)NS * AN : 0));
-}
-
 static int stream_blocks3(size_t n) {
     size_t b = (n + NTHREADS - 1) / NTHREADS;
     return (int)(b < (size_t)MAX_STREAM_BLOCKS ? (b > 0 ? b : 1) : MAX_STREAM_BLOCKS);
@@ -990,42 +1339,62 @@ struct S3 {
     }
 };
 
-template <typename T, int MODE, int SMAG>
-static cudaError_t launch_split(const Geo& G, const T* u, const T* v, const T* Fu, const double* f, T* out,
+// Planes per CTA of the column pass: the split with the fewest rounds of CTAs
+// times steps (the eight lead-in steps of a march cost about three full ones).
+static int column_planes(const Geo& G, int slots) {
+    const long long cols = ((long long)G.nx * G.ny + CW - 1) / CW;
+    int best = G.nz;
+    double least = 1e300;
+    for (int parts = 1; parts <= 16; ++parts) {
+        const int zc = (G.nz + parts - 1) / parts;
+        if (zc < 8 && parts > 1) break;
+        const long long ctas = cols * ((G.nz + zc - 1) / zc);
+        const double cost = (double)((ctas + slots - 1) / slots) * (zc + 3.0);
+        if (cost < least) {
+            least = cost;
+            best = zc;
+        }
+    }
+    return best;
+}
+
+template <typename T, int KIND, int SMAG>
+static cudaError_t launch_split(int mode, const Geo& G, const T* u, const T* v, const T* Fu, const double* f, T* out,
                                 T* out2, double* part, Ctl* ctl, int check_done, cudaStream_t s) {
     if (G.s3 == nullptr) return cudaErrorInvalidValue;
+    using SH = PlaneShape<T, KIND, SMAG>;
     S3<T> sc(G);
-    const size_t smp = plane_smem<T, MODE>(SMAG), sms = slab_smem<T, MODE>(SMAG);
-    static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
-    if (!configured) {
-        cudaError_t e = set_smem(plane3d<T, MODE, SMAG>, smp);
-        if (e != cudaSuccess) return e;
-        if ((e = set_smem(slab3d<T, MODE, SMAG>, sms)) != cudaSuccess) return e;
-        configured = true;
+    static std::atomic<int> slots{0};   // resident column CTAs; set once, concurrent first calls are harmless
+    cudaError_t e;
+    if (slots.load() == 0) {
+        int dev = 0, nsm = 0, per = 0;
+        if ((e = set_smem(plane3d<T, KIND, SMAG>, SH::smem)) != cudaSuccess || (e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, column3d<T, KIND, SMAG>, COL_THREADS, 0)) != cudaSuccess)
+            return e;
+        slots = std::max(1, nsm * per);
     }
     if (SMAG) {
         dim3 gk((G.nx + KX - 1) / KX, (G.ny + KY - 1) / KY, (G.nz + SZB - 1) / SZB);
-        strain3d<T, MODE, 0><<<gk, NTHREADS, 0, s>>>(G, u, v, sc.s0, sc.s1, part, ctl, check_done);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        strain3d<T, KIND, 0><<<gk, NTHREADS, 0, s>>>(G, u, v, sc.s0, sc.s1, part, ctl, check_done);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    dim3 gp((G.nx + PX - 1) / PX, (G.ny + PY - 1) / PY, G.nz);
-    plane3d<T, MODE, SMAG><<<gp, NTHREADS, smp, s>>>(G, u, v, sc.s0, sc.s1, sc.P, ctl, check_done);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    constexpr int TX = SlabT<T>::TX, TZ = SlabT<T>::TZ;
-    dim3 gs((G.nz + TZ - 1) / TZ, (G.nx + TX - 1) / TX, G.ny);
-    slab3d<T, MODE, SMAG><<<gs, NTHREADS, sms, s>>>(G, u, v, Fu, f, sc.s0, sc.s1, sc.P, out, out2, part, ctl,
+    dim3 gp((G.nx + PX - 1) / PX, (G.ny + SH::PY - 1) / SH::PY, G.nz);
+    plane3d<T, KIND, SMAG><<<gp, NTHREADS, SH::smem, s>>>(G, u, v, sc.s0, sc.s1, sc.P, ctl, check_done);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int zc = column_planes(G, slots.load());
+    dim3 gc((unsigned)(((size_t)G.nx * G.ny + CW - 1) / CW), (G.nz + zc - 1) / zc);
+    column3d<T, KIND, SMAG><<<gc, COL_THREADS, 0, s>>>(G, mode, zc, u, v, Fu, f, sc.s0, sc.s1, sc.P, out, out2, part, ctl,
                                                      check_done);
     return cudaGetLastError();
 }
 
-template <typename T, int MODE>
-static cudaError_t launch_split_m(const Geo& G, const T* u, const T* v, const T* Fu, const double* f, T* out,
+template <typename T, int KIND>
+static cudaError_t launch_split_k(int mode, const Geo& G, const T* u, const T* v, const T* Fu, const double* f, T* out,
                                   T* out2, double* part, Ctl* ctl, int check_done, cudaStream_t s) {
-    if (G.sgs == 2) return launch_split<T, MODE, 2>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-    return G.smag ? launch_split<T, MODE, 1>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s)
-                  : launch_split<T, MODE, 0>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+    if (G.sgs == 2) return launch_split<T, KIND, 2>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+    return G.smag ? launch_split<T, KIND, 1>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s)
+                  : launch_split<T, KIND, 0>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1039,24 +1408,7 @@ static cudaError_t launch_split_m(const Geo& G, const T* u, const T* v, const T*
 // at the walls), which equals D_j applied to D_j dp evaluated with its ghosts.
 // Fields: 0 u, 1 v, 2 w, 3 theta, 4 p; planes [z][y][x].
 //
-// A thread owns W consecutive points along x (16 bytes where nx allows it, one
-// point otherwise): rows load, stage and store as vectors.
 // ---------------------------------------------------------------------------
-template <typename T, int W> struct VecT;
-template <> struct VecT<float, 4> { using type = float4; };
-template <> struct VecT<double, 2> { using type = double2; };
-template <> struct VecT<float, 1> { using type = float; };
-template <> struct VecT<double, 1> { using type = double; };
-
-template <typename T, int W>
-__device__ __forceinline__ void vload(const T* p, T (&v)[W]) {
-    *reinterpret_cast<typename VecT<T, W>::type*>(v) = *reinterpret_cast<const typename VecT<T, W>::type*>(p);
-}
-template <typename T, int W>
-__device__ __forceinline__ void vstore(T* p, const T (&v)[W]) {
-    *reinterpret_cast<typename VecT<T, W>::type*>(p) = *reinterpret_cast<const typename VecT<T, W>::type*>(v);
-}
-
 // e[0 .. W+4) = row[gx-2 .. gx+W+2) of a periodic row (gx and nx multiples of W)
 template <typename T, int W>
 __device__ __forceinline__ void row_taps(const T* __restrict__ row, int gx, int nx, T (&e)[W + 4]) {
@@ -1109,8 +1461,8 @@ __global__ void __launch_bounds__(NTHREADS)
 schur_rhs3d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int check_done) {
     pdl_wait();
     if (check_done && ctl->done) return;
-    const T cdiv = T(G.schur_cdiv);
-    const T ix = T(G.inv_dx), iy = T(G.inv_dy), iz = T(G.inv_dz);
+    const T cdiv = GC(schur_cdiv);
+    const T ix = GC(inv_dx), iy = GC(inv_dy), iz = GC(inv_dz);
     const T one[4] = {T(1), T(1), T(1), T(1)};
     const size_t np = (size_t)G.npt;
     const unsigned nv = G.npt / W, nxv = G.nx / W, nxy = nxv * G.ny;
@@ -1151,20 +1503,6 @@ struct HelmC {                      // coefficients of a sweep in the type of th
     T c0, cx[4], cy[4], cz[4];      // res = rhs + c0 x + sum_k c_k (x_{+k} + x_{-k})
 };
 
-template <typename T, int W> struct HelmTile;      // threads along x, y
-template <> struct HelmTile<float, 4> { static constexpr int NXT = 16, NYT = 16; };
-template <> struct HelmTile<double, 2> { static constexpr int NXT = 32, NYT = 8; };
-template <typename T> struct HelmTile<T, 1> { static constexpr int NXT = 32, NYT = 8; };
-
-template <typename T, int W>
-__device__ __forceinline__ void cpa(T* dst, const T* src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (W * sizeof(T) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"(W * (int)sizeof(T)) : "memory");
-}
-
 template <typename T, int W, int FIRST, int LAST>
 __global__ void __launch_bounds__(NTHREADS, 2)
 helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, const T* __restrict__ xin,
@@ -1177,7 +1515,7 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
     __shared__ __align__(16) T pl[2][SP];
     pdl_wait();
     const int done = check_done ? ctl->done : 0;
-    const T ith = T(ctl->cheb[5][k][0]), a1 = T(ctl->cheb[5][k][1]), a2 = T(ctl->cheb[5][k][2]);
+    const T ith = cheb_coef<T>(ctl, 5, k, 0), a1 = cheb_coef<T>(ctl, 5, k, 1), a2 = cheb_coef<T>(ctl, 5, k, 2);
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int z0 = blockIdx.z * zb, nzb = min(zb, G.nz - z0);
     const size_t nxy = (size_t)G.ny * G.nx;
@@ -1308,9 +1646,9 @@ __global__ void __launch_bounds__(NTHREADS)
 schur_back3d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ctl* ctl, int check_done) {
     pdl_wait();
     if (check_done && ctl->done) return;
-    const T cgrad = T(G.schur_cgrad), hdt = T(G.half_dt);
-    const T ith_t = T(ctl->cheb[3][0][0]);
-    const T ix = T(G.inv_dx), iy = T(G.inv_dy), iz = T(G.inv_dz);
+    const T cgrad = GC(schur_cgrad), hdt = GC(half_dt);
+    const T ith_t = cheb_coef<T>(ctl, 3, 0, 0);
+    const T ix = GC(inv_dx), iy = GC(inv_dy), iz = GC(inv_dz);
     const T one[4] = {T(1), T(1), T(1), T(1)};
     const size_t np = (size_t)G.npt;
     const T* dp = z + 4 * np;
@@ -1348,8 +1686,7 @@ schur_back3d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ct
         final_sums(part, gridDim.x, 1, tot);
         if (threadIdx.x == 0) {
             const double zn = sqrt(tot[0]);
-            ctl->eps_jv = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
-            ctl->eps_part = 0;
+            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
         }
     }
 }
@@ -1360,16 +1697,10 @@ schur_back3d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ct
 int stencil3d_part_blocks(const Geo& G) {
     // largest reduction grid any 3-D kernel launches
     using namespace d3;
-    const long long slab = (long long)((G.nz + SlabT<float>::TZ - 1) / SlabT<float>::TZ) *
-                           ((G.nx + SlabT<float>::TX - 1) / SlabT<float>::TX) * G.ny;
-    const long long slab64 = (long long)((G.nz + SlabT<double>::TZ - 1) / SlabT<double>::TZ) *
-                             ((G.nx + SlabT<double>::TX - 1) / SlabT<double>::TX) * G.ny;
-    const long long cheb = (long long)((G.nx + PX - 1) / PX) * ((G.ny + PY - 1) / PY) * G.nz * 5;
+    const long long column = ((long long)G.nx * G.ny + CW - 1) / CW * ((G.nz + 7) / 8);     // marches of eight planes at least
+    const long long cheb = (long long)((G.nx + 31) / 32) * ((G.ny + 7) / 8) * ((G.nz + 7) / 8) * 5;   // smallest tile and march
     const long long strain = (long long)((G.nx + KX - 1) / KX) * ((G.ny + KY - 1) / KY) * G.nz;
-    long long m = slab > slab64 ? slab : slab64;
-    if (cheb > m) m = cheb;
-    if (strain > m) m = strain;
-    return (int)m;
+    return (int)std::max(column, std::max(cheb, strain));
 }
 
 size_t stencil3d_scratch_bytes(const Geo& G) { return 7 * (size_t)G.npt * sizeof(double); }
@@ -1378,15 +1709,12 @@ template <typename T>
 cudaError_t launch_stencil3d(int mode, const Geo& G, const T* u, const T* v, const T* Fu, const double* f,
                              T* out, T* out2, double* part, Ctl* ctl, int check_done, cudaStream_t s) {
     using namespace d3;
-    switch (mode) {
-        case d3::MODE_F: return launch_split_m<T, d3::MODE_F>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-        case d3::MODE_RHS: return launch_split_m<T, d3::MODE_RHS>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-        case d3::MODE_RES: return launch_split_m<T, d3::MODE_RES>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-        case d3::MODE_JV: return launch_split_m<T, d3::MODE_JV>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-        case d3::MODE_RHSRES:
-            return launch_split_m<T, d3::MODE_RHSRES>(G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
-        default: return cudaErrorInvalidValue;
-    }
+    if (mode < d3::MODE_F || mode > d3::MODE_RHSRES) return cudaErrorInvalidValue;
+    if (mode != d3::MODE_JV) return launch_split_k<T, ONE>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+    // the plain forward difference is the float64 path's; float32 takes launch_jv_diff3d
+    if constexpr (sizeof(T) == sizeof(double))
+        return launch_split_k<T, SHIFT>(mode, G, u, v, Fu, f, out, out2, part, ctl, check_done, s);
+    return cudaErrorNotSupported;
 }
 template cudaError_t launch_stencil3d<float>(int, const Geo&, const float*, const float*, const float*,
                                              const double*, float*, float*, double*, Ctl*, int, cudaStream_t);
@@ -1396,25 +1724,72 @@ template cudaError_t launch_stencil3d<double>(int, const Geo&, const double*, co
 cudaError_t launch_jv_diff3d(const Geo& G, const float* u, const float* v, float* out, Ctl* ctl, int check_done,
                              cudaStream_t s) {
     using namespace d3;
-    return launch_split_m<float, d3::MODE_DJV>(G, u, v, nullptr, nullptr, out, nullptr, nullptr, ctl, check_done, s);
+    return launch_split_k<float, PAIR>(d3::MODE_JV, G, u, v, nullptr, nullptr, out, nullptr, nullptr, ctl, check_done, s);
 }
 
 template <typename T>
 cudaError_t launch_eddy3d(const Geo& G, const T* u, T* nu, double* part, Ctl* ctl, cudaStream_t s) {
     using namespace d3;
     dim3 gk((G.nx + KX - 1) / KX, (G.ny + KY - 1) / KY, (G.nz + SZB - 1) / SZB);
-    strain3d<T, d3::MODE_F, 1><<<gk, NTHREADS, 0, s>>>(G, u, nullptr, nullptr, nu, part, ctl, 0);
+    strain3d<T, ONE, 1><<<gk, NTHREADS, 0, s>>>(G, u, nullptr, nullptr, nu, part, ctl, 0);
     return cudaGetLastError();
 }
 template cudaError_t launch_eddy3d<float>(const Geo&, const float*, float*, double*, Ctl*, cudaStream_t);
 template cudaError_t launch_eddy3d<double>(const Geo&, const double*, double*, double*, Ctl*, cudaStream_t);
 
-template <typename T, int SMAG>
-static cudaError_t launch_pc3(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
-                              const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
-                              long long* launches) {
+// Points per thread of the marching sweeps: 16 bytes where the rows are
+// multiples of that, else 8 bytes of float32, else one.  Every plane of the
+// workspace vectors starts a multiple of npt elements in, so nx decides the
+// alignment; r and z of the per-call entry may be the caller's (8-byte aligned)
+// float64 arrays.
+template <typename T>
+static int row_vector(const Geo& G, const T* r, const T* z) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z);
+    if (G.nx % (16 / sizeof(T)) == 0 && (a & 15) == 0) return 16 / sizeof(T);
+    return sizeof(T) == 4 && G.nx % 2 == 0 && (a & 7) == 0 ? 2 : 1;
+}
+
+template <typename T, int W, int SMAG>
+static cudaError_t launch_pc3_w(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb_, T* da, T* db,
+                                const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
+                                long long* launches) {
     using namespace d3;
-    dim3 grid((G.nx + PX - 1) / PX, (G.ny + PY - 1) / PY, ((G.nz + CZB - 1) / CZB) * 5);
+    constexpr int SMS = 152;
+    constexpr int TX = HelmTile<T, W>::NXT * W, TY = HelmTile<T, W>::NYT;
+    const int gx = (G.nx + TX - 1) / TX, gy = (G.ny + TY - 1) / TY;
+    // planes per CTA: the longest march that still gives every SM two CTAs of the
+    // four diffused fields (each march reads eight planes beyond its own)
+    int zb = 64;
+    while (zb > 8 && 4LL * gx * gy * ((G.nz + zb - 1) / zb) < 2 * SMS) zb /= 2;
+    dim3 grid(gx, gy, ((G.nz + zb - 1) / zb) * 5);
+    const T* zin = nullptr;
+    const T* din = nullptr;
+    T* zbuf[2] = {za, zb_};
+    T* dbuf[2] = {da, db};
+    for (int k = 1; k <= sweeps - 1; ++k) {
+        const bool first = k == 1, last = k == sweeps - 1;
+        T* zo = last ? z : zbuf[k & 1];
+        T* dO = dbuf[k & 1];
+        auto* kern = first ? (last ? cheb3d<T, W, SMAG, 1, 1> : cheb3d<T, W, SMAG, 1, 0>)
+                           : (last ? cheb3d<T, W, SMAG, 0, 1> : cheb3d<T, W, SMAG, 0, 0>);
+        const cudaError_t e = launch_pdl(kern, grid, dim3(NTHREADS), 0, s, G, k, zb, r, zin, din, zo, dO, nu, part, ctl,
+                                         check_done);
+        if (launches) ++*launches;
+        if (e != cudaSuccess) return e;
+        zin = zo;
+        din = dO;
+    }
+    return cudaSuccess;
+}
+
+// float64: the sweep with shared fluxes.
+template <int SMAG>
+static cudaError_t launch_pc3_shared(const Geo& G, int sweeps, const double* r, double* z, double* za, double* zb,
+                                     double* da, double* db, const double* nu, double* part, Ctl* ctl, int check_done,
+                                     cudaStream_t s, long long* launches) {
+    using namespace d3;
+    using T = double;
+    dim3 grid((G.nx + CX - 1) / CX, (G.ny + CY - 1) / CY, ((G.nz + CZB - 1) / CZB) * 5);
     const T* zin = nullptr;
     const T* din = nullptr;
     T* zbuf[2] = {za, zb};
@@ -1423,21 +1798,31 @@ static cudaError_t launch_pc3(const Geo& G, int sweeps, const T* r, T* z, T* za,
         const bool first = k == 1, last = k == sweeps - 1;
         T* zo = last ? z : zbuf[k & 1];
         T* dO = dbuf[k & 1];
-        if (first && last)
-            cheb3d<T, SMAG, 1, 1><<<grid, NTHREADS, 0, s>>>(G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else if (first)
-            cheb3d<T, SMAG, 1, 0><<<grid, NTHREADS, 0, s>>>(G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else if (last)
-            cheb3d<T, SMAG, 0, 1><<<grid, NTHREADS, 0, s>>>(G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else
-            cheb3d<T, SMAG, 0, 0><<<grid, NTHREADS, 0, s>>>(G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
+        auto* kern = first ? (last ? cheb3d_shared<T, SMAG, 1, 1> : cheb3d_shared<T, SMAG, 1, 0>)
+                           : (last ? cheb3d_shared<T, SMAG, 0, 1> : cheb3d_shared<T, SMAG, 0, 0>);
+        kern<<<grid, NTHREADS, 0, s>>>(G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
         if (launches) ++*launches;
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         zin = zo;
         din = dO;
     }
     return cudaSuccess;
+}
+
+template <typename T, int SMAG>
+static cudaError_t launch_pc3(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
+                              const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
+                              long long* launches) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        return launch_pc3_shared<SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+    } else {
+        switch (row_vector<T>(G, r, z)) {
+            case 4: return launch_pc3_w<T, 4, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+            case 2: return launch_pc3_w<T, 2, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+            default: return launch_pc3_w<T, 1, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+        }
+    }
 }
 
 // Acoustic Schur complement (3-D): rhs in da, iterates in xa / xb, directions
@@ -1497,13 +1882,12 @@ static cudaError_t launch_schur3d_w(const Geo& G, int sweeps, const T* r, T* z, 
 template <typename T>
 static cudaError_t launch_schur3d(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
                                   double* part, Ctl* ctl, int check_done, cudaStream_t s, long long* launches) {
-    // 16-byte rows: every plane of the workspace vectors starts a multiple of npt
-    // elements in, so nx decides the alignment; r and z of the per-call entry may
-    // be the caller's (8-byte aligned) float64 arrays
-    constexpr int W = 16 / sizeof(T);
-    const bool vec = G.nx % W == 0 && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z)) & 15) == 0;
-    return vec ? launch_schur3d_w<T, W>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches)
-               : launch_schur3d_w<T, 1>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches);
+    const int w = row_vector<T>(G, r, z);
+    if (w == 16 / sizeof(T))
+        return launch_schur3d_w<T, 16 / sizeof(T)>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches);
+    if constexpr (sizeof(T) == sizeof(float))
+        if (w == 2) return launch_schur3d_w<T, 2>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches);
+    return launch_schur3d_w<T, 1>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches);
 }
 
 template <typename T>

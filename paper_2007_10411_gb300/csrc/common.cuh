@@ -93,6 +93,7 @@ struct Ctl {
     double target;       // eta * beta0
     double res2;         // ||W R||^2 of the last residual evaluation
     double unorm2;       // ||W u||^2 of the same state
+    double eps_num, inv_eps_num;     // sqrt(eps_mach (1 + ||W u||)) of that state, and its reciprocal
     double eps_mach;     // unit roundoff of the stencil precision
     double eps_jv;       // finite-difference step of the next Jacobian-vector product (put_eps)
     double kmax;         // max eddy coefficient K_M (preconditioner bounds)
@@ -111,23 +112,30 @@ struct Ctl {
     double cheb[6][MAX_PC_SWEEPS][3];   // slot 5: pressure Helmholtz of the Schur complement
     float chebf[6][MAX_PC_SWEEPS][3];   // the same in float32
     unsigned int counter[8];         // last-block counters, one per kernel family
-    double scale[5];                 // field scales (Geo::scale), set once
-    // eps_jv scale_f and its reciprocal rounded to float32, for the float32 3-D passes: formed
-    // once in float64 with the step instead of by every block
+    double scale[5], inv_scale[5];   // field scales (Geo::scale) and their reciprocals, set once
+    // eps_jv scale_f and its reciprocal, formed once with the step instead of by every block
+    // of a Jacobian product (a float64 division is some 25 issues of 64 cycles)
+    double ev[5], cf[5];
     float evf[5], cff[5];
 };
 
-// The one writer of a finite-difference step that is not pending (eps_part).
-__device__ __forceinline__ void put_eps(Ctl* ctl, double e) {
-    ctl->eps_jv = e;
-    ctl->eps_part = 0;
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        const double s = ctl->scale[f], es = e * s;
-        ctl->evf[f] = (float)es;
-        ctl->cff[f] = (float)(es != 0.0 ? 1.0 / es : 0.0);
+// A finite-difference step e that is not pending (eps_part) and its reciprocal:
+// called by threads 0 .. 4 of one block (thread f forms field f's values).
+__device__ __forceinline__ void put_eps(Ctl* ctl, double e, double ie) {
+    const int f = threadIdx.x;
+    if (f == 0) {
+        ctl->eps_jv = e;
+        ctl->eps_part = 0;
+    }
+    if (f < 5) {
+        const double v = e * ctl->scale[f], r = ie * ctl->inv_scale[f];
+        ctl->ev[f] = v;
+        ctl->cf[f] = r;
+        ctl->evf[f] = (float)v;
+        ctl->cff[f] = (float)r;
     }
 }
+
 
 template <typename T>
 __device__ __forceinline__ T cheb_coef(const Ctl* ctl, int f, int k, int i) {
@@ -187,6 +195,30 @@ __device__ __forceinline__ double root(double x) {
     return __fma_rn(__fma_rn(-g, g, x), h, g);
 }
 __device__ __forceinline__ float root(float x) { return sqrtf(x); }
+
+// sqrt(x) and 1 / sqrt(x) of a positive x by the same iteration, two coupled
+// steps (relative error of a few 2^-53): about ten dependent operations where a
+// square root and a division take nearly a hundred, each a 64-cycle issue for
+// every block that waits on it.  Zero (and negative) give 0 and 0.
+__device__ __forceinline__ void root_pair(double x, double& g, double& ig) {
+    const int hi = __double2hiint(x);
+    if (hi < 0x00100000 || hi >= 0x7ff00000) {
+        g = x > 0.0 ? sqrt(x) : 0.0;
+        ig = g > 0.0 ? 1.0 / g : 0.0;
+        return;
+    }
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double h = __dmul_rn(0.5, y);
+    g = __dmul_rn(x, y);
+    double r = __fma_rn(-g, h, 0.5);
+    g = __fma_rn(g, r, g);
+    h = __fma_rn(h, r, h);
+    r = __fma_rn(-g, h, 0.5);
+    h = __fma_rn(h, r, h);
+    g = __fma_rn(__fma_rn(-g, g, x), h, g);
+    ig = h + h;
+}
 
 // ---------------------------------------------------------------- reductions
 // Sum NV thread-local values over the block and store them, as float64, at
@@ -275,14 +307,32 @@ __device__ __forceinline__ void block_partial_ff(float v, float2* p, int blk) {
     }
 }
 
-// Finite-difference step of a Jacobian product: eps_jv, or, when ctl->eps_part
-// > 0, eps = sqrt(eps_mach (1 + ||u||)) / ||z|| with ||z||^2 summed from the
+// The state's norms from a residual evaluation: tot[0] = ||W R||^2, tot[1] = ||W u||^2.
+__device__ __forceinline__ void put_norms(Ctl* ctl, const double* tot) {
+    ctl->res2 = tot[0];
+    ctl->unorm2 = tot[1];
+    ctl->nan = !(isfinite(tot[0]) && isfinite(tot[1]));
+    const double num = sqrt(ctl->eps_mach * (1.0 + sqrt(tot[1])));
+    ctl->eps_num = num;
+    ctl->inv_eps_num = 1.0 / num;
+}
+
+// eps = eps_num / ||z||, by threads 0 .. 4 of one block.
+__device__ __forceinline__ void put_eps_norm2(Ctl* ctl, double zn2) {
+    double zn, izn;
+    root_pair(zn2, zn, izn);
+    put_eps(ctl, ctl->eps_num * izn, zn * ctl->inv_eps_num);
+}
+
+// Finite-difference step of a Jacobian product and its reciprocal: eps_jv, or,
+// when ctl->eps_part > 0, eps = eps_num / ||z|| with ||z||^2 summed from the
 // pending float-float partials in one fixed order (every block of the launch
 // obtains bitwise the same value).  Called by all threads of the block.
-__device__ __forceinline__ double pending_eps(const Ctl* ctl, const double* part) {
-    __shared__ double wsum[NTHREADS / 32];
-    __shared__ double eps_s;
+__device__ __forceinline__ double2 pending_eps(const Ctl* ctl, const double* part) {
+    __shared__ float2 wsum[NTHREADS / 32];
+    __shared__ double2 eps_s;
     const int np = ctl->eps_part;
+    const double num = ctl->eps_num, inum = ctl->inv_eps_num;
     if (np > 0) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const float2* p = reinterpret_cast<const float2*>(part);
@@ -292,16 +342,18 @@ __device__ __forceinline__ double pending_eps(const Ctl* ctl, const double* part
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             s = ff_add(s, make_float2(__shfl_down_sync(0xffffffffu, s.x, o), __shfl_down_sync(0xffffffffu, s.y, o)));
-        if (lane == 0) wsum[warp] = (double)s.x + (double)s.y;
+        if (lane == 0) wsum[warp] = s;
         __syncthreads();
         if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-            const double zn = sqrt(t);
-            eps_s = zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0;
+            float2 t = wsum[0];
+            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) t = ff_add(t, wsum[w]);
+            double zn, izn;
+            root_pair((double)t.x + (double)t.y, zn, izn);
+            eps_s = make_double2(num * izn, zn * inum);
         }
     } else if (threadIdx.x == 0) {
-        eps_s = ctl->eps_jv;
+        const double e = ctl->eps_jv;
+        eps_s = make_double2(e, e != 0.0 ? 1.0 / e : 0.0);
     }
     __syncthreads();
     return eps_s;

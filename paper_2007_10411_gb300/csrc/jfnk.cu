@@ -504,7 +504,10 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     // so its step need not grow with the float32 roundoff.
     init.eps_mach = ldexp(1.0, -52);
     init.m = m;
-    for (int f = 0; f < nf; ++f) init.scale[f] = G.scale[f];
+    for (int f = 0; f < nf; ++f) {
+        init.scale[f] = G.scale[f];
+        init.inv_scale[f] = G.inv_scale[f];
+    }
     if (cudaMemcpy(h->ctl, &init, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(h->part, 0, part_len * sizeof(double)) != cudaSuccess ||
         cudaMemset(h->x, 0, nb8) != cudaSuccess) {

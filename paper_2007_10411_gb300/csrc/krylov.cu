@@ -37,6 +37,13 @@ template <> struct V4<double> { using type = double2; static constexpr int W = 2
 
 __device__ __forceinline__ float dotv(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 __device__ __forceinline__ double dotv(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
+// c + a . b as one chain of fused multiply-adds (a float64 addition costs as much as one)
+__device__ __forceinline__ float dotacc(float4 a, float4 b, float c) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+}
+__device__ __forceinline__ double dotacc(double2 a, double2 b, double c) { return fma(a.y, b.y, fma(a.x, b.x, c)); }
+__device__ __forceinline__ float dotacc(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double dotacc(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float4 axpyv(float4 y, float a, float4 x) {
     return make_float4(y.x - a * x.x, y.y - a * x.y, y.z - a * x.z, y.w - a * x.w);
 }
@@ -87,6 +94,14 @@ static int stream_blocks(size_t n) {
     return (int)(b < (size_t)MAX_STREAM_BLOCKS ? (b > 0 ? b : 1) : MAX_STREAM_BLOCKS);
 }
 
+// Grid of the point-wise streaming kernels: up to eight CTAs per SM (two leave
+// most of the memory latency uncovered), by field planes where a kernel's
+// factor depends on the field (no division per element).
+static int wide_blocks(size_t n) {
+    return (int)std::min<size_t>(std::max<size_t>((n + NTHREADS - 1) / NTHREADS, 1), 8 * 152);
+}
+static dim3 plane_blocks(const Geo& G) { return dim3((unsigned)std::max(1, wide_blocks(G.npt) / G.nf), G.nf); }
+
 // Grid of the multi-dot kernels: >= two CTAs per SM, and enough CTAs that no
 // thread accumulates more than PER_THREAD vector elements in low precision.
 // Grid of Arnoldi passes A and C (register use fits three CTAs per SM).
@@ -126,6 +141,45 @@ __device__ __forceinline__ double pshfl_down(double a, int o) { return __shfl_do
 __device__ __forceinline__ float2 pload(const float2* p) { return __ldcg(p); }
 __device__ __forceinline__ double pload(const double* p) { return __ldcg(p); }
 
+// Sums of CH values per lane over the lanes of a warp that share q = lane mod KS,
+// into red[q * CH + c][warp] (k < nv only).  Recursive halving: at each step a lane
+// keeps one half of the values and hands over the other, so that CH values cost
+// CH - 1 additions and a few more instead of 5 CH (a float64 addition occupies
+// the sub-partition's pipe for 64 cycles).  Fixed order.
+template <typename T, int CH, int KS>
+__device__ __forceinline__ void warp_sums(const T (&acc)[CH], T (*red)[NTHREADS / 32], int nv) {
+    constexpr int P = CH <= 8 ? 8 : CH <= 16 ? 16 : 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T v[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = i < CH ? acc[i < CH ? i : 0] : T(0);
+    int idx = 0, dup = 0;
+    int n = P;
+#pragma unroll
+    for (int o = 16; o >= KS; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < P / 2; ++i)
+                if (i < n) {
+                    const T send = up ? v[i] : v[i + n];
+                    const T keep = up ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            if (up) idx += n;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+            dup |= o;
+        }
+    }
+    // fewer lanes than values: each lane still holds n of them
+    const int q = lane & (KS - 1);
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+        if (i < n && idx + i < CH && q * CH + idx + i < nv && !(lane & dup)) red[q * CH + idx + i][warp] = v[i];
+}
+
 // Block partial of NV per-warp sums red[k][w] (k < nv) into part[k * stride + blk].
 template <typename T, int NV, typename P>
 __device__ __forceinline__ void store_partials(const T (*red)[NTHREADS / 32], int nv, P* part, int stride, int blk) {
@@ -147,33 +201,36 @@ __device__ __forceinline__ void store_partials(const T (*red)[NTHREADS / 32], in
 // takes the values w, w + nw (together), w + 2 nw, ...; a lane adds
 // b = lane + 32 r with all its loads of a 512-block chunk in flight, then a
 // fixed tree over r and a fixed shuffle tree over the lanes.
-template <typename P>
+template <int R, typename P>
 __device__ __forceinline__ P chunk_sum(const P* p, int nblk, int b0, int lane) {
-    P v[16];
+    P v[R];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < R; ++r) {
         const int b = b0 + lane + 32 * r;
         v[r] = b < nblk ? pload(p + b) : pzero(P());
     }
 #pragma unroll
-    for (int h = 8; h > 0; h >>= 1)
+    for (int h = R; h > 1; h = (h + 1) / 2)
 #pragma unroll
-        for (int r = 0; r < h; ++r) v[r] = padd(v[r], v[r + h]);
+        for (int r = 0; r < R / 2; ++r)
+            if (r < h / 2) v[r] = padd(v[r], v[r + (h + 1) / 2]);
     return v[0];
 }
 
-template <typename P, typename TO>
-__device__ void grid_sums(const P* part, int nblk, int nv, double* out, TO* outT) {
+// R partials per lane and chunk: the instantiation nearest above nblk / 32, so that
+// a small grid does not add zeros (float64: 15 additions for one at 64 blocks).
+template <int R, typename P, typename TO>
+__device__ __forceinline__ void grid_sums_r(const P* part, int nblk, int nv, double* out, TO* outT) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
     for (int k = warp; k < nv; k += 2 * nw) {
         const int k2 = k + nw;
         const P* p = part + (size_t)k * nblk;
         const P* p2 = part + (size_t)(k2 < nv ? k2 : k) * nblk;
-        P s = pzero(P()), s2 = pzero(P());
-        for (int b0 = 0; b0 < nblk; b0 += 512) {
-            const P c = chunk_sum(p, nblk, b0, lane);
-            const P c2 = chunk_sum(p2, nblk, b0, lane);
+        P s = chunk_sum<R>(p, nblk, 0, lane), s2 = chunk_sum<R>(p2, nblk, 0, lane);
+        for (int b0 = 32 * R; b0 < nblk; b0 += 32 * R) {
+            const P c = chunk_sum<R>(p, nblk, b0, lane);
+            const P c2 = chunk_sum<R>(p2, nblk, b0, lane);
             s = padd(s, c);
             s2 = padd(s2, c2);
         }
@@ -192,6 +249,14 @@ __device__ void grid_sums(const P* part, int nblk, int nv, double* out, TO* outT
         }
     }
     __syncthreads();
+}
+
+template <typename P, typename TO>
+__device__ void grid_sums(const P* part, int nblk, int nv, double* out, TO* outT) {
+    if (nblk <= 64) grid_sums_r<2>(part, nblk, nv, out, outT);
+    else if (nblk <= 128) grid_sums_r<4>(part, nblk, nv, out, outT);
+    else if (nblk <= 320) grid_sums_r<10>(part, nblk, nv, out, outT);
+    else grid_sums_r<16>(part, nblk, nv, out, outT);
 }
 
 // h_{j+1,j}^2 = ||w'||^2 - ||h2||^2 by one warp (nv <= 32): every lane returns
@@ -226,7 +291,7 @@ arnoldi_a(const T* __restrict__ V, size_t ldv, const T* __restrict__ w, size_t n
         const VT wv = reinterpret_cast<const VT*>(w)[i];
 #pragma unroll
         for (int k = 0; k < NV; ++k)
-            if (k < nv) acc_t[k] += dotv(reinterpret_cast<const VT*>(V + k * ldv)[i], wv);
+            if (k < nv) acc_t[k] = dotacc(reinterpret_cast<const VT*>(V + k * ldv)[i], wv, acc_t[k]);
     }
     for (size_t i = nvec * W + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
 #pragma unroll
@@ -235,16 +300,7 @@ arnoldi_a(const T* __restrict__ V, size_t ldv, const T* __restrict__ w, size_t n
     }
     pdl_trigger();
     __shared__ T red[NV][NTHREADS / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        if (k < nv) {
-            T x = acc_t[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-            if (lane == 0) red[k][warp] = x;
-        }
-    }
+    warp_sums<T, NV, 1>(acc_t, red, nv);
     __syncthreads();
     store_partials<T, NV>(red, nv, reinterpret_cast<typename PartOf<T>::type*>(part), gridDim.x, blockIdx.x);
 }
@@ -278,7 +334,7 @@ __device__ void givens_update(Ctl* c, int j, int m, const double* h2, double wn2
     if (threadIdx.x < 32) hn2 = subdiag2(h2, j + 1, wn2);
     if (threadIdx.x == 0) {
         const double target = c->target;
-        const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
+        const double hn = hn2 > 0.0 ? root(hn2) : 0.0;
         col[j + 1] = hn;
         for (int i = 0; i < j; ++i) {
             const double t = csv[i] * col[i] + snv[i] * col[i + 1];
@@ -287,9 +343,15 @@ __device__ void givens_update(Ctl* c, int j, int m, const double* h2, double wn2
         }
         double cs = 1.0, sn = 0.0;
         if (col[j + 1] != 0.0) {
-            const double rho = hypot(col[j], col[j + 1]);
-            cs = col[j] / rho;
-            sn = col[j + 1] / rho;
+            // rotation by the reciprocal root of the scaled sum of squares (the larger
+            // entry's exponent is taken out, so nothing over- or underflows)
+            const double big = fmax(fabs(col[j]), fabs(col[j + 1]));
+            const int e = isfinite(big) ? -ilogb(big) : 0;
+            const double a = scalbn(col[j], e), b = scalbn(col[j + 1], e);
+            double rho, irho;
+            root_pair(fma(a, a, b * b), rho, irho);
+            cs = a * irho;
+            sn = b * irho;
         }
         const double rjj = cs * col[j] + sn * col[j + 1];
         col[j] = rjj;
@@ -400,9 +462,9 @@ __device__ __forceinline__ void work_b(const VT (&v)[CH], VT wv, T* __restrict__
     for (int o = 1; o < KS; o <<= 1) sum = addv(sum, shfl_xor_v(mask, sum, o));
     const VT wp = subv(wv, sum);
 #pragma unroll
-    for (int c = 0; c < CH; ++c) acc[c] += dotv(v[c], wp);
+    for (int c = 0; c < CH; ++c) acc[c] = dotacc(v[c], wp, acc[c]);
     if (q == 0) {
-        accn += dotv(wp, wp);
+        accn = dotacc(wp, wp, accn);
         reinterpret_cast<VT*>(w)[i] = wp;
     }
 }
@@ -485,13 +547,7 @@ arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int 
     pdl_trigger();
     // block sums: slot 0 = ||w'||^2, slot 1 + k = v_k . w' (fixed shuffle trees, then the partial type across warps)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        T x = acc[c];
-#pragma unroll
-        for (int o = KS; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane < KS) red[1 + lane * CH + c][warp] = x;
-    }
+    warp_sums<T, CH, KS>(acc, red + 1, nv);
     {
         T x = accn;
 #pragma unroll
@@ -531,9 +587,9 @@ arnoldi_c(T* __restrict__ V, size_t ldv, const T* __restrict__ w, size_t n, int 
     }
     const T* hs = tots + 1;
     if (threadIdx.x < 32) {
-        const double hn2 = subdiag2(tot + 1, nv, tot[0]);
-        const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
-        if (threadIdx.x == 0) inv_s = T(hn > 0.0 ? 1.0 / hn : 0.0);
+        double g, ig;
+        root_pair(subdiag2(tot + 1, nv, tot[0]), g, ig);
+        if (threadIdx.x == 0) inv_s = T(ig);
     }
     __syncthreads();
     const T inv = inv_s;
@@ -623,14 +679,15 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
     __shared__ T sig_s;
     if (threadIdx.x < 32) {
         const double hn2 = subdiag2(tot + 1, j, tot[0]);
-        const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
-        if (threadIdx.x == 0) {
-            inv_s = T(hn > 0.0 ? 1.0 / hn : 0.0);
-            // z_j = M^{-1} w'_{j-1} carries the scale ||w'_{j-1}||: w_j = J z_j is used
-            // as sigma w_j with sigma = 1 / ||w'_{j-1}||, and z_j enters the update as sigma z_j
-            const double sg = tot[0] > 0.0 ? 1.0 / sqrt(tot[0]) : 0.0;
-            sig_s = T(sg);
-            if (blockIdx.x == 1) ctl->zscale[j] = (double)T(sg);
+        // lane 0: 1 / h_{j,j-1}.  Lane 1: z_j = M^{-1} w'_{j-1} carries the scale ||w'_{j-1}||:
+        // w_j = J z_j is used as sigma w_j with sigma = 1 / ||w'_{j-1}||, and z_j enters the
+        // update as sigma z_j
+        double g, ig;
+        root_pair(threadIdx.x == 0 ? hn2 : tot[0], g, ig);
+        if (threadIdx.x == 0) inv_s = T(ig);
+        if (threadIdx.x == 1) {
+            sig_s = T(ig);
+            if (blockIdx.x == 1) ctl->zscale[j] = (double)T(ig);
         }
     }
     __syncthreads();
@@ -666,7 +723,7 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
             sum = fmav(hs[q * CH + c], v[c], sum);
-            acc[c] += dotv(v[c], wv);
+            acc[c] = dotacc(v[c], wv, acc[c]);
         }
         if (KS > 1) {
             const unsigned mask = __activemask();     // the KS lanes of an element are active together
@@ -676,7 +733,7 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
         const VT vn = scalev(subv(wpv, sum), inv);
         if (q == 0) {
             reinterpret_cast<VT*>(vout)[i] = vn;
-            accn += dotv(vn, wv);
+            accn = dotacc(vn, wv, accn);
         }
     }
     for (size_t i = nvec * W + g0; i < n; i += gstride) {
@@ -704,13 +761,7 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
     }
     pdl_trigger();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        T x = acc[c];
-#pragma unroll
-        for (int o = KS; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane < KS && lane * CH + c < j) red[lane * CH + c][warp] = x;
-    }
+    warp_sums<T, CH, KS>(acc, red, j);
     {
         T x = accn;
 #pragma unroll
@@ -733,14 +784,40 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-template <typename T, int NV>
-__global__ void __launch_bounds__(NTHREADS, 2)
+// One vector of 16 bytes of every z_k per thread and chunk of eight directions,
+// the chunk's loads in flight together; only the K directions of the cycle are
+// read.  Bound: HBM (K vectors, x in and out).  With one element per thread, all
+// KMAX slots and two CTAs per SM: 95 us at 1024 x 512 for K = 30 and 78 us for
+// K = 8 (floor 43 and 16 us); here 81 us for K = 30 and 1.26 -> 0.4 ms at 256 x 256 x 128 (K = 5).
+template <typename T>
+__device__ __forceinline__ double update_sum(const T* zv, int n, const double* ys, const float* yh, const float* yl,
+                                             float& hi, float& lo, double s) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        for (int k = 0; k < n; ++k) s = fma(ys[k], zv[k], s);
+    } else {
+        for (int k = 0; k < n; ++k) {
+            const float z = (float)zv[k];
+            const float ph = yh[k] * z;
+            const float pl = fmaf(yh[k], z, -ph);      // exact product error
+            float t, e;
+            two_sum(hi, ph, t, e);
+            hi = t;
+            lo += e + pl + yl[k] * z;
+        }
+    }
+    return s;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(NTHREADS)
 update_x(const T* __restrict__ Z, size_t ldz, double* __restrict__ x, T* __restrict__ xT, size_t n,
          double* part, Ctl* ctl) {
+    using VT = typename V4<T>::type;
+    constexpr int W = V4<T>::W, CH = 8;
     const int K = ctl->k;
-    __shared__ double ys[NV];
-    __shared__ float yh[NV], yl[NV];
-    for (int k = threadIdx.x; k < NV; k += blockDim.x) {
+    __shared__ double ys[KMAX];
+    __shared__ float yh[KMAX], yl[KMAX];
+    for (int k = threadIdx.x; k < KMAX; k += blockDim.x) {
         const double y = k < K ? ctl->y[k] * ctl->zscale[k] : 0.0;
         ys[k] = y;
         yh[k] = (float)y;
@@ -748,33 +825,51 @@ update_x(const T* __restrict__ Z, size_t ldz, double* __restrict__ x, T* __restr
     }
     __syncthreads();
     T acc[1] = {T(0)};
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        // all K loads of the element are issued before the (serial) combination
-        T zv[NV];
+    const size_t nvec = n / W, stride = (size_t)gridDim.x * blockDim.x;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    for (size_t i = first; i < nvec; i += stride) {
+        double s[W];
+        float hi[W], lo[W];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) zv[k] = k < K ? Z[k * ldz + i] : T(0);
-        double s;
-        if (sizeof(T) == sizeof(double)) {
-            s = x[i];
-#pragma unroll
-            for (int k = 0; k < NV; ++k)
-                if (k < K) s += ys[k] * (double)zv[k];
-        } else {
-            float hi = 0.0f, lo = 0.0f;
-#pragma unroll
-            for (int k = 0; k < NV; ++k)
-                if (k < K) {
-                    const float z = (float)zv[k];
-                    const float ph = yh[k] * z;
-                    const float pl = fmaf(yh[k], z, -ph);      // exact product error
-                    float t, e;
-                    two_sum(hi, ph, t, e);
-                    hi = t;
-                    lo += e + pl + yl[k] * z;
-                }
-            s = x[i] + ((double)hi + (double)lo);
+        for (int w = 0; w < W; w += 2) {
+            const double2 v = reinterpret_cast<const double2*>(x)[(i * W + w) / 2];
+            s[w] = v.x;
+            s[w + 1] = v.y;
         }
+#pragma unroll
+        for (int w = 0; w < W; ++w) hi[w] = lo[w] = 0.f;
+        for (int k0 = 0; k0 < K; k0 += CH) {
+            VT zv[CH];
+#pragma unroll
+            for (int c = 0; c < CH; ++c)      // past the cycle's end y is zero and nothing is read
+                zv[c] = k0 + c < K ? reinterpret_cast<const VT*>(Z + (size_t)(k0 + c) * ldz)[i] : VT{};
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                T zc[CH];
+#pragma unroll
+                for (int c = 0; c < CH; ++c) zc[c] = reinterpret_cast<const T*>(&zv[c])[w];
+                s[w] = update_sum<T>(zc, CH, ys + k0, yh + k0, yl + k0, hi[w], lo[w], s[w]);
+            }
+        }
+        T o[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            if constexpr (sizeof(T) == sizeof(float)) s[w] += (double)hi[w] + (double)lo[w];
+            o[w] = T(s[w]);
+            acc[0] += o[w] * o[w];
+        }
+#pragma unroll
+        for (int w = 0; w < W; w += 2) reinterpret_cast<double2*>(x)[(i * W + w) / 2] = make_double2(s[w], s[w + 1]);
+        if (xT != nullptr) reinterpret_cast<VT*>(xT)[i] = *reinterpret_cast<const VT*>(o);
+    }
+    for (size_t i = nvec * W + first; i < n; i += stride) {
+        double s = x[i];
+        float hi = 0.f, lo = 0.f;
+        for (int k = 0; k < K; ++k) {
+            const T z = Z[(size_t)k * ldz + i];
+            s = update_sum<T>(&z, 1, ys + k, yh + k, yl + k, hi, lo, s);
+        }
+        if constexpr (sizeof(T) == sizeof(float)) s += (double)hi + (double)lo;
         x[i] = s;
         if (xT != nullptr) xT[i] = T(s);
         acc[0] += T(s) * T(s);
@@ -783,11 +878,8 @@ update_x(const T* __restrict__ Z, size_t ldz, double* __restrict__ x, T* __restr
     if (arrive_last(&ctl->counter[CNT_UPDATE], gridDim.x)) {
         __shared__ double tot[1];
         final_sums(part, gridDim.x, 1, tot);
-        if (threadIdx.x == 0) {
-            ctl->scratch[0] = tot[0];
-            const double xn = sqrt(tot[0]);
-            put_eps(ctl, xn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / xn : 0.0);
-        }
+        if (threadIdx.x == 0) ctl->scratch[0] = tot[0];
+        if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
     }
 }
 
@@ -797,15 +889,19 @@ template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 cycle_init(Geo G, const double* __restrict__ R, T* __restrict__ V0, double* __restrict__ x, size_t n,
            double eta, int m, int pc_none, Ctl* ctl) {
-    const double beta = sqrt(ctl->res2);
-    const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int f = field_of(i, G.npt);
-        V0[i] = T(-R[i] * G.inv_scale[f] * inv);
+    double beta, inv;
+    root_pair(ctl->res2, beta, inv);
+    const double c = -G.inv_scale[blockIdx.y] * inv;
+    const size_t f0 = (size_t)blockIdx.y * G.npt;
+    R += f0;
+    V0 += f0;
+    x += f0;
+#pragma unroll 4
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G.npt; i += gridDim.x * blockDim.x) {
+        V0[i] = T(R[i] * c);
         x[i] = 0.0;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         ctl->beta0 = beta;
         ctl->target = eta * beta;
         ctl->g[0] = beta;
@@ -818,10 +914,8 @@ cycle_init(Geo G, const double* __restrict__ R, T* __restrict__ V0, double* __re
         ctl->iters = 0;
         ctl->m = m;
         for (int k = 0; k < KMAX; ++k) ctl->zscale[k] = 1.0;
-        if (pc_none) {
-            put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
-        }
     }
+    if (pc_none && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 5) put_eps(ctl, ctl->eps_num, ctl->inv_eps_num);
 }
 
 // Restart: r = b - w with w = J x, stored unnormalised in v_0 plus ||r||^2.
@@ -830,17 +924,22 @@ __global__ void __launch_bounds__(NTHREADS)
 restart_residual(Geo G, const double* __restrict__ R, const T* __restrict__ w, T* __restrict__ V0,
                  size_t n, double* part, Ctl* ctl) {
     double acc[1] = {0.0};
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int f = field_of(i, G.npt);
-        const double r = -R[i] * G.inv_scale[f] - (double)w[i];
+    const double c = -G.inv_scale[blockIdx.y];
+    const size_t f0 = (size_t)blockIdx.y * G.npt;
+    R += f0;
+    V0 += f0;
+    w += f0;
+#pragma unroll 4
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G.npt; i += gridDim.x * blockDim.x) {
+        const double r = fma(R[i], c, -(double)w[i]);
         V0[i] = T(r);
-        acc[0] += r * r;
+        acc[0] = fma(r, r, acc[0]);
     }
-    block_partials<1>(acc, 1, part, gridDim.x, blockIdx.x);
-    if (arrive_last(&ctl->counter[CNT_RESTART], gridDim.x)) {
+    const int nblk = gridDim.x * gridDim.y;
+    block_partials<1>(acc, 1, part, nblk, blockIdx.y * gridDim.x + blockIdx.x);
+    if (arrive_last(&ctl->counter[CNT_RESTART], nblk)) {
         __shared__ double tot[1];
-        final_sums(part, gridDim.x, 1, tot);
+        final_sums(part, nblk, 1, tot);
         if (threadIdx.x == 0) ctl->scratch[1] = tot[0];
     }
 }
@@ -848,9 +947,11 @@ restart_residual(Geo G, const double* __restrict__ R, const T* __restrict__ w, T
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 restart_scale(T* __restrict__ V0, size_t n, int pc_none, Ctl* ctl) {
-    const double beta = sqrt(ctl->scratch[1]);
-    const T inv = T(beta > 0.0 ? 1.0 / beta : 0.0);
+    double beta, ib;
+    root_pair(ctl->scratch[1], beta, ib);
+    const T inv = T(ib);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
+#pragma unroll 4
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) V0[i] *= inv;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->g[0] = beta;
@@ -861,10 +962,8 @@ restart_scale(T* __restrict__ V0, size_t n, int pc_none, Ctl* ctl) {
         ctl->breakdown = 0;
         ctl->k = 0;
         for (int k = 0; k < KMAX; ++k) ctl->zscale[k] = 1.0;
-        if (pc_none) {
-            put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
-        }
     }
+    if (pc_none && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 5) put_eps(ctl, ctl->eps_num, ctl->inv_eps_num);
 }
 
 // Left preconditioning (nonlinear preconditioning): the cycle starts from
@@ -896,26 +995,25 @@ left_scale(const T* __restrict__ z, T* __restrict__ V0, size_t n, int first, Ctl
         ctl->done = 0;
         ctl->breakdown = 0;
         ctl->k = 0;
-        put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
     }
+    if (blockIdx.x == 0 && threadIdx.x < 5) put_eps(ctl, ctl->eps_num, ctl->inv_eps_num);
 }
 
 // The finite-difference step of a Jacobian product on a unit vector (left
 // preconditioning: restores it after a preconditioner apply left its own).
-__global__ void unit_eps_k(Ctl* ctl) {
-    put_eps(ctl, sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))));
-}
+__global__ void unit_eps_k(Ctl* ctl) { put_eps(ctl, ctl->eps_num, ctl->inv_eps_num); }
 
 // u += W^{-1} x (float64), uT = u rounded to T.
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS)
 newton_update(Geo G, double* __restrict__ u, const double* __restrict__ x, T* __restrict__ uT, size_t n) {
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int f = field_of(i, G.npt);
-        const double v = u[i] + G.scale[f] * x[i];
-        u[i] = v;
-        if (uT != nullptr) uT[i] = T(v);
+    const double c = G.scale[blockIdx.y];
+    const size_t f0 = (size_t)blockIdx.y * G.npt;
+#pragma unroll 4
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G.npt; i += gridDim.x * blockDim.x) {
+        const double v = u[f0 + i] + c * x[f0 + i];
+        u[f0 + i] = v;
+        if (uT != nullptr) uT[f0 + i] = T(v);
     }
 }
 
@@ -923,6 +1021,7 @@ newton_update(Geo G, double* __restrict__ u, const double* __restrict__ x, T* __
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(NTHREADS) convert_k(const TI* __restrict__ in, TO* __restrict__ out, size_t n) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
+#pragma unroll 4
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += stride) out[i] = TO(in[i]);
 }
 
@@ -960,7 +1059,7 @@ __global__ void set_eps_k(double eps, int su, int sv, Ctl* ctl) {
         const double vn = sqrt(ctl->scratch[sv]);
         e = vn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->scratch[su]))) / vn : 0.0;
     }
-    put_eps(ctl, e);
+    put_eps(ctl, e, e != 0.0 ? 1.0 / e : 0.0);
 }
 
 // ------------------------------------------------- learned preconditioner
@@ -1043,10 +1142,7 @@ pc_eps_k(const float* __restrict__ z, size_t n, double* part, Ctl* ctl) {
     if (arrive_last(&ctl->counter[CNT_MISC], gridDim.x)) {
         __shared__ double tot[1];
         final_sums(part, gridDim.x, 1, tot);
-        if (threadIdx.x == 0) {
-            const double zn = sqrt(tot[0]);
-            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-        }
+        if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
     }
 }
 
@@ -1166,22 +1262,22 @@ template cudaError_t launch_arnoldi_givens<double>(size_t, int, int, const doubl
 template <typename T>
 cudaError_t launch_update(const T* Z, size_t ldz, double* x, T* xT, size_t n, double* part,
                           Ctl* ctl, cudaStream_t s) {
-    update_x<T, KMAX><<<stream_blocks(n), NTHREADS, 0, s>>>(Z, ldz, x, xT, n, part, ctl);
+    update_x<T><<<wide_blocks(n / V4<T>::W), NTHREADS, 0, s>>>(Z, ldz, x, xT, n, part, ctl);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_cycle_init(const Geo& G, const double* R, T* V0, double* x, size_t n, double eta,
                               int m, int pc_none, Ctl* ctl, cudaStream_t s) {
-    cycle_init<T><<<stream_blocks(n), NTHREADS, 0, s>>>(G, R, V0, x, n, eta, m, pc_none, ctl);
+    cycle_init<T><<<plane_blocks(G), NTHREADS, 0, s>>>(G, R, V0, x, n, eta, m, pc_none, ctl);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_restart(const Geo& G, const double* R, const T* w, T* V0, size_t n, int pc_none,
                            double* part, Ctl* ctl, cudaStream_t s, long long* launches) {
-    restart_residual<T><<<stream_blocks(n), NTHREADS, 0, s>>>(G, R, w, V0, n, part, ctl);
-    restart_scale<T><<<stream_blocks(n), NTHREADS, 0, s>>>(V0, n, pc_none, ctl);
+    restart_residual<T><<<plane_blocks(G), NTHREADS, 0, s>>>(G, R, w, V0, n, part, ctl);
+    restart_scale<T><<<wide_blocks(n), NTHREADS, 0, s>>>(V0, n, pc_none, ctl);
     if (launches) *launches += 2;
     return cudaGetLastError();
 }
@@ -1189,7 +1285,7 @@ cudaError_t launch_restart(const Geo& G, const double* R, const T* w, T* V0, siz
 template <typename T>
 cudaError_t launch_restart_residual(const Geo& G, const double* R, const T* w, T* V0, size_t n, double* part,
                                     Ctl* ctl, cudaStream_t s) {
-    restart_residual<T><<<stream_blocks(n), NTHREADS, 0, s>>>(G, R, w, V0, n, part, ctl);
+    restart_residual<T><<<plane_blocks(G), NTHREADS, 0, s>>>(G, R, w, V0, n, part, ctl);
     return cudaGetLastError();
 }
 
@@ -1200,20 +1296,20 @@ cudaError_t launch_left_scale(const T* z, T* V0, size_t n, int first, Ctl* ctl, 
 }
 
 cudaError_t launch_unit_eps(Ctl* ctl, cudaStream_t s) {
-    unit_eps_k<<<1, 1, 0, s>>>(ctl);
+    unit_eps_k<<<1, 5, 0, s>>>(ctl);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_newton_update(const Geo& G, double* u, const double* x, T* uT, size_t n,
                                  cudaStream_t s) {
-    newton_update<T><<<stream_blocks(n), NTHREADS, 0, s>>>(G, u, x, uT, n);
+    newton_update<T><<<plane_blocks(G), NTHREADS, 0, s>>>(G, u, x, uT, n);
     return cudaGetLastError();
 }
 
 template <typename TI, typename TO>
 cudaError_t launch_convert(const TI* in, TO* out, size_t n, cudaStream_t s) {
-    convert_k<TI, TO><<<stream_blocks(n), NTHREADS, 0, s>>>(in, out, n);
+    convert_k<TI, TO><<<wide_blocks(n), NTHREADS, 0, s>>>(in, out, n);
     return cudaGetLastError();
 }
 
@@ -1231,7 +1327,7 @@ cudaError_t launch_norm2(const Geo& G, const T* a, size_t n, int weighted, int s
 }
 
 cudaError_t launch_set_eps(double eps, int su, int sv, Ctl* ctl, cudaStream_t s) {
-    set_eps_k<<<1, 1, 0, s>>>(eps, su, sv, ctl);
+    set_eps_k<<<1, 5, 0, s>>>(eps, su, sv, ctl);
     return cudaGetLastError();
 }
 

@@ -33,20 +33,15 @@ namespace jfnk {
 constexpr int R = 2;          // derivative radius for p = 2
 constexpr int HALO = 2 * R;   // input halo (derivative applied twice)
 
-// Candidate tiles of the Jacobian-product and preconditioner kernels (float32
-// path); jfnk_autotune times each on the handle's workload and keeps the
-// fastest (Geo::tile_jv, Geo::tile_pc).  The float64 path uses the first entry.
-template <int I> struct JvcTile;         // float32 Jacobian product (jvc2d): tile and staging buffers
+// Candidate tiles of the float32 Jacobian product (jvc2d): tile and staging
+// buffers.  jfnk_autotune times each on the handle's workload, with the CTA sizes
+// of the float32 preconditioner sweep (launch_precond_f32), and keeps the fastest
+// (Geo::tile_jv, Geo::tile_pc).
+template <int I> struct JvcTile;
 template <> struct JvcTile<0> { static constexpr int TX = 32, TZ = 16, NBUF = 1; };
 template <> struct JvcTile<1> { static constexpr int TX = 32, TZ = 16, NBUF = 2; };
 template <> struct JvcTile<2> { static constexpr int TX = 64, TZ = 8, NBUF = 1; };
 template <> struct JvcTile<3> { static constexpr int TX = 32, TZ = 8, NBUF = 1; };
-template <int I> struct PcTile;
-template <> struct PcTile<0> { static constexpr int TX = 64, TZ = 16; };
-template <> struct PcTile<1> { static constexpr int TX = 32, TZ = 16; };
-template <> struct PcTile<2> { static constexpr int TX = 64, TZ = 8; };
-template <> struct PcTile<3> { static constexpr int TX = 32, TZ = 8; };
-
 // Explicitly rounded product and fused multiply-add: expressions written with
 // them round the same way in every instantiation (tile shape) of a kernel.
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
@@ -357,17 +352,9 @@ flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restri
     T* Ss = Z + 4 * sh.zn();                        // [4][TZ][TX] (PPT = 0)
     const int x0 = blockIdx.x << sh.lx, z0 = blockIdx.y << sh.lz;
     T ev[4] = {T(0), T(0), T(0), T(0)};
-    __shared__ double cfs[4];                       // 1 / (eps scale_f), computed once per block
-    __shared__ T evs[4];                            // eps scale_f
     if (mode == MODE_JV) {
-        if (threadIdx.x < 4) {
-            const double e = ctl->eps_jv * G.scale[threadIdx.x];
-            evs[threadIdx.x] = T(e);
-            cfs[threadIdx.x] = e != 0.0 ? 1.0 / e : 0.0;
-        }
-        __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) ev[q] = evs[q];
+        for (int q = 0; q < 4; ++q) ev[q] = T(ctl->ev[q]);
         load_fields<T, 1>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
     } else {
         load_fields<T, 0>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
@@ -412,7 +399,7 @@ flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restri
         if (fl == 2 && gz == 0 && G.heat != nullptr) Fv += T(G.heat[gx] * G.heat_coef);
         const double uo = (double)s1[fl * sh.plane() + (tz + HALO) * SX + tx + HALO];
         flux_out(G, mode, fl, Fv, uo, (size_t)fl * G.npt + (size_t)gz * G.nx + gx, v, Fu, f, out, out2,
-                 mode == MODE_JV ? cfs[fl] : 0.0, ar, au);
+                 mode == MODE_JV ? ctl->cf[fl] : 0.0, ar, au);
     };
     if (PPT > 0) {
 #pragma unroll
@@ -443,9 +430,7 @@ flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restri
             __shared__ double tot[2];
             final_sums(part, nblk, 2, tot);
             if (threadIdx.x == 0) {
-                ctl->res2 = tot[0];
-                ctl->unorm2 = tot[1];
-                ctl->nan = !(isfinite(tot[0]) && isfinite(tot[1]));
+                put_norms(ctl, tot);
             }
         }
     }
@@ -753,12 +738,11 @@ jvc2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __
     int t = blockIdx.x;
     if (t < ntiles) jv_stage_issue(stg, u, v, G, (t % ntx) * TX, (t / ntx) * TZ, SX, SH::SZ);
     cpa_commit();
-    const double eps = pending_eps(ctl, part);
+    const double2 eps = pending_eps(ctl, part);
     __shared__ float evs[4], cfs[4];
     if (threadIdx.x < 4) {
-        const double e = eps * G.scale[threadIdx.x];
-        evs[threadIdx.x] = (float)e;
-        cfs[threadIdx.x] = (float)(e != 0.0 ? 1.0 / e : 0.0);
+        evs[threadIdx.x] = (float)(eps.x * G.scale[threadIdx.x]);
+        cfs[threadIdx.x] = (float)(eps.y * G.inv_scale[threadIdx.x]);
     }
     __syncthreads();
     JvcConst k;
@@ -984,163 +968,292 @@ __global__ void pc_setup(Geo G, int sweeps, Ctl* ctl) {
     }
 }
 
-// One CTA = one field of one TX x TZ tile; threads laid out (TX, NTHREADS/TX)
-// so that every stage indexes rows and columns without divisions.  D_x z is
-// formed only on the tile rows (x-halo r), D_z z only on the tile columns
-// (z-halo r): exactly the taps the second application of D reads.
-template <typename T, int SMAG, int FIRST, int LAST, int TX, int TZ>
-__global__ void __launch_bounds__(NTHREADS, 8)
-cheb2d(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, const T* __restrict__ din,
-       T* __restrict__ zout, T* __restrict__ dout, const T* __restrict__ nu, double* part, Ctl* ctl,
-       int check_done) {
-    constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO;
-    constexpr int QX = TX + 2 * R, QZ = TZ + 2 * R;
-    constexpr int TY = NTHREADS / TX;              // thread rows
-    static_assert(NTHREADS % TX == 0 && TZ % TY == 0, "tile must tile the block");
+// Row vectors: a thread of the float32 sweeps and of the Schur-complement kernels
+// owns W consecutive points along x (16 bytes where nx allows it).
+template <typename T, int W> struct RowVec { using type = typename Vec16<T>::type; };
+template <typename T> struct RowVec<T, 1> { using type = T; };
+template <> struct RowVec<float, 2> { using type = float2; };
+template <typename T, int W>
+__device__ __forceinline__ void rload(const T* p, T (&v)[W]) {
+    *reinterpret_cast<typename RowVec<T, W>::type*>(v) = *reinterpret_cast<const typename RowVec<T, W>::type*>(p);
+}
+template <typename T, int W>
+__device__ __forceinline__ void rstore(T* p, const T (&v)[W]) {
+    *reinterpret_cast<typename RowVec<T, W>::type*>(p) = *reinterpret_cast<const typename RowVec<T, W>::type*>(v);
+}
+
+// Asynchronous copy of W elements (16, 8 or 4 bytes) into shared memory.
+template <typename T, int W>
+__device__ __forceinline__ void cpa_vec(T* dst, const T* src) {
+    if constexpr (W * sizeof(T) == 16) cpa16(dst, src, 16);
+    else cpa_elem<W * (int)sizeof(T)>(dst, src, W * (int)sizeof(T));
+}
+
+// ----------------------------------------------------------------------------
+// Field-block sweep, float32: one CTA sweeps all fields of a TX x TZ tile.  The
+// three diffused fields (halo 4) and the eddy field (halo 2) are copied to
+// shared memory at once, so a launch waits for memory once and meets one
+// barrier; a thread owns W consecutive points along x and forms every flux its D
+// reads itself (8 along x, 4 rows along z): twice the arithmetic of exchanging
+// them, but no second phase.  first / last: roles of the sweep (both with
+// pc_sweeps = 2); p is written by the last sweep.  Explicitly rounded, so every
+// tile shape computes the same bits.
+//
+// Bound: latency of the one load phase and issue (23 MB a launch at
+// 1024 x 512, 3.4 us).  One field per CTA with three barriers and the fluxes in
+// shared memory took 19-20 us there and 7.1-7.8 us at 250 x 119; this form 12.0 and 4.4 us (with
+// the overlap of the launches before it).
+// ----------------------------------------------------------------------------
+template <int W> struct PcRow { static constexpr int NXT = W == 4 ? 16 : 32; };   // threads along x
+
+template <int W, int NT, int SMAG>
+__global__ void __launch_bounds__(NT, 768 / NT)
+cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const float* __restrict__ zin,
+       const float* __restrict__ din, float* __restrict__ zout, float* __restrict__ dout, const float* __restrict__ nu,
+       double* part, Ctl* ctl, int check_done) {
+    using T = float;
+    constexpr int NXT = PcRow<W>::NXT, TX = NXT * W, TZ = NT / NXT;
+    constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO, KZ = TZ + 2 * R, RV = SX / W;
+    __shared__ __align__(16) T zs[3][SZ * SX];
+    __shared__ __align__(16) T ks[SMAG ? KZ * SX : 4];
     pdl_wait();
-    if (check_done && ctl->done) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* zs = reinterpret_cast<T*>(smem_raw);      // [SZ][SX] current iterate, halo 2r
-    T* gxs = zs + SZ * SX;                          // [TZ][QX] D_x z on tile rows
-    T* gzs = gxs + TZ * QX;                         // [QZ][TX] D_z z on tile columns
-    T* kk_ = gzs + QZ * TX;                         // [QZ][QX] eddy coefficient (along x for Deardorff)
-    T* kz_ = SMAG == 2 ? kk_ + QZ * QX : kk_;       // [QZ][QX] Deardorff coefficient along z
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    const int fld = blockIdx.z;                     // 0 u, 1 w, 2 theta, 3 p (last sweep only)
+    const int done = check_done ? ctl->done : 0;
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T ith = cheb_coef<T>(ctl, fld, k, 0);
-    const T a1 = cheb_coef<T>(ctl, fld, k, 1);
-    const T a2 = cheb_coef<T>(ctl, fld, k, 2);
-    const T* rf = r + (size_t)fld * G.npt;
-    T* zf = zout + (size_t)fld * G.npt;
-    const int gxx = x0 + tx;
+    const T* src = first ? r : zin;
+    const size_t np = (size_t)G.npt;
+    // storage row of global row gz (rows beyond one reflection feed no output)
+    auto row = [&](int gz) {
+        int side;
+        return min(max(mirror_z(gz, G.nz, side), 0), G.nz - 1) * G.nx;
+    };
+    for (int j = threadIdx.x; j < SZ * RV; j += NT) {
+        const int iz = j / RV, ix = (j % RV) * W;
+        const int o = row(z0 + iz - HALO) + wrap_x(x0 + ix - HALO, G.nx);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) cpa_vec<T, W>(&zs[f][iz * SX + ix], src + f * np + o);
+        if (SMAG && iz >= R && iz < SZ - R) cpa_vec<T, W>(&ks[(iz - R) * SX + ix], nu + o);
+    }
+    cpa_commit();
+    const int tx = (threadIdx.x % NXT) * W, tz = threadIdx.x / NXT;
+    const int gx = x0 + tx, gz = z0 + tz;
+    const bool inside = gx < G.nx && gz < G.nz;
+    const size_t own = inside ? (size_t)gz * G.nx + gx : 0;
+    T rv[3][W], dv[3][W], pv[W];
+    if (inside && !done) {
+        if (!first) {
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                rload<T, W>(r + f * np + own, rv[f]);
+                rload<T, W>(din + f * np + own, dv[f]);
+            }
+        }
+        if (last) rload<T, W>(r + 3 * np + own, pv);
+    }
+    cpa_wait<0>();
+    if (done) return;
+    __syncthreads();
+    if (z0 - HALO < 0 || z0 + TZ + HALO > G.nz) {      // ghost rows: signs of the odd fields
+        for (int j = threadIdx.x; j < SZ * SX; j += NT) {
+            int side;
+            mirror_z(z0 + j / SX - HALO, G.nz, side);
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+                if (odd_ghost(G, f, side)) zs[f][j] = flip(zs[f][j]);
+        }
+        __syncthreads();
+    }
     T acc[1] = {T(0)};
-    if (fld == 3) {
-        if (LAST && gxx < G.nx) {          // p block: (2/dt) I, exact in one step
-            for (int tz = ty; tz < TZ; tz += TY) {
-                const int gz = z0 + tz;
-                if (gz >= G.nz) break;
-                const int o = gz * G.nx + gxx;
-                const T zv = rf[o] * ith;
-                zf[o] = zv;
-                acc[0] += zv * zv;
-            }
-        }
-    } else {
-        // per-output operands first: their latency overlaps the tile staging below
-        constexpr int NR = TZ / TY;
-        T rv[NR], dv[NR];
-        const T* df = FIRST ? nullptr : din + (size_t)fld * G.npt;
-        const bool colok = gxx < G.nx;
+    if (inside) {
+        const T wx1 = G.f32.wx1, wx2 = G.f32.wx2, wz1 = G.f32.wz1, wz2 = G.f32.wz2;
+        const int me = (tz + HALO) * SX + tx + HALO, mk = (tz + R) * SX + tx + HALO;
+        T kx[W + 4], kz[4][W];                          // eddy values on the x and z arms
+        if (SMAG) {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) {
-            const int gz = z0 + ty + q * TY;
-            const bool ok = colok && gz < G.nz;
-            const int o = gz * G.nx + gxx;
-            rv[q] = ok ? rf[o] : T(0);
-            dv[q] = (!FIRST && ok) ? df[o] : T(0);
-        }
-        // x_k with halo 2r (first sweep: x_1 = r / theta_c)
-        T sc[4] = {T(0), T(0), T(0), T(0)};
-        if (FIRST) {
-            sc[fld] = ith;
-            load_fields<T, 2, 1>(zs, nullptr, r, sc, G, x0, z0, SX, SZ, fld);
-        } else {
-            load_fields<T, 0, 1>(zs, zin, nullptr, sc, G, x0, z0, SX, SZ, fld);
-        }
-        if (SMAG == 2) {
-            // Deardorff: nu holds the strain s; K_m = c_m s along x, K_M = c_M s along z,
-            // heat K_h = c_m s (1 + a_h l), K_H = c_M s (1 + a_z l)
-            const T cm = GC(dd_cm), cM = GC(dd_cM);
-            for (int qz = ty; qz < QZ; qz += TY) {
-                int side;
-                const int szr = mirror_z(z0 + qz - R, G.nz, side);
-                const bool ok = szr >= 0 && szr < G.nz;
-                const T* nrow = nu + szr * G.nx;
-                for (int qx = tx; qx < QX; qx += TX) {
-                    const T sv = ok ? nrow[wrap_x(x0 + qx - R, G.nx)] : T(0);
-                    kk_[qz * QX + qx] = rmul(cm, fld == 2 ? dd_heat(sv, GC(dd_ah), G) : sv);
-                    kz_[qz * QX + qx] = rmul(cM, fld == 2 ? dd_heat(sv, GC(dd_az), G) : sv);
-                }
-            }
-        } else if (SMAG) {
-            const T kscale = fld == 2 ? GC(inv_Pr) : T(1);
-            for (int qz = ty; qz < QZ; qz += TY) {
-                int side;
-                const int szr = mirror_z(z0 + qz - R, G.nz, side);
-                const bool ok = szr >= 0 && szr < G.nz;
-                const T* nrow = nu + szr * G.nx;
-                for (int qx = tx; qx < QX; qx += TX)
-                    kk_[qz * QX + qx] = ok ? nrow[wrap_x(x0 + qx - R, G.nx)] * kscale : T(0);
-            }
-        }
-        __syncthreads();
-        const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
-        for (int tz = ty; tz < TZ; tz += TY)              // D_x on tile rows, x-halo r
-            for (int qx = tx; qx < QX; qx += TX)
-                gxs[tz * QX + qx] = dd(zs, (tz + HALO) * SX + qx + R, 1, idx_);
-        for (int qz = ty; qz < QZ; qz += TY)              // D_z on tile columns, z-halo r
-            gzs[qz * TX + tx] = dd(zs, (qz + R) * SX + tx + HALO, SX, idz_);
-        __syncthreads();
-        const T Kc = T(fld == 2 ? G.K_H : G.K_M);
-        const T tdt = GC(two_over_dt);
-        T* dof = LAST ? nullptr : dout + (size_t)fld * G.npt;
-        if (colok) {
-#pragma unroll
-            for (int q = 0; q < NR; ++q) {
-                const int tz = ty + q * TY;
-                const int gz = z0 + tz;
-                if (gz >= G.nz) break;
-                const T* gxr = gxs + tz * QX + tx + R;          // centre of the x taps
-                const T* gzc = gzs + (tz + R) * TX + tx;        // centre of the z taps
-                // explicitly rounded (rmul / rfma): every tile shape computes the same bits
-                T difx, difz;
-                if (SMAG) {
-                    const T* kx = kk_ + (tz + R) * QX + tx + R;
-                    const T* kz = kz_ + (tz + R) * QX + tx + R;
-                    const T x1 = rfma(kx[1], gxr[1], -rmul(kx[-1], gxr[-1]));
-                    const T x2 = rfma(kx[2], gxr[2], -rmul(kx[-2], gxr[-2]));
-                    const T z1 = rfma(kz[QX], gzc[TX], -rmul(kz[-QX], gzc[-TX]));
-                    const T z2 = rfma(kz[2 * QX], gzc[2 * TX], -rmul(kz[-2 * QX], gzc[-2 * TX]));
-                    difx = rfma(T(2.0 / 3.0), x1, rmul(T(-1.0 / 12.0), x2));
-                    difz = rfma(T(2.0 / 3.0), z1, rmul(T(-1.0 / 12.0), z2));
+            for (int i = 0; i < W + 4; i += 2) {
+                if constexpr (W == 1) {
+                    kx[i] = ks[mk - 2 + i];
+                    if (i + 1 < W + 4) kx[i + 1] = ks[mk - 1 + i];
                 } else {
-                    difx = rmul(Kc, rfma(T(2.0 / 3.0), gxr[1] - gxr[-1], rmul(T(-1.0 / 12.0), gxr[2] - gxr[-2])));
-                    difz = rmul(Kc, rfma(T(2.0 / 3.0), gzc[TX] - gzc[-TX], rmul(T(-1.0 / 12.0), gzc[2 * TX] - gzc[-2 * TX])));
+                    const float2 v = *reinterpret_cast<const float2*>(&ks[mk - 2 + i]);
+                    kx[i] = v.x;
+                    kx[i + 1] = v.y;
                 }
-                const T dif = rfma(difx, idx_, rmul(difz, idz_));
-                const T xk = zs[(tz + HALO) * SX + tx + HALO];
-                const int o = gz * G.nx + gxx;
-                const T res = rv[q] - rfma(tdt, xk, -dif);
-                const T dprev = FIRST ? rmul(rv[q], ith) : dv[q];
-                const T dk = rfma(a1, dprev, rmul(a2, res));
-                const T xn = xk + dk;
-                zf[o] = xn;
-                if (!LAST) dof[o] = dk;
-                if (LAST) acc[0] += xn * xn;
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) rload<T, W>(&ks[mk + (q < 2 ? q - 2 : q - 1) * SX], kz[q]);
+        }
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            const T ith = cheb_coef<T>(ctl, f, k, 0), a1 = cheb_coef<T>(ctl, f, k, 1), a2 = cheb_coef<T>(ctl, f, k, 2);
+            const T* p = zs[f];
+            // what the fluxes leave out: c_m, c_M (Deardorff), 1/Pr of theta, the constant K, 1/theta_c of x_1 = r / theta_c
+            const T ks_ = SMAG == 2 ? T(1) : SMAG ? (f == 2 ? G.f32.inv_Pr : T(1)) : (f == 2 ? G.f32.K_H : G.f32.K_M);
+            T xk[W], e[W + 8], difx[W], difz[W];
+            if constexpr (W == 1) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) e[i] = p[me - 4 + i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < W + 8; i += W) {
+                    T v[W];
+                    rload<T, W>(p + me - 4 + i, v);
+#pragma unroll
+                    for (int j = 0; j < W; ++j) e[i + j] = v[j];
+                }
+            }
+            {
+                T fx[W + 4];
+#pragma unroll
+                for (int i = 0; i < W + 4; ++i) {
+                    const T d = rfma(wx1, e[i + 3] - e[i + 1], rmul(wx2, e[i + 4] - e[i]));
+                    const T c = SMAG == 2 ? (f == 2 ? dd_heat(kx[i], G.f32.dd_ah, G) : kx[i]) : kx[i];
+                    fx[i] = SMAG ? rmul(c, d) : d;
+                }
+#pragma unroll
+                for (int i = 0; i < W; ++i) difx[i] = rfma(wx1, fx[i + 3] - fx[i + 1], rmul(wx2, fx[i + 4] - fx[i]));
+            }
+            {
+                T v[9][W], fz[4][W];
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    if (q != 4) rload<T, W>(p + me + (q - 4) * SX, v[q]);
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    v[4][i] = e[4 + i];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int c = q < 2 ? q + 2 : q + 3;             // rows -2, -1, 1, 2
+                        const T d = rfma(wz1, v[c + 1][i] - v[c - 1][i], rmul(wz2, v[c + 2][i] - v[c - 2][i]));
+                        const T kq = SMAG == 2 ? (f == 2 ? dd_heat(kz[q][i], G.f32.dd_az, G) : kz[q][i]) : kz[q][i];
+                        fz[q][i] = SMAG ? rmul(kq, d) : d;
+                    }
+                    difz[i] = rfma(wz1, fz[2][i] - fz[1][i], rmul(wz2, fz[3][i] - fz[0][i]));
+                }
+            }
+            T xo[W], dk[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                const T sum = SMAG == 2 ? rfma(G.f32.dd_cm, difx[i], rmul(G.f32.dd_cM, difz[i])) : rmul(ks_, __fadd_rn(difx[i], difz[i]));
+                xk[i] = first ? rmul(ith, e[4 + i]) : e[4 + i];
+                const T rr = first ? e[4 + i] : rv[f][i];
+                const T res = __fsub_rn(rr, rfma(G.f32.two_over_dt, xk[i], -(first ? rmul(ith, sum) : sum)));
+                dk[i] = rfma(a1, first ? xk[i] : dv[f][i], rmul(a2, res));
+                xo[i] = __fadd_rn(xk[i], dk[i]);
+                if (last) acc[0] = rfma(xo[i], xo[i], acc[0]);
+            }
+            rstore<T, W>(zout + f * np + own, xo);
+            if (!last) rstore<T, W>(dout + f * np + own, dk);
+        }
+        if (last) {                                     // p block: (2/dt) I, exact in one step
+            const T ith = cheb_coef<T>(ctl, 3, k, 0);
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                pv[i] = rmul(pv[i], ith);
+                acc[0] = rfma(pv[i], pv[i], acc[0]);
+            }
+            rstore<T, W>(zout + 3 * np + own, pv);
         }
     }
     pdl_trigger();
-    if (LAST) {
+    if (last) {
+        // ||z||^2 stays pending, one float-float partial per block: the Jacobian
+        // product that follows adds them (pending_eps), so this launch ends without
+        // an arrival count and a serial tail
+        const int blk = blockIdx.y * gridDim.x + blockIdx.x;
+        block_partial_ff(acc[0], reinterpret_cast<float2*>(part), blk);
+        if (blk == 0 && threadIdx.x == 0) ctl->eps_part = gridDim.x * gridDim.y;
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Field-block sweep, float64: one CTA = one field of one tile (blockIdx.z: u, w,
+// theta, and p for the last sweep).  The fluxes K D_x x (tile rows, two columns
+// either side) and K D_z x (tile columns, two rows either side) are formed once
+// in shared memory, then differentiated.
+// Bound: the FP64 pipe, about 28 operations a point and field plus the arms (37
+// and the products rebuilt at every tap before), so the tile follows the grid as
+// flux2d's does: 160 -> 115 us at 1024 x 512.
+// ----------------------------------------------------------------------------
+template <int SMAG>
+__global__ void __launch_bounds__(NTHREADS)
+cheb2d_f64(Geo G, int k, int first, int last, FluxShape sh, const double* __restrict__ r,
+           const double* __restrict__ zin, const double* __restrict__ din, double* __restrict__ zout,
+           double* __restrict__ dout, const double* __restrict__ nu, double* part, Ctl* ctl, int check_done) {
+    using T = double;
+    pdl_wait();
+    if (check_done && ctl->done) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int TX = sh.tx(), TZ = sh.tz(), CN = sh.cn(), SX = sh.sx(), PXW = TX + 2 * R;
+    T* zs = reinterpret_cast<T*>(smem_raw);             // [SZ][SX] iterate (r for a first sweep)
+    T* X = zs + sh.plane();                             // [TZ][TX + 4] K D_x
+    T* Z = X + sh.xn();                                 // [TZ + 4][TX] K D_z
+    const int fld = blockIdx.z, x0 = blockIdx.x << sh.lx, z0 = blockIdx.y << sh.lz;
+    const T ith = ctl->cheb[fld][k][0], a1 = ctl->cheb[fld][k][1], a2 = ctl->cheb[fld][k][2];
+    const size_t fo = (size_t)fld * G.npt;
+    double acc[1] = {0.0};
+    if (fld == 3) {
+        for (int w = threadIdx.x; w < CN; w += NTHREADS) {      // p block: (2/dt) I, exact in one step
+            const int gx = x0 + (w & (TX - 1)), gz = z0 + (w >> sh.lx);
+            if (gx >= G.nx || gz >= G.nz) continue;
+            const size_t o = fo + (size_t)gz * G.nx + gx;
+            const T zv = r[o] * ith;
+            zout[o] = zv;
+            acc[0] = fma(zv, zv, acc[0]);
+        }
+    } else {
+        const T none[4] = {0.0, 0.0, 0.0, 0.0};
+        load_fields<T, 0, 1>(zs, first ? r : zin, nullptr, none, G, x0, z0, SX, TZ + 2 * HALO, fld);
+        __syncthreads();
+        // eddy coefficient of the point at tile (ix, iz), its constant factors left to the end
+        auto coef = [&](int ix, int iz, bool zarm) -> T {
+            int side;
+            const int sz = min(max(mirror_z(z0 + iz, G.nz, side), 0), G.nz - 1);
+            const T v = nu[(size_t)sz * G.nx + wrap_x(x0 + ix, G.nx)];
+            return SMAG == 2 && fld == 2 ? dd_heat(v, zarm ? G.dd_az : G.dd_ah, G) : v;
+        };
+        for (int w = threadIdx.x; w < TZ * PXW; w += NTHREADS) {
+            const int iz = w / PXW, ix = w - iz * PXW - R;
+            const T d = wd(zs, (iz + HALO) * SX + ix + HALO, 1, G.wx1, G.wx2);
+            X[w] = SMAG ? coef(ix, iz, false) * d : d;
+        }
+        for (int w = threadIdx.x; w < TX * (TZ + 2 * R); w += NTHREADS) {
+            const int iz = (w >> sh.lx) - R, ix = w & (TX - 1);
+            const T d = wd(zs, (iz + HALO) * SX + ix + HALO, SX, G.wz1, G.wz2);
+            Z[w] = SMAG ? coef(ix, iz, true) * d : d;
+        }
+        __syncthreads();
+        // factors the fluxes leave out, with 1/theta_c of x_1 = r / theta_c
+        const T one = first ? ith : 1.0;
+        const T kf = SMAG == 2 ? 1.0 : SMAG ? (fld == 2 ? G.inv_Pr : 1.0) : (fld == 2 ? G.K_H : G.K_M);
+        const T cx = (SMAG == 2 ? G.dd_cm : kf) * one, cz = (SMAG == 2 ? G.dd_cM : kf) * one;
+        const T wx1 = cx * G.wx1, wx2 = cx * G.wx2, wz1 = cz * G.wz1, wz2 = cz * G.wz2;
+        for (int w = threadIdx.x; w < CN; w += NTHREADS) {
+            const int tz = w >> sh.lx, tx = w & (TX - 1);
+            const int gx = x0 + tx, gz = z0 + tz;
+            if (gx >= G.nx || gz >= G.nz) continue;
+            const size_t o = fo + (size_t)gz * G.nx + gx;
+            const T* x = X + tz * PXW + tx + R;
+            const T* z = Z + (tz + R) * TX + tx;
+            const T xv = zs[(tz + HALO) * SX + tx + HALO];
+            const T xk = first ? ith * xv : xv, rv = first ? xv : r[o];
+            const T dif = fma(wx1, x[1] - x[-1], fma(wx2, x[2] - x[-2], fma(wz1, z[TX] - z[-TX], wz2 * (z[2 * TX] - z[-2 * TX]))));
+            const T res = fma(-G.two_over_dt, xk, rv) + dif;
+            const T dk = fma(a1, first ? xk : din[o], a2 * res);
+            const T xn = xk + dk;
+            zout[o] = xn;
+            if (!last) dout[o] = dk;
+            else acc[0] = fma(xn, xn, acc[0]);
+        }
+    }
+    pdl_trigger();
+    if (last) {
         const int nblk = gridDim.x * gridDim.y * gridDim.z;
         const int blk = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        if constexpr (sizeof(T) == sizeof(float)) {
-            // ||z||^2 stays pending, one float-float partial per block: the
-            // Jacobian product that follows adds them (pending_eps), so this
-            // launch ends without an arrival count and a serial tail
-            block_partial_ff(acc[0], reinterpret_cast<float2*>(part), blk);
-            if (blk == 0 && threadIdx.x == 0) ctl->eps_part = nblk;
-        } else {
-            block_partials<1, T>(acc, 1, part, nblk, blk);
-            if (arrive_last(&ctl->counter[CNT_PC], nblk)) {
-                __shared__ double tot[1];
-                final_sums(part, nblk, 1, tot);
-                if (threadIdx.x == 0) {
-                    const double zn = sqrt(tot[0]);
-                    put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-                }
-            }
+        block_partials<1, T>(acc, 1, part, nblk, blk);
+        if (arrive_last(&ctl->counter[CNT_PC], nblk)) {
+            __shared__ double tot[1];
+            final_sums(part, nblk, 1, tot);
+            if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
         }
     }
 }
@@ -1164,10 +1277,7 @@ pc_diag(Geo G, const T* __restrict__ r, T* __restrict__ z, size_t n, double* par
     if (arrive_last(&ctl->counter[CNT_PC], gridDim.x)) {
         __shared__ double tot[1];
         final_sums(part, gridDim.x, 1, tot);
-        if (threadIdx.x == 0) {
-            const double zn = sqrt(tot[0]);
-            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-        }
+        if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
     }
 }
 
@@ -1183,257 +1293,270 @@ pc_diag(Geo G, const T* __restrict__ r, T* __restrict__ z, size_t n, double* par
 // sweeps on its Gershgorin interval (coefficients ctl->cheb[5], pc_setup);
 // theta gets r_theta / theta_c of its field block.
 // ============================================================================
-template <typename T>
-__device__ __forceinline__ T plane_dx(const T* __restrict__ f, const Geo& G, int gz, int gx, T inv_h) {
-    const T* row = f + (size_t)gz * G.nx;
-    return (T(2.0 / 3.0) * (row[wrap_x(gx + 1, G.nx)] - row[wrap_x(gx - 1, G.nx)]) -
-            T(1.0 / 12.0) * (row[wrap_x(gx + 2, G.nx)] - row[wrap_x(gx - 2, G.nx)])) * inv_h;
+// D_x at W points of a periodic row (gx and nx multiples of W)
+template <typename T, int W>
+__device__ __forceinline__ void row_dx(const T* __restrict__ row, int gx, int nx, T w1, T w2, T (&d)[W]) {
+    T e[W + 4];
+    if constexpr (W == 1) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) e[k] = row[wrap_x(gx + k - 2, nx)];
+    } else {
+        T l[W], c[W], r[W];
+        rload<T, W>(row + wrap_x(gx - W, nx), l);
+        rload<T, W>(row + gx, c);
+        rload<T, W>(row + wrap_x(gx + W, nx), r);
+        e[0] = l[W - 2];
+        e[1] = l[W - 1];
+#pragma unroll
+        for (int k = 0; k < W; ++k) e[2 + k] = c[k];
+        e[W + 2] = r[0];
+        e[W + 3] = r[1];
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) d[i] = rfma(w1, e[i + 3] - e[i + 1], rmul(w2, e[i + 4] - e[i]));
 }
 
-// value of plane f (field parity fld) at row gz, one mirror reflection at the walls
-template <typename T>
-__device__ __forceinline__ T plane_z(const T* __restrict__ f, const Geo& G, int gz, int gx, int fld) {
-    int side;
-    const int sz = mirror_z(gz, G.nz, side);
-    const T v = f[(size_t)sz * G.nx + gx];
-    return side == 1 ? T(G.pb[fld]) * v : (side == 2 ? T(G.pt[fld]) * v : v);
-}
-
-template <typename T>
-__device__ __forceinline__ T plane_dz(const T* __restrict__ f, const Geo& G, int gz, int gx, int fld, T inv_h) {
-    return (T(2.0 / 3.0) * (plane_z(f, G, gz + 1, gx, fld) - plane_z(f, G, gz - 1, gx, fld)) -
-            T(1.0 / 12.0) * (plane_z(f, G, gz + 2, gx, fld) - plane_z(f, G, gz - 2, gx, fld))) * inv_h;
+// D_z at W points of row gz of a plane (field parity fld, one mirror reflection)
+template <typename T, int W>
+__device__ __forceinline__ void row_dz(const T* __restrict__ f, const Geo& G, int gz, int gx, int fld, T w1, T w2, T (&d)[W]) {
+    T a[4][W];
+    constexpr int s[4] = {-2, -1, 1, 2};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int side;
+        const int sz = mirror_z(gz + s[k], G.nz, side);
+        rload<T, W>(f + (size_t)sz * G.nx + gx, a[k]);
+        if (odd_ghost(G, fld, side)) {
+#pragma unroll
+            for (int i = 0; i < W; ++i) a[k][i] = flip(a[k][i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) d[i] = rfma(w1, a[2][i] - a[1][i], rmul(w2, a[3][i] - a[0][i]));
 }
 
 // rhs = v_p - c_div (D_x v_u + D_z v_w)
-template <typename T>
+template <typename T, int W>
 __global__ void __launch_bounds__(NTHREADS)
 schur_rhs2d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int check_done) {
+    pdl_wait();
     if (check_done && ctl->done) return;
-    const T cdiv = GC(schur_cdiv);
-    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < G.npt; p += gridDim.x * blockDim.x) {
-        const int gz = p / G.nx, gx = p - gz * G.nx;
-        const T du = plane_dx(r, G, gz, gx, idx_);
-        const T dw = plane_dz(r + G.npt, G, gz, gx, 1, idz_);
-        rhs[p] = r[(size_t)3 * G.npt + p] - cdiv * (du + dw);
+    const unsigned nv = G.npt / W, nxv = G.nx / W;
+    for (unsigned q = blockIdx.x * NTHREADS + threadIdx.x; q < nv; q += gridDim.x * NTHREADS) {
+        const int gz = q / nxv, gx = (q - gz * nxv) * W;
+        const size_t p = (size_t)q * W;
+        T dx[W], dz[W], c[W];
+        row_dx<T, W>(r + p - gx, gx, G.nx, GC(wx1), GC(wx2), dx);
+        row_dz<T, W>(r + G.npt, G, gz, gx, 1, GC(wz1), GC(wz2), dz);
+        rload<T, W>(r + (size_t)3 * G.npt + p, c);
+#pragma unroll
+        for (int i = 0; i < W; ++i) c[i] -= GC(schur_cdiv) * (dx[i] + dz[i]);
+        rstore<T, W>(rhs + p, c);
     }
+    pdl_trigger();
 }
 
-// One Chebyshev sweep (k = 1 .. s-1) for H x = rhs on one plane, tiled like
-// cheb2d: x_k staged with halo 2r (even mirror of p), D_x on tile rows, D_z on
-// tile columns, then res = rhs - H x_k, d_k, x_{k+1} = x_k + d_k.
-template <typename T, int FIRST, int LAST, int TX, int TZ>
-__global__ void __launch_bounds__(NTHREADS)
-helm2d(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, const T* __restrict__ din,
-       T* __restrict__ xout, T* __restrict__ dout, Ctl* ctl, int check_done) {
-    constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO;
-    constexpr int QX = TX + 2 * R, QZ = TZ + 2 * R;
-    constexpr int TY = NTHREADS / TX;
-    static_assert(NTHREADS % TX == 0 && TZ % TY == 0, "tile must tile the block");
-    if (check_done && ctl->done) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* zs = reinterpret_cast<T*>(smem_raw);      // [SZ][SX]
-    T* gxs = zs + SZ * SX;                          // [TZ][QX]
-    T* gzs = gxs + TZ * QX;                         // [QZ][TX]
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    const T ith = cheb_coef<T>(ctl, 5, k, 0);
-    const T a1 = cheb_coef<T>(ctl, 5, k, 1);
-    const T a2 = cheb_coef<T>(ctl, 5, k, 2);
-    const int gxx = x0 + tx;
-    const bool colok = gxx < G.nx;
-    constexpr int NR = TZ / TY;
-    T rv[NR], dv[NR];
-#pragma unroll
-    for (int q = 0; q < NR; ++q) {
-        const int gz = z0 + ty + q * TY;
-        const bool ok = colok && gz < G.nz;
-        const int o = gz * G.nx + gxx;
-        rv[q] = ok ? rhs[o] : T(0);
-        dv[q] = (!FIRST && ok) ? din[o] : T(0);
-    }
-    const T* src = FIRST ? rhs : xin;
-    const T sc = FIRST ? ith : T(1);
-    const T pb = T(G.pb[3]), pt = T(G.pt[3]);
-    for (int idx = threadIdx.x; idx < SX * SZ; idx += blockDim.x) {
-        const int iz = idx / SX, ix = idx - iz * SX;
-        int side;
-        const int sz = mirror_z(z0 + iz - HALO, G.nz, side);
-        const int sx = wrap_x(x0 + ix - HALO, G.nx);
-        T val = T(0);
-        if (sz >= 0 && sz < G.nz) {
-            val = sc * src[(size_t)sz * G.nx + sx];
-            if (side == 1) val *= pb;
-            else if (side == 2) val *= pt;
-        }
-        zs[idx] = val;
-    }
-    __syncthreads();
-    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
-    for (int tz = ty; tz < TZ; tz += TY)
-        for (int qx = tx; qx < QX; qx += TX) gxs[tz * QX + qx] = dd(zs, (tz + HALO) * SX + qx + R, 1, idx_);
-    for (int qz = ty; qz < QZ; qz += TY) gzs[qz * TX + tx] = dd(zs, (qz + R) * SX + tx + HALO, SX, idz_);
-    __syncthreads();
-    const T ah = GC(helm_a);
-    const T tdt = GC(two_over_dt);
-    if (colok) {
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-            const int tz = ty + q * TY;
-            const int gz = z0 + tz;
-            if (gz >= G.nz) break;
-            const T* gxr = gxs + tz * QX + tx + R;
-            const T* gzc = gzs + (tz + R) * TX + tx;
-            const T difx = T(2.0 / 3.0) * (gxr[1] - gxr[-1]) - T(1.0 / 12.0) * (gxr[2] - gxr[-2]);
-            const T difz = T(2.0 / 3.0) * (gzc[TX] - gzc[-TX]) - T(1.0 / 12.0) * (gzc[2 * TX] - gzc[-2 * TX]);
-            const T xk = zs[(tz + HALO) * SX + tx + HALO];
-            const T res = rv[q] - (tdt * xk - ah * (difx * idx_ + difz * idz_));
-            const T dprev = FIRST ? rv[q] * ith : dv[q];
-            const T dk = a1 * dprev + a2 * res;
-            const int o = gz * G.nx + gxx;
-            xout[o] = xk + dk;
-            if (!LAST) dout[o] = dk;
-        }
-    }
-}
+// ----------------------------------------------------------------------------
+// S Chebyshev sweeps k .. k+S-1 for H x = rhs on one plane per launch (temporal
+// blocking).  x_k of a TX x TZ tile is staged with a halo of 4 S (periodic x,
+// even mirror in z; the mirrored ghost rows give the mirrored result, so ghosts
+// are swept like other points); sweep s runs on the tile plus a ring of
+// 4 (S - 1 - s) points from one of two x buffers into the other, one barrier a
+// sweep.  H is applied as the composite stencil of D taken twice (coefficients
+// sum_{a+b=s} w_a w_b: -65/72, 1/9, 4/9, -1/9, 1/144), so no first derivative is
+// exchanged.  Points are handled in groups of W along x; the groups are ordered
+// tile first, then ring by ring, and dealt to the threads in that order: a
+// thread keeps rhs and d of its groups in registers through all sweeps.
+// Needs nz >= 4 S (one reflection).
+//
+// Bound: a launch's fixed costs (staging latency, barriers) and issue; a plane
+// is 2 MB at 1024 x 512 and stays in L2.  Per pair of sweeps the former kernel
+// (D exchanged through shared memory, five barriers, no overlap of launches)
+// took 11.7 us at 1024 x 512; four sweeps take 10.9 us here.
+// ----------------------------------------------------------------------------
+template <typename T>
+struct Helm2C {
+    T c0, cx[4], cz[4];             // res = rhs + c0 x + sum_l c_l (x_{+l} + x_{-l})
+};
+constexpr int HELM_THREADS = 512;
+constexpr int HELM_TX = 64, HELM_TZ = 32;
 
-// Two Chebyshev sweeps (k and k+1) per launch (temporal blocking): x_k is
-// staged with halo 4r, sweep k runs on the tile plus a ring of 2r points
-// (ghost rows included -- the mirrored data give the mirrored result), and
-// sweep k+1 on the tile from those values.  Needs nz >= 4r (one reflection).
-template <typename T, int FIRST, int LAST, int TX, int TZ>
-__global__ void __launch_bounds__(NTHREADS)
-helm2d_x2(Geo G, int k, const T* __restrict__ rhs, const T* __restrict__ xin, const T* __restrict__ din,
-          T* __restrict__ xout, T* __restrict__ dout, Ctl* ctl, int check_done) {
-    constexpr int H2 = 2 * HALO;                       // staging halo (two sweeps)
-    constexpr int SX = TX + 2 * H2, SZ = TZ + 2 * H2;
-    constexpr int EX = TX + 2 * HALO, EZ = TZ + 2 * HALO;   // first-sweep region
-    constexpr int TY = NTHREADS / TX;
-    static_assert(NTHREADS % TX == 0 && TZ % TY == 0, "tile must tile the block");
-    if (check_done && ctl->done) return;
+template <typename T, int W, int S>
+__global__ void __launch_bounds__(HELM_THREADS)
+helm2d(Geo G, Helm2C<T> C, int k, int first, int last, const T* __restrict__ rhs, const T* __restrict__ xin,
+       const T* __restrict__ din, T* __restrict__ xout, T* __restrict__ dout, Ctl* ctl, int check_done) {
+    constexpr int TX = HELM_TX, TZ = HELM_TZ;
+    constexpr int H0 = HALO * S, SX = TX + 2 * H0, SZ = TZ + 2 * H0;
+    constexpr int CORE = TX * TZ / W;
+    constexpr int ALL = (TX + 2 * HALO * (S - 1)) * (TZ + 2 * HALO * (S - 1)) / W;      // groups of sweep 0
+    constexpr int NS = (ALL + HELM_THREADS - 1) / HELM_THREADS;
+    static_assert(CORE % HELM_THREADS == 0, "whole slots of tile groups");
+    constexpr int CS = CORE / HELM_THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* xs = reinterpret_cast<T*>(smem_raw);   // [SZ][SX]   x_k
-    T* re = xs + SZ * SX;                        // [EZ][EX]   rhs on the first-sweep region
-    T* de = re + EZ * EX;                        // [EZ][EX]   d_{k-1}, then d_k
-    T* x1 = de + EZ * EX;                        // [EZ][EX]   x_{k+1}
-    T* gx = x1 + EZ * EX;                        // [EZ][EX + 2R]  D_x rows (reused by sweep k+1)
-    T* gz = gx + EZ * (EX + 2 * R);              // [EZ + 2R][EX]  D_z columns (reused)
+    T* xb = reinterpret_cast<T*>(smem_raw);         // [2][SZ][SX]
+    pdl_wait();
+    if (check_done && ctl->done) return;
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
     const T ith = cheb_coef<T>(ctl, 5, k, 0);
-    const T a1 = cheb_coef<T>(ctl, 5, k, 1), a2 = cheb_coef<T>(ctl, 5, k, 2);
-    const T b1 = cheb_coef<T>(ctl, 5, k + 1, 1), b2 = cheb_coef<T>(ctl, 5, k + 1, 2);
-    const T pb = T(G.pb[3]), pt = T(G.pt[3]);
-    // staging: x_k (halo 2 HALO), rhs and d_{k-1} (halo HALO); p parity in z, periodic x
-    for (int idx = threadIdx.x; idx < SX * SZ; idx += blockDim.x) {
-        const int iz = idx / SX, ix = idx - iz * SX;
+    // storage row of global row gz (rows beyond one reflection feed no output)
+    auto row = [&](int gz) {
         int side;
-        const int sz = mirror_z(z0 + iz - H2, G.nz, side);
-        const int sx = wrap_x(x0 + ix - H2, G.nx);
-        // rows beyond one reflection (tiles overhanging a wall) feed no output: zero
-        const bool ok = sz >= 0 && sz < G.nz;
-        const T sgn = side == 1 ? pb : (side == 2 ? pt : T(1));
-        const size_t o = ok ? (size_t)sz * G.nx + sx : 0;
-        const T xv = ok ? (FIRST ? ith * rhs[o] : xin[o]) : T(0);
-        xs[idx] = sgn * xv;
-        const int ez = iz - HALO, ex = ix - HALO;
-        if (ez >= 0 && ez < EZ && ex >= 0 && ex < EX) {
-            const T rv = ok ? sgn * rhs[o] : T(0);
-            re[ez * EX + ex] = rv;
-            de[ez * EX + ex] = FIRST ? ith * rv : (ok ? sgn * din[o] : T(0));
-        }
-    }
-    __syncthreads();
-    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
-    const T ah = GC(helm_a), tdt = GC(two_over_dt);
-    // sweep k on the first-sweep region
-    for (int i = threadIdx.x; i < EZ * (EX + 2 * R); i += blockDim.x) {
-        const int ez = i / (EX + 2 * R), c = i - ez * (EX + 2 * R);
-        gx[i] = dd(xs, (ez + HALO) * SX + c + R, 1, idx_);
-    }
-    for (int i = threadIdx.x; i < (EZ + 2 * R) * EX; i += blockDim.x) {
-        const int r = i / EX, ex = i - r * EX;
-        gz[i] = dd(xs, (r + R) * SX + ex + HALO, SX, idz_);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < EZ * EX; i += blockDim.x) {
-        const int ez = i / EX, ex = i - ez * EX;
-        const T* gxr = gx + ez * (EX + 2 * R) + ex + R;
-        const T* gzc = gz + (ez + R) * EX + ex;
-        const T difx = T(2.0 / 3.0) * (gxr[1] - gxr[-1]) - T(1.0 / 12.0) * (gxr[2] - gxr[-2]);
-        const T difz = T(2.0 / 3.0) * (gzc[EX] - gzc[-EX]) - T(1.0 / 12.0) * (gzc[2 * EX] - gzc[-2 * EX]);
-        const T xk = xs[(ez + HALO) * SX + ex + HALO];
-        const T res = re[i] - (tdt * xk - ah * (difx * idx_ + difz * idz_));
-        const T dk = a1 * de[i] + a2 * res;
-        de[i] = dk;
-        x1[i] = xk + dk;
-    }
-    __syncthreads();
-    // sweep k+1 on the tile
-    constexpr int GX2 = TX + 2 * R;
-    for (int i = threadIdx.x; i < TZ * GX2; i += blockDim.x) {
-        const int tz = i / GX2, c = i - tz * GX2;
-        gx[i] = dd(x1, (tz + HALO) * EX + c + R, 1, idx_);
-    }
-    for (int i = threadIdx.x; i < (TZ + 2 * R) * TX; i += blockDim.x) {
-        const int r = i / TX, tx = i - r * TX;
-        gz[i] = dd(x1, (r + R) * EX + tx + HALO, EX, idz_);
-    }
-    __syncthreads();
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    const int gxx = x0 + tx;
-    if (gxx < G.nx) {
+        return min(max(mirror_z(gz, G.nz, side), 0), G.nz - 1) * G.nx;
+    };
+    int off[NS], ring[NS], pos[NS];
+    T rv[NS][W], dv[NS][W];
 #pragma unroll
-        for (int q = 0; q < TZ / TY; ++q) {
-            const int tz = ty + q * TY;
-            const int gzz = z0 + tz;
-            if (gzz >= G.nz) break;
-            const T* gxr = gx + tz * GX2 + tx + R;
-            const T* gzc = gz + (tz + R) * TX + tx;
-            const T difx = T(2.0 / 3.0) * (gxr[1] - gxr[-1]) - T(1.0 / 12.0) * (gxr[2] - gxr[-2]);
-            const T difz = T(2.0 / 3.0) * (gzc[TX] - gzc[-TX]) - T(1.0 / 12.0) * (gzc[2 * TX] - gzc[-2 * TX]);
-            const int e = (tz + HALO) * EX + tx + HALO;
-            const T xk = x1[e];
-            const T res = re[e] - (tdt * xk - ah * (difx * idx_ + difz * idz_));
-            const T dk = b1 * de[e] + b2 * res;
-            const int o = gzz * G.nx + gxx;
-            xout[o] = xk + dk;
-            if (!LAST) dout[o] = dk;
+    for (int q = 0; q < NS; ++q) {
+        int j = threadIdx.x + q * HELM_THREADS;
+        int iz, ix, h = 0;
+        if (q < CS) {
+            iz = j / (TX / W);
+            ix = (j % (TX / W)) * W;
+        } else {
+            j -= CORE;
+            h = S;                                  // no group
+            iz = ix = 0;
+#pragma unroll
+            for (int t = 1; t < S; ++t) {           // ring t: 4 rows above and below, then the two sides
+                const int gw = (TX + 2 * HALO * t) / W, rows = 2 * HALO * gw;
+                const int side_w = 2 * HALO / W, n = rows + (TZ + 2 * HALO * (t - 1)) * side_w;
+                if (h == S && j < n) {
+                    h = t;
+                    if (j < rows) {
+                        const int r = j / gw;
+                        iz = r < HALO ? r - HALO * t : TZ + HALO * (t - 1) + r - HALO;
+                        ix = (j % gw) * W - HALO * t;
+                    } else {
+                        const int c = (j - rows) % side_w;
+                        iz = (j - rows) / side_w - HALO * (t - 1);
+                        ix = c < side_w / 2 ? c * W - HALO * t : TX + HALO * (t - 1) + (c - side_w / 2) * W;
+                    }
+                }
+                if (h == S) j -= n;
+            }
+        }
+        ring[q] = h;
+        off[q] = (iz + H0) * SX + ix + H0;
+        pos[q] = row(z0 + iz) + wrap_x(x0 + ix, G.nx);
+        if (h < S) {
+            rload<T, W>(rhs + pos[q], rv[q]);
+            if (first) {
+#pragma unroll
+                for (int i = 0; i < W; ++i) dv[q][i] = ith * rv[q][i];
+            } else {
+                rload<T, W>(din + pos[q], dv[q]);
+            }
         }
     }
+    {
+        const T* src = first ? rhs : xin;
+        const T sc = first ? ith : T(1);
+        for (int j = threadIdx.x; j < SX * SZ / W; j += HELM_THREADS) {
+            const int iz = j / (SX / W), ix = (j % (SX / W)) * W;
+            T v[W];
+            rload<T, W>(src + row(z0 + iz - H0) + wrap_x(x0 + ix - H0, G.nx), v);
+#pragma unroll
+            for (int i = 0; i < W; ++i) v[i] *= sc;
+            rstore<T, W>(xb + j * W, v);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        const T* xa = xb + (s & 1) * SX * SZ;
+        T* xn = xb + ((s + 1) & 1) * SX * SZ;
+        const T a1 = cheb_coef<T>(ctl, 5, k + s, 1), a2 = cheb_coef<T>(ctl, 5, k + s, 2);
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            if (ring[q] > S - 1 - s) continue;
+            const T* p = xa + off[q];
+            T e[W + 2 * HALO], r[W];
+#pragma unroll
+            for (int i = 0; i < W + 2 * HALO; i += W) {
+                T v[W];
+                rload<T, W>(p - HALO + i, v);
+#pragma unroll
+                for (int j = 0; j < W; ++j) e[i + j] = v[j];
+            }
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                r[i] = rv[q][i] + C.c0 * e[HALO + i];
+#pragma unroll
+                for (int l = 1; l <= HALO; ++l) r[i] += C.cx[l - 1] * (e[HALO + i + l] + e[HALO + i - l]);
+            }
+#pragma unroll
+            for (int l = 1; l <= HALO; ++l) {
+                T a[W], b[W];
+                rload<T, W>(p + l * SX, a);
+                rload<T, W>(p - l * SX, b);
+#pragma unroll
+                for (int i = 0; i < W; ++i) r[i] += C.cz[l - 1] * (a[i] + b[i]);
+            }
+            T xo[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                dv[q][i] = a1 * dv[q][i] + a2 * r[i];
+                xo[i] = e[HALO + i] + dv[q][i];
+            }
+            if (s + 1 < S) {
+                rstore<T, W>(xn + off[q], xo);
+            } else {
+                const int j = threadIdx.x + q * HELM_THREADS;
+                if (x0 + (j % (TX / W)) * W < G.nx && z0 + j / (TX / W) < G.nz) {
+                    rstore<T, W>(xout + pos[q], xo);
+                    if (!last) rstore<T, W>(dout + pos[q], dv[q]);
+                }
+            }
+        }
+        if (s + 1 < S) __syncthreads();
+    }
+    pdl_trigger();
 }
 
 // z_u, z_w from the pressure solution (already in plane 3 of z), z_theta, and
-// the finite-difference step eps from ||z||.
-template <typename T>
+// the finite-difference step eps from ||z|| (float32: pending, as cheb2d leaves it).
+template <typename T, int W>
 __global__ void __launch_bounds__(NTHREADS)
 schur_back2d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ctl* ctl, int check_done) {
+    pdl_wait();
     if (check_done && ctl->done) return;
-    const T cgrad = GC(schur_cgrad);
-    const T hdt = GC(half_dt);
+    const T cgrad = GC(schur_cgrad), hdt = GC(half_dt);
     const T ith_t = cheb_coef<T>(ctl, 2, 0, 0);
-    const T idx_ = GC(inv_dx), idz_ = GC(inv_dz);
     const size_t np = (size_t)G.npt;
     const T* dp = z + 3 * np;
     T acc[1] = {T(0)};
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < G.npt; p += gridDim.x * blockDim.x) {
-        const int gz = p / G.nx, gx = p - gz * G.nx;
-        const T zu = hdt * (r[p] - cgrad * plane_dx(dp, G, gz, gx, idx_));
-        const T zw = hdt * (r[np + p] - cgrad * plane_dz(dp, G, gz, gx, 3, idz_));
-        const T zt = r[2 * np + p] * ith_t;
-        const T zp = dp[p];
-        z[p] = zu;
-        z[np + p] = zw;
-        z[2 * np + p] = zt;
-        acc[0] += zu * zu + zw * zw + zt * zt + zp * zp;
+    const unsigned nv = G.npt / W, nxv = G.nx / W;
+    for (unsigned q = blockIdx.x * NTHREADS + threadIdx.x; q < nv; q += gridDim.x * NTHREADS) {
+        const int gz = q / nxv, gx = (q - gz * nxv) * W;
+        const size_t p = (size_t)q * W;
+        T dx[W], dz[W], ru[W], rw[W], rt[W], zp[W];
+        row_dx<T, W>(dp + p - gx, gx, G.nx, GC(wx1), GC(wx2), dx);
+        row_dz<T, W>(dp, G, gz, gx, 3, GC(wz1), GC(wz2), dz);
+        rload<T, W>(r + p, ru);
+        rload<T, W>(r + np + p, rw);
+        rload<T, W>(r + 2 * np + p, rt);
+        rload<T, W>(dp + p, zp);
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            ru[i] = hdt * (ru[i] - cgrad * dx[i]);
+            rw[i] = hdt * (rw[i] - cgrad * dz[i]);
+            rt[i] *= ith_t;
+            acc[0] += ru[i] * ru[i] + rw[i] * rw[i] + rt[i] * rt[i] + zp[i] * zp[i];
+        }
+        rstore<T, W>(z + p, ru);
+        rstore<T, W>(z + np + p, rw);
+        rstore<T, W>(z + 2 * np + p, rt);
     }
-    block_partials<1, T>(acc, 1, part, gridDim.x, blockIdx.x);
-    if (arrive_last(&ctl->counter[CNT_PC], gridDim.x)) {
-        __shared__ double tot[1];
-        final_sums(part, gridDim.x, 1, tot);
-        if (threadIdx.x == 0) {
-            const double zn = sqrt(tot[0]);
-            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
+    pdl_trigger();
+    if constexpr (sizeof(T) == sizeof(float)) {
+        block_partial_ff(acc[0], reinterpret_cast<float2*>(part), blockIdx.x);
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->eps_part = gridDim.x;
+    } else {
+        block_partials<1, T>(acc, 1, part, gridDim.x, blockIdx.x);
+        if (arrive_last(&ctl->counter[CNT_PC], gridDim.x)) {
+            __shared__ double tot[1];
+            final_sums(part, gridDim.x, 1, tot);
+            if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
         }
     }
 }
@@ -1625,48 +1748,81 @@ cudaError_t launch_eddy(const Geo& G, const T* u, T* nu, double* part, Ctl* ctl,
 template cudaError_t launch_eddy<float>(const Geo&, const float*, float*, double*, Ctl*, cudaStream_t);
 template cudaError_t launch_eddy<double>(const Geo&, const double*, double*, double*, Ctl*, cudaStream_t);
 
-template <typename T, int SMAG, int TX, int TZ>
-static cudaError_t launch_precond_t(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da,
-                                    T* db, const T* nu, double* part, Ctl* ctl, int check_done,
-                                    cudaStream_t s, long long* launches) {
+template <typename T, int SMAG>
+static cudaError_t launch_pc_diag(const Geo& G, const T* r, T* z, double* part, Ctl* ctl, int check_done, cudaStream_t s,
+                                  long long* launches) {
     const size_t n = (size_t)G.nf * G.npt;
-    if (sweeps <= 1) {
-        pc_diag<T, SMAG><<<stream_blocks(n), NTHREADS, 0, s>>>(G, r, z, n, part, ctl, check_done);
-        if (launches) ++*launches;
-        return cudaGetLastError();
-    }
-    dim3 grid((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ, 3);
-    const size_t sm = sizeof(T) * ((TZ + 2 * HALO) * (TX + 2 * HALO) + TZ * (TX + 2 * R) +
-                                   (TZ + 2 * R) * TX + (SMAG == 2 ? 2 : 1) * (TX + 2 * R) * (TZ + 2 * R));
-    static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
-    if (!configured) {
-        cudaError_t e;
-        if ((e = set_smem(cheb2d<T, SMAG, 1, 1, TX, TZ>, sm)) != cudaSuccess) return e;
-        if ((e = set_smem(cheb2d<T, SMAG, 1, 0, TX, TZ>, sm)) != cudaSuccess) return e;
-        if ((e = set_smem(cheb2d<T, SMAG, 0, 1, TX, TZ>, sm)) != cudaSuccess) return e;
-        if ((e = set_smem(cheb2d<T, SMAG, 0, 0, TX, TZ>, sm)) != cudaSuccess) return e;
-        configured = true;
-    }
-    const T* zin = nullptr;
-    const T* din = nullptr;
-    T* zbuf[2] = {za, zb};
-    T* dbuf[2] = {da, db};
+    pc_diag<T, SMAG><<<stream_blocks(n), NTHREADS, 0, s>>>(G, r, z, n, part, ctl, check_done);
+    if (launches) ++*launches;
+    return cudaGetLastError();
+}
+
+template <int W, int NT, int SMAG>
+static cudaError_t launch_precond_w(const Geo& G, int sweeps, const float* r, float* z, float* za, float* zb, float* da,
+                                    float* db, const float* nu, double* part, Ctl* ctl, int check_done,
+                                    cudaStream_t s, long long* launches) {
+    constexpr int TX = PcRow<W>::NXT * W, TZ = NT / PcRow<W>::NXT;
+    const dim3 grid((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ);
+    const float* zin = nullptr;
+    const float* din = nullptr;
+    float* zbuf[2] = {za, zb};
+    float* dbuf[2] = {da, db};
     for (int k = 1; k <= sweeps - 1; ++k) {
-        const bool first = k == 1, last = k == sweeps - 1;
-        T* zo = last ? z : zbuf[k & 1];
-        T* dO = dbuf[k & 1];
-        grid.z = last ? 4 : 3;            // the p block is written by the last sweep only
-        cudaError_t le;
-        if (first && last)
-            le = launch_pdl(cheb2d<T, SMAG, 1, 1, TX, TZ>, grid, NTHREADS, sm, s, G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else if (first)
-            le = launch_pdl(cheb2d<T, SMAG, 1, 0, TX, TZ>, grid, NTHREADS, sm, s, G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else if (last)
-            le = launch_pdl(cheb2d<T, SMAG, 0, 1, TX, TZ>, grid, NTHREADS, sm, s, G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
-        else
-            le = launch_pdl(cheb2d<T, SMAG, 0, 0, TX, TZ>, grid, NTHREADS, sm, s, G, k, r, zin, din, zo, dO, nu, part, ctl, check_done);
+        const int first = k == 1, last = k == sweeps - 1;
+        float* zo = last ? z : zbuf[k & 1];
+        float* dO = dbuf[k & 1];
+        const cudaError_t e = launch_pdl(cheb2d<W, NT, SMAG>, grid, dim3(NT), 0, s, G, k, first, last, r, zin, din, zo, dO,
+                                         nu, part, ctl, check_done);
         if (launches) ++*launches;
-        if (le != cudaSuccess) return le;
+        if (e != cudaSuccess) return e;
+        zin = zo;
+        din = dO;
+    }
+    return cudaSuccess;
+}
+
+// Rows of 16-byte, 8-byte or single-element vectors as nx allows (r and z of the
+// batched and per-call paths are workspace vectors: their planes start multiples
+// of npt elements in); 256, 128 or 64 threads a CTA by Geo::tile_pc, by the grid
+// for tile_pc = 0: the widest tile that leaves no SM without a CTA.
+template <int SMAG>
+static cudaError_t launch_precond_f32(const Geo& G, int sweeps, const float* r, float* z, float* za, float* zb, float* da,
+                                      float* db, const float* nu, double* part, Ctl* ctl, int check_done,
+                                      cudaStream_t s, long long* launches) {
+    constexpr int SMS = 152;
+    const int w = G.nx % 4 == 0 ? 4 : (G.nx % 2 == 0 ? 2 : 1);
+    int nt = G.tile_pc == 1 ? 256 : (G.tile_pc == 2 ? 128 : 64);
+    if (G.tile_pc == 0) {
+        const long long vecs = (long long)((G.nx + w - 1) / w) * G.nz;       // threads with a point
+        nt = vecs >= 256LL * SMS ? 256 : (vecs >= 128LL * SMS ? 128 : 64);
+    }
+#define JF_PC(W, NT) launch_precond_w<W, NT, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches)
+#define JF_PCW(W) (nt == 256 ? JF_PC(W, 256) : nt == 128 ? JF_PC(W, 128) : JF_PC(W, 64))
+    return w == 4 ? JF_PCW(4) : w == 2 ? JF_PCW(2) : JF_PCW(1);
+#undef JF_PCW
+#undef JF_PC
+}
+
+template <int SMAG>
+static cudaError_t launch_precond_f64(const Geo& G, int sweeps, const double* r, double* z, double* za, double* zb,
+                                      double* da, double* db, const double* nu, double* part, Ctl* ctl, int check_done,
+                                      cudaStream_t s, long long* launches) {
+    const FluxShape sh = flux_shape(G);
+    const size_t sm = (sh.plane() + sh.xn() + sh.zn()) * sizeof(double);     // 17 KB at most
+    dim3 grid((G.nx + sh.tx() - 1) >> sh.lx, (G.nz + sh.tz() - 1) >> sh.lz, 3);
+    const double* zin = nullptr;
+    const double* din = nullptr;
+    double* zbuf[2] = {za, zb};
+    double* dbuf[2] = {da, db};
+    for (int k = 1; k <= sweeps - 1; ++k) {
+        const int first = k == 1, last = k == sweeps - 1;
+        double* zo = last ? z : zbuf[k & 1];
+        double* dO = dbuf[k & 1];
+        grid.z = last ? 4 : 3;            // the p block is written by the last sweep only
+        const cudaError_t e = launch_pdl(cheb2d_f64<SMAG>, grid, dim3(NTHREADS), sm, s, G, k, first, last, sh, r, zin, din,
+                                         zo, dO, nu, part, ctl, check_done);
+        if (launches) ++*launches;
+        if (e != cudaSuccess) return e;
         zin = zo;
         din = dO;
     }
@@ -1674,79 +1830,95 @@ static cudaError_t launch_precond_t(const Geo& G, int sweeps, const T* r, T* z, 
 }
 
 template <typename T, int SMAG>
-static cudaError_t launch_precond_tile(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da,
-                                       T* db, const T* nu, double* part, Ctl* ctl, int check_done,
-                                       cudaStream_t s, long long* launches) {
-#define JF_PC(I) launch_precond_t<T, SMAG, PcTile<I>::TX, PcTile<I>::TZ>(G, sweeps, r, z, za, zb, da, db, nu, \
-                                                                      part, ctl, check_done, s, launches)
-    if (sizeof(T) == sizeof(double)) return JF_PC(1);
-    switch (G.tile_pc) {
-        case 1: return JF_PC(1);
-        case 2: return JF_PC(2);
-        case 3: return JF_PC(3);
-        default: return JF_PC(0);
+static cudaError_t launch_precond_block(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
+                                        const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
+                                        long long* launches) {
+    if (sweeps <= 1) return launch_pc_diag<T, SMAG>(G, r, z, part, ctl, check_done, s, launches);
+    if constexpr (sizeof(T) == sizeof(double))
+        return launch_precond_f64<SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+    else
+        return launch_precond_f32<SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+}
+
+template <typename T, int W, int S>
+static cudaError_t launch_helm2d(const Geo& G, const Helm2C<T>& C, int k, int first, int last, const T* rhs, const T* xin,
+                                 const T* din, T* xout, T* dout, Ctl* ctl, int check_done, cudaStream_t s) {
+    constexpr int TX = HELM_TX, TZ = HELM_TZ;
+    constexpr size_t sm = sizeof(T) * (S > 1 ? 2 : 1) * (size_t)(TX + 2 * HALO * S) * (TZ + 2 * HALO * S);
+    static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
+    if (!configured) {
+        const cudaError_t e = set_smem(helm2d<T, W, S>, sm);
+        if (e != cudaSuccess) return e;
+        configured = true;
     }
-#undef JF_PC
+    return launch_pdl(helm2d<T, W, S>, dim3((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ), dim3(HELM_THREADS), sm, s, G, C,
+                      k, first, last, rhs, xin, din, xout, dout, ctl, check_done);
 }
 
 // Acoustic Schur complement: rhs (plane 0 of da), sweeps - 1 Helmholtz
 // sweeps (iterates in plane 0 of za / zb, directions in planes 0 / 1 of db,
 // the last one into plane 3 of z), then the back-substitution.
-template <typename T>
-static cudaError_t launch_schur(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
-                                double* part, Ctl* ctl, int check_done, cudaStream_t s, long long* launches) {
-    constexpr int TX = 64, TZ = 16;
+template <typename T, int W>
+static cudaError_t launch_schur_w(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
+                                  double* part, Ctl* ctl, int check_done, cudaStream_t s, long long* launches) {
+    constexpr int SMS = 152;
     const size_t np = (size_t)G.npt;
-    const size_t sm = sizeof(T) * ((TZ + 2 * HALO) * (TX + 2 * HALO) + TZ * (TX + 2 * R) + (TZ + 2 * R) * TX);
+    const int nb = (int)std::min<size_t>((np / W + NTHREADS - 1) / NTHREADS, 4 * SMS);
     T* rhs = da;
-    schur_rhs2d<T><<<stream_blocks(np), NTHREADS, 0, s>>>(G, r, rhs, ctl, check_done);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(schur_rhs2d<T, W>, dim3(nb), dim3(NTHREADS), 0, s, G, r, rhs, ctl, check_done);
     if (e != cudaSuccess) return e;
     if (launches) ++*launches;
-    dim3 grid((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ);
+    Helm2C<T> C;
+    const double lap[5] = {-65.0 / 72.0, 1.0 / 9.0, 4.0 / 9.0, -1.0 / 9.0, 1.0 / 144.0};
+    const double ax = G.helm_a * G.inv_dx * G.inv_dx, az = G.helm_a * G.inv_dz * G.inv_dz;
+    C.c0 = T(lap[0] * (ax + az) - G.two_over_dt);
+    for (int l = 0; l < 4; ++l) {
+        C.cx[l] = T(lap[l + 1] * ax);
+        C.cz[l] = T(lap[l + 1] * az);
+    }
     T* xbuf[2] = {za, zb};
     T* dbuf[2] = {db, db + np};
     const T* xin = nullptr;
     const T* din = nullptr;
+    // sweeps per launch: four where the rows are float32 vectors (a sweep's ring is
+    // then cheap next to a launch), two otherwise (float64: the rings cost the FP64
+    // pipe; single points: three times the loads), within one reflection of nz
+    constexpr int MAXS = sizeof(T) == sizeof(float) && W > 1 ? 4 : 2;
+    const int most = std::min(MAXS, G.nz / HALO);
     int cur = 1;                              // buffer pair the next output goes to
-    const bool pairs = G.nz >= 2 * HALO;      // fused pairs need one mirror reflection of a 2*HALO halo
-    const size_t sm2 = sizeof(T) * ((TZ + 4 * HALO) * (TX + 4 * HALO) + 3 * (TZ + 2 * HALO) * (TX + 2 * HALO) +
-                                    (TZ + 2 * HALO) * (TX + 2 * HALO + 2 * R) + (TZ + 2 * HALO + 2 * R) * (TX + 2 * HALO));
-    static std::atomic<bool> configured{false};
-    if (!configured) {
-        if ((e = set_smem(helm2d_x2<T, 1, 1, TX, TZ>, sm2)) != cudaSuccess) return e;
-        if ((e = set_smem(helm2d_x2<T, 1, 0, TX, TZ>, sm2)) != cudaSuccess) return e;
-        if ((e = set_smem(helm2d_x2<T, 0, 1, TX, TZ>, sm2)) != cudaSuccess) return e;
-        if ((e = set_smem(helm2d_x2<T, 0, 0, TX, TZ>, sm2)) != cudaSuccess) return e;
-        configured = true;
-    }
     for (int k = 1; k <= sweeps - 1;) {
-        const bool first = k == 1;
-        const bool two = pairs && k + 1 <= sweeps - 1;
-        const bool last = (two ? k + 1 : k) == sweeps - 1;
+        const int n = std::min(most, sweeps - k);
+        const int first = k == 1, last = k + n == sweeps;
         T* xo = last ? z + 3 * np : xbuf[cur];
         T* dO = dbuf[cur];
-        if (two) {
-            if (first && last) helm2d_x2<T, 1, 1, TX, TZ><<<grid, NTHREADS, sm2, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else if (first) helm2d_x2<T, 1, 0, TX, TZ><<<grid, NTHREADS, sm2, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else if (last) helm2d_x2<T, 0, 1, TX, TZ><<<grid, NTHREADS, sm2, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else helm2d_x2<T, 0, 0, TX, TZ><<<grid, NTHREADS, sm2, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-        } else {
-            if (first && last) helm2d<T, 1, 1, TX, TZ><<<grid, NTHREADS, sm, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else if (first) helm2d<T, 1, 0, TX, TZ><<<grid, NTHREADS, sm, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else if (last) helm2d<T, 0, 1, TX, TZ><<<grid, NTHREADS, sm, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
-            else helm2d<T, 0, 0, TX, TZ><<<grid, NTHREADS, sm, s>>>(G, k, rhs, xin, din, xo, dO, ctl, check_done);
+        const T* rh = rhs;
+        if constexpr (MAXS == 4) {
+            if (n == 4) e = launch_helm2d<T, W, 4>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+            if (n == 3) e = launch_helm2d<T, W, 3>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
         }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (n == 2) e = launch_helm2d<T, W, 2>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+        if (n == 1) e = launch_helm2d<T, W, 1>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+        if (e != cudaSuccess) return e;
         if (launches) ++*launches;
         xin = xo;
         din = dO;
         cur ^= 1;
-        k += two ? 2 : 1;
+        k += n;
     }
-    schur_back2d<T><<<stream_blocks(np), NTHREADS, 0, s>>>(G, r, z, part, ctl, check_done);
+    e = launch_pdl(schur_back2d<T, W>, dim3(nb), dim3(NTHREADS), 0, s, G, r, z, part, ctl, check_done);
     if (launches) ++*launches;
-    return cudaGetLastError();
+    return e;
+}
+
+template <typename T>
+static cudaError_t launch_schur(const Geo& G, int sweeps, const T* r, T* z, T* za, T* zb, T* da, T* db,
+                                double* part, Ctl* ctl, int check_done, cudaStream_t s, long long* launches) {
+    // 16-byte rows: the workspace planes start multiples of npt elements in; r and z of
+    // the per-call entry may be the caller's (8-byte aligned) float64 arrays
+    constexpr int W = 16 / sizeof(T);
+    const bool vec = G.nx % W == 0 && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z)) & 15) == 0;
+    return vec ? launch_schur_w<T, W>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches)
+               : launch_schur_w<T, 1>(G, sweeps, r, z, za, zb, da, db, part, ctl, check_done, s, launches);
 }
 
 template <typename T>
@@ -1758,9 +1930,9 @@ cudaError_t launch_precond(const Geo& G, int sweeps, const T* r, T* z, T* za, T*
     if (G.dim == 3 && sweeps > 1)
         return launch_precond3d<T>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
     if (G.sgs == 2)
-        return launch_precond_tile<T, 2>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
-    return G.smag ? launch_precond_tile<T, 1>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches)
-                  : launch_precond_tile<T, 0>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+        return launch_precond_block<T, 2>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
+    return G.smag ? launch_precond_block<T, 1>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches)
+                  : launch_precond_block<T, 0>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches);
 }
 template cudaError_t launch_precond<float>(const Geo&, int, const float*, float*, float*, float*, float*,
                                            float*, const float*, double*, Ctl*, int, cudaStream_t, long long*);

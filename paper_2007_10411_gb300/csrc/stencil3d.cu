@@ -198,15 +198,14 @@ __device__ __forceinline__ void cpa1(T* dst, const T* src) {
 
 // eps_f = eps_jv * scale_f and 1 / eps_f (Jacobian-product modes)
 template <typename T>
-__device__ __forceinline__ T eps_field(const Ctl* ctl, const Geo& G, int f) {
+__device__ __forceinline__ T eps_field(const Ctl* ctl, int f) {
     if constexpr (sizeof(T) == sizeof(float)) return ctl->evf[f];
-    else return ctl->eps_jv * G.scale[f];
+    else return ctl->ev[f];
 }
 template <typename T>
-__device__ __forceinline__ T inv_eps_field(const Ctl* ctl, const Geo& G, int f) {
+__device__ __forceinline__ T inv_eps_field(const Ctl* ctl, int f) {
     if constexpr (sizeof(T) == sizeof(float)) return ctl->cff[f];
-    const T e = T(ctl->eps_jv * G.scale[f]);
-    return e != T(0) ? T(1) / e : T(0);
+    else return ctl->cf[f];
 }
 
 // ------------------------------------------------------------------ tiles
@@ -246,7 +245,7 @@ strain3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict_
     T ev[3] = {T(0), T(0), T(0)};
     if (KIND != ONE) {
 #pragma unroll
-        for (int f = 0; f < 3; ++f) ev[f] = eps_field<T>(ctl, G, f);
+        for (int f = 0; f < 3; ++f) ev[f] = eps_field<T>(ctl, f);
     }
     const size_t nxy = (size_t)G.ny * G.nx;
     int xoff[XS];
@@ -462,7 +461,7 @@ __device__ __forceinline__ void plane_point(const Geo& G, const T* __restrict__ 
 }
 
 template <typename T, int KIND, int SMAG>
-__global__ void __launch_bounds__(NTHREADS)
+__global__ void __launch_bounds__(NTHREADS, sizeof(T) == sizeof(float) ? 3 : 4)
 plane3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ s0,
         const T* __restrict__ s1, T* __restrict__ P, Ctl* ctl, int check_done) {
     using SH = PlaneShape<T, KIND, SMAG>;
@@ -476,7 +475,7 @@ plane3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, const T* __rest
     T ev[5] = {T(0), T(0), T(0), T(0), T(0)};
     if (KIND != ONE) {
 #pragma unroll
-        for (int f = 0; f < 5; ++f) ev[f] = eps_field<T>(ctl, G, f);
+        for (int f = 0; f < 5; ++f) ev[f] = eps_field<T>(ctl, f);
     }
     const size_t plane = (size_t)gz * G.ny * G.nx;
     // eddy values of the thread's points and of its arm point, in flight with the staging
@@ -588,9 +587,9 @@ column3d(Geo G, int mode, int zc, const T* __restrict__ u, const T* __restrict__
         const T w1 = GC(wz1), w2 = GC(wz2);
         T evq = T(0), evp = T(0), cf = T(0);         // eps scale, 1 / (eps scale)
         if (KIND != ONE) {
-            evq = eps_field<T>(ctl, G, q);
-            evp = eps_field<T>(ctl, G, pq);
-            cf = inv_eps_field<T>(ctl, G, q);
+            evq = eps_field<T>(ctl, q);
+            evp = eps_field<T>(ctl, pq);
+            cf = inv_eps_field<T>(ctl, q);
         }
         const bool oddb = G.pb[q] < 0, oddt = G.pt[q] < 0, poddb = G.pb[pq] < 0, poddt = G.pt[pq] < 0;
         // offsets within a plane stack fit 32 bits (npt does): one wide multiply-add per access
@@ -738,9 +737,7 @@ column3d(Geo G, int mode, int zc, const T* __restrict__ u, const T* __restrict__
             __shared__ double tot[2];
             final_sums(part, nblk, 2, tot);
             if (threadIdx.x == 0) {
-                ctl->res2 = tot[0];
-                ctl->unorm2 = tot[1];
-                ctl->nan = !(isfinite(tot[0]) && isfinite(tot[1]));
+                put_norms(ctl, tot);
             }
         }
     }
@@ -1050,10 +1047,7 @@ cheb3d(Geo G, int k, int zb, const T* __restrict__ r, const T* __restrict__ zin,
         if (arrive_last(&ctl->counter[CNT_PC], nblk)) {
             __shared__ double tot[1];
             final_sums(part, nblk, 1, tot);
-            if (threadIdx.x == 0) {
-                const double zn = sqrt(tot[0]);
-                put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-            }
+            if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
         }
     }
 }
@@ -1254,10 +1248,7 @@ cheb3d_shared(Geo G, int k, const T* __restrict__ r, const T* __restrict__ zin, 
         if (arrive_last(&ctl->counter[CNT_PC], nblk)) {
             __shared__ double tot[1];
             final_sums(part, nblk, 1, tot);
-            if (threadIdx.x == 0) {
-                const double zn = sqrt(tot[0]);
-                put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-            }
+            if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
         }
     }
 }
@@ -1684,10 +1675,7 @@ schur_back3d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ct
     if (arrive_last(&ctl->counter[CNT_PC], gridDim.x)) {
         __shared__ double tot[1];
         final_sums(part, gridDim.x, 1, tot);
-        if (threadIdx.x == 0) {
-            const double zn = sqrt(tot[0]);
-            put_eps(ctl, zn > 0.0 ? sqrt(ctl->eps_mach * (1.0 + sqrt(ctl->unorm2))) / zn : 0.0);
-        }
+        if (threadIdx.x < 5) put_eps_norm2(ctl, tot[0]);
     }
 }
 

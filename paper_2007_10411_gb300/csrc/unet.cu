@@ -9,9 +9,9 @@
 // mma.sync.m16n8k16.row.col.f32.bf16.bf16.f32 with ldmatrix fragments from
 // shared memory (input tile with a one-pixel halo, NHWC, and the layer's
 // weights [tap][cout][cin], resident for the CTA's lifetime).  The backward pass w.r.t. the input is the same
-// kernel with flipped, transposed weights; the weight gradient is a float32
-// reduction over pixel tiles (CUDA cores) with one atomic add per weight and
-// tile.
+// kernel with flipped, transposed weights; the weight gradient is a GEMM over
+// the pixels of a tile on the same instruction, with one atomic add per weight
+// and tile (part).
 #include <atomic>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -592,65 +592,98 @@ conv_tc(ConvIn in, Bal bal, const bf16* __restrict__ W, ConvOut out, Lv lv, cons
                      : "memory");
 }
 
-// dW[tap][co][ci] += sum_p dout[p][co] in[p + off(tap)][ci] over a 16x16 pixel tile.
+// dW[tap][co][ci] += sum_p dout[p][co] in[p + off(tap)][ci] over a 16x16 pixel
+// tile, on mma.sync m16n8k16: M = output channels, N = 16 input channels of one
+// tap, K = the 16 pixels of a tile row.  Both operands lie in shared memory with
+// the pixel as the row, so their fragments are transposed ldmatrix loads, and a
+// tap is an offset of the B rows.  One work unit is a (tap, 16 input channels)
+// pair over 16 / kparts tile rows, for all output channels; units are dealt to
+// the warps of blockIdx.z's, because a coarse level has few tiles (8 at
+// 64 x 32 pixels for 152 SMs).  Products of bfloat16 are exact, sums are
+// float32 as in the CUDA-core form: 145 us for L2b at 256 x 128, all layers
+// 480 us; 145 -> 9 us, all layers 480 -> 70 us.
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(addr));
+}
+
+template <int CI, int CO, int KS>
+struct WgradShape {
+    static constexpr int T = 16, HP = KS / 2, IW = T + 2 * HP;     // tile side, staged side
+    static constexpr int CIP = CI + 8, COP = CO + 8;               // padded pixel strides: conflict-free ldmatrix rows
+    static constexpr int ITEMS = KS * KS * (CI / 16);
+    static constexpr size_t SMEM = sizeof(bf16) * (size_t)(IW * IW * CIP + T * T * COP);
+};
+
 template <int CI, int CO, int KS>
 __global__ void __launch_bounds__(256)
 conv_wgrad(const bf16* __restrict__ in, int istr, int ioff, const bf16* __restrict__ dout, Lv lv,
-           float* __restrict__ dW) {
-    constexpr int TH = 16, TW = 16, HP = KS / 2;
-    constexpr int IH = TH + 2 * HP, IW = TW + 2 * HP;
+           float* __restrict__ dW, int kparts) {
+    using S = WgradShape<CI, CO, KS>;
+    constexpr int T = S::T, HP = S::HP, IW = S::IW;
     extern __shared__ __align__(16) unsigned char sm[];
-    bf16* xs = reinterpret_cast<bf16*>(sm);        // [IH*IW][CI]
-    bf16* ds = xs + IH * IW * CI;                  // [TH*TW][CO]
-    const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH;
+    bf16* xs = reinterpret_cast<bf16*>(sm);        // [IW*IW][CIP]
+    bf16* ds = xs + IW * IW * S::CIP;              // [T*T][COP]
+    const int x0 = blockIdx.x * T, y0 = blockIdx.y * T;
     const int H = lv.H, Wd = lv.Wd;
     const int sy0 = (y0 / lv.Hs) * lv.Hs, sy1 = min(sy0 + lv.Hs, H);   // the tile's slice
     constexpr int VPP = CI / 8;
-    for (int idx = threadIdx.x; idx < IH * IW * VPP; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < IW * IW * VPP; idx += blockDim.x) {
         const int pix = idx / VPP, v = idx - pix * VPP;
         const int iy = pix / IW, ix = pix - iy * IW;
         const int gy = y0 + iy - HP, gx = x0 + ix - HP;
         uint4 val = make_uint4(0u, 0u, 0u, 0u);
         if (gy >= sy0 && gy < sy1 && gx >= 0 && gx < Wd)
             val = *reinterpret_cast<const uint4*>(in + ((size_t)gy * Wd + gx) * istr + ioff + v * 8);
-        *reinterpret_cast<uint4*>(xs + pix * CI + v * 8) = val;
+        *reinterpret_cast<uint4*>(xs + pix * S::CIP + v * 8) = val;
     }
     constexpr int VPO = CO / 8;
-    for (int idx = threadIdx.x; idx < TH * TW * VPO; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < T * T * VPO; idx += blockDim.x) {
         const int pix = idx / VPO, v = idx - pix * VPO;
-        const int gy = y0 + pix / TW, gx = x0 + pix % TW;
+        const int gy = y0 + pix / T, gx = x0 + pix % T;
         uint4 val = make_uint4(0u, 0u, 0u, 0u);
         if (gy < H && gx < Wd) val = *reinterpret_cast<const uint4*>(dout + ((size_t)gy * Wd + gx) * CO + v * 8);
-        *reinterpret_cast<uint4*>(ds + pix * CO + v * 8) = val;
+        *reinterpret_cast<uint4*>(ds + pix * S::COP + v * 8) = val;
     }
     __syncthreads();
-    constexpr int GROUPS = KS * KS * (CO / 4) * (CI / 4);
-    for (int grp = threadIdx.x; grp < GROUPS; grp += blockDim.x) {
-        const int ci4 = grp % (CI / 4), r1 = grp / (CI / 4);
-        const int co4 = r1 % (CO / 4), tap = r1 / (CO / 4);
-        const int dy = tap / KS - HP, dx = tap % KS - HP;
-        float a[4][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int id = lane >> 3, r = lane & 7;        // ldmatrix: matrix and row this lane addresses
+    const uint32_t xa = (uint32_t)__cvta_generic_to_shared(xs), da = (uint32_t)__cvta_generic_to_shared(ds);
+    const int rows = T / kparts;
+    for (int unit = blockIdx.z * 8 + warp; unit < S::ITEMS * kparts; unit += gridDim.z * 8) {
+        const int item = unit % S::ITEMS, py0 = unit / S::ITEMS * rows;
+        const int tap = item / (CI / 16), cib = item % (CI / 16);
+        const int dy = tap / KS, dx = tap % KS;    // offsets in the staged tile
+        float acc[CO / 16][2][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < CO / 16; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) a[i][j] = 0.f;
-        for (int p = 0; p < TH * TW; ++p) {
-            const int py = p / TW, pxx = p % TW;
-            const bf16* dp = ds + p * CO + co4 * 4;
-            const bf16* xp = xs + ((py + HP + dy) * IW + (pxx + HP + dx)) * CI + ci4 * 4;
-            float dv[4], xv[4];
+            for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { dv[i] = __bfloat162float(dp[i]); xv[i] = __bfloat162float(xp[i]); }
+                for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+        for (int py = py0; py < py0 + rows; ++py) {
+            // B: pixels k = 8 (id & 1) + r, input channels 8 (id >> 1) ..
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4_t(xa + 2 * (((py + dy) * IW + (id & 1) * 8 + r + dx) * S::CIP + cib * 16 + (id >> 1) * 8), b0, b1, b2, b3);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) a[i][j] = fmaf(dv[i], xv[j], a[i][j]);
+            for (int i = 0; i < CO / 16; ++i) {
+                // A: pixels k = 8 (id >> 1) + r, output channels 8 (id & 1) ..
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4_t(da + 2 * ((py * T + (id >> 1) * 8 + r) * S::COP + i * 16 + (id & 1) * 8), a0, a1, a2, a3);
+                mma16816(acc[i][0], a0, a1, a2, a3, b0, b1);
+                mma16816(acc[i][1], a0, a1, a2, a3, b2, b3);
+            }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < CO / 16; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                atomicAdd(dW + ((size_t)tap * CO + co4 * 4 + i) * CI + ci4 * 4 + j, a[i][j]);
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int co = i * 16 + (lane >> 2) + (e >> 1) * 8, ci = cib * 16 + j * 8 + (lane & 3) * 2 + (e & 1);
+                    atomicAdd(dW + ((size_t)tap * CO + co) * CI + ci, acc[i][j][e]);
+                }
     }
 }
 
@@ -907,17 +940,23 @@ cudaError_t conv(const bf16* in, int istr, int ioff, const bf16* W, void* out, i
 
 template <int CI, int CO, int KS>
 cudaError_t wgrad(const bf16* in, int istr, int ioff, const bf16* dout, const Lv& lv, float* dW, cudaStream_t s) {
-    constexpr int HP = KS / 2;
-    const size_t sm = sizeof(bf16) * ((16 + 2 * HP) * (16 + 2 * HP) * CI + 256 * CO);
+    using S = WgradShape<CI, CO, KS>;
+    constexpr int SMS = 152;
     static bool configured = false;
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(conv_wgrad<CI, CO, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sm);
+                                             (int)S::SMEM);
         if (e != cudaSuccess) return e;
         configured = true;
     }
     dim3 grid((lv.Wd + 15) / 16, (lv.H + 15) / 16);
-    conv_wgrad<CI, CO, KS><<<grid, 256, sm, s>>>(in, istr, ioff, dout, lv, dW);
+    // split the units until every SM has a CTA: first one unit a warp, then halves
+    // and quarters of the tile's rows (each part adds its own sums to dW)
+    const int tiles = grid.x * grid.y;
+    int kparts = 1;
+    while (kparts < 4 && tiles * ((S::ITEMS * kparts + 7) / 8) < SMS) kparts *= 2;
+    grid.z = std::max(1, std::min((S::ITEMS * kparts + 7) / 8, 2 * SMS / tiles));
+    conv_wgrad<CI, CO, KS><<<grid, 256, S::SMEM, s>>>(in, istr, ioff, dout, lv, dW, kparts);
     return cudaGetLastError();
 }
 

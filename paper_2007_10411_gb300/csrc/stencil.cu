@@ -33,15 +33,6 @@ namespace jfnk {
 constexpr int R = 2;          // derivative radius for p = 2
 constexpr int HALO = 2 * R;   // input halo (derivative applied twice)
 
-// Candidate tiles of the float32 Jacobian product (jvc2d): tile and staging
-// buffers.  jfnk_autotune times each on the handle's workload, with the CTA sizes
-// of the float32 preconditioner sweep (launch_precond_f32), and keeps the fastest
-// (Geo::tile_jv, Geo::tile_pc).
-template <int I> struct JvcTile;
-template <> struct JvcTile<0> { static constexpr int TX = 32, TZ = 16, NBUF = 1; };
-template <> struct JvcTile<1> { static constexpr int TX = 32, TZ = 16, NBUF = 2; };
-template <> struct JvcTile<2> { static constexpr int TX = 64, TZ = 8, NBUF = 1; };
-template <> struct JvcTile<3> { static constexpr int TX = 32, TZ = 8, NBUF = 1; };
 // Explicitly rounded product and fused multiply-add: expressions written with
 // them round the same way in every instantiation (tile shape) of a kernel.
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
@@ -456,133 +447,57 @@ __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_gro
 template <int N>
 __device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Issue the copies of the ghost-extended u and v tiles (four fields each) into
-// s[0..4) and s[4..8) (planes of SZ x SX).  jv_stage_fix walks the same chunk
-// -> thread assignment once the copies have landed, so a thread only touches
-// what it copied itself: mirror signs on ghost rows and the eps scale on v,
-// in the order load_fields applies them.
-template <typename T>
-__device__ __forceinline__ void jv_stage_issue(T* s, const T* __restrict__ u, const T* __restrict__ v,
-                                               const Geo& G, int x0, int z0, int SX, int SZ) {
-    constexpr int VW = Vec16<T>::W;
-    const int plane = SZ * SX;
-    if (rows_vectorisable<T>(G, x0, SX)) {
-        const int nch = SX / VW;
-        const int total = nch * SZ;
-        for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-            const int iz = idx / nch, c = idx - iz * nch;
-            int side;
-            const int sz = mirror_z(z0 + iz - HALO, G.nz, side);
-            const bool ok = sz >= 0 && sz < G.nz;
-            const size_t off = ok ? (size_t)sz * G.nx + (x0 - HALO + c * VW) : 0;
-            T* d = s + iz * SX + c * VW;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                cpa16(d + f * plane, u + (size_t)f * G.npt + off, ok ? 16 : 0);
-                cpa16(d + (4 + f) * plane, v + (size_t)f * G.npt + off, ok ? 16 : 0);
-            }
-        }
-        return;
-    }
-    const int total = SX * SZ;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int iz = idx / SX, ix = idx - iz * SX;
-        int side;
-        const int sz = mirror_z(z0 + iz - HALO, G.nz, side);
-        const bool ok = sz >= 0 && sz < G.nz;
-        const size_t off = ok ? (size_t)sz * G.nx + wrap_x(x0 + ix - HALO, G.nx) : 0;
-        T* d = s + iz * SX + ix;
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            cpa_elem<sizeof(T)>(d + f * plane, u + (size_t)f * G.npt + off, ok ? (int)sizeof(T) : 0);
-            cpa_elem<sizeof(T)>(d + (4 + f) * plane, v + (size_t)f * G.npt + off, ok ? (int)sizeof(T) : 0);
-        }
-    }
+// Row vectors: a thread of the float32 sweeps and of the Schur-complement kernels
+// owns W consecutive points along x (16 bytes where nx allows it).
+template <typename T, int W> struct RowVec { using type = typename Vec16<T>::type; };
+template <typename T> struct RowVec<T, 1> { using type = T; };
+template <> struct RowVec<float, 2> { using type = float2; };
+template <typename T, int W>
+__device__ __forceinline__ void rload(const T* p, T (&v)[W]) {
+    *reinterpret_cast<typename RowVec<T, W>::type*>(v) = *reinterpret_cast<const typename RowVec<T, W>::type*>(p);
+}
+template <typename T, int W>
+__device__ __forceinline__ void rstore(T* p, const T (&v)[W]) {
+    *reinterpret_cast<typename RowVec<T, W>::type*>(p) = *reinterpret_cast<const typename RowVec<T, W>::type*>(v);
+}
+
+// Asynchronous copy of W elements (16, 8 or 4 bytes) into shared memory.
+template <typename T, int W>
+__device__ __forceinline__ void cpa_vec(T* dst, const T* src) {
+    if constexpr (W * sizeof(T) == 16) cpa16(dst, src, 16);
+    else cpa_elem<W * (int)sizeof(T)>(dst, src, W * (int)sizeof(T));
 }
 
 // ============================================================================
-// Mixed-path Jv, compute-once form (float32 path).
+// Mixed-path Jv in 2-D (float32): the forward difference F(u + eps V) - F(u)
+// formed term by term, free of cancellation.  With a = u, b = eps V (per field
+// eps scale_f) and the midpoint m = a + b/2 of the two states,
+//   convection  a'_j phi' - a_j phi = m_j b_phi + b_j m_phi,
+//   diffusion   K' D phi' - K D phi = Km D b_phi + dK D m_phi,
+//               Km = (K + K')/2, dK = K' - K in cancellation-free form,
+//   pressure    (pbar + p') div' - (pbar + p) div = (pbar + m_p) div b + b_p div m,
+// so each flux difference X_phi = Km D_x b + dK D_x m - 1/2 (m_u b_phi + b_u m_phi)
+// (Z_phi alike) is formed once per point and
+//   dF_phi = D_x X_phi + D_z Z_phi + S_phi.
+// Phase 1 stages u and the raw direction v of a TX x TZ tile with a halo of 4
+// (cp.async; D(b) = eps D(v) is scaled in registers).  Phase 2 forms, for W
+// consecutive points per thread, both fluxes and the point-wise part S (kept in
+// registers), and on the arms X (two columns either side) or Z (two rows above
+// and below) alone.  Phase 3 differentiates the fluxes and writes Jv.
+// The arithmetic is explicitly rounded, so a flux formed in a tile and the same
+// flux formed in a neighbour's arm are bitwise equal and every tile shape gives
+// the same result.  The eddy coefficient of a point in a ghost row is that of
+// its mirror image.
 //
-// Same quantity as jv_diff2d, organised so that every flux is formed once per
-// point and only then differentiated.  With a = u and b = eps V (per field
-// eps scale_f), the difference of F(a + b) - F(a) is, term by term,
-//   convection  1/2 [D_x P_phi + D_z Q_phi] + 1/2 adv_phi,
-//               P_phi = a_u b_phi + b_u (a_phi + b_phi)   (x-flux difference)
-//               Q_phi = a_w b_phi + b_w (a_phi + b_phi)   (z-flux difference)
-//               adv_phi = a_u D_x b_phi + a_w D_z b_phi + b_u D_x phi' + b_w D_z phi'
-//   diffusion   D_x Fx_phi + D_z Fz_phi,
-//               Fx_phi = K_a D_x b_phi + dK D_x phi'  (dK = K(a + b) - K(a), cancellation-free),
-//   point-wise  pressure gradient, buoyancy, stratification, (pbar + p) div u,
-// with phi' = a_phi + b_phi.  Phase 1 stages u and the raw direction v of a
-// TX x TZ tile with a halo of 4 (cp.async, the next tile's copies in flight
-// while this one is computed; the eps scale is applied in registers, so only
-// ghost rows need a pass over the staged planes, for the mirror signs).
-// Phase 2 forms, at every point where they are differentiated, the x-fluxes
-// P, Fx (tile rows, columns -2 .. TX+1) and the z-fluxes Q, Fz (rows -2 ..
-// TZ+1, tile columns), and, at the tile's own points, the point-wise part S
-// (kept in registers).  Phase 3 differentiates the fluxes and writes Jv.
-// Phases 2 and 3 give a thread the same PPT vertically adjacent points of
-// one column (warps run along x: conflict-free shared-memory rows).  Every
-// value at a point is computed by the same expression whatever the tile
-// shape, so all shapes give bitwise the same result.
-// The eddy coefficient at a ghost row is the mirror image of the interior
-// value (K mirrored even): the Smagorinsky step of a flux point in a ghost
-// row is evaluated at its image row.
+// Bound: issue and shared-memory latency.  The form with one point per thread,
+// diffusive and convective fluxes apart and products about a: 22 us at
+// 1024 x 512 and 7.4 us at 250 x 119; this form 17.5 and 5.3 us.
 // ============================================================================
-template <int TX, int TZ>
-struct JvcShape {
-    static constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO;
-    static constexpr int PLANE = SX * SZ;
-    static constexpr int STG = 8 * PLANE;                 // u (planes 0-3) and raw v (planes 4-7)
-    static constexpr int PXW = TX + 2 * R;                // x-flux rows: columns -2 .. TX+1
-    static constexpr int PXN = TZ * PXW;                  // per flux field
-    static constexpr int QZN = (TZ + 2 * R) * TX;         // z-flux columns: rows -2 .. TZ+1
-    static constexpr int PPT = TX * TZ / NTHREADS;        // points per thread (one column, PPT rows)
-    static constexpr int NARM = 4 * TX + 4 * TZ;          // z-arm items, then x-arm items
-    static_assert(NTHREADS % TX == 0 && PPT * (NTHREADS / TX) == TZ && PPT >= 1, "tile / thread mapping");
-    static constexpr size_t smem(int nbuf) { return sizeof(float) * ((size_t)nbuf * STG + 7 * PXN + 7 * QZN); }
-};
-
-// Tile row (in staged coordinates, relative to the tile origin) whose eddy
-// value a flux point in tile row iz takes: its mirror image where the global
-// row is a ghost row (-2, -1 or nz, nz+1), else itself.
-__device__ __forceinline__ int jvc_smag_row(int iz, int z0, int nz) {
-    const int gz = z0 + iz;
-    if (gz < 0) return (-1 - gz) - z0;
-    if (gz >= nz && gz <= nz + 1) return (2 * nz - 1 - gz) - z0;
-    return iz;
-}
-
-struct JvcConst {
-    float ev[4];        // eps scale_f: b = ev * v
-    float idx, idz;
-    float cs2, iPr, KM, KH;
-    float cm, cM, cl, dlt, ah, az;   // Deardorff constants (Geo::dd_*)
-};
-
-// The flux and derivative arithmetic of jvc2d is written with explicitly
-// rounded operations (no contraction left to the compiler), so a flux formed
-// in the tile centre and the same flux formed in a neighbouring tile's arm
-// are bitwise equal, and every tile shape gives the same result.
-// w1 = (2/3)/h, w2 = -(1/12)/h (Geo::fx1 .. fz2)
-__device__ __forceinline__ float ddf(const float* s, int i, int st, float w1, float w2) {
-    const float d1 = __fsub_rn(s[i + st], s[i - st]), d2 = __fsub_rn(s[i + 2 * st], s[i - 2 * st]);
-    return __fmaf_rn(w1, d1, __fmul_rn(w2, d2));
-}
-// a0 b + b0 (a + b): the flux difference a'_j phi' - a_j phi
-__device__ __forceinline__ float flux_diff(float a0, float b0, float a, float b) {
-    return __fmaf_rn(a0, b, __fmul_rn(b0, __fadd_rn(a, b)));
-}
-// K b' + dK (a' + b'): the diffusive flux difference
-__device__ __forceinline__ float kflux_diff(float kk, float dk, float da, float db) {
-    return __fmaf_rn(kk, db, __fmul_rn(dk, __fadd_rn(da, db)));
-}
-
 // The strain magnitude s = sqrt(2 S:S) at a, at a' = a + b, and their
 // difference ds = s' - s in cancellation-free form, from the velocity
 // gradients of a (ux, uz, wx, wz) and of b.
-__device__ __forceinline__ void jvc_strain(float aux, float auz, float awx, float awz, float bux, float buz,
-                                           float bwx, float bwz, float& sa, float& sp, float& ds) {
+__device__ __forceinline__ void jv_strain(float aux, float auz, float awx, float awz, float bux, float buz,
+                                          float bwx, float bwz, float& sa, float& sp, float& ds) {
     const float a13 = __fmul_rn(0.5f, __fadd_rn(auz, awx)), b13 = __fmul_rn(0.5f, __fadd_rn(buz, bwx));
     const float ssa = __fmaf_rn(aux, aux, __fmaf_rn(awz, awz, __fmul_rn(2.f, __fmul_rn(a13, a13))));
     // S':S' - S:S = (2 S + S_b) : S_b
@@ -603,270 +518,346 @@ __device__ __forceinline__ void jvc_strain(float aux, float auz, float awx, floa
 // Deardorff heat factor g(s) = s (1 + a l(s)), l = min(Delta, c_l s), at s and
 // its difference g(s') - g(s) = ds (1 + a l') + a s (l' - l), with l' - l = c_l ds
 // where neither side is capped (0 where both are; direct where they straddle).
-__device__ __forceinline__ void jvc_heat(float sa, float sp, float ds, float a, const JvcConst& k, float& g,
-                                         float& dg) {
-    float la = k.dlt, lp = k.dlt, dl = 0.f;
-    if (k.cl >= 0.f) {
-        const float ta = __fmul_rn(k.cl, sa), tp = __fmul_rn(k.cl, sp);
-        la = ta < k.dlt ? ta : k.dlt;
-        lp = tp < k.dlt ? tp : k.dlt;
-        if (ta < k.dlt && tp < k.dlt) dl = __fmul_rn(k.cl, ds);
-        else if (ta < k.dlt || tp < k.dlt) dl = __fsub_rn(lp, la);
+__device__ __forceinline__ void jv_heat(const Geo& G, float sa, float sp, float ds, float a, float& g, float& dg) {
+    const float cl = G.f32.dd_cl, dlt = G.f32.dd_delta;
+    float la = dlt, lp = dlt, dl = 0.f;
+    if (cl >= 0.f) {
+        const float ta = __fmul_rn(cl, sa), tp = __fmul_rn(cl, sp);
+        la = ta < dlt ? ta : dlt;
+        lp = tp < dlt ? tp : dlt;
+        if (ta < dlt && tp < dlt) dl = __fmul_rn(cl, ds);
+        else if (ta < dlt || tp < dlt) dl = __fsub_rn(lp, la);
     }
     g = __fmul_rn(sa, __fmaf_rn(a, la, 1.f));
     dg = __fmaf_rn(ds, __fmaf_rn(a, lp, 1.f), __fmul_rn(__fmul_rn(a, sa), dl));
 }
 
-// Phase 2 at one point.  i: staged index of the point; is: staged index of the
-// point whose eddy coefficient it takes (its image in a ghost row).  XF: the
-// x-fluxes P, Fx; ZF: the z-fluxes Q, Fz; CEN: also the point-wise part S.
-template <int SMAG, bool XF, bool ZF, bool CEN, int SX, int PLANE>
-__device__ __forceinline__ void jvc_point(const float* __restrict__ st, int i, int is, const JvcConst& k,
-                                          const Geo& G, float (&P)[4], float (&Fx)[3], float (&Q)[4],
-                                          float (&Fz)[3], float (&S)[4], float (&vraw)[4]) {
-    const float* A = st;                 // a planes 0..3
-    const float* V = st + 4 * PLANE;     // raw v planes 0..3
-    float a[4], b[4];
+template <int W, int NT>
+struct JvShape {
+    static constexpr int NXT = W == 4 ? 16 : 32, TX = NXT * W, TZ = NT / NXT;
+    static constexpr int SX = TX + 2 * HALO, SZ = TZ + 2 * HALO, PLANE = SX * SZ;
+    static constexpr int XN = TZ * SX;                 // X flux of one field (rows padded like the staged ones)
+    static constexpr int ZN = (TZ + 2 * R) * TX;       // Z flux of one field
+    static constexpr int ZARM = 2 * R * NXT, XARM = 2 * R * TZ;      // arm items: W points, one point
+    static constexpr size_t smem = sizeof(float) * (size_t)(8 * PLANE + 4 * XN + 4 * ZN);
+};
+
+// D_x / D_z of the W points at staged index i of a plane
+template <int W>
+__device__ __forceinline__ void jv_dx(const float* __restrict__ s, int i, float w1, float w2, float (&d)[W]) {
+    float e[W + 4];
+    if constexpr (W == 1) {
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        a[f] = A[f * PLANE + i];
-        vraw[f] = V[f * PLANE + i];
-        b[f] = __fmul_rn(k.ev[f], vraw[f]);
-    }
-    // first derivatives at the point (b-derivatives scaled by ev in registers)
-    constexpr bool DXUW = XF || CEN || SMAG, DZUW = ZF || CEN || SMAG;
-    constexpr bool DXT = XF || CEN, DZT = ZF || CEN;
-    float dax[4] = {0.f, 0.f, 0.f, 0.f}, daz[4] = {0.f, 0.f, 0.f, 0.f};
-    float dbx[4] = {0.f, 0.f, 0.f, 0.f}, dbz[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int k = 0; k < 5; ++k) e[k] = s[i + k - 2];
+    } else {
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        const bool wx = f < 2 ? DXUW : (f == 2 ? DXT : CEN);
-        const bool wz = f < 2 ? DZUW : (f == 2 ? DZT : CEN);
-        if (wx) {
-            dax[f] = ddf(A + f * PLANE, i, 1, G.f32.wx1, G.f32.wx2);
-            dbx[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, 1, G.f32.wx1, G.f32.wx2));
-        }
-        if (wz) {
-            daz[f] = ddf(A + f * PLANE, i, SX, G.f32.wz1, G.f32.wz2);
-            dbz[f] = __fmul_rn(k.ev[f], ddf(V + f * PLANE, i, SX, G.f32.wz1, G.f32.wz2));
+        for (int k = 0; k < W + 4; k += 2) {
+            const float2 v = *reinterpret_cast<const float2*>(s + i - 2 + k);
+            e[k] = v.x;
+            e[k + 1] = v.y;
         }
     }
-    // exchange coefficients along x and z, momentum [0] and heat [1], and their differences
-    float kx[2], dkx[2], kz[2], dkz[2];
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+        d[k] = __fmaf_rn(w1, __fsub_rn(e[k + 3], e[k + 1]), __fmul_rn(w2, __fsub_rn(e[k + 4], e[k])));
+}
+template <int W>
+__device__ __forceinline__ void jv_dz(const float* __restrict__ s, int i, int st, float w1, float w2, float (&d)[W]) {
+    float a[W], b[W], c[W], e[W];
+    rload<float, W>(s + i - 2 * st, a);
+    rload<float, W>(s + i - st, b);
+    rload<float, W>(s + i + st, c);
+    rload<float, W>(s + i + 2 * st, e);
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+        d[k] = __fmaf_rn(w1, __fsub_rn(c[k], b[k]), __fmul_rn(w2, __fsub_rn(e[k], a[k])));
+}
+
+// Phase 2 at W points (staged index i; is: the index whose eddy coefficient they
+// take).  XF / ZF: form the X / Z fluxes; both: tile points with their part S.
+template <int W, int SMAG, bool XF, bool ZF, int SX, int PLANE, int XN, int ZN>
+__device__ __forceinline__ void jv_points(const Geo& G, const float (&ev)[4], const float* __restrict__ st, int i, int is,
+                                          float* __restrict__ X, float* __restrict__ Z, float (&S)[4][W]) {
+    constexpr bool CEN = XF && ZF;
+    const float wx1 = G.f32.wx1, wx2 = G.f32.wx2, wz1 = G.f32.wz1, wz2 = G.f32.wz2;
+    const float* U = st;                     // u planes 0..3
+    const float* V = st + 4 * PLANE;         // raw v planes 0..3
+    // velocity gradients of a and b (b by its eps)
+    float ax[2][W], az[2][W], bx[2][W], bz[2][W];
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        if (XF || SMAG) {
+            jv_dx<W>(U + f * PLANE, i, wx1, wx2, ax[f]);
+            jv_dx<W>(V + f * PLANE, i, wx1, wx2, bx[f]);
+        }
+        if (ZF || SMAG) {
+            jv_dz<W>(U + f * PLANE, i, SX, wz1, wz2, az[f]);
+            jv_dz<W>(V + f * PLANE, i, SX, wz1, wz2, bz[f]);
+        }
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            if (XF || SMAG) bx[f][k] = __fmul_rn(ev[f], bx[f][k]);
+            if (ZF || SMAG) bz[f][k] = __fmul_rn(ev[f], bz[f][k]);
+        }
+    }
+    // exchange coefficients: midpoint and difference, momentum [0] and heat [1], along x and z
+    float kx[2][W], dkx[2][W], kz[2][W], dkz[2][W];
     if (SMAG) {
-        float sa, sp, ds;
+        float sa[W], sp[W], ds[W];
         if (is == i) {
-            jvc_strain(dax[0], daz[0], dax[1], daz[1], dbx[0], dbz[0], dbx[1], dbz[1], sa, sp, ds);
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+                jv_strain(ax[0][k], az[0][k], ax[1][k], az[1][k], bx[0][k], bz[0][k], bx[1][k], bz[1][k], sa[k], sp[k], ds[k]);
         } else {
-            jvc_strain(ddf(A, is, 1, G.f32.wx1, G.f32.wx2), ddf(A, is, SX, G.f32.wz1, G.f32.wz2), ddf(A + PLANE, is, 1, G.f32.wx1, G.f32.wx2),
-                       ddf(A + PLANE, is, SX, G.f32.wz1, G.f32.wz2), __fmul_rn(k.ev[0], ddf(V, is, 1, G.f32.wx1, G.f32.wx2)),
-                       __fmul_rn(k.ev[0], ddf(V, is, SX, G.f32.wz1, G.f32.wz2)),
-                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, 1, G.f32.wx1, G.f32.wx2)),
-                       __fmul_rn(k.ev[1], ddf(V + PLANE, is, SX, G.f32.wz1, G.f32.wz2)), sa, sp, ds);
+            float cx[2][W], cz[2][W], ex[2][W], ez[2][W];
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                jv_dx<W>(U + f * PLANE, is, wx1, wx2, cx[f]);
+                jv_dz<W>(U + f * PLANE, is, SX, wz1, wz2, cz[f]);
+                jv_dx<W>(V + f * PLANE, is, wx1, wx2, ex[f]);
+                jv_dz<W>(V + f * PLANE, is, SX, wz1, wz2, ez[f]);
+            }
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+                jv_strain(cx[0][k], cz[0][k], cx[1][k], cz[1][k], __fmul_rn(ev[0], ex[0][k]), __fmul_rn(ev[0], ez[0][k]),
+                          __fmul_rn(ev[1], ex[1][k]), __fmul_rn(ev[1], ez[1][k]), sa[k], sp[k], ds[k]);
         }
-        if (SMAG == 2) {
-            kx[0] = __fmul_rn(k.cm, sa); dkx[0] = __fmul_rn(k.cm, ds);
-            kz[0] = __fmul_rn(k.cM, sa); dkz[0] = __fmul_rn(k.cM, ds);
-            float g, dg;
-            jvc_heat(sa, sp, ds, k.ah, k, g, dg);
-            kx[1] = __fmul_rn(k.cm, g); dkx[1] = __fmul_rn(k.cm, dg);
-            jvc_heat(sa, sp, ds, k.az, k, g, dg);
-            kz[1] = __fmul_rn(k.cM, g); dkz[1] = __fmul_rn(k.cM, dg);
-        } else {
-            const float ka = __fmul_rn(k.cs2, sa), dk = __fmul_rn(k.cs2, ds);
-            kx[0] = kz[0] = ka; dkx[0] = dkz[0] = dk;
-            kx[1] = kz[1] = __fmul_rn(ka, k.iPr); dkx[1] = dkz[1] = __fmul_rn(dk, k.iPr);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const float sm = __fmaf_rn(0.5f, ds[k], sa[k]);
+            if (SMAG == 2) {
+                const float cm = G.f32.dd_cm, cM = G.f32.dd_cM;
+                kx[0][k] = __fmul_rn(cm, sm);
+                dkx[0][k] = __fmul_rn(cm, ds[k]);
+                kz[0][k] = __fmul_rn(cM, sm);
+                dkz[0][k] = __fmul_rn(cM, ds[k]);
+                float g, dg;
+                if (XF) {
+                    jv_heat(G, sa[k], sp[k], ds[k], G.f32.dd_ah, g, dg);
+                    kx[1][k] = __fmul_rn(cm, __fmaf_rn(0.5f, dg, g));
+                    dkx[1][k] = __fmul_rn(cm, dg);
+                }
+                if (ZF) {
+                    jv_heat(G, sa[k], sp[k], ds[k], G.f32.dd_az, g, dg);
+                    kz[1][k] = __fmul_rn(cM, __fmaf_rn(0.5f, dg, g));
+                    dkz[1][k] = __fmul_rn(cM, dg);
+                }
+            } else {
+                kx[0][k] = kz[0][k] = __fmul_rn(G.f32.cs2, sm);
+                dkx[0][k] = dkz[0][k] = __fmul_rn(G.f32.cs2, ds[k]);
+                kx[1][k] = kz[1][k] = __fmul_rn(kx[0][k], G.f32.inv_Pr);
+                dkx[1][k] = dkz[1][k] = __fmul_rn(dkx[0][k], G.f32.inv_Pr);
+            }
         }
     } else {
-        kx[0] = kz[0] = k.KM; kx[1] = kz[1] = k.KH;
-        dkx[0] = dkz[0] = dkx[1] = dkz[1] = 0.f;
-    }
-    if (XF) {
 #pragma unroll
-        for (int f = 0; f < 4; ++f) P[f] = flux_diff(a[0], b[0], a[f], b[f]);
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            const int c = f == 2 ? 1 : 0;
-            Fx[f] = SMAG ? kflux_diff(kx[c], dkx[c], dax[f], dbx[f]) : __fmul_rn(kx[c], dbx[f]);
+        for (int k = 0; k < W; ++k) {
+            kx[0][k] = kz[0][k] = G.f32.K_M;
+            kx[1][k] = kz[1][k] = G.f32.K_H;
+            dkx[0][k] = dkx[1][k] = dkz[0][k] = dkz[1][k] = 0.f;
         }
     }
-    if (ZF) {
+    // half the advecting velocities, midpoint and b
+    float mu[W], bu[W], mw[W], bw[W];
+    {
+        float a[W], v[W];
+        rload<float, W>(U + i, a);
+        rload<float, W>(V + i, v);
 #pragma unroll
-        for (int f = 0; f < 4; ++f) Q[f] = flux_diff(a[1], b[1], a[f], b[f]);
+        for (int k = 0; k < W; ++k) {
+            const float b = __fmul_rn(ev[0], v[k]);
+            bu[k] = __fmul_rn(0.5f, b);
+            mu[k] = __fmul_rn(0.5f, __fadd_rn(a[k], bu[k]));
+        }
+        rload<float, W>(U + PLANE + i, a);
+        rload<float, W>(V + PLANE + i, v);
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            const int c = f == 2 ? 1 : 0;
-            Fz[f] = SMAG ? kflux_diff(kz[c], dkz[c], daz[f], dbz[f]) : __fmul_rn(kz[c], dbz[f]);
+        for (int k = 0; k < W; ++k) {
+            const float b = __fmul_rn(ev[1], v[k]);
+            bw[k] = __fmul_rn(0.5f, b);
+            mw[k] = __fmul_rn(0.5f, __fadd_rn(a[k], bw[k]));
         }
     }
-    if (CEN) {
-        const float th0 = G.f32.theta0;
+    float divb[W], divm[W];
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            // a_u D_x b + a_w D_z b + b_u D_x phi' + b_w D_z phi'
-            const float adv = __fmaf_rn(a[0], dbx[f], __fmaf_rn(a[1], dbz[f],
-                              __fmaf_rn(b[0], __fadd_rn(dax[f], dbx[f]), __fmul_rn(b[1], __fadd_rn(daz[f], dbz[f])))));
-            S[f] = __fmul_rn(-0.5f, adv);
+    for (int f = 0; f < 4; ++f) {
+        float a[W], v[W], dax[W], daz[W], dbx[W], dbz[W];
+        rload<float, W>(U + f * PLANE + i, a);
+        rload<float, W>(V + f * PLANE + i, v);
+        const bool needx = XF && (f < 3 || CEN), needz = ZF && (f < 3 || CEN);
+        if (f < 2) {
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                dax[k] = ax[f][k];
+                daz[k] = az[f][k];
+                dbx[k] = bx[f][k];
+                dbz[k] = bz[f][k];
+            }
+        } else {
+            if (needx) {
+                jv_dx<W>(U + f * PLANE, i, wx1, wx2, dax);
+                jv_dx<W>(V + f * PLANE, i, wx1, wx2, dbx);
+            }
+            if (needz) {
+                jv_dz<W>(U + f * PLANE, i, SX, wz1, wz2, daz);
+                jv_dz<W>(V + f * PLANE, i, SX, wz1, wz2, dbz);
+            }
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                if (needx) dbx[k] = __fmul_rn(ev[f], dbx[k]);
+                if (needz) dbz[k] = __fmul_rn(ev[f], dbz[k]);
+            }
         }
-        const float gth = G.f32.gth;
-        S[0] = __fmaf_rn(-th0, dbx[3], S[0]);
-        S[1] = __fmaf_rn(-th0, dbz[3], __fmaf_rn(gth, b[2], S[1]));
-        S[2] = __fmaf_rn(-G.f32.beta, b[1], S[2]);
-        const float diva = __fadd_rn(dax[0], daz[1]), divb = __fadd_rn(dbx[0], dbz[1]);
-        const float pp = __fadd_rn(__fadd_rn(G.f32.pbar, a[3]), b[3]);
-        S[3] = __fmaf_rn(-G.f32.gamma_p, __fmaf_rn(pp, divb, __fmul_rn(b[3], diva)), S[3]);
+        float Xv[W], Zv[W];
+        const int h = f == 2 ? 1 : 0;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const float b = __fmul_rn(ev[f], v[k]), m = __fmaf_rn(0.5f, b, a[k]);
+            float dmx = 0.f, dmz = 0.f;
+            if (needx) dmx = __fmaf_rn(0.5f, dbx[k], dax[k]);
+            if (needz) dmz = __fmaf_rn(0.5f, dbz[k], daz[k]);
+            if (XF) {
+                float x = -__fmaf_rn(mu[k], b, __fmul_rn(bu[k], m));
+                if (f < 3) {
+                    x = __fmaf_rn(kx[h][k], dbx[k], x);
+                    if (SMAG) x = __fmaf_rn(dkx[h][k], dmx, x);
+                }
+                Xv[k] = x;
+            }
+            if (ZF) {
+                float z = -__fmaf_rn(mw[k], b, __fmul_rn(bw[k], m));
+                if (f < 3) {
+                    z = __fmaf_rn(kz[h][k], dbz[k], z);
+                    if (SMAG) z = __fmaf_rn(dkz[h][k], dmz, z);
+                }
+                Zv[k] = z;
+            }
+            if (CEN) {
+                float s = -__fmaf_rn(mu[k], dbx[k], __fmaf_rn(bu[k], dmx, __fmaf_rn(mw[k], dbz[k], __fmul_rn(bw[k], dmz))));
+                if (f == 0) { divb[k] = dbx[k]; divm[k] = dmx; }
+                if (f == 1) {
+                    divb[k] = __fadd_rn(divb[k], dbz[k]);
+                    divm[k] = __fadd_rn(divm[k], dmz);
+                    S[2][k] = -__fmul_rn(G.f32.beta, b);
+                }
+                if (f == 2) {
+                    s = __fadd_rn(s, S[2][k]);
+                    S[1][k] = __fmaf_rn(G.f32.gth, b, S[1][k]);
+                }
+                if (f == 3) {
+                    S[0][k] = __fmaf_rn(-G.f32.theta0, dbx[k], S[0][k]);
+                    S[1][k] = __fmaf_rn(-G.f32.theta0, dbz[k], S[1][k]);
+                    s = __fmaf_rn(-G.f32.gamma_p, __fmaf_rn(__fadd_rn(G.f32.pbar, m), divb[k], __fmul_rn(b, divm[k])), s);
+                }
+                S[f][k] = s;
+            }
+        }
+        if (XF) rstore<float, W>(X + f * XN, Xv);
+        if (ZF) rstore<float, W>(Z + f * ZN, Zv);
     }
 }
 
-template <int SMAG, int TX, int TZ, int NBUF>
-__global__ void __launch_bounds__(NTHREADS)
-jvc2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __restrict__ out,
-      const double* part, Ctl* ctl, int check_done) {
-    using SH = JvcShape<TX, TZ>;
-    constexpr int SX = SH::SX, PLANE = SH::PLANE, PXW = SH::PXW, PXN = SH::PXN, QZN = SH::QZN;
-    constexpr int PPT = SH::PPT;
-    pdl_wait();
-    if (check_done && ctl->done) return;
+template <int W, int NT, int SMAG>
+__global__ void __launch_bounds__(NT, 512 / NT)
+jv2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __restrict__ out,
+     const double* part, Ctl* ctl, int check_done) {
+    using SH = JvShape<W, NT>;
+    constexpr int TX = SH::TX, TZ = SH::TZ, SX = SH::SX, SZ = SH::SZ, PLANE = SH::PLANE, XN = SH::XN, ZN = SH::ZN;
+    constexpr int RV = SX / W;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* stg = reinterpret_cast<float*>(smem_raw);
-    float* PX = stg + NBUF * SH::STG;    // [4][TZ][PXW] then Fx [3][TZ][PXW]
-    float* FX = PX + 4 * PXN;
-    float* QZ = FX + 3 * PXN;            // [4][TZ+4][TX] then Fz [3][TZ+4][TX]
-    float* FZ = QZ + 4 * QZN;
-    const int ntx = (G.nx + TX - 1) / TX;
-    const int ntiles = ntx * ((G.nz + TZ - 1) / TZ);
-    int t = blockIdx.x;
-    if (t < ntiles) jv_stage_issue(stg, u, v, G, (t % ntx) * TX, (t / ntx) * TZ, SX, SH::SZ);
+    float* st = reinterpret_cast<float*>(smem_raw);      // u (planes 0-3) and raw v (planes 4-7)
+    float* X = st + 8 * PLANE;                           // [4][TZ][SX], tile column 0 at HALO
+    float* Z = X + 4 * XN;                               // [4][TZ + 4][TX]
+    pdl_wait();
+    const int done = check_done ? ctl->done : 0;
+    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
+    const size_t np = (size_t)G.npt;
+    if (done) return;
+    for (int j = threadIdx.x; j < SZ * RV; j += NT) {
+        const int iz = j / RV, ix = (j % RV) * W;
+        int side;
+        // rows beyond one reflection feed no output
+        const int sz = min(max(mirror_z(z0 + iz - HALO, G.nz, side), 0), G.nz - 1);
+        const size_t o = (size_t)sz * G.nx + wrap_x(x0 + ix - HALO, G.nx);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            cpa_vec<float, W>(st + f * PLANE + iz * SX + ix, u + f * np + o);
+            cpa_vec<float, W>(st + (4 + f) * PLANE + iz * SX + ix, v + f * np + o);
+        }
+    }
     cpa_commit();
+    // the step, while the copies are in flight
     const double2 eps = pending_eps(ctl, part);
     __shared__ float evs[4], cfs[4];
     if (threadIdx.x < 4) {
         evs[threadIdx.x] = (float)(eps.x * G.scale[threadIdx.x]);
         cfs[threadIdx.x] = (float)(eps.y * G.inv_scale[threadIdx.x]);
     }
+    cpa_wait<0>();
     __syncthreads();
-    JvcConst k;
+    float ev[4];
 #pragma unroll
-    for (int f = 0; f < 4; ++f) k.ev[f] = evs[f];
-    k.idx = G.f32.inv_dx;
-    k.idz = G.f32.inv_dz;
-    k.cs2 = G.f32.cs2;
-    k.iPr = G.f32.inv_Pr;
-    k.KM = G.f32.K_M;
-    k.KH = G.f32.K_H;
-    k.cm = G.f32.dd_cm;
-    k.cM = G.f32.dd_cM;
-    k.cl = G.f32.dd_cl;
-    k.dlt = G.f32.dd_delta;
-    k.ah = G.f32.dd_ah;
-    k.az = G.f32.dd_az;
-    const float tdt = G.f32.two_over_dt;
-    const int col = threadIdx.x % TX, r0 = (threadIdx.x / TX) * PPT;
-    for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
-        const int x0 = (t % ntx) * TX, z0 = (t / ntx) * TZ;
-        float* sa = stg + (NBUF == 2 ? (it & 1) * SH::STG : 0);
-        if (NBUF == 2) {
-            // double buffer: the next tile's copies go out before this tile is computed
-            const int tn = t + gridDim.x;
-            if (tn < ntiles)
-                jv_stage_issue(stg + ((it + 1) & 1) * SH::STG, u, v, G, (tn % ntx) * TX, (tn / ntx) * TZ, SX,
-                               SH::SZ);
-            cpa_commit();
-            cpa_wait<1>();
-        } else {
-            cpa_wait<0>();
-        }
-        __syncthreads();
-        if (z0 - HALO < 0 || z0 + TZ + HALO > G.nz) {
-            // mirror signs of the ghost rows (u and v planes alike)
-            for (int e = threadIdx.x; e < SH::SZ * SX; e += blockDim.x) {
-                const int iz = e / SX;
-                int side;
-                const int sz = mirror_z(z0 + iz - HALO, G.nz, side);
-                if (side == 0 || sz < 0 || sz >= G.nz) continue;
+    for (int f = 0; f < 4; ++f) ev[f] = evs[f];
+    if (z0 - HALO < 0 || z0 + TZ + HALO > G.nz) {        // ghost rows: signs of the odd fields
+        for (int j = threadIdx.x; j < PLANE; j += NT) {
+            int side;
+            mirror_z(z0 + j / SX - HALO, G.nz, side);
 #pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    const float sg = side == 1 ? (float)G.pb[f] : (float)G.pt[f];
-                    if (sg != 1.f) {
-                        sa[f * PLANE + e] *= sg;
-                        sa[(4 + f) * PLANE + e] *= sg;
-                    }
+            for (int f = 0; f < 4; ++f)
+                if (odd_ghost(G, f, side)) {
+                    st[f * PLANE + j] = flip(st[f * PLANE + j]);
+                    st[(4 + f) * PLANE + j] = flip(st[(4 + f) * PLANE + j]);
                 }
-            }
-            __syncthreads();
-        }
-        // phase 2a: this thread's points (fluxes of every kind, S and the raw direction)
-        float Sv[PPT][4], Vc[PPT][4];
-#pragma unroll
-        for (int q = 0; q < PPT; ++q) {
-            const int iz = r0 + q;
-            const int i = (iz + HALO) * SX + col + HALO;
-            const int is = SMAG ? (jvc_smag_row(iz, z0, G.nz) + HALO) * SX + col + HALO : i;
-            float P[4], Fx[3], Q[4], Fz[3];
-            jvc_point<SMAG, true, true, true, SX, PLANE>(sa, i, is, k, G, P, Fx, Q, Fz, Sv[q], Vc[q]);
-            const int ip = iz * PXW + col + R, iq = (iz + R) * TX + col;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) { PX[f * PXN + ip] = P[f]; QZ[f * QZN + iq] = Q[f]; }
-#pragma unroll
-            for (int f = 0; f < 3; ++f) { FX[f * PXN + ip] = Fx[f]; FZ[f * QZN + iq] = Fz[f]; }
-        }
-        // phase 2b: the arms -- z-fluxes of rows -2, -1, TZ, TZ+1; x-fluxes of columns -2, -1, TX, TX+1
-        for (int w = threadIdx.x; w < SH::NARM; w += blockDim.x) {
-            float P[4], Fx[3], Q[4], Fz[3], S_[4], V_[4];
-            if (w < 4 * TX) {
-                const int a = w / TX, cx = w - a * TX;
-                const int iz = a < 2 ? a - 2 : TZ + a - 2;
-                const int i = (iz + HALO) * SX + cx + HALO;
-                const int is = SMAG ? (jvc_smag_row(iz, z0, G.nz) + HALO) * SX + cx + HALO : i;
-                jvc_point<SMAG, false, true, false, SX, PLANE>(sa, i, is, k, G, P, Fx, Q, Fz, S_, V_);
-                const int iq = (iz + R) * TX + cx;
-#pragma unroll
-                for (int f = 0; f < 4; ++f) QZ[f * QZN + iq] = Q[f];
-#pragma unroll
-                for (int f = 0; f < 3; ++f) FZ[f * QZN + iq] = Fz[f];
-            } else {
-                const int w2 = w - 4 * TX;
-                const int a = w2 / TZ, iz = w2 - a * TZ;
-                const int cx = a < 2 ? a - 2 : TX + a - 2;
-                const int i = (iz + HALO) * SX + cx + HALO;
-                const int is = SMAG ? (jvc_smag_row(iz, z0, G.nz) + HALO) * SX + cx + HALO : i;
-                jvc_point<SMAG, true, false, false, SX, PLANE>(sa, i, is, k, G, P, Fx, Q, Fz, S_, V_);
-                const int ip = iz * PXW + cx + R;
-#pragma unroll
-                for (int f = 0; f < 4; ++f) PX[f * PXN + ip] = P[f];
-#pragma unroll
-                for (int f = 0; f < 3; ++f) FX[f * PXN + ip] = Fx[f];
-            }
         }
         __syncthreads();
-        if (NBUF == 1) {
-            // single buffer: the staged planes are dead now; the next tile's copies
-            // land while this one's fluxes are differentiated
-            const int tn = t + gridDim.x;
-            if (tn < ntiles) jv_stage_issue(stg, u, v, G, (tn % ntx) * TX, (tn / ntx) * TZ, SX, SH::SZ);
-            cpa_commit();
-        }
-        // phase 3: differentiate the fluxes, add S, write J v = 2 v / dt - dF / (eps scale_f)
-#pragma unroll
-        for (int q = 0; q < PPT; ++q) {
-            const int iz = r0 + q;
-            const int gz = z0 + iz, gx = x0 + col;
-            if (gz >= G.nz || gx >= G.nx) continue;
-            const int ip = iz * PXW + col + R, iq = (iz + R) * TX + col;
-            const size_t o = (size_t)gz * G.nx + gx;
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                const float conv = __fadd_rn(ddf(PX + f * PXN, ip, 1, G.f32.wx1, G.f32.wx2),
-                                             ddf(QZ + f * QZN, iq, TX, G.f32.wz1, G.f32.wz2));
-                float dF = __fmaf_rn(-0.5f, conv, Sv[q][f]);
-                if (f < 3)
-                    dF = __fadd_rn(dF, __fadd_rn(ddf(FX + f * PXN, ip, 1, G.f32.wx1, G.f32.wx2),
-                                                 ddf(FZ + f * QZN, iq, TX, G.f32.wz1, G.f32.wz2)));
-                out[(size_t)f * G.npt + o] = __fmaf_rn(tdt, Vc[q][f], __fmul_rn(-cfs[f], dF));
-            }
-        }
-        __syncthreads();     // staging buffer and flux arrays are reused by the next tile
     }
+    auto eddy_index = [&](int iz, int ix) {              // staged index of the point whose eddy value (iz, ix) takes
+        return (flux_eddy_row(iz, z0, G.nz) + HALO) * SX + ix + HALO;
+    };
+    const int tx = (threadIdx.x % SH::NXT) * W, tz = threadIdx.x / SH::NXT;
+    float S[4][W];
+    if (x0 + tx <= G.nx + 1 && z0 + tz <= G.nz + 1) {    // else it feeds no output
+        const int i = (tz + HALO) * SX + tx + HALO;
+        jv_points<W, SMAG, true, true, SX, PLANE, XN, ZN>(G, ev, st, i, SMAG ? eddy_index(tz, tx) : i,
+                                                          X + tz * SX + tx + HALO, Z + (tz + R) * TX + tx, S);
+    }
+    // the arms: Z of rows -2, -1, TZ, TZ+1 (W points an item), X of columns -2, -1, TX, TX+1
+    for (int w = threadIdx.x; w < SH::ZARM + SH::XARM; w += NT) {
+        if (w < SH::ZARM) {
+            const int a = w / SH::NXT, ix = (w % SH::NXT) * W, iz = a < 2 ? a - 2 : TZ + a - 2;
+            if (x0 + ix > G.nx + 1 || z0 + iz > G.nz + 1) continue;
+            const int i = (iz + HALO) * SX + ix + HALO;
+            float none[4][W];
+            jv_points<W, SMAG, false, true, SX, PLANE, XN, ZN>(G, ev, st, i, SMAG ? eddy_index(iz, ix) : i, X,
+                                                               Z + (iz + R) * TX + ix, none);
+        } else {
+            const int a = (w - SH::ZARM) & 3, iz = (w - SH::ZARM) >> 2, ix = a < 2 ? a - 2 : TX + a - 2;
+            if (x0 + ix > G.nx + 1 || z0 + iz > G.nz + 1) continue;
+            const int i = (iz + HALO) * SX + ix + HALO;
+            float none[4][1];
+            jv_points<1, SMAG, true, false, SX, PLANE, XN, ZN>(G, ev, st, i, SMAG ? eddy_index(iz, ix) : i,
+                                                               X + iz * SX + ix + HALO, Z, none);
+        }
+    }
+    __syncthreads();
+    if (x0 + tx < G.nx && z0 + tz < G.nz) {
+        const float wx1 = G.f32.wx1, wx2 = G.f32.wx2, wz1 = G.f32.wz1, wz2 = G.f32.wz2;
+        const size_t o = (size_t)(z0 + tz) * G.nx + x0 + tx;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            float dx[W], dz[W], vc[W], r[W];
+            jv_dx<W>(X + f * XN, tz * SX + tx + HALO, wx1, wx2, dx);
+            jv_dz<W>(Z + f * ZN, (tz + R) * TX + tx, TX, wz1, wz2, dz);
+            rload<float, W>(st + (4 + f) * PLANE + (tz + HALO) * SX + tx + HALO, vc);
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                const float dF = __fadd_rn(S[f][k], __fadd_rn(dx[k], dz[k]));
+                r[k] = __fmaf_rn(G.f32.two_over_dt, vc[k], __fmul_rn(-cfs[f], dF));
+            }
+            rstore<float, W>(out + f * np + o, r);
+        }
+    }
+    pdl_trigger();
 }
 
 // ============================================================================
@@ -966,27 +957,6 @@ __global__ void pc_setup(Geo G, int sweeps, Ctl* ctl) {
         put(k, degenerate ? 0.0 : rho_new * rho, rho_new * two_over_delta);
         rho = rho_new;
     }
-}
-
-// Row vectors: a thread of the float32 sweeps and of the Schur-complement kernels
-// owns W consecutive points along x (16 bytes where nx allows it).
-template <typename T, int W> struct RowVec { using type = typename Vec16<T>::type; };
-template <typename T> struct RowVec<T, 1> { using type = T; };
-template <> struct RowVec<float, 2> { using type = float2; };
-template <typename T, int W>
-__device__ __forceinline__ void rload(const T* p, T (&v)[W]) {
-    *reinterpret_cast<typename RowVec<T, W>::type*>(v) = *reinterpret_cast<const typename RowVec<T, W>::type*>(p);
-}
-template <typename T, int W>
-__device__ __forceinline__ void rstore(T* p, const T (&v)[W]) {
-    *reinterpret_cast<typename RowVec<T, W>::type*>(p) = *reinterpret_cast<const typename RowVec<T, W>::type*>(v);
-}
-
-// Asynchronous copy of W elements (16, 8 or 4 bytes) into shared memory.
-template <typename T, int W>
-__device__ __forceinline__ void cpa_vec(T* dst, const T* src) {
-    if constexpr (W * sizeof(T) == 16) cpa16(dst, src, 16);
-    else cpa_elem<W * (int)sizeof(T)>(dst, src, W * (int)sizeof(T));
 }
 
 // ----------------------------------------------------------------------------
@@ -1689,49 +1659,39 @@ template cudaError_t launch_stencil<float>(int, const Geo&, const float*, const 
 template cudaError_t launch_stencil<double>(int, const Geo&, const double*, const double*, const double*,
                                             const double*, double*, double*, double*, Ctl*, int, cudaStream_t);
 
-// float32: the compute-once kernel jvc2d, persistent (one CTA per resident
-// slot, capped at the tile count), double-buffered staging.
-template <int SMAG, int TX, int TZ, int NBUF>
-static cudaError_t launch_jvc_t(const Geo& G, const float* u, const float* v, float* out, const double* part,
-                                Ctl* ctl, int check_done, cudaStream_t s) {
-    static std::atomic<int> slots{0};   // resident CTAs on the device; set once (races are benign)
-    const size_t sm = JvcShape<TX, TZ>::smem(NBUF);
-    if (slots.load() == 0) {
-        cudaError_t e = set_smem(jvc2d<SMAG, TX, TZ, NBUF>, sm);
+template <int W, int NT, int SMAG>
+static cudaError_t launch_jv_t(const Geo& G, const float* u, const float* v, float* out, const double* part, Ctl* ctl,
+                               int check_done, cudaStream_t s) {
+    using SH = JvShape<W, NT>;
+    static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
+    if (!configured) {
+        const cudaError_t e = set_smem(jv2d<W, NT, SMAG>, SH::smem);
         if (e != cudaSuccess) return e;
-        int dev = 0, nsm = 0, per = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-            (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jvc2d<SMAG, TX, TZ, NBUF>, NTHREADS, sm)) !=
-                cudaSuccess)
-            return e;
-        slots = std::max(1, nsm * per);
+        configured = true;
     }
-    const int ntiles = ((G.nx + TX - 1) / TX) * ((G.nz + TZ - 1) / TZ);
-    const int grid = std::min(ntiles, slots.load());
-    return launch_pdl(jvc2d<SMAG, TX, TZ, NBUF>, dim3(grid), NTHREADS, sm, s, G, u, v, out, part, ctl, check_done);
+    return launch_pdl(jv2d<W, NT, SMAG>, dim3((G.nx + SH::TX - 1) / SH::TX, (G.nz + SH::TZ - 1) / SH::TZ), dim3(NT),
+                      SH::smem, s, G, u, v, out, part, ctl, check_done);
 }
 
+// Rows of 16-byte, 8-byte or single-element vectors as nx allows (u and v are
+// workspace vectors: their planes start multiples of npt elements in); 256 or 128
+// threads a CTA by Geo::tile_jv, 256 for tile_jv = 0.
 template <int SMAG>
-static cudaError_t launch_jvc_tile(const Geo& G, const float* u, const float* v, float* out, const double* part,
-                                   Ctl* ctl, int check_done, cudaStream_t s) {
-#define JF_JVC(I) launch_jvc_t<SMAG, JvcTile<I>::TX, JvcTile<I>::TZ, JvcTile<I>::NBUF>(G, u, v, out, part, ctl, \
-                                                                                     check_done, s)
-    switch (G.tile_jv) {
-        case 1: return JF_JVC(1);
-        case 2: return JF_JVC(2);
-        case 3: return JF_JVC(3);
-        default: return JF_JVC(0);
-    }
-#undef JF_JVC
+static cudaError_t launch_jv(const Geo& G, const float* u, const float* v, float* out, const double* part, Ctl* ctl,
+                             int check_done, cudaStream_t s) {
+    const bool small = G.tile_jv == 2;
+#define JF_JV(W) (small ? launch_jv_t<W, 128, SMAG>(G, u, v, out, part, ctl, check_done, s) \
+                        : launch_jv_t<W, 256, SMAG>(G, u, v, out, part, ctl, check_done, s))
+    return G.nx % 4 == 0 ? JF_JV(4) : G.nx % 2 == 0 ? JF_JV(2) : JF_JV(1);
+#undef JF_JV
 }
 
 cudaError_t launch_jv_diff(const Geo& G, const float* u, const float* v, float* out, double* part, Ctl* ctl,
                            int check_done, cudaStream_t s) {
     if (G.dim == 3) return launch_jv_diff3d(G, u, v, out, ctl, check_done, s);
-    if (G.sgs == 2) return launch_jvc_tile<2>(G, u, v, out, part, ctl, check_done, s);
-    return G.smag ? launch_jvc_tile<1>(G, u, v, out, part, ctl, check_done, s)
-                  : launch_jvc_tile<0>(G, u, v, out, part, ctl, check_done, s);
+    if (G.sgs == 2) return launch_jv<2>(G, u, v, out, part, ctl, check_done, s);
+    return G.smag ? launch_jv<1>(G, u, v, out, part, ctl, check_done, s)
+                  : launch_jv<0>(G, u, v, out, part, ctl, check_done, s);
 }
 
 static int stream_blocks(size_t n) {

@@ -867,7 +867,7 @@ static jfnk_status fused_step(jfnk_handle* h, const T* uT, bool learned, bool ar
         kt_end(h, JFNK_KF_ARNOLDI_A, 2 * vb);
     } else {
         CK(launch_arnoldi_ca<T>(V, ld, wb[(j - 1) & 1], wj, n, j, m, h->partB, h->part, h->ctl, s));
-        nblkA = arnoldi_ca_parts<T>(n);
+        nblkA = arnoldi_ca_parts<T>(n, j);
         kt_end(h, JFNK_KF_ARNOLDI_A, (j + 3) * vb);   // reads v_0..v_{j-1}, w'_{j-1}, w_j; writes v_j
     }
     kt_begin(h, JFNK_KF_ARNOLDI_B);

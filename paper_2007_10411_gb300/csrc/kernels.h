@@ -68,12 +68,12 @@ cudaError_t launch_arnoldi_c(T* V, size_t ldv, const T* w, size_t n, int nv, int
 // Right-preconditioned path, lagged second projection: pass CA of step j
 // forms v_j from w'_{j-1} (wprev) and pass B's partials of step j-1, runs the
 // Givens update of column j-1, and leaves h1 = [v_0..v_j]^T w_j as partials of
-// arnoldi_ca_parts(n) blocks for launch_arnoldi_b_from.
+// arnoldi_ca_parts(n, j) blocks for launch_arnoldi_b_from.
 template <typename T>
 cudaError_t launch_arnoldi_ca(T* V, size_t ldv, const T* wprev, const T* w, size_t n, int j, int m,
                               const double* partB, double* partA, Ctl* ctl, cudaStream_t s);
 template <typename T>
-int arnoldi_ca_parts(size_t n);
+int arnoldi_ca_parts(size_t n, int j);
 template <typename T>
 cudaError_t launch_arnoldi_b_from(const T* V, size_t ldv, T* w, size_t n, int nv, const double* partA, int nblkA,
                                   double* partB, Ctl* ctl, cudaStream_t s);

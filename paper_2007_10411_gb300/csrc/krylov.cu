@@ -438,6 +438,19 @@ template <> __device__ __forceinline__ double2 zerov<double2>() { return make_do
 template <> __device__ __forceinline__ float zerov<float>() { return 0.f; }
 template <> __device__ __forceinline__ double zerov<double>() { return 0.0; }
 
+// Lanes per element of passes B and CA: float32 one up to NV = 16, two above;
+// float64 one always.  A float64 FMA occupies a sub-partition's pipe for 64
+// cycles, so what a pass costs is its FMAs (2 per basis entry) and everything a
+// split adds: with four lanes an element the shuffled sums and the padding of
+// the instantiation were a third of the arithmetic (381 us at nv = 28,
+// 1024 x 512, for 183 us of FMAs).  One lane keeps all entries (up to 32 double2
+// and their sums: one CTA per SM above NV = 16, 8 warps of 32 loads each in
+// flight) and skips the empty ones four at a time (SKIP): 222 us at nv = 28,
+// 175 against 270 at 17 .. 24, 130 against 192 at 13 .. 16.
+template <typename T, int NV> constexpr int LANES = sizeof(T) == sizeof(double) || NV <= 16 ? 1 : 2;
+template <typename T, int NV> constexpr int MIN_CTAS = sizeof(T) == sizeof(double) && NV > 16 ? 1 : 2;
+template <typename T> constexpr bool SKIP = sizeof(T) == sizeof(double);
+
 // Pass B loads of one element (a VT vector of W entries, or a scalar in the
 // tail) for lane q of its group, which owns basis vectors q*CH .. q*CH+CH-1.
 template <typename T, typename VT, int CH>
@@ -452,17 +465,23 @@ __device__ __forceinline__ void load_b(const T* __restrict__ V, size_t ldv, size
 // Pass B arithmetic of one element: the group's partial sums of V h1 meet by
 // shuffles, w' = w - V h1 is stored by lane 0, every lane dots its vectors with w'.
 template <typename T, typename VT, int CH, int KS>
-__device__ __forceinline__ void work_b(const VT (&v)[CH], VT wv, T* __restrict__ w, size_t i, int q, const T* h1s,
+__device__ __forceinline__ void work_b(const VT (&v)[CH], VT wv, T* __restrict__ w, size_t i, int nv, int q, const T* h1s,
                                        T (&acc)[CH], T& accn) {
     VT sum = zerov<VT>();
 #pragma unroll
-    for (int c = 0; c < CH; ++c) sum = fmav(h1s[q * CH + c], v[c], sum);
+    for (int c4 = 0; c4 < CH; c4 += 4)
+        if (!SKIP<T> || c4 < nv)
+#pragma unroll
+            for (int c = c4; c < c4 + 4; ++c) sum = fmav(h1s[q * CH + c], v[c], sum);
     const unsigned mask = __activemask();     // the KS lanes of a group are active together
 #pragma unroll
     for (int o = 1; o < KS; o <<= 1) sum = addv(sum, shfl_xor_v(mask, sum, o));
     const VT wp = subv(wv, sum);
 #pragma unroll
-    for (int c = 0; c < CH; ++c) acc[c] = dotacc(v[c], wp, acc[c]);
+    for (int c4 = 0; c4 < CH; c4 += 4)
+        if (!SKIP<T> || c4 < nv)
+#pragma unroll
+            for (int c = c4; c < c4 + 4; ++c) acc[c] = dotacc(v[c], wp, acc[c]);
     if (q == 0) {
         accn = dotacc(wp, wp, accn);
         reinterpret_cast<VT*>(w)[i] = wp;
@@ -476,22 +495,20 @@ __device__ __forceinline__ void work_b(const VT (&v)[CH], VT wv, T* __restrict__
 // with at most eight entries per lane the next element's loads are issued
 // before the current one is combined (software pipeline).
 template <typename T, int NV>
-__global__ void __launch_bounds__(NTHREADS, 2)
+__global__ void __launch_bounds__(NTHREADS, MIN_CTAS<T, NV>)
 arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int nv,
           const double* partA, int nblkA, double* part, Ctl* ctl, int jscale) {
     pdl_wait();
     const int done = ctl->done;     // no writer during this launch; read beside the partials
     // jscale >= 0: w is used as zscale[jscale] w (lagged second projection, see arnoldi_ca)
     const T sig = jscale >= 0 ? T(ctl->zscale[jscale]) : T(1);
-    // one lane per element up to NV = 16, two above (four for a float64 basis at
-    // NV = 32, where two would not fit the registers): a lane keeps up to sixteen
-    // loads in flight, and the instantiation nearest above nv (8, 12, 16, 24, 32)
-    // leaves few of its entries empty
-    constexpr int KS = NV <= 16 ? 1 : ((sizeof(T) == sizeof(double) && NV > 24) ? 4 : 2), CH = NV / KS;
+    // a lane keeps up to sixteen (float64: thirty-two) loads in flight, and the
+    // instantiation nearest above nv (8, 12, 16, 24, 32) leaves few entries empty
+    constexpr int KS = LANES<T, NV>, CH = NV / KS;
     // the next element's loads are issued ahead (software pipeline) where the
     // registers allow it; twelve or more entries per lane are deep enough without
     constexpr bool PF = CH <= 8;
-    static_assert(CH * KS == NV && CH <= 16, "lane split");
+    static_assert(CH * KS == NV && CH % 4 == 0, "lane split");
     __shared__ double h1d[NV];
     __shared__ T h1s[NV];
     __shared__ T red[NV + 1][NTHREADS / 32];
@@ -517,7 +534,7 @@ arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int 
             const size_t i = wk.at(cc);
             VT v[CH];
             load_b<T, VT, CH>(V, ldv, i, nv, q, v);
-            work_b<T, VT, CH, KS>(v, scalev(reinterpret_cast<const VT*>(w)[i], sig), w, i, q, h1s, acc, accn);
+            work_b<T, VT, CH, KS>(v, scalev(reinterpret_cast<const VT*>(w)[i], sig), w, i, nv, q, h1s, acc, accn);
         }
     } else {
         VT vn[CH], wn = zerov<VT>();
@@ -536,13 +553,13 @@ arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int 
                 load_b<T, VT, CH>(V, ldv, inext, nv, q, vn);
                 wn = scalev(reinterpret_cast<const VT*>(w)[inext], sig);
             }
-            work_b<T, VT, CH, KS>(v, wv, w, i, q, h1s, acc, accn);
+            work_b<T, VT, CH, KS>(v, wv, w, i, nv, q, h1s, acc, accn);
         }
     }
     for (size_t i = nvec * W + g0; i < n; i += gstride) {
         T v[CH];
         load_b<T, T, CH>(V, ldv, i, nv, q, v);
-        work_b<T, T, CH, KS>(v, sig * w[i], w, i, q, h1s, acc, accn);
+        work_b<T, T, CH, KS>(v, sig * w[i], w, i, nv, q, h1s, acc, accn);
     }
     pdl_trigger();
     // block sums: slot 0 = ||w'||^2, slot 1 + k = v_k . w' (fixed shuffle trees, then the partial type across warps)
@@ -654,7 +671,7 @@ arnoldi_c(T* __restrict__ V, size_t ldv, const T* __restrict__ w, size_t n, int 
 // once; block 0 runs the Hessenberg / Givens update of column j-1 (as pass
 // C's block 0 does).  Partials (j + 1 values) are indexed by streaming block.
 template <typename T, int NV>
-__global__ void __launch_bounds__(NTHREADS, 2)
+__global__ void __launch_bounds__(NTHREADS, MIN_CTAS<T, NV>)
 arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* __restrict__ w, size_t n,
            int j, int m, const double* partB, int nblkB, double* partA, Ctl* ctl) {
     pdl_wait();
@@ -693,11 +710,10 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
     __syncthreads();
     const T inv = inv_s;
     const T sig = sig_s;
-    // KS lanes per element (one up to NV = 16, two above; four for a float64
-    // basis at NV = 32): a lane loads all its basis entries before it combines
+    // KS lanes per element: a lane loads all its basis entries before it combines
     // them, so that they are in flight together; the lanes' parts of V h2 meet
     // by shuffles and lane 0 stores v_j
-    constexpr int KS = NV <= 16 ? 1 : ((sizeof(T) == sizeof(double) && NV > 24) ? 4 : 2), CH = NV / KS;
+    constexpr int KS = LANES<T, NV>, CH = NV / KS;
     const int q = threadIdx.x & (KS - 1);
     T acc[CH];
 #pragma unroll
@@ -721,10 +737,13 @@ arnoldi_ca(T* __restrict__ V, size_t ldv, const T* __restrict__ wprev, const T* 
         const VT wv = scalev(reinterpret_cast<const VT*>(w)[i], sig);
         VT sum = zerov<VT>();
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            sum = fmav(hs[q * CH + c], v[c], sum);
-            acc[c] = dotacc(v[c], wv, acc[c]);
-        }
+        for (int c4 = 0; c4 < CH; c4 += 4)
+            if (!SKIP<T> || c4 < j)
+#pragma unroll
+                for (int c = c4; c < c4 + 4; ++c) {
+                    sum = fmav(hs[q * CH + c], v[c], sum);
+                    acc[c] = dotacc(v[c], wv, acc[c]);
+                }
         if (KS > 1) {
             const unsigned mask = __activemask();     // the KS lanes of an element are active together
 #pragma unroll
@@ -1154,7 +1173,12 @@ pc_eps_k(const float* __restrict__ z, size_t n, double* part, Ctl* ctl) {
 template <typename T> static int grid_a(size_t n) {
     return std::max(dot_blocks(n / V4<T>::W), reduce_blocks(n / V4<T>::W));
 }
-template <typename T> static int grid_b(size_t n) { return reduce_blocks(n / V4<T>::W); }
+// Pass B and CA above 16 float64 vectors hold one CTA per SM (MIN_CTAS).
+template <typename T> static bool one_per_sm(int nv) { return sizeof(T) == sizeof(double) && nv > 16; }
+template <typename T> static int grid_b(size_t n, int nv) {
+    const int b = reduce_blocks(n / V4<T>::W);
+    return one_per_sm<T>(nv) ? std::min(b, 152) : b;
+}
 template <typename T> static int grid_c(size_t n) {
     return std::min(dot_blocks(n / V4<T>::W) + 1, MAX_DOT_BLOCKS);
 }
@@ -1178,7 +1202,7 @@ cudaError_t launch_arnoldi_a(const T* V, size_t ldv, const T* w, size_t n, int n
 template <typename T>
 cudaError_t launch_arnoldi_b(const T* V, size_t ldv, T* w, size_t n, int nv, const double* partA,
                              double* partB, Ctl* ctl, cudaStream_t s) {
-    const int nb = grid_b<T>(n), na = grid_a<T>(n);
+    const int nb = grid_b<T>(n, nv), na = grid_a<T>(n);
     if (nv <= 8) return launch_pdl(arnoldi_b<T, 8>, nb, NTHREADS, 0, s, V, ldv, w, n, nv, partA, na, partB, ctl, -1);
     if (nv <= 12) return launch_pdl(arnoldi_b<T, 12>, nb, NTHREADS, 0, s, V, ldv, w, n, nv, partA, na, partB, ctl, -1);
     if (nv <= 16) return launch_pdl(arnoldi_b<T, 16>, nb, NTHREADS, 0, s, V, ldv, w, n, nv, partA, na, partB, ctl, -1);
@@ -1189,7 +1213,7 @@ cudaError_t launch_arnoldi_b(const T* V, size_t ldv, T* w, size_t n, int nv, con
 template <typename T>
 cudaError_t launch_arnoldi_c(T* V, size_t ldv, const T* w, size_t n, int nv, int m, const double* partB,
                              Ctl* ctl, cudaStream_t s) {
-    const int nc = grid_c<T>(n), nb = grid_b<T>(n);
+    const int nc = grid_c<T>(n), nb = grid_b<T>(n, nv);
     if (nv <= 8) return launch_pdl(arnoldi_c<T, 8>, nc, NTHREADS, 0, s, V, ldv, w, n, nv, m, partB, nb, ctl);
     if (nv <= 16) return launch_pdl(arnoldi_c<T, 16>, nc, NTHREADS, 0, s, V, ldv, w, n, nv, m, partB, nb, ctl);
     return launch_pdl(arnoldi_c<T, 32>, nc, NTHREADS, 0, s, V, ldv, w, n, nv, m, partB, nb, ctl);
@@ -1200,20 +1224,20 @@ cudaError_t launch_arnoldi_c(T* V, size_t ldv, const T* w, size_t n, int nv, int
 // Two CTAs per SM are resident (register use): the Givens block and the
 // streaming blocks fit one wave.
 constexpr int MAX_CA_BLOCKS = 2 * 152;
-template <typename T> static int grid_ca(size_t n) {
-    return std::min(dot_blocks(n / V4<T>::W), MAX_CA_BLOCKS - 1) + 1;
+template <typename T> static int grid_ca(size_t n, int j) {
+    return std::min(dot_blocks(n / V4<T>::W), (one_per_sm<T>(j + 1) ? 152 : MAX_CA_BLOCKS) - 1) + 1;
 }
 template <typename T>
-int arnoldi_ca_parts(size_t n) {
-    return grid_ca<T>(n) - 1;
+int arnoldi_ca_parts(size_t n, int j) {
+    return grid_ca<T>(n, j) - 1;
 }
-template int arnoldi_ca_parts<float>(size_t);
-template int arnoldi_ca_parts<double>(size_t);
+template int arnoldi_ca_parts<float>(size_t, int);
+template int arnoldi_ca_parts<double>(size_t, int);
 
 template <typename T>
 cudaError_t launch_arnoldi_ca(T* V, size_t ldv, const T* wprev, const T* w, size_t n, int j, int m,
                               const double* partB, double* partA, Ctl* ctl, cudaStream_t s) {
-    const int nc = grid_ca<T>(n), nb = grid_b<T>(n);
+    const int nc = grid_ca<T>(n, j), nb = grid_b<T>(n, j);     // pass B of step j - 1 ran over j vectors
     if (j + 1 <= 8)
         return launch_pdl(arnoldi_ca<T, 8>, nc, NTHREADS, 0, s, V, ldv, wprev, w, n, j, m, partB, nb, partA, ctl);
     if (j + 1 <= 12)
@@ -1233,7 +1257,7 @@ template cudaError_t launch_arnoldi_ca<double>(double*, size_t, const double*, c
 template <typename T>
 cudaError_t launch_arnoldi_b_from(const T* V, size_t ldv, T* w, size_t n, int nv, const double* partA, int nblkA,
                                   double* partB, Ctl* ctl, cudaStream_t s) {
-    const int nb = grid_b<T>(n);
+    const int nb = grid_b<T>(n, nv);
     const int js = nv > 1 ? nv - 1 : -1;    // step j = nv - 1 >= 1 follows pass CA: w is scaled
     if (nv <= 8) return launch_pdl(arnoldi_b<T, 8>, nb, NTHREADS, 0, s, V, ldv, w, n, nv, partA, nblkA, partB, ctl, js);
     if (nv <= 12) return launch_pdl(arnoldi_b<T, 12>, nb, NTHREADS, 0, s, V, ldv, w, n, nv, partA, nblkA, partB, ctl, js);
@@ -1250,7 +1274,7 @@ template cudaError_t launch_arnoldi_b_from<double>(const double*, size_t, double
 // with its Givens block and no streaming blocks), after pass B of step nv - 1.
 template <typename T>
 cudaError_t launch_arnoldi_givens(size_t n, int nv, int m, const double* partB, Ctl* ctl, cudaStream_t s) {
-    const int nb = grid_b<T>(n);
+    const int nb = grid_b<T>(n, nv);
     T* none = nullptr;
     if (nv <= 8) return launch_pdl(arnoldi_c<T, 8>, 1, NTHREADS, 0, s, none, (size_t)0, (const T*)none, n, nv, m, partB, nb, ctl);
     if (nv <= 16) return launch_pdl(arnoldi_c<T, 16>, 1, NTHREADS, 0, s, none, (size_t)0, (const T*)none, n, nv, m, partB, nb, ctl);

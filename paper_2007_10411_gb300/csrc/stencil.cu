@@ -971,13 +971,15 @@ __global__ void pc_setup(Geo G, int sweeps, Ctl* ctl) {
 //
 // Bound: latency of the one load phase and issue (23 MB a launch at
 // 1024 x 512, 3.4 us).  One field per CTA with three barriers and the fluxes in
-// shared memory took 19-20 us there and 7.1-7.8 us at 250 x 119; this form 12.0 and 4.4 us (with
-// the overlap of the launches before it).
+// shared memory took 19-20 us there and 7.1-7.8 us at 250 x 119; this form 11.2 and 4.4 us (with
+// the overlap of the launches before it; 12.0 us at 1024 x 512 with the first
+// field's loads hoisted over the loop and 72 registers, three CTAs per SM: 1024
+// threads an SM need 64).
 // ----------------------------------------------------------------------------
 template <int W> struct PcRow { static constexpr int NXT = W == 4 ? 16 : 32; };   // threads along x
 
 template <int W, int NT, int SMAG>
-__global__ void __launch_bounds__(NT, 768 / NT)
+__global__ void __launch_bounds__(NT, 1024 / NT)
 cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const float* __restrict__ zin,
        const float* __restrict__ din, float* __restrict__ zout, float* __restrict__ dout, const float* __restrict__ nu,
        double* part, Ctl* ctl, int check_done) {
@@ -1008,17 +1010,8 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
     const int gx = x0 + tx, gz = z0 + tz;
     const bool inside = gx < G.nx && gz < G.nz;
     const size_t own = inside ? (size_t)gz * G.nx + gx : 0;
-    T rv[3][W], dv[3][W], pv[W];
-    if (inside && !done) {
-        if (!first) {
-#pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                rload<T, W>(r + f * np + own, rv[f]);
-                rload<T, W>(din + f * np + own, dv[f]);
-            }
-        }
-        if (last) rload<T, W>(r + 3 * np + own, pv);
-    }
+    T pv[W];
+    if (inside && !done && last) rload<T, W>(r + 3 * np + own, pv);
     cpa_wait<0>();
     if (done) return;
     __syncthreads();
@@ -1036,29 +1029,17 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
     if (inside) {
         const T wx1 = G.f32.wx1, wx2 = G.f32.wx2, wz1 = G.f32.wz1, wz2 = G.f32.wz2;
         const int me = (tz + HALO) * SX + tx + HALO, mk = (tz + R) * SX + tx + HALO;
-        T kx[W + 4], kz[4][W];                          // eddy values on the x and z arms
-        if (SMAG) {
-#pragma unroll
-            for (int i = 0; i < W + 4; i += 2) {
-                if constexpr (W == 1) {
-                    kx[i] = ks[mk - 2 + i];
-                    if (i + 1 < W + 4) kx[i + 1] = ks[mk - 1 + i];
-                } else {
-                    const float2 v = *reinterpret_cast<const float2*>(&ks[mk - 2 + i]);
-                    kx[i] = v.x;
-                    kx[i + 1] = v.y;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) rload<T, W>(&ks[mk + (q < 2 ? q - 2 : q - 1) * SX], kz[q]);
-        }
-#pragma unroll
+#pragma unroll 1
         for (int f = 0; f < 3; ++f) {
             const T ith = cheb_coef<T>(ctl, f, k, 0), a1 = cheb_coef<T>(ctl, f, k, 1), a2 = cheb_coef<T>(ctl, f, k, 2);
             const T* p = zs[f];
             // what the fluxes leave out: c_m, c_M (Deardorff), 1/Pr of theta, the constant K, 1/theta_c of x_1 = r / theta_c
             const T ks_ = SMAG == 2 ? T(1) : SMAG ? (f == 2 ? G.f32.inv_Pr : T(1)) : (f == 2 ? G.f32.K_H : G.f32.K_M);
-            T xk[W], e[W + 8], difx[W], difz[W];
+            T rv[W], dv[W], xk[W], e[W + 8], difx[W], difz[W];
+            if (!first) {
+                rload<T, W>(r + f * np + own, rv);
+                rload<T, W>(din + f * np + own, dv);
+            }
             if constexpr (W == 1) {
 #pragma unroll
                 for (int i = 0; i < 9; ++i) e[i] = p[me - 4 + i];
@@ -1072,7 +1053,20 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
                 }
             }
             {
-                T fx[W + 4];
+                T fx[W + 4], kx[W + 4];                 // kx: eddy values on the x arm
+                if (SMAG) {
+#pragma unroll
+                    for (int i = 0; i < W + 4; i += 2) {
+                        if constexpr (W == 1) {
+                            kx[i] = ks[mk - 2 + i];
+                            if (i + 1 < W + 4) kx[i + 1] = ks[mk - 1 + i];
+                        } else {
+                            const float2 v = *reinterpret_cast<const float2*>(&ks[mk - 2 + i]);
+                            kx[i] = v.x;
+                            kx[i + 1] = v.y;
+                        }
+                    }
+                }
 #pragma unroll
                 for (int i = 0; i < W + 4; ++i) {
                     const T d = rfma(wx1, e[i + 3] - e[i + 1], rmul(wx2, e[i + 4] - e[i]));
@@ -1083,10 +1077,14 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
                 for (int i = 0; i < W; ++i) difx[i] = rfma(wx1, fx[i + 3] - fx[i + 1], rmul(wx2, fx[i + 4] - fx[i]));
             }
             {
-                T v[9][W], fz[4][W];
+                T v[9][W], fz[4][W], kz[4][W];          // kz: eddy values on the z arm
 #pragma unroll
                 for (int q = 0; q < 9; ++q)
                     if (q != 4) rload<T, W>(p + me + (q - 4) * SX, v[q]);
+                if (SMAG) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) rload<T, W>(&ks[mk + (q < 2 ? q - 2 : q - 1) * SX], kz[q]);
+                }
 #pragma unroll
                 for (int i = 0; i < W; ++i) {
                     v[4][i] = e[4 + i];
@@ -1105,9 +1103,9 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
             for (int i = 0; i < W; ++i) {
                 const T sum = SMAG == 2 ? rfma(G.f32.dd_cm, difx[i], rmul(G.f32.dd_cM, difz[i])) : rmul(ks_, __fadd_rn(difx[i], difz[i]));
                 xk[i] = first ? rmul(ith, e[4 + i]) : e[4 + i];
-                const T rr = first ? e[4 + i] : rv[f][i];
+                const T rr = first ? e[4 + i] : rv[i];
                 const T res = __fsub_rn(rr, rfma(G.f32.two_over_dt, xk[i], -(first ? rmul(ith, sum) : sum)));
-                dk[i] = rfma(a1, first ? xk[i] : dv[f][i], rmul(a2, res));
+                dk[i] = rfma(a1, first ? xk[i] : dv[i], rmul(a2, res));
                 xo[i] = __fadd_rn(xk[i], dk[i]);
                 if (last) acc[0] = rfma(xo[i], xo[i], acc[0]);
             }
@@ -1675,7 +1673,8 @@ static cudaError_t launch_jv_t(const Geo& G, const float* u, const float* v, flo
 
 // Rows of 16-byte, 8-byte or single-element vectors as nx allows (u and v are
 // workspace vectors: their planes start multiples of npt elements in); 256 or 128
-// threads a CTA by Geo::tile_jv, 256 for tile_jv = 0.
+// threads a CTA by Geo::tile_jv, 256 for tile_jv = 0 (a step with 256 / 128 at
+// 1024 x 512: 52.9 / 57.1 ms, at 250 x 119: 3.91 / 4.01 ms: a smaller tile has more arms).
 template <int SMAG>
 static cudaError_t launch_jv(const Geo& G, const float* u, const float* v, float* out, const double* part, Ctl* ctl,
                              int check_done, cudaStream_t s) {
@@ -1744,7 +1743,9 @@ static cudaError_t launch_precond_w(const Geo& G, int sweeps, const float* r, fl
 // Rows of 16-byte, 8-byte or single-element vectors as nx allows (r and z of the
 // batched and per-call paths are workspace vectors: their planes start multiples
 // of npt elements in); 256, 128 or 64 threads a CTA by Geo::tile_pc, by the grid
-// for tile_pc = 0: the widest tile that leaves no SM without a CTA.
+// for tile_pc = 0: 256 where that leaves no SM without a CTA, else 128 (a step at
+// 1024 x 512 with 256 / 128 / 64: 52.9 / 53.6 / 55.5 ms, at 250 x 119: 3.83 /
+// 3.81 / 3.90 ms).
 template <int SMAG>
 static cudaError_t launch_precond_f32(const Geo& G, int sweeps, const float* r, float* z, float* za, float* zb, float* da,
                                       float* db, const float* nu, double* part, Ctl* ctl, int check_done,
@@ -1754,7 +1755,7 @@ static cudaError_t launch_precond_f32(const Geo& G, int sweeps, const float* r, 
     int nt = G.tile_pc == 1 ? 256 : (G.tile_pc == 2 ? 128 : 64);
     if (G.tile_pc == 0) {
         const long long vecs = (long long)((G.nx + w - 1) / w) * G.nz;       // threads with a point
-        nt = vecs >= 256LL * SMS ? 256 : (vecs >= 128LL * SMS ? 128 : 64);
+        nt = vecs >= 256LL * SMS ? 256 : 128;
     }
 #define JF_PC(W, NT) launch_precond_w<W, NT, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches)
 #define JF_PCW(W) (nt == 256 ? JF_PC(W, 256) : nt == 128 ? JF_PC(W, 128) : JF_PC(W, 64))

@@ -381,6 +381,101 @@ strain3d(Geo G, const T* __restrict__ u, const T* __restrict__ v, T* __restrict_
     }
 }
 
+// The difference form's strain pass in float32, two points along x per thread: no
+// shared memory and no barrier.  A thread reads its row's neighbours (x -+ 2, y -+ 1,
+// y -+ 2) as 8-byte pairs through the L1 and keeps its columns' z-2 .. z+2 in
+// registers; eps v enters as eps D(v).  For an even nx; strain3d above otherwise,
+// and in float64, where the FP64 pipe bounds the pass.
+// Bound: load latency and issue (134 MB, 20 us at 256 x 256 x 64): 67 -> 54 us there.
+__global__ void __launch_bounds__(NTHREADS, 2)
+strain3d_pairs(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __restrict__ s0,
+               float* __restrict__ s1, const Ctl* ctl, int check_done) {
+    if (check_done && ctl->done) return;
+    const int gx = (blockIdx.x * KX + threadIdx.x % KX) * 2, gy = blockIdx.y * KY + threadIdx.x / KX;
+    if (gx >= G.nx || gy >= G.ny) return;
+    const int z0 = blockIdx.z * SZB, z1 = min(z0 + SZB, G.nz);
+    const int nxy = G.ny * G.nx, own = gy * G.nx + gx;
+    const int xl = gy * G.nx + wrap(gx - 2, G.nx), xr = gy * G.nx + wrap(gx + 2, G.nx);
+    int yo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) yo[q] = wrap(gy + (q < 2 ? q - 2 : q - 1), G.ny) * G.nx + gx;
+    float ev[3];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) ev[f] = eps_field<float>(ctl, f);
+    auto pair = [&](int st, int f, int z, int o) {
+        return __ldg(reinterpret_cast<const float2*>((st ? v : u) + (size_t)f * G.npt + (size_t)z * nxy + o));
+    };
+    // mirror ghosts with each component's parity
+    auto col = [&](int st, int f, int z) {
+        int side;
+        const int sz = mirror(z, G.nz, side);
+        const float2 a = pair(st, f, sz, own);
+        const bool odd = (side == 1 && G.pb[f] < 0) || (side == 2 && G.pt[f] < 0);
+        return odd ? make_float2(flip(a.x), flip(a.y)) : a;
+    };
+    const float wx1 = G.f32.wx1, wx2 = G.f32.wx2, wy1 = G.f32.wy1, wy2 = G.f32.wy2, wz1 = G.f32.wz1, wz2 = G.f32.wz2;
+    float2 w[2][3][5];
+#pragma unroll
+    for (int st = 0; st < 2; ++st)
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[st][f][q] = col(st, f, z0 - 2 + q);
+    for (int z = z0; z < z1; ++z) {
+        float g[2][3][3][2];      // [u, eps v][component][axis][point]
+#pragma unroll
+        for (int st = 0; st < 2; ++st)
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                w[st][f][4] = col(st, f, z + 2);
+                const float2 l = pair(st, f, z, xl), r = pair(st, f, z, xr);
+                const float2 d2 = pair(st, f, z, yo[0]), d1 = pair(st, f, z, yo[1]);
+                const float2 u1 = pair(st, f, z, yo[2]), u2 = pair(st, f, z, yo[3]);
+                const float2(&c)[5] = w[st][f];
+                g[st][f][0][0] = wx1 * (c[2].y - l.y) + wx2 * (r.x - l.x);
+                g[st][f][0][1] = wx1 * (r.x - c[2].x) + wx2 * (r.y - l.y);
+                g[st][f][1][0] = wy1 * (u1.x - d1.x) + wy2 * (u2.x - d2.x);
+                g[st][f][1][1] = wy1 * (u1.y - d1.y) + wy2 * (u2.y - d2.y);
+                g[st][f][2][0] = wz1 * (c[3].x - c[1].x) + wz2 * (c[4].x - c[0].x);
+                g[st][f][2][1] = wz1 * (c[3].y - c[1].y) + wz2 * (c[4].y - c[0].y);
+                if (st)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        g[1][f][d][0] *= ev[f];
+                        g[1][f][d][1] *= ev[f];
+                    }
+            }
+        float sa[2], ds[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            float dA = 0.f, oA = 0.f, dD = 0.f, oD = 0.f;     // diagonal and off-diagonal sums of S:S, S':S' - S:S
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int j = (i + 1) % 3;
+                const float a = g[0][i][i][e], b = g[1][i][i][e];
+                const float ao = g[0][i][j][e] + g[0][j][i][e], bo = g[1][i][j][e] + g[1][j][i][e];
+                dA += a * a;
+                dD += (2.f * a + b) * b;
+                oA += ao * ao;
+                oD += (2.f * ao + bo) * bo;
+            }
+            const float q = 2.f * dA + oA, d = 2.f * dD + oD, t = q + d;     // 2 S:S and its difference
+            sa[e] = root(q);
+            const float den = sa[e] + root(t > 0.f ? t : 0.f);
+            ds[e] = den > 0.f ? d / den : 0.f;
+        }
+        const size_t p = (size_t)z * nxy + own;
+        *reinterpret_cast<float2*>(s0 + p) = make_float2(sa[0], sa[1]);
+        *reinterpret_cast<float2*>(s1 + p) = make_float2(ds[0], ds[1]);
+#pragma unroll
+        for (int st = 0; st < 2; ++st)
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[st][f][q] = w[st][f][q + 1];
+    }
+}
+
 // ============================================================================
 // Plane pass: x and y terms of every field and the point-wise terms, for a
 // PX x PYT tile of plane z = blockIdx.z; writes their sum to P.  The fluxes
@@ -1367,7 +1462,16 @@ static cudaError_t launch_split(int mode, const Geo& G, const T* u, const T* v, 
     }
     if (SMAG) {
         dim3 gk((G.nx + KX - 1) / KX, (G.ny + KY - 1) / KY, (G.nz + SZB - 1) / SZB);
-        strain3d<T, KIND, 0><<<gk, NTHREADS, 0, s>>>(G, u, v, sc.s0, sc.s1, part, ctl, check_done);
+        bool pairs = false;
+        if constexpr (KIND == PAIR && sizeof(T) == sizeof(float)) {
+            auto at = [](const void* q) { return reinterpret_cast<uintptr_t>(q); };
+            pairs = G.nx % 2 == 0 && ((at(u) | at(v) | at(sc.s0) | at(sc.s1)) & 7) == 0;
+            if (pairs) {
+                gk.x = (G.nx / 2 + KX - 1) / KX;
+                strain3d_pairs<<<gk, NTHREADS, 0, s>>>(G, u, v, sc.s0, sc.s1, ctl, check_done);
+            }
+        }
+        if (!pairs) strain3d<T, KIND, 0><<<gk, NTHREADS, 0, s>>>(G, u, v, sc.s0, sc.s1, part, ctl, check_done);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     dim3 gp((G.nx + PX - 1) / PX, (G.ny + SH::PY - 1) / SH::PY, G.nz);

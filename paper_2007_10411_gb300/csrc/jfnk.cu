@@ -434,7 +434,7 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     const int m = h->m;
     int maxblk = std::max(MAX_STREAM_BLOCKS, MAX_DOT_BLOCKS);
     maxblk = std::max(maxblk, dim == 3 ? stencil3d_part_blocks(G) : stencil_part_blocks(G));
-    {   // multi-dot grids: up to n / (4 * NTHREADS * 64) CTAs
+    {   // multi-dot grids: n / (4 * NTHREADS * 64) CTAs (float64: 2), to whole rounds less than twice that
         const size_t rb = h->n / ((size_t)NTHREADS * 64) + 1;
         maxblk = std::max(maxblk, (int)std::min(rb, (size_t)MAX_REDUCE_BLOCKS));
     }

@@ -491,9 +491,9 @@ __device__ __forceinline__ void work_b(const VT (&v)[CH], VT wv, T* __restrict__
 // Pass B, split over KS lanes per element: h1 from pass A's partials (every
 // block, grid_sums), w' = w - V h1 (stored over w), ||w'||^2 and h2 = V^T w'
 // into this pass's partials.  Each lane keeps its CH basis entries in
-// registers for both uses, so every basis vector is read from memory once;
-// with at most eight entries per lane the next element's loads are issued
-// before the current one is combined (software pipeline).
+// registers for both uses, so every basis vector is read from memory once.
+// (Loading the next element ahead with eight entries a lane: 11.8 against 10.6 us
+// at 1024 x 512, nv <= 8; the other warps cover the latency already.)
 template <typename T, int NV>
 __global__ void __launch_bounds__(NTHREADS, MIN_CTAS<T, NV>)
 arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int nv,
@@ -505,9 +505,6 @@ arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int 
     // a lane keeps up to sixteen (float64: thirty-two) loads in flight, and the
     // instantiation nearest above nv (8, 12, 16, 24, 32) leaves few entries empty
     constexpr int KS = LANES<T, NV>, CH = NV / KS;
-    // the next element's loads are issued ahead (software pipeline) where the
-    // registers allow it; twelve or more entries per lane are deep enough without
-    constexpr bool PF = CH <= 8;
     static_assert(CH * KS == NV && CH % 4 == 0, "lane split");
     __shared__ double h1d[NV];
     __shared__ T h1s[NV];
@@ -529,32 +526,11 @@ arnoldi_b(const T* __restrict__ V, size_t ldv, T* __restrict__ w, size_t n, int 
     const size_t g0 = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) / KS;
     const size_t gstride = (size_t)gridDim.x * blockDim.x / KS;
     const Walk wk = make_walk(g0, gstride, nvec, !(nv & 1));
-    if constexpr (!PF) {
-        for (size_t cc = 0; cc < wk.cnt; ++cc) {
-            const size_t i = wk.at(cc);
-            VT v[CH];
-            load_b<T, VT, CH>(V, ldv, i, nv, q, v);
-            work_b<T, VT, CH, KS>(v, scalev(reinterpret_cast<const VT*>(w)[i], sig), w, i, nv, q, h1s, acc, accn);
-        }
-    } else {
-        VT vn[CH], wn = zerov<VT>();
-        if (wk.cnt > 0) {
-            load_b<T, VT, CH>(V, ldv, wk.at(0), nv, q, vn);
-            wn = scalev(reinterpret_cast<const VT*>(w)[wk.at(0)], sig);
-        }
-        for (size_t cc = 0; cc < wk.cnt; ++cc) {
-            const size_t i = wk.at(cc);
-            VT v[CH];
-#pragma unroll
-            for (int c = 0; c < CH; ++c) v[c] = vn[c];
-            const VT wv = wn;
-            if (cc + 1 < wk.cnt) {
-                const size_t inext = wk.at(cc + 1);
-                load_b<T, VT, CH>(V, ldv, inext, nv, q, vn);
-                wn = scalev(reinterpret_cast<const VT*>(w)[inext], sig);
-            }
-            work_b<T, VT, CH, KS>(v, wv, w, i, nv, q, h1s, acc, accn);
-        }
+    for (size_t cc = 0; cc < wk.cnt; ++cc) {
+        const size_t i = wk.at(cc);
+        VT v[CH];
+        load_b<T, VT, CH>(V, ldv, i, nv, q, v);
+        work_b<T, VT, CH, KS>(v, scalev(reinterpret_cast<const VT*>(w)[i], sig), w, i, nv, q, h1s, acc, accn);
     }
     for (size_t i = nvec * W + g0; i < n; i += gstride) {
         T v[CH];
@@ -1173,11 +1149,16 @@ pc_eps_k(const float* __restrict__ z, size_t n, double* part, Ctl* ctl) {
 template <typename T> static int grid_a(size_t n) {
     return std::max(dot_blocks(n / V4<T>::W), reduce_blocks(n / V4<T>::W));
 }
+// Grids above one round of resident CTAs (two per SM) are whole rounds: the 320
+// blocks that PER_THREAD asks for at 256 x 256 x 64 ran 16 of them after the
+// other 304 (in us at nv <= 8 / 12 / 16 / 24: 137 / 153 / 170 / 235, with 608 blocks
+// 93 / 120 / 137 / 174).
 // Pass B and CA above 16 float64 vectors hold one CTA per SM (MIN_CTAS).
 template <typename T> static bool one_per_sm(int nv) { return sizeof(T) == sizeof(double) && nv > 16; }
 template <typename T> static int grid_b(size_t n, int nv) {
     const int b = reduce_blocks(n / V4<T>::W);
-    return one_per_sm<T>(nv) ? std::min(b, 152) : b;
+    if (one_per_sm<T>(nv)) return std::min(b, 152);
+    return b > MAX_STREAM_BLOCKS ? std::min((b + MAX_STREAM_BLOCKS - 1) / MAX_STREAM_BLOCKS * MAX_STREAM_BLOCKS, MAX_REDUCE_BLOCKS) : b;
 }
 template <typename T> static int grid_c(size_t n) {
     return std::min(dot_blocks(n / V4<T>::W) + 1, MAX_DOT_BLOCKS);

@@ -862,7 +862,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
         if kj["launches"] and pipe is not None:
             live_us = kj["ms"] / kj["launches"] * 1e3
             fp64["fp64_pipe"] = {
-                "kernel": "stencil2d<double, MODE_JV> (float64 Jacobian product)", "bound": "fp64 pipe",
+                "kernel": "flux2d<double> (float64 Jacobian product)", "bound": "fp64 pipe",
                 "live_us_per_launch": live_us, "ncu_us_per_launch": pipe[1], "ncu_pipe_frac": pipe[0],
                 "frac": pipe[0] * pipe[1] / live_us,
                 "how": "FP64-pipe busy fraction from one ncu capture (profiles/ncu_traffic.txt), scaled by the "

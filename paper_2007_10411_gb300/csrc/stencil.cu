@@ -87,22 +87,25 @@ template <> struct Vec16<double> {
     __device__ static double2 neg(double2 x) { return make_double2(flip(x.x), flip(x.y)); }
 };
 
-// True when the whole x-range [x0 - HALO, x0 - HALO + SX) of a tile is inside the
-// grid and rows start on 16-byte boundaries: the tile rows load as 16-byte vectors.
+// Every row of every plane of the arrays starts on a 16-byte boundary: planes are
+// nx * nz elements apart, and the base may be the caller's array, which need only
+// be aligned to its element (8 bytes).
 template <typename T>
-__device__ __forceinline__ bool rows_vectorisable(const Geo& G, int x0, int SX) {
-    return x0 - HALO >= 0 && x0 - HALO + SX <= G.nx && (G.nx % Vec16<T>::W) == 0;
+static bool rows_aligned(const Geo& G, const T* a, const T* b = nullptr) {
+    return G.nx % Vec16<T>::W == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
 }
 
 // Stage 1: s[f][SZ][SX] <- (LOADMODE 0) u, (1) u + ev*v, (2) ev*v for fields
-// f0 .. f0+NF-1, ghost-extended (periodic x, signed mirror z).
+// f0 .. f0+NF-1, ghost-extended (periodic x, signed mirror z).  aligned: the
+// host's rows_aligned(u, v); a tile whose x-range [x0 - HALO, x0 - HALO + SX)
+// lies inside the grid then loads its rows as 16-byte vectors.
 template <typename T, int LOADMODE, int NF = 4>
 __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const T* __restrict__ v,
-                                            const T (&ev)[4], const Geo& G, int x0, int z0,
+                                            const T (&ev)[4], const Geo& G, int aligned, int x0, int z0,
                                             int SX, int SZ, int f0 = 0) {
     using VT = typename Vec16<T>::type;
     constexpr int VW = Vec16<T>::W;
-    if (rows_vectorisable<T>(G, x0, SX)) {
+    if (aligned && x0 - HALO >= 0 && x0 - HALO + SX <= G.nx) {
         const int nch = SX / VW;
         const int total = nch * SZ;
         for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
@@ -146,7 +149,7 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
             if (ok) {
                 const size_t o = (size_t)f * G.npt + off;
                 if (LOADMODE == 0) val = u[o];
-                else if (LOADMODE == 1) val = u[o] + ev[f] * v[o];
+                else if (LOADMODE == 1) val = rfma(ev[f], v[o], u[o]);
                 else val = ev[f] * v[o];
                 if (odd_ghost(G, f, side)) val = flip(val);
             }
@@ -330,7 +333,7 @@ __device__ __forceinline__ void flux_out(const Geo& G, int mode, int fl, T Fv, d
 // sub-partitions' FP64 pipes.
 template <typename T, int SMAG, int PPT>
 __global__ void __launch_bounds__(NTHREADS)
-flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
+flux2d(Geo G, int mode, FluxShape sh, int aligned, const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ Fu,
        const double* __restrict__ f, T* __restrict__ out, T* __restrict__ out2, double* __restrict__ part, Ctl* ctl,
        int check_done) {
     pdl_wait();
@@ -346,9 +349,9 @@ flux2d(Geo G, int mode, FluxShape sh, const T* __restrict__ u, const T* __restri
     if (mode == MODE_JV) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) ev[q] = T(ctl->ev[q]);
-        load_fields<T, 1>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
+        load_fields<T, 1>(s1, u, v, ev, G, aligned, x0, z0, SX, TZ + 2 * HALO);
     } else {
-        load_fields<T, 0>(s1, u, v, ev, G, x0, z0, SX, TZ + 2 * HALO);
+        load_fields<T, 0>(s1, u, v, ev, G, aligned, x0, z0, SX, TZ + 2 * HALO);
     }
     __syncthreads();
     T S[PPT > 0 ? PPT : 1][4];
@@ -1144,7 +1147,7 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
 // ----------------------------------------------------------------------------
 template <int SMAG>
 __global__ void __launch_bounds__(NTHREADS)
-cheb2d_f64(Geo G, int k, int first, int last, FluxShape sh, const double* __restrict__ r,
+cheb2d_f64(Geo G, int k, int first, int last, FluxShape sh, int aligned, const double* __restrict__ r,
            const double* __restrict__ zin, const double* __restrict__ din, double* __restrict__ zout,
            double* __restrict__ dout, const double* __restrict__ nu, double* part, Ctl* ctl, int check_done) {
     using T = double;
@@ -1170,7 +1173,7 @@ cheb2d_f64(Geo G, int k, int first, int last, FluxShape sh, const double* __rest
         }
     } else {
         const T none[4] = {0.0, 0.0, 0.0, 0.0};
-        load_fields<T, 0, 1>(zs, first ? r : zin, nullptr, none, G, x0, z0, SX, TZ + 2 * HALO, fld);
+        load_fields<T, 0, 1>(zs, first ? r : zin, nullptr, none, G, aligned, x0, z0, SX, TZ + 2 * HALO, fld);
         __syncthreads();
         // eddy coefficient of the point at tile (ix, iz), its constant factors left to the end
         auto coef = [&](int ix, int iz, bool zarm) -> T {
@@ -1624,10 +1627,11 @@ static cudaError_t launch_flux_t(const FluxShape& sh, int mode, const Geo& G, co
     }
     const size_t sm = sh.elems() * sizeof(T);
     dim3 grid((G.nx + sh.tx() - 1) >> sh.lx, (G.nz + sh.tz() - 1) >> sh.lz);
+    const int aligned = rows_aligned(G, u, mode == MODE_JV ? v : nullptr);
     if (mode == MODE_JV)
-        return launch_pdl(flux2d<T, SMAG, PPT>, grid, NTHREADS, sm, s, G, mode, sh, u, v, Fu, f, out, out2, part, ctl,
-                          check_done);
-    flux2d<T, SMAG, PPT><<<grid, NTHREADS, sm, s>>>(G, mode, sh, u, v, Fu, f, out, out2, part, ctl, check_done);
+        return launch_pdl(flux2d<T, SMAG, PPT>, grid, NTHREADS, sm, s, G, mode, sh, aligned, u, v, Fu, f, out, out2, part,
+                          ctl, check_done);
+    flux2d<T, SMAG, PPT><<<grid, NTHREADS, sm, s>>>(G, mode, sh, aligned, u, v, Fu, f, out, out2, part, ctl, check_done);
     return cudaGetLastError();
 }
 
@@ -1780,8 +1784,8 @@ static cudaError_t launch_precond_f64(const Geo& G, int sweeps, const double* r,
         double* zo = last ? z : zbuf[k & 1];
         double* dO = dbuf[k & 1];
         grid.z = last ? 4 : 3;            // the p block is written by the last sweep only
-        const cudaError_t e = launch_pdl(cheb2d_f64<SMAG>, grid, dim3(NTHREADS), sm, s, G, k, first, last, sh, r, zin, din,
-                                         zo, dO, nu, part, ctl, check_done);
+        const cudaError_t e = launch_pdl(cheb2d_f64<SMAG>, grid, dim3(NTHREADS), sm, s, G, k, first, last, sh,
+                                         (int)rows_aligned(G, first ? r : zin), r, zin, din, zo, dO, nu, part, ctl, check_done);
         if (launches) ++*launches;
         if (e != cudaSuccess) return e;
         zin = zo;

@@ -450,6 +450,16 @@ __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_gro
 template <int N>
 __device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+// Grid of a kernel with one CTA per tile: tile columns along x, tile rows along y
+// and, past the 65 535 that y holds (heights above 8 x 65 535 points), along z too.
+// The last rows may then lie past the wall; they feed no output.
+static dim3 tile_grid(int cols, int rows) {
+    constexpr int MAX_Y = 65535;
+    const int nz = (rows + MAX_Y - 1) / MAX_Y;
+    return dim3(cols, (rows + nz - 1) / nz, nz);
+}
+__device__ __forceinline__ int tile_row() { return blockIdx.z * gridDim.y + blockIdx.y; }
+
 // Row vectors: a thread of the float32 sweeps and of the Schur-complement kernels
 // owns W consecutive points along x (16 bytes where nx allows it).
 template <typename T, int W> struct RowVec { using type = typename Vec16<T>::type; };
@@ -773,9 +783,9 @@ jv2d(Geo G, const float* __restrict__ u, const float* __restrict__ v, float* __r
     float* Z = X + 4 * XN;                               // [4][TZ + 4][TX]
     pdl_wait();
     const int done = check_done ? ctl->done : 0;
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
+    const int x0 = blockIdx.x * TX, z0 = tile_row() * TZ;
     const size_t np = (size_t)G.npt;
-    if (done) return;
+    if (done || z0 >= G.nz) return;
     for (int j = threadIdx.x; j < SZ * RV; j += NT) {
         const int iz = j / RV, ix = (j % RV) * W;
         int side;
@@ -993,7 +1003,7 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
     __shared__ __align__(16) T ks[SMAG ? KZ * SX : 4];
     pdl_wait();
     const int done = check_done ? ctl->done : 0;
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
+    const int x0 = blockIdx.x * TX, z0 = tile_row() * TZ;
     const T* src = first ? r : zin;
     const size_t np = (size_t)G.npt;
     // storage row of global row gz (rows beyond one reflection feed no output)
@@ -1130,9 +1140,9 @@ cheb2d(Geo G, int k, int first, int last, const float* __restrict__ r, const flo
         // ||z||^2 stays pending, one float-float partial per block: the Jacobian
         // product that follows adds them (pending_eps), so this launch ends without
         // an arrival count and a serial tail
-        const int blk = blockIdx.y * gridDim.x + blockIdx.x;
+        const int blk = tile_row() * gridDim.x + blockIdx.x;
         block_partial_ff(acc[0], reinterpret_cast<float2*>(part), blk);
-        if (blk == 0 && threadIdx.x == 0) ctl->eps_part = gridDim.x * gridDim.y;
+        if (blk == 0 && threadIdx.x == 0) ctl->eps_part = gridDim.x * gridDim.y * gridDim.z;
     }
 }
 
@@ -1602,6 +1612,7 @@ static FluxShape flux_shape(const Geo& G) {
     FluxShape best = cand[3];
     double least = 1e300;
     for (const FluxShape& c : cand) {
+        if ((G.nz + c.tz() - 1) >> c.lz > 65535 && &c != &cand[3]) continue;      // more rows than gridDim.y holds
         const long long tiles = (long long)((G.nx + c.tx() - 1) >> c.lx) * ((G.nz + c.tz() - 1) >> c.lz);
         const double cw = c.cn() / 32.0, aw = 4.0 * (c.tx() + c.tz()) / 32.0;
         const double cost = (double)((tiles + SMS - 1) / SMS) *
@@ -1671,7 +1682,7 @@ static cudaError_t launch_jv_t(const Geo& G, const float* u, const float* v, flo
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(jv2d<W, NT, SMAG>, dim3((G.nx + SH::TX - 1) / SH::TX, (G.nz + SH::TZ - 1) / SH::TZ), dim3(NT),
+    return launch_pdl(jv2d<W, NT, SMAG>, tile_grid((G.nx + SH::TX - 1) / SH::TX, (G.nz + SH::TZ - 1) / SH::TZ), dim3(NT),
                       SH::smem, s, G, u, v, out, part, ctl, check_done);
 }
 
@@ -1725,7 +1736,7 @@ static cudaError_t launch_precond_w(const Geo& G, int sweeps, const float* r, fl
                                     float* db, const float* nu, double* part, Ctl* ctl, int check_done,
                                     cudaStream_t s, long long* launches) {
     constexpr int TX = PcRow<W>::NXT * W, TZ = NT / PcRow<W>::NXT;
-    const dim3 grid((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ);
+    const dim3 grid = tile_grid((G.nx + TX - 1) / TX, (G.nz + TZ - 1) / TZ);
     const float* zin = nullptr;
     const float* din = nullptr;
     float* zbuf[2] = {za, zb};

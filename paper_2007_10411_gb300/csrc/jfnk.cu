@@ -271,17 +271,17 @@ static double pc_bytes(const jfnk_handle* h) {
     const double P = (double)h->npt * (h->mixed ? 4.0 : 8.0);
     const int s = h->opts.pc_sweeps;
     if (h->G.pc_schur) {
-        // rhs: velocities and v_p -> rhs; each Helmholtz launch (one sweep, or two
-        // in 2-D where nz >= 8) reads x (rhs on the first), rhs and d and writes x
-        // and d (not on the last); back: velocities, v_theta, dp -> z but z_p
+        // rhs: velocities and v_p -> rhs; each Helmholtz launch (3-D: one sweep, 2-D:
+        // schur2d_sweeps) reads x (rhs on the first), rhs and d and writes x and d
+        // (not on the last); back: velocities, v_theta, dp -> z but z_p
         const int nf = h->G.nf;
+        const size_t elem = h->mixed ? sizeof(float) : sizeof(double);
+        const bool vec = h->G.nx % (16 / elem) == 0;      // the workspace's vectors are 16-byte aligned
         double b = nf + (2.0 * nf - 1.0);     // rhs kernel + back-substitution
-        const bool pairs = h->G.dim == 2 && h->G.nz >= 8;
         for (int k = 1; k <= s - 1;) {
-            const bool two = pairs && k + 1 <= s - 1;
-            const bool first = k == 1, last = (two ? k + 1 : k) == s - 1;
-            b += (first ? 1.0 : 3.0) + (last ? 1.0 : 2.0);
-            k += two ? 2 : 1;
+            const int n = h->G.dim == 2 ? schur2d_sweeps(h->G, elem, vec, s - k) : 1;
+            b += (k == 1 ? 1.0 : 3.0) + (k + n == s ? 1.0 : 2.0);
+            k += n;
         }
         return b * P;
     }

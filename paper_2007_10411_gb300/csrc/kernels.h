@@ -28,6 +28,10 @@ cudaError_t launch_precond(const Geo& G, int sweeps, const T* r, T* z, T* za, T*
                            const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
                            long long* launches);
 
+// 2-D Schur complement: Helmholtz sweeps that one launch does when `left` remain
+// (elem: bytes of an element; vec: rows are whole 16-byte vectors).
+int schur2d_sweeps(const Geo& G, size_t elem, bool vec, int left);
+
 // Chebyshev coefficients of the preconditioner blocks from ctl->kmax (or the constant K).
 cudaError_t launch_pc_setup(const Geo& G, int sweeps, Ctl* ctl, cudaStream_t s);
 

@@ -1831,6 +1831,14 @@ static cudaError_t launch_helm2d(const Geo& G, const Helm2C<T>& C, int k, int fi
                       k, first, last, rhs, xin, din, xout, dout, ctl, check_done);
 }
 
+// Helmholtz sweeps of one launch with `left` still to do: at most four where the
+// rows are float32 vectors (a sweep's ring is then cheap next to a launch), two
+// otherwise (float64: the rings cost the FP64 pipe; single points: three times the
+// loads), within one reflection of nz.
+int schur2d_sweeps(const Geo& G, size_t elem, bool vec, int left) {
+    return std::min(std::min(elem == sizeof(float) && vec ? 4 : 2, G.nz / HALO), left);
+}
+
 // Acoustic Schur complement: rhs (plane 0 of da), sweeps - 1 Helmholtz
 // sweeps (iterates in plane 0 of za / zb, directions in planes 0 / 1 of db,
 // the last one into plane 3 of z), then the back-substitution.
@@ -1856,19 +1864,14 @@ static cudaError_t launch_schur_w(const Geo& G, int sweeps, const T* r, T* z, T*
     T* dbuf[2] = {db, db + np};
     const T* xin = nullptr;
     const T* din = nullptr;
-    // sweeps per launch: four where the rows are float32 vectors (a sweep's ring is
-    // then cheap next to a launch), two otherwise (float64: the rings cost the FP64
-    // pipe; single points: three times the loads), within one reflection of nz
-    constexpr int MAXS = sizeof(T) == sizeof(float) && W > 1 ? 4 : 2;
-    const int most = std::min(MAXS, G.nz / HALO);
     int cur = 1;                              // buffer pair the next output goes to
     for (int k = 1; k <= sweeps - 1;) {
-        const int n = std::min(most, sweeps - k);
+        const int n = schur2d_sweeps(G, sizeof(T), W > 1, sweeps - k);
         const int first = k == 1, last = k + n == sweeps;
         T* xo = last ? z + 3 * np : xbuf[cur];
         T* dO = dbuf[cur];
         const T* rh = rhs;
-        if constexpr (MAXS == 4) {
+        if constexpr (sizeof(T) == sizeof(float) && W > 1) {
             if (n == 4) e = launch_helm2d<T, W, 4>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
             if (n == 3) e = launch_helm2d<T, W, 3>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
         }

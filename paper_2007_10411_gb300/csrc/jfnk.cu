@@ -265,8 +265,8 @@ static void kt_end(jfnk_handle* h, int fam, double bytes) {
     h->kt_count += 1;
 }
 
-// Algorithmic HBM bytes of one preconditioner apply (every input read once,
-// every output written once, per field plane).
+// Algorithmic HBM bytes of one preconditioner apply: every input of a launch read
+// once, every output written once.
 static double pc_bytes(const jfnk_handle* h) {
     const double P = (double)h->npt * (h->mixed ? 4.0 : 8.0);
     const int s = h->opts.pc_sweeps;
@@ -285,11 +285,14 @@ static double pc_bytes(const jfnk_handle* h) {
         }
         return b * P;
     }
-    if (s <= 1) return 2.0 * 4.0 * P;
+    // field block: r, d (not on the first), x -> x, d (not on the last) of the diffused
+    // fields (all but p) and the eddy field once a launch; p on the last
+    const int nf = h->G.nf;
+    if (s <= 1) return 2.0 * nf * P;
     double b = 0.0;
     for (int k = 1; k <= s - 1; ++k) {
         const bool first = k == 1, last = k == s - 1;
-        b += 3.0 * P * (1.0 + (first ? 0.0 : 2.0) + 1.0 + (last ? 0.0 : 1.0) + (h->G.smag ? 1.0 : 0.0));
+        b += P * ((nf - 1) * (1.0 + (first ? 0.0 : 2.0) + 1.0 + (last ? 0.0 : 1.0)) + (h->G.smag ? 1.0 : 0.0));
     }
     return b + 2.0 * P;
 }

@@ -199,12 +199,13 @@ __device__ __forceinline__ float root(float x) { return sqrtf(x); }
 // sqrt(x) and 1 / sqrt(x) of a positive x by the same iteration, two coupled
 // steps (relative error of a few 2^-53): about ten dependent operations where a
 // square root and a division take nearly a hundred, each a 64-cycle issue for
-// every block that waits on it.  Zero (and negative) give 0 and 0.
+// every block that waits on it.  Zero (and negative) give 0 and 0, infinity gives
+// infinity and 0, NaN gives NaN twice: a norm that is not a number stays visible.
 __device__ __forceinline__ void root_pair(double x, double& g, double& ig) {
     const int hi = __double2hiint(x);
     if (hi < 0x00100000 || hi >= 0x7ff00000) {
-        g = x > 0.0 ? sqrt(x) : 0.0;
-        ig = g > 0.0 ? 1.0 / g : 0.0;
+        g = x > 0.0 ? sqrt(x) : (x <= 0.0 ? 0.0 : x);
+        ig = g > 0.0 ? 1.0 / g : g;
         return;
     }
     double y;

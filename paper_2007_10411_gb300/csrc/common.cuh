@@ -84,9 +84,10 @@ struct Ctl {
     int iters;           // Krylov iterations in this Newton solve
     int m;               // restart length
     int ncap;            // training pairs recorded for the learned preconditioner
-    int eps_part;        // > 0: ||z||^2 of the last preconditioner apply is pending as that many
-                         // float-float partials at the head of the partial buffer (float32 2-D
-                         // field-block path); the Jacobian-product kernel forms eps from them.
+    int eps_part;        // ||z||^2 of the last preconditioner apply is pending at the head of the
+                         // partial buffer, and the Jacobian-product kernel forms eps from it:
+                         // > 0: that many float-float partials (float32 2-D field blocks);
+                         // < 0: minus that many float64 partials (float32 2-D Schur complement);
                          // 0: eps_jv holds the step.  Every writer of eps_jv clears it.
     int pad_;
     double beta0;        // ||b|| of the Newton system
@@ -326,30 +327,43 @@ __device__ __forceinline__ void put_eps_norm2(Ctl* ctl, double zn2) {
 }
 
 // Finite-difference step of a Jacobian product and its reciprocal: eps_jv, or,
-// when ctl->eps_part > 0, eps = eps_num / ||z|| with ||z||^2 summed from the
-// pending float-float partials in one fixed order (every block of the launch
-// obtains bitwise the same value).  Called by all threads of the block.
+// when ctl->eps_part is not 0, eps = eps_num / ||z|| with ||z||^2 summed from the
+// pending partials.  The first four warps add them (a float64 addition takes a
+// sub-partition's pipe for 64 cycles; more warps would queue for it), across the
+// warps in float64, in one fixed order: every block of the launch, whatever its
+// size, obtains bitwise the same value.  Called by all threads of a block of at
+// least 128.
 __device__ __forceinline__ double2 pending_eps(const Ctl* ctl, const double* part) {
-    __shared__ float2 wsum[NTHREADS / 32];
+    constexpr int NT = 128;
+    __shared__ double wsum[NT / 32];
     __shared__ double2 eps_s;
     const int np = ctl->eps_part;
     const double num = ctl->eps_num, inum = ctl->inv_eps_num;
-    if (np > 0) {
+    if (np != 0) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const float2* p = reinterpret_cast<const float2*>(part);
-        float2 s = make_float2(0.f, 0.f);
+        if (np > 0 && threadIdx.x < NT) {
+            const float2* p = reinterpret_cast<const float2*>(part);
+            float2 s = make_float2(0.f, 0.f);
 #pragma unroll 8
-        for (int b = threadIdx.x; b < np; b += blockDim.x) s = ff_add(s, __ldcg(p + b));
+            for (int b = threadIdx.x; b < np; b += NT) s = ff_add(s, __ldcg(p + b));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            s = ff_add(s, make_float2(__shfl_down_sync(0xffffffffu, s.x, o), __shfl_down_sync(0xffffffffu, s.y, o)));
-        if (lane == 0) wsum[warp] = s;
+            for (int o = 16; o > 0; o >>= 1)
+                s = ff_add(s, make_float2(__shfl_down_sync(0xffffffffu, s.x, o), __shfl_down_sync(0xffffffffu, s.y, o)));
+            if (lane == 0) wsum[warp] = (double)s.x + (double)s.y;
+        } else if (threadIdx.x < NT) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int b = threadIdx.x; b < -np; b += NT) s += __ldcg(part + b);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (lane == 0) wsum[warp] = s;
+        }
         __syncthreads();
         if (threadIdx.x == 0) {
-            float2 t = wsum[0];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) t = ff_add(t, wsum[w]);
+            double t = wsum[0];
+            for (int w = 1; w < NT / 32; ++w) t += wsum[w];
             double zn, izn;
-            root_pair((double)t.x + (double)t.y, zn, izn);
+            root_pair(t, zn, izn);
             eps_s = make_double2(num * izn, zn * inum);
         }
     } else if (threadIdx.x == 0) {

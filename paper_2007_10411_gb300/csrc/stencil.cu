@@ -1495,7 +1495,7 @@ helm2d(Geo G, Helm2C<T> C, int k, int first, int last, const T* __restrict__ rhs
 }
 
 // z_u, z_w from the pressure solution (already in plane 3 of z), z_theta, and
-// the finite-difference step eps from ||z|| (float32: pending, as cheb2d leaves it).
+// the finite-difference step eps from ||z|| (float32: pending, as float64 partials).
 template <typename T, int W>
 __global__ void __launch_bounds__(NTHREADS)
 schur_back2d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ctl* ctl, int check_done) {
@@ -1529,11 +1529,10 @@ schur_back2d(Geo G, const T* __restrict__ r, T* __restrict__ z, double* part, Ct
         rstore<T, W>(z + 2 * np + p, rt);
     }
     pdl_trigger();
+    block_partials<1, T>(acc, 1, part, gridDim.x, blockIdx.x);
     if constexpr (sizeof(T) == sizeof(float)) {
-        block_partial_ff(acc[0], reinterpret_cast<float2*>(part), blockIdx.x);
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->eps_part = gridDim.x;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->eps_part = -(int)gridDim.x;      // float64 partials
     } else {
-        block_partials<1, T>(acc, 1, part, gridDim.x, blockIdx.x);
         if (arrive_last(&ctl->counter[CNT_PC], gridDim.x)) {
             __shared__ double tot[1];
             final_sums(part, gridDim.x, 1, tot);

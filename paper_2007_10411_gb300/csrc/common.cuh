@@ -223,6 +223,18 @@ __device__ __forceinline__ void root_pair(double x, double& g, double& ig) {
 }
 
 // ---------------------------------------------------------------- reductions
+// c + a . b.  float32: the four products meet each other first, so that the running
+// sum is rounded once a vector instead of once an element.  float64: one chain of
+// fused multiply-adds, because an addition occupies the FP64 pipe for as long as a
+// fused multiply-add (two roundings of the running sum a vector instead of one, at
+// 2^-53 each; the passes would take a quarter longer with a separate addition).
+__device__ __forceinline__ float dotacc(float4 a, float4 b, float c) {
+    return c + fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+__device__ __forceinline__ double dotacc(double2 a, double2 b, double c) { return fma(a.y, b.y, fma(a.x, b.x, c)); }
+__device__ __forceinline__ float dotacc(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double dotacc(double a, double b, double c) { return fma(a, b, c); }
+
 // Sum NV thread-local values over the block and store them, as float64, at
 // part[k * stride + blk] (k < nv).  Deterministic (fixed shuffle tree).  The
 // tree runs in the type of the thread values: float32 kernels reduce their

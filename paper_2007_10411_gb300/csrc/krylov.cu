@@ -37,13 +37,6 @@ template <> struct V4<double> { using type = double2; static constexpr int W = 2
 
 __device__ __forceinline__ float dotv(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 __device__ __forceinline__ double dotv(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
-// c + a . b as one chain of fused multiply-adds (a float64 addition costs as much as one)
-__device__ __forceinline__ float dotacc(float4 a, float4 b, float c) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
-}
-__device__ __forceinline__ double dotacc(double2 a, double2 b, double c) { return fma(a.y, b.y, fma(a.x, b.x, c)); }
-__device__ __forceinline__ float dotacc(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double dotacc(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float4 axpyv(float4 y, float a, float4 x) {
     return make_float4(y.x - a * x.x, y.y - a * x.y, y.z - a * x.z, y.w - a * x.w);
 }

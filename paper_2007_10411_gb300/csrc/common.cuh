@@ -25,7 +25,7 @@ constexpr int MAX_PC_SWEEPS = 64;
 // instruction and sub-partition): a dozen per thread cost several microseconds
 // of a 20 us launch.
 struct GeoF {
-    float inv_dx, inv_dy, inv_dz, wx1, wx2, wy1, wy2, wz1, wz2;
+    float inv_dx, inv_dy, inv_dz, wx1, wx2, wy1, wy2, wz1, wz2, ex, ey, ez;
     float theta0, beta, pbar, gth, gamma_p, K_M, K_H, cs2, inv_Pr;
     float dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
     float two_over_dt, helm_a, schur_cdiv, schur_cgrad, half_dt;
@@ -49,6 +49,11 @@ struct Geo {
     double dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
     // derivative weights with 1/h folded in: D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
     double wx1, wx2, wy1, wy2, wz1, wz2;
+    // relative difference of 2/3 times 1/h (each rounded) from w1, and of -1/12 times 1/h
+    // from w2 = -w1/8: D f = w (1 + e) (...).  The divergence of a nearly solenoidal flow
+    // is a small part of its terms, so what the rounding of one axis's weight adds counts
+    // in full, and the pressure equation multiplies it by gamma_p pbar.
+    double ex, ey, ez;
     double gth;                       // g / theta0
     double inv_Pr;
     double two_over_dt;

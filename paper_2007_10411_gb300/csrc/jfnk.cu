@@ -358,6 +358,10 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     G.wy2 = -1.0 / 12.0 / dy;
     G.wz1 = 2.0 / 3.0 / dz;
     G.wz2 = -1.0 / 12.0 / dz;
+    auto lost = [](double w, double inv_h) { return fma(2.0 / 3.0, inv_h, -w) / w; };
+    G.ex = lost(G.wx1, G.inv_dx);
+    G.ey = lost(G.wy1, G.inv_dy);
+    G.ez = lost(G.wz1, G.inv_dz);
     G.gth = strat->g / strat->theta0;
     G.theta0 = strat->theta0;
     G.beta = strat->beta;
@@ -409,6 +413,9 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     F.wy2 = (float)G.wy2;
     F.wz1 = (float)G.wz1;
     F.wz2 = (float)G.wz2;
+    F.ex = (float)lost(F.wx1, G.inv_dx);
+    F.ey = (float)lost(F.wy1, G.inv_dy);
+    F.ez = (float)lost(F.wz1, G.inv_dz);
     F.theta0 = (float)G.theta0;
     F.beta = (float)G.beta;
     F.pbar = (float)G.pbar;

@@ -189,6 +189,18 @@ __device__ __forceinline__ T advect(T s, T mj, T bj, T dm, T db) {
     return KIND == PAIR ? s - mj * db - bj * dm : s - bj * db;
 }
 
+// -gamma_p (pbar + p) times a part of the divergence, added to the small terms s:
+// p the state's (midpoint's) pressure, div the part (of b), divm the same of m, lost
+// what the rounded weights left out of div.  The parts of the three axes nearly cancel
+// each other; gamma_p (pbar + p) is the same factor in both passes, and the large
+// product is rounded once, last.
+template <typename T, int KIND>
+__device__ __forceinline__ T pressure_part(const Geo& G, T s, T p, T b, T div, T divm, T lost) {
+    const T g = GC(gamma_p) * (GC(pbar) + p);
+    if (KIND == PAIR) s = fma(-GC(gamma_p), b * divm, s);
+    return fma(-g, div, fma(-g, lost, s));
+}
+
 // Asynchronous copy of one element into shared memory.
 template <typename T>
 __device__ __forceinline__ void cpa1(T* dst, const T* src) {
@@ -519,7 +531,7 @@ __device__ __forceinline__ void plane_point(const Geo& G, const T* __restrict__ 
     coefs<T, KIND, SMAG>(G, na, ds, false, km, dk);
     const T bu = T(0.5) * B[c], bv = T(0.5) * B[SP + c];
     const T mu = KIND == PAIR ? T(0.5) * M[c] : T(0), mv = KIND == PAIR ? T(0.5) * M[SP + c] : T(0);
-    T divb = T(0), divm = T(0);
+    T divb = T(0), divm = T(0), dive = T(0);
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
         const T b = B[f * SP + c], m = KIND == PAIR ? M[f * SP + c] : T(0);
@@ -539,14 +551,13 @@ __device__ __forceinline__ void plane_point(const Geo& G, const T* __restrict__ 
             // the small advective terms first: the large linear ones are rounded once
             s = advect<T, KIND>(s, mu, bu, dmx, dbx);
             s = advect<T, KIND>(s, mv, bv, dmy, dby);
-            if (f == 0) { divb = dbx; divm = dmx; }
-            if (f == 1) { divb += dby; divm += dmy; }
+            if (f == 0) { divb = dbx; divm = dmx; dive = GC(ex) * dbx; }
+            if (f == 1) { divb += dby; divm += dmy; dive = fma(GC(ey), dby, dive); }
             if (f == 2) s += GC(gth) * B[3 * SP + c];
             if (f == 3) s -= GC(beta) * B[2 * SP + c];
             if (f == 4) {       // pressure equation, x and y parts of the divergence; gradient of p
-                T t = (GC(pbar) + (KIND == PAIR ? m : b)) * divb;
-                if (KIND == PAIR) t += b * divm;
-                s -= GC(gamma_p) * t;
+                // (what the weights lost, Geo::ex, with the small terms: see pressure_part)
+                s = pressure_part<T, KIND>(G, s, KIND == PAIR ? m : b, b, divb, divm, dive);
                 S[0] -= GC(theta0) * dbx;
                 S[1] -= GC(theta0) * dby;
             }
@@ -765,9 +776,9 @@ column3d(Geo G, int mode, int zc, const T* __restrict__ u, const T* __restrict__
                 if (q == IP) {
                     Z[r2] = flux_p<T, KIND>(mw, bw, m[r2], b[r2]);
                     const T dw = w1 * (c[r1] - c[r3]) + w2 * (c[r0] - c[r4]);
-                    T t = (GC(pbar) + (KIND == PAIR ? m[r2] : b[r2])) * dw;
-                    if (KIND == PAIR) t += b[r2] * (w1 * (d[r1] - d[r3]) + w2 * (d[r0] - d[r4]));
-                    s = advect<T, KIND>(s, mw, bw, dm, db) - GC(gamma_p) * t;
+                    const T dwm = KIND == PAIR ? w1 * (d[r1] - d[r3]) + w2 * (d[r0] - d[r4]) : T(0);
+                    s = pressure_part<T, KIND>(G, advect<T, KIND>(s, mw, bw, dm, db), KIND == PAIR ? m[r2] : b[r2], b[r2], dw, dwm,
+                                               GC(ez) * dw);
                 } else {
                     T km[2], dk[2];
                     coefs<T, KIND, SMAG>(G, ka, kd, true, km, dk);

@@ -260,16 +260,17 @@ __device__ __forceinline__ void flux_point(const Geo& G, const FluxShape& sh, co
         }
     }
     const T hu = rmul(T(0.5), U[i]), hw = rmul(T(0.5), W[i]);
+    // K D phi - 1/2 u_j phi: see flux_sum
     if (XF) {
-        X[0] = rfma(kx, ux, -rmul(hu, U[i]));
-        X[XN] = rfma(kx, wx, -rmul(hu, W[i]));
-        X[2 * XN] = rfma(kxh, tx, -rmul(hu, H[i]));
+        X[0] = flux_sum(kx, ux, hu, U[i]);
+        X[XN] = flux_sum(kx, wx, hu, W[i]);
+        X[2 * XN] = flux_sum(kxh, tx, hu, H[i]);
         X[3 * XN] = -rmul(hu, P[i]);
     }
     if (ZF) {
-        Z[0] = rfma(kz, uz, -rmul(hw, U[i]));
-        Z[ZN] = rfma(kz, wz, -rmul(hw, W[i]));
-        Z[2 * ZN] = rfma(kzh, tz, -rmul(hw, H[i]));
+        Z[0] = flux_sum(kz, uz, hw, U[i]);
+        Z[ZN] = flux_sum(kz, wz, hw, W[i]);
+        Z[2 * ZN] = flux_sum(kzh, tz, hw, H[i]);
         Z[3 * ZN] = -rmul(hw, P[i]);
     }
     if (XF && ZF) {

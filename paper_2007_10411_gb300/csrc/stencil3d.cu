@@ -175,7 +175,7 @@ __device__ __forceinline__ T flux_of(T km, T dk, T mj, T bj, T m, T b, T dm, T d
         x += km * db;
         return SMAG ? x + dk * dm : x;
     } else {
-        return dk * db - bj * b;
+        return flux_sum(dk, db, bj, b);
     }
 }
 // The same for p, which is not diffused.

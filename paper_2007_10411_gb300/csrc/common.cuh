@@ -76,6 +76,11 @@ __device__ __forceinline__ T geo_const(double d, float f) {
 }
 #define GC(name) geo_const<T>(G.name, G.f32.name)
 
+// D applied twice, from the first differences g_k = x_{k+1} - x_k of a line:
+// sum_s c_s x_s (c_s = sum_{a+b=s} w_a w_b: -65/72, 1/9, 4/9, -1/9, 1/144 for |s| = 0 .. 4,
+// which add up to zero) = sum_{k=0..3} C_k (g_k - g_{-1-k}) with C_k = sum_{s>k} c_s.
+constexpr double HELM_DIFF[4] = {65.0 / 144.0, 49.0 / 144.0, -15.0 / 144.0, 1.0 / 144.0};
+
 constexpr int NUM_TILE_SHAPES = 4;
 
 // Solver control block in device memory.  Written by the "last block" of the

@@ -1343,12 +1343,18 @@ schur_rhs2d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int c
 // blocking).  x_k of a TX x TZ tile is staged with a halo of 4 S (periodic x,
 // even mirror in z; the mirrored ghost rows give the mirrored result, so ghosts
 // are swept like other points); sweep s runs on the tile plus a ring of
-// 4 (S - 1 - s) points from one of two x buffers into the other, one barrier a
-// sweep.  H is applied as the composite stencil of D taken twice (coefficients
-// sum_{a+b=s} w_a w_b: -65/72, 1/9, 4/9, -1/9, 1/144), so no first derivative is
-// exchanged.  Points are handled in groups of W along x; the groups are ordered
-// tile first, then ring by ring, and dealt to the threads in that order: a
+// 4 (S - 1 - s) points.  Points are handled in groups of W along x; the groups are
+// ordered tile first, then ring by ring, and dealt to the threads in that order: a
 // thread keeps rhs and d of its groups in registers through all sweeps.
+// float32: from one of two x buffers into the other, one barrier a sweep.  H is
+// applied as the composite stencil of D taken twice, so no first derivative is
+// exchanged, and in the first differences of x (HELM_DIFF), as D of D x is: x itself,
+// times coefficients of which the sum is zero, cancels, and lost up to 40 times as
+// much (p after 32 sweeps at 1024 x 512: relative error 4.7e-6, now 1.2e-7 as with D
+// taken twice; 1 % of a launch).
+// float64: D_x x and D_z x are exchanged, then differentiated again: the FP64 pipe
+// counts operations, 20 a point and the arms against 33 in first differences (a Schur
+// step at 1024 x 256: 12.2 against 19.0 ms).
 // Needs nz >= 4 S (one reflection).
 //
 // Bound: a launch's fixed costs (staging latency, barriers) and issue; a plane
@@ -1358,7 +1364,8 @@ schur_rhs2d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int c
 // ----------------------------------------------------------------------------
 template <typename T>
 struct Helm2C {
-    T c0, cx[4], cz[4];             // res = rhs + c0 x + sum_l c_l (x_{+l} + x_{-l})
+    T c0, cx[4], cz[4];             // res = rhs + c0 x + sum_k c_k (g_k - g_{-1-k}), g_k = x_{k+1} - x_k along each axis
+                                    // (float64: cx, cz 0 and 1, the outer D's weights times a)
 };
 constexpr int HELM_THREADS = 512;
 constexpr int HELM_TX = 64, HELM_TZ = 32;
@@ -1375,7 +1382,9 @@ helm2d(Geo G, Helm2C<T> C, int k, int first, int last, const T* __restrict__ rhs
     static_assert(CORE % HELM_THREADS == 0, "whole slots of tile groups");
     constexpr int CS = CORE / HELM_THREADS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* xb = reinterpret_cast<T*>(smem_raw);         // [2][SZ][SX]
+    T* xb = reinterpret_cast<T*>(smem_raw);         // [2][SZ][SX]; float64: x, D_x x, D_z x
+    constexpr bool TWICE = sizeof(T) == sizeof(double);
+    static_assert(!TWICE || W == 1, "float64: single points");
     pdl_wait();
     if (check_done && ctl->done) return;
     const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
@@ -1445,40 +1454,72 @@ helm2d(Geo G, Helm2C<T> C, int k, int first, int last, const T* __restrict__ rhs
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        const T* xa = xb + (s & 1) * SX * SZ;
-        T* xn = xb + ((s + 1) & 1) * SX * SZ;
+        const T* xa = TWICE ? xb : xb + (s & 1) * SX * SZ;
+        T* xn = TWICE ? xb : xb + ((s + 1) & 1) * SX * SZ;
+        [[maybe_unused]] T *gx = xb + SX * SZ, *gz = gx + SX * SZ;      // float64: D_x x, D_z x where this sweep reads them
         const T a1 = cheb_coef<T>(ctl, 5, k + s, 1), a2 = cheb_coef<T>(ctl, 5, k + s, 2);
+        if constexpr (TWICE) {
+            const int h = HALO * (S - 1 - s), RX = TX + 2 * h, RZ = TZ + 2 * h, o = (H0 - h) * SX + H0 - h;
+            for (int j = threadIdx.x; j < RZ * (RX + 2 * R); j += HELM_THREADS) {
+                const int i = o + j / (RX + 2 * R) * SX + j % (RX + 2 * R) - R;
+                gx[i] = wd(xa, i, 1, GC(wx1), GC(wx2));
+            }
+            for (int j = threadIdx.x; j < (RZ + 2 * R) * RX; j += HELM_THREADS) {
+                const int i = o + (j / RX - R) * SX + j % RX;
+                gz[i] = wd(xa, i, SX, GC(wz1), GC(wz2));
+            }
+            __syncthreads();
+        }
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
             if (ring[q] > S - 1 - s) continue;
             const T* p = xa + off[q];
-            T e[W + 2 * HALO], r[W];
-#pragma unroll
-            for (int i = 0; i < W + 2 * HALO; i += W) {
-                T v[W];
-                rload<T, W>(p - HALO + i, v);
-#pragma unroll
-                for (int j = 0; j < W; ++j) e[i + j] = v[j];
-            }
-#pragma unroll
-            for (int i = 0; i < W; ++i) {
-                r[i] = rv[q][i] + C.c0 * e[HALO + i];
-#pragma unroll
-                for (int l = 1; l <= HALO; ++l) r[i] += C.cx[l - 1] * (e[HALO + i + l] + e[HALO + i - l]);
-            }
-#pragma unroll
-            for (int l = 1; l <= HALO; ++l) {
-                T a[W], b[W];
-                rload<T, W>(p + l * SX, a);
-                rload<T, W>(p - l * SX, b);
-#pragma unroll
-                for (int i = 0; i < W; ++i) r[i] += C.cz[l - 1] * (a[i] + b[i]);
-            }
             T xo[W];
+            if constexpr (TWICE) {
+                const T *x = gx + off[q], *z = gz + off[q];
+                const T xk = *p;
+                const T r = rfma(C.c0, xk, rv[q][0]) + rfma(C.cx[0], x[1] - x[-1], rfma(C.cx[1], x[2] - x[-2],
+                            rfma(C.cz[0], z[SX] - z[-SX], rmul(C.cz[1], z[2 * SX] - z[-2 * SX]))));
+                dv[q][0] = rfma(a1, dv[q][0], rmul(a2, r));
+                xo[0] = xk + dv[q][0];
+            } else {
+                T e[W + 2 * HALO], r[W];
 #pragma unroll
-            for (int i = 0; i < W; ++i) {
-                dv[q][i] = a1 * dv[q][i] + a2 * r[i];
-                xo[i] = e[HALO + i] + dv[q][i];
+                for (int i = 0; i < W + 2 * HALO; i += W) {
+                    T v[W];
+                    rload<T, W>(p - HALO + i, v);
+#pragma unroll
+                    for (int j = 0; j < W; ++j) e[i + j] = v[j];
+                }
+                T g[W + 2 * HALO - 1];                      // first differences along the row
+#pragma unroll
+                for (int i = 0; i < W + 2 * HALO - 1; ++i) g[i] = e[i + 1] - e[i];
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    r[i] = rv[q][i] + C.c0 * e[HALO + i];
+#pragma unroll
+                    for (int l = 0; l < HALO; ++l) r[i] += C.cx[l] * (g[HALO + i + l] - g[HALO - 1 + i - l]);
+                }
+                T pa[W], pb[W];
+#pragma unroll
+                for (int i = 0; i < W; ++i) pa[i] = pb[i] = e[HALO + i];
+#pragma unroll
+                for (int l = 1; l <= HALO; ++l) {
+                    T a[W], b[W];
+                    rload<T, W>(p + l * SX, a);
+                    rload<T, W>(p - l * SX, b);
+#pragma unroll
+                    for (int i = 0; i < W; ++i) {
+                        r[i] += C.cz[l - 1] * ((a[i] - pa[i]) - (pb[i] - b[i]));
+                        pa[i] = a[i];
+                        pb[i] = b[i];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    dv[q][i] = a1 * dv[q][i] + a2 * r[i];
+                    xo[i] = e[HALO + i] + dv[q][i];
+                }
             }
             if (s + 1 < S) {
                 rstore<T, W>(xn + off[q], xo);
@@ -1820,7 +1861,8 @@ template <typename T, int W, int S>
 static cudaError_t launch_helm2d(const Geo& G, const Helm2C<T>& C, int k, int first, int last, const T* rhs, const T* xin,
                                  const T* din, T* xout, T* dout, Ctl* ctl, int check_done, cudaStream_t s) {
     constexpr int TX = HELM_TX, TZ = HELM_TZ;
-    constexpr size_t sm = sizeof(T) * (S > 1 ? 2 : 1) * (size_t)(TX + 2 * HALO * S) * (TZ + 2 * HALO * S);
+    constexpr int PLANES = sizeof(T) == sizeof(double) ? 3 : S > 1 ? 2 : 1;
+    constexpr size_t sm = sizeof(T) * PLANES * (size_t)(TX + 2 * HALO * S) * (TZ + 2 * HALO * S);
     static std::atomic<bool> configured{false};   // set once; concurrent first calls are harmless
     if (!configured) {
         const cudaError_t e = set_smem(helm2d<T, W, S>, sm);
@@ -1853,12 +1895,19 @@ static cudaError_t launch_schur_w(const Geo& G, int sweeps, const T* r, T* z, T*
     if (e != cudaSuccess) return e;
     if (launches) ++*launches;
     Helm2C<T> C;
-    const double lap[5] = {-65.0 / 72.0, 1.0 / 9.0, 4.0 / 9.0, -1.0 / 9.0, 1.0 / 144.0};
     const double ax = G.helm_a * G.inv_dx * G.inv_dx, az = G.helm_a * G.inv_dz * G.inv_dz;
-    C.c0 = T(lap[0] * (ax + az) - G.two_over_dt);
+    C.c0 = T(-G.two_over_dt);
     for (int l = 0; l < 4; ++l) {
-        C.cx[l] = T(lap[l + 1] * ax);
-        C.cz[l] = T(lap[l + 1] * az);
+        C.cx[l] = T(HELM_DIFF[l] * ax);
+        C.cz[l] = T(HELM_DIFF[l] * az);
+    }
+    constexpr bool TWICE = sizeof(T) == sizeof(double);      // D applied twice by single points
+    constexpr int WH = TWICE ? 1 : W;
+    if (TWICE) {
+        C.cx[0] = T(G.helm_a * G.wx1);
+        C.cx[1] = T(G.helm_a * G.wx2);
+        C.cz[0] = T(G.helm_a * G.wz1);
+        C.cz[1] = T(G.helm_a * G.wz2);
     }
     T* xbuf[2] = {za, zb};
     T* dbuf[2] = {db, db + np};
@@ -1872,11 +1921,11 @@ static cudaError_t launch_schur_w(const Geo& G, int sweeps, const T* r, T* z, T*
         T* dO = dbuf[cur];
         const T* rh = rhs;
         if constexpr (sizeof(T) == sizeof(float) && W > 1) {
-            if (n == 4) e = launch_helm2d<T, W, 4>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
-            if (n == 3) e = launch_helm2d<T, W, 3>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+            if (n == 4) e = launch_helm2d<T, WH, 4>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+            if (n == 3) e = launch_helm2d<T, WH, 3>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
         }
-        if (n == 2) e = launch_helm2d<T, W, 2>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
-        if (n == 1) e = launch_helm2d<T, W, 1>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+        if (n == 2) e = launch_helm2d<T, WH, 2>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
+        if (n == 1) e = launch_helm2d<T, WH, 1>(G, C, k, first, last, rh, xin, din, xo, dO, ctl, check_done, s);
         if (e != cudaSuccess) return e;
         if (launches) ++*launches;
         xin = xo;

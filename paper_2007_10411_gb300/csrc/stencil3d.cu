@@ -1509,9 +1509,9 @@ static cudaError_t launch_split_k(int mode, const Geo& G, const T* u, const T* v
 //   H dp = v_p - c_div (D_x v_u + D_y v_v + D_z v_w),  H = (2/dt) I - a sum_j D_j D_j,
 //   z_i = (dt/2)(v_i - c_grad D_i dp),  z_theta = v_theta / theta_c,
 // with H applied point-wise as the composite stencil of the first derivative
-// taken twice along each axis (coefficients c_s = sum_{a+b=s} w_a w_b: -65/72,
-// 1/9, 4/9, -1/9, 1/144 for |s| = 0..4) on the ghost-extended plane (p even
-// at the walls), which equals D_j applied to D_j dp evaluated with its ghosts.
+// taken twice along each axis (in float32 in the line's first differences, HELM_DIFF:
+// p errs 20 % less; in float64, where the FP64 pipe counts operations, 25 against 36,
+// through its coefficients) on the ghost-extended plane (p even at the walls), which equals D_j applied to D_j dp evaluated with its ghosts.
 // Fields: 0 u, 1 v, 2 w, 3 theta, 4 p; planes [z][y][x].
 //
 // ---------------------------------------------------------------------------
@@ -1606,7 +1606,9 @@ schur_rhs3d(Geo G, const T* __restrict__ r, T* __restrict__ rhs, Ctl* ctl, int c
 // ---------------------------------------------------------------------------
 template <typename T>
 struct HelmC {                      // coefficients of a sweep in the type of the sweep
-    T c0, cx[4], cy[4], cz[4];      // res = rhs + c0 x + sum_k c_k (x_{+k} + x_{-k})
+    // float32: res = rhs + c0 x + sum_k c_k (g_k - g_{-1-k}), g_k = x_{k+1} - x_k along each axis
+    // float64: res = rhs + c0 x + lap0 x + sum_k c_k (x_{+k+1} + x_{-k-1})
+    T c0, lap0, cx[4], cy[4], cz[4];
 };
 
 template <typename T, int W, int FIRST, int LAST>
@@ -1618,6 +1620,7 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
     // ring of the tile in vectors: HALO rows above and below, HALO columns either side
     constexpr int NH = (2 * HALO * TX + 2 * HALO * TY) / W, HS = (NH + NTHREADS - 1) / NTHREADS;
     static_assert(NXT * NYT == NTHREADS, "one vector per thread");
+    constexpr bool DIFF = sizeof(T) == sizeof(float);
     __shared__ __align__(16) T pl[2][SP];
     pdl_wait();
     const int done = check_done ? ctl->done : 0;
@@ -1666,10 +1669,14 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
             if (hdst[q] >= 0) cpa<T, W>(&pl[t & 1][hdst[q]], src + pz + hsrc[q]);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    T xw[9][W], xn[W], rv[W], dv[W];
+    T xw[9][W], gz[8][W], xn[W], rv[W], dv[W];      // the column's values and (float32: kept instead of those below) differences
     ring(0);
 #pragma unroll
     for (int q = 0; q < 8; ++q) vload<T, W>(src + plane(q - 4) + own, xw[q]);
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+#pragma unroll
+        for (int i = 0; i < W; ++i) gz[q][i] = xw[q + 1][i] - xw[q][i];
     vload<T, W>(src + plane(4) + own, xn);
     vload<T, W>(rhs + plane(0) + own, rv);
     if (!FIRST) vload<T, W>(din + plane(0) + own, dv);
@@ -1709,13 +1716,19 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
         }
 #pragma unroll
         for (int i = 0; i < W; ++i) e[HALO + i] = xw[4][i];
+        // the differences first: they are small (float64: the coefficients' form, see above)
+        T g[W + 2 * HALO - 1], pa[W], pb[W];
+#pragma unroll
+        for (int i = 0; i < W + 2 * HALO - 1; ++i) g[i] = e[i + 1] - e[i];
 #pragma unroll
         for (int i = 0; i < W; ++i) {
-            s[i] = C.c0 * xw[4][i];
+            gz[7][i] = xw[8][i] - xw[7][i];
+            pa[i] = pb[i] = xw[4][i];
+            s[i] = DIFF ? T(0) : C.lap0 * xw[4][i];
 #pragma unroll
-            for (int l = 1; l <= 4; ++l) {
-                s[i] += C.cx[l - 1] * (e[HALO + i + l] + e[HALO + i - l]);
-                s[i] += C.cz[l - 1] * (xw[4 + l][i] + xw[4 - l][i]);
+            for (int l = 3; l >= 0; --l) {
+                s[i] += C.cx[l] * (DIFF ? g[HALO + i + l] - g[HALO - 1 + i - l] : e[HALO + 1 + i + l] + e[HALO - 1 + i - l]);
+                s[i] += C.cz[l] * (DIFF ? gz[4 + l][i] - gz[3 - l][i] : xw[5 + l][i] + xw[3 - l][i]);
             }
         }
 #pragma unroll
@@ -1724,8 +1737,14 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
             vload<T, W>(p + me + l * SX, a);
             vload<T, W>(p + me - l * SX, b);
 #pragma unroll
-            for (int i = 0; i < W; ++i) s[i] += C.cy[l - 1] * (a[i] + b[i]);
+            for (int i = 0; i < W; ++i) {
+                s[i] += C.cy[l - 1] * (DIFF ? (a[i] - pa[i]) - (pb[i] - b[i]) : a[i] + b[i]);
+                pa[i] = a[i];
+                pb[i] = b[i];
+            }
         }
+#pragma unroll
+        for (int i = 0; i < W; ++i) s[i] += C.c0 * xw[4][i];
         T xo[W], dk[W];
 #pragma unroll
         for (int i = 0; i < W; ++i) {
@@ -1740,9 +1759,12 @@ helm3d(Geo G, HelmC<T> C, int k, int zb, int rev, const T* __restrict__ rhs, con
             if (!LAST) vstore<T, W>(dout + o, dk);
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int i = 0; i < W; ++i) {
 #pragma unroll
-            for (int i = 0; i < W; ++i) xw[q][i] = xw[q + 1][i];
+            for (int q = DIFF ? 4 : 0; q < 8; ++q) xw[q][i] = xw[q + 1][i];
+#pragma unroll
+            for (int q = 0; q < 7; ++q) gz[q][i] = gz[q + 1][i];
+        }
     }
     pdl_trigger();
 }
@@ -1943,14 +1965,16 @@ static cudaError_t launch_schur3d_w(const Geo& G, int sweeps, const T* r, T* z, 
     if (e != cudaSuccess) return e;
     if (launches) ++*launches;
     HelmC<T> C;
-    const double lap[5] = {-65.0 / 72.0, 1.0 / 9.0, 4.0 / 9.0, -1.0 / 9.0, 1.0 / 144.0};
     const double ax = G.helm_a * G.inv_dx * G.inv_dx, ay = G.helm_a * G.inv_dy * G.inv_dy,
                  az = G.helm_a * G.inv_dz * G.inv_dz;
-    C.c0 = T(lap[0] * (ax + ay + az) - G.two_over_dt);
+    constexpr double lap[5] = {-65.0 / 72.0, 1.0 / 9.0, 4.0 / 9.0, -1.0 / 9.0, 1.0 / 144.0};
+    C.c0 = T(-G.two_over_dt);
+    C.lap0 = T(lap[0] * (ax + ay + az));
     for (int l = 0; l < 4; ++l) {
-        C.cx[l] = T(lap[l + 1] * ax);
-        C.cy[l] = T(lap[l + 1] * ay);
-        C.cz[l] = T(lap[l + 1] * az);
+        const double c = sizeof(T) == sizeof(float) ? HELM_DIFF[l] : lap[l + 1];
+        C.cx[l] = T(c * ax);
+        C.cy[l] = T(c * ay);
+        C.cz[l] = T(c * az);
     }
     constexpr int TX = HelmTile<T, W>::NXT * W, TY = HelmTile<T, W>::NYT;
     const int gx = (G.nx + TX - 1) / TX, gy = (G.ny + TY - 1) / TY;

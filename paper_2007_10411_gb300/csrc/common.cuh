@@ -28,8 +28,7 @@ struct GeoF {
     float inv_dx, inv_dy, inv_dz, wx1, wx2, wy1, wy2, wz1, wz2, ex, ey, ez;
     float theta0, beta, pbar, gth, gamma_p, K_M, K_H, cs2, inv_Pr;
     float dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
-    float two_over_dt, helm_a, schur_cdiv, schur_cgrad, half_dt;
-    float scale[5];
+    float two_over_dt, schur_cdiv, schur_cgrad, half_dt;
 };
 
 // Geometry and physics constants, passed by value to the stencil kernels.

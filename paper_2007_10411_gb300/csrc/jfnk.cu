@@ -432,11 +432,9 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     F.dd_ah = (float)G.dd_ah;
     F.dd_az = (float)G.dd_az;
     F.two_over_dt = (float)G.two_over_dt;
-    F.helm_a = (float)G.helm_a;
     F.schur_cdiv = (float)G.schur_cdiv;
     F.schur_cgrad = (float)G.schur_cgrad;
     F.half_dt = (float)G.half_dt;
-    for (int f = 0; f < nf; ++f) F.scale[f] = (float)G.scale[f];
 
     const size_t eT = h->mixed ? sizeof(float) : sizeof(double);
     const size_t nb8 = h->ld * sizeof(double);

@@ -35,28 +35,8 @@ template <typename T> struct V4;
 template <> struct V4<float> { using type = float4; static constexpr int W = 4; };
 template <> struct V4<double> { using type = double2; static constexpr int W = 2; };
 
-__device__ __forceinline__ float dotv(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
-__device__ __forceinline__ double dotv(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
-__device__ __forceinline__ float4 axpyv(float4 y, float a, float4 x) {
-    return make_float4(y.x - a * x.x, y.y - a * x.y, y.z - a * x.z, y.w - a * x.w);
-}
-__device__ __forceinline__ double2 axpyv(double2 y, double a, double2 x) {
-    return make_double2(y.x - a * x.x, y.y - a * x.y);
-}
 __device__ __forceinline__ float4 scalev(float4 x, float a) { return make_float4(a * x.x, a * x.y, a * x.z, a * x.w); }
 __device__ __forceinline__ double2 scalev(double2 x, double a) { return make_double2(a * x.x, a * x.y); }
-
-__device__ __forceinline__ float4 reload(const float4* p) {
-    float4 r;
-    asm volatile("ld.global.ca.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
-    return r;
-}
-__device__ __forceinline__ double2 reload(const double2* p) {
-    double2 r;
-    asm volatile("ld.global.ca.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "l"(p));
-    return r;
-}
 
 // Field of vector entry i (planes of npt entries); 32-bit division where it fits.
 __device__ __forceinline__ int field_of(size_t i, int npt) {
@@ -423,8 +403,6 @@ __device__ __forceinline__ float4 subv(float4 a, float4 b) { return make_float4(
 __device__ __forceinline__ double2 subv(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float subv(float a, float b) { return a - b; }
 __device__ __forceinline__ double subv(double a, double b) { return a - b; }
-__device__ __forceinline__ float dotv(float a, float b) { return a * b; }
-__device__ __forceinline__ double dotv(double a, double b) { return a * b; }
 template <typename VT> __device__ __forceinline__ VT zerov();
 template <> __device__ __forceinline__ float4 zerov<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 template <> __device__ __forceinline__ double2 zerov<double2>() { return make_double2(0.0, 0.0); }

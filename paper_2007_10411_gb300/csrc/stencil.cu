@@ -40,12 +40,6 @@ __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a,
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-template <typename T>
-__device__ __forceinline__ T dd(const T* s, int i, int st, T inv_h) {
-    const T d1 = s[i + st] - s[i - st], d2 = s[i + 2 * st] - s[i - 2 * st];
-    return rmul(rfma(T(2.0 / 3.0), d1, rmul(T(-1.0 / 12.0), d2)), inv_h);
-}
-
 // Source row / sign of a ghost-extended z index.  side: 0 interior, 1 bottom, 2 top.
 __device__ __forceinline__ int mirror_z(int gz, int nz, int& side) {
     side = 0;
@@ -73,7 +67,6 @@ template <> struct Vec16<float> {
     __device__ static float4 fma(float a, float4 x, float4 y) {
         return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
     }
-    __device__ static float4 mul(float a, float4 x) { return make_float4(a * x.x, a * x.y, a * x.z, a * x.w); }
     __device__ static float4 neg(float4 x) { return make_float4(flip(x.x), flip(x.y), flip(x.z), flip(x.w)); }
 };
 template <> struct Vec16<double> {
@@ -83,7 +76,6 @@ template <> struct Vec16<double> {
     __device__ static double2 fma(double a, double2 x, double2 y) {
         return make_double2(::fma(a, x.x, y.x), ::fma(a, x.y, y.y));
     }
-    __device__ static double2 mul(double a, double2 x) { return make_double2(a * x.x, a * x.y); }
     __device__ static double2 neg(double2 x) { return make_double2(flip(x.x), flip(x.y)); }
 };
 
@@ -95,8 +87,8 @@ static bool rows_aligned(const Geo& G, const T* a, const T* b = nullptr) {
     return G.nx % Vec16<T>::W == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
 }
 
-// Stage 1: s[f][SZ][SX] <- (LOADMODE 0) u, (1) u + ev*v, (2) ev*v for fields
-// f0 .. f0+NF-1, ghost-extended (periodic x, signed mirror z).  aligned: the
+// Stage 1: s[f][SZ][SX] <- (LOADMODE 0) u, (1) u + ev*v for fields f0 .. f0+NF-1,
+// ghost-extended (periodic x, signed mirror z).  aligned: the
 // host's rows_aligned(u, v); a tile whose x-range [x0 - HALO, x0 - HALO + SX)
 // lies inside the grid then loads its rows as 16-byte vectors.
 template <typename T, int LOADMODE, int NF = 4>
@@ -122,10 +114,9 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
                 if (ok) {
                     const size_t o = (size_t)f * G.npt + off;
                     if (LOADMODE == 0) val = *reinterpret_cast<const VT*>(u + o);
-                    else if (LOADMODE == 1)
+                    else
                         val = Vec16<T>::fma(ev[f], *reinterpret_cast<const VT*>(v + o),
                                             *reinterpret_cast<const VT*>(u + o));
-                    else val = Vec16<T>::mul(ev[f], *reinterpret_cast<const VT*>(v + o));
                     if (odd_ghost(G, f, side)) val = Vec16<T>::neg(val);
                 }
                 *reinterpret_cast<VT*>(s + (q * SZ + iz) * SX + c * VW) = val;
@@ -149,8 +140,7 @@ __device__ __forceinline__ void load_fields(T* s, const T* __restrict__ u, const
             if (ok) {
                 const size_t o = (size_t)f * G.npt + off;
                 if (LOADMODE == 0) val = u[o];
-                else if (LOADMODE == 1) val = rfma(ev[f], v[o], u[o]);
-                else val = ev[f] * v[o];
+                else val = rfma(ev[f], v[o], u[o]);
                 if (odd_ghost(G, f, side)) val = flip(val);
             }
             s[(q * SZ + iz) * SX + ix] = val;

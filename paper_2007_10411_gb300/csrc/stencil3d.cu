@@ -48,10 +48,6 @@ constexpr int R = 2;
 constexpr int HALO = 2 * R;
 constexpr int MODE_F = 0, MODE_RHS = 1, MODE_RES = 2, MODE_JV = 3, MODE_RHSRES = 4;
 
-template <typename T>
-__device__ __forceinline__ T dd(const T* s, int i, int st, T ih) {
-    return (T(2.0 / 3.0) * (s[i + st] - s[i - st]) - T(1.0 / 12.0) * (s[i + 2 * st] - s[i - 2 * st])) * ih;
-}
 // D f from the four neighbours f(-2), f(-1), f(+1), f(+2)
 template <typename T>
 __device__ __forceinline__ T d5(T m2, T m1, T p1, T p2, T ih) {

@@ -576,7 +576,9 @@ extern "C" jfnk_status jfnk_kernel_timing_read(jfnk_handle* h, jfnk_kernel_time*
 
 // Time every tile candidate of the float32 Jacobian-product and preconditioner
 // kernels on this handle's grid (inputs: u and a direction built from it) and
-// keep the fastest; tiles[0..1] (may be NULL) receive the chosen indices.
+// keep the fastest; tiles[0..1] (may be NULL) receive the chosen indices.  An index
+// that launches what a smaller one launches is left out: the choice between the two
+// would be noise.
 template <typename T>
 static jfnk_status autotune_impl(jfnk_handle* h, const double* u, int* tiles) {
     cudaStream_t s = h->stream;
@@ -596,10 +598,15 @@ static jfnk_status autotune_impl(jfnk_handle* h, const double* u, int* tiles) {
     const int reps = 16;
     float best_jv = 1e30f, best_pc = 1e30f;
     int arg_jv = 0, arg_pc = 0;
+    auto repeats = [&](int (*threads)(const Geo&, int), int c) {
+        for (int b = 0; b < c; ++b)
+            if (threads(G, b) == threads(G, c)) return true;
+        return false;
+    };
     for (int c = 0; c < NUM_TILE_SHAPES; ++c) {
         G.tile_jv = c;
         G.tile_pc = c;
-        for (int pass = 0; pass < 4; ++pass) {          // pass 0 warms up (and sets shared-memory limits)
+        for (int pass = 0; pass < 4 && !repeats(jv2d_threads, c); ++pass) {          // pass 0 warms up (and sets shared-memory limits)
             CK(cudaEventRecord(e0, s));
             for (int r = 0; r < reps; ++r) CK(launch_jv_diff(G, uT, dir, (T*)h->w, h->part, h->ctl, 0, s));
             CK(cudaEventRecord(e1, s));
@@ -608,7 +615,7 @@ static jfnk_status autotune_impl(jfnk_handle* h, const double* u, int* tiles) {
             CK(cudaEventElapsedTime(&ms, e0, e1));
             if (pass > 0 && ms < best_jv) { best_jv = ms; arg_jv = c; }   // best of three timings
         }
-        if (h->opts.precond != JFNK_PC_NONE && h->opts.pc_sweeps > 1) {
+        if (h->opts.precond != JFNK_PC_NONE && h->opts.pc_sweeps > 1 && !repeats(cheb2d_threads, c)) {
             for (int pass = 0; pass < 4; ++pass) {
                 CK(cudaEventRecord(e0, s));
                 for (int r = 0; r < reps; ++r)

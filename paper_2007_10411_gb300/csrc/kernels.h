@@ -28,6 +28,11 @@ cudaError_t launch_precond(const Geo& G, int sweeps, const T* r, T* z, T* za, T*
                            const T* nu, double* part, Ctl* ctl, int check_done, cudaStream_t s,
                            long long* launches);
 
+// Threads per CTA of the float32 2-D Jacobian product and field-block sweep with tile
+// index `tile` on this grid; 0 where the index has no effect (3-D, Schur complement).
+int jv2d_threads(const Geo& G, int tile);
+int cheb2d_threads(const Geo& G, int tile);
+
 // 2-D Schur complement: Helmholtz sweeps that one launch does when `left` remain
 // (elem: bytes of an element; vec: rows are whole 16-byte vectors).
 int schur2d_sweeps(const Geo& G, size_t elem, bool vec, int left);

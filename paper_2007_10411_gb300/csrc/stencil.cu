@@ -1721,10 +1721,12 @@ static cudaError_t launch_jv_t(const Geo& G, const float* u, const float* v, flo
 // workspace vectors: their planes start multiples of npt elements in); 256 or 128
 // threads a CTA by Geo::tile_jv, 256 for tile_jv = 0 (a step with 256 / 128 at
 // 1024 x 512: 52.9 / 57.1 ms, at 250 x 119: 3.91 / 4.01 ms: a smaller tile has more arms).
+int jv2d_threads(const Geo& G, int tile) { return G.dim == 3 ? 0 : (tile == 2 ? 128 : 256); }
+
 template <int SMAG>
 static cudaError_t launch_jv(const Geo& G, const float* u, const float* v, float* out, const double* part, Ctl* ctl,
                              int check_done, cudaStream_t s) {
-    const bool small = G.tile_jv == 2;
+    const bool small = jv2d_threads(G, G.tile_jv) == 128;
 #define JF_JV(W) (small ? launch_jv_t<W, 128, SMAG>(G, u, v, out, part, ctl, check_done, s) \
                         : launch_jv_t<W, 256, SMAG>(G, u, v, out, part, ctl, check_done, s))
     return G.nx % 4 == 0 ? JF_JV(4) : G.nx % 2 == 0 ? JF_JV(2) : JF_JV(1);
@@ -1792,17 +1794,20 @@ static cudaError_t launch_precond_w(const Geo& G, int sweeps, const float* r, fl
 // for tile_pc = 0: 256 where that leaves no SM without a CTA, else 128 (a step at
 // 1024 x 512 with 256 / 128 / 64: 52.9 / 53.6 / 55.5 ms, at 250 x 119: 3.83 /
 // 3.81 / 3.90 ms).
+int cheb2d_threads(const Geo& G, int tile) {
+    constexpr int SMS = 152;
+    if (G.dim == 3 || G.pc_schur) return 0;
+    if (tile != 0) return tile == 1 ? 256 : (tile == 2 ? 128 : 64);
+    const int w = G.nx % 4 == 0 ? 4 : (G.nx % 2 == 0 ? 2 : 1);
+    return (long long)((G.nx + w - 1) / w) * G.nz >= 256LL * SMS ? 256 : 128;       // threads with a point
+}
+
 template <int SMAG>
 static cudaError_t launch_precond_f32(const Geo& G, int sweeps, const float* r, float* z, float* za, float* zb, float* da,
                                       float* db, const float* nu, double* part, Ctl* ctl, int check_done,
                                       cudaStream_t s, long long* launches) {
-    constexpr int SMS = 152;
     const int w = G.nx % 4 == 0 ? 4 : (G.nx % 2 == 0 ? 2 : 1);
-    int nt = G.tile_pc == 1 ? 256 : (G.tile_pc == 2 ? 128 : 64);
-    if (G.tile_pc == 0) {
-        const long long vecs = (long long)((G.nx + w - 1) / w) * G.nz;       // threads with a point
-        nt = vecs >= 256LL * SMS ? 256 : 128;
-    }
+    const int nt = cheb2d_threads(G, G.tile_pc);
 #define JF_PC(W, NT) launch_precond_w<W, NT, SMAG>(G, sweeps, r, z, za, zb, da, db, nu, part, ctl, check_done, s, launches)
 #define JF_PCW(W) (nt == 256 ? JF_PC(W, 256) : nt == 128 ? JF_PC(W, 128) : JF_PC(W, 64))
     return w == 4 ? JF_PCW(4) : w == 2 ? JF_PCW(2) : JF_PCW(1);

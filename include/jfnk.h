@@ -422,9 +422,12 @@ jfnk_status jfnk_set_precond(jfnk_handle* h, int precond);
 /* Choose the tile shapes of the float32 Jacobian-product and preconditioner
  * stencils for this handle's grid: every candidate is timed on the handle's
  * stream with inputs derived from the device state u (unchanged), and the
- * fastest is kept.  tiles (host, may be NULL) receives {jv, pc} indices.
- * Synchronises the stream; results of the kernels are unaffected (every
- * shape computes the same values).  A float64 handle keeps its single shape. */
+ * fastest is kept (indices that launch the same kernel are one candidate).
+ * tiles (host, may be NULL) receives {jv, pc} indices.  Synchronises the stream.
+ * Every shape computes the same values; a step may differ in its last bits, because
+ * the preconditioner's tiles decide in which order the squares of ||z||, from which the
+ * finite-difference step follows, are added.  The tiles of the float64 kernels follow
+ * the grid: on a float64 handle the call reports the indices set and changes nothing. */
 jfnk_status jfnk_autotune(jfnk_handle* h, const double* u, int* tiles);
 
 /* Set the tile-shape indices (0 .. JFNK_NUM_TILE_SHAPES-1) directly. */

@@ -640,7 +640,7 @@ static jfnk_status autotune_impl(jfnk_handle* h, const double* u, int* tiles) {
 
 extern "C" jfnk_status jfnk_autotune(jfnk_handle* h, const double* u, int* tiles) {
     if (!h || !u) return JFNK_ERR_INVALID_ARG;
-    if (!h->mixed) {                       // the float64 kernels have a single tile shape
+    if (!h->mixed) {                       // the float64 kernels' tiles follow the grid (flux_shape)
         if (tiles) { tiles[0] = h->G.tile_jv; tiles[1] = h->G.tile_pc; }
         return JFNK_OK;
     }

@@ -17,9 +17,11 @@
 // its partial sums, and every block of the NEXT pass adds all of them in one
 // fixed order (grid_sums), so that no pass ends in a serial last-block tail
 // and all blocks hold bitwise the same coefficients.  A thread accumulates
-// its partial dot products in the basis precision over at most 64 vector
-// elements (the grid grows with n), then the block and grid sums run in
-// float64.
+// its partial dot products in the basis precision: pass A, and pass B of a
+// float32 basis, over at most 64 vectors (the grid grows with n); pass CA, pass C
+// and pass B of more than sixteen float64 vectors on one round of resident CTAs,
+// over n / (grid threads) of them.  The sums of a block and of the grid run in
+// float-float pairs (float32) or float64.
 #include <math.h>
 
 #include <algorithm>
@@ -233,9 +235,8 @@ __device__ void grid_sums(const P* part, int nblk, int nv, double* out, TO* outT
 }
 
 // h_{j+1,j}^2 = ||w'||^2 - ||h2||^2 by one warp (nv <= 32): every lane returns
-// the same value.  The Givens block and the streaming blocks of pass C both
-// call it, so the Hessenberg entry and the normalisation of v_{j+1} are the
-// same number.
+// the same value.  The Givens block takes its root, the streaming blocks the
+// reciprocal of it (root, root_pair: they agree to a few 2^-53).
 __device__ __forceinline__ double subdiag2(const double* h2, int nv, double wn2) {
     const int lane = threadIdx.x & 31;
     double q = lane < nv ? h2[lane] * h2[lane] : 0.0;
@@ -417,7 +418,10 @@ template <> __device__ __forceinline__ double zerov<double>() { return 0.0; }
 // 1024 x 512, for 183 us of FMAs).  One lane keeps all entries (up to 32 double2
 // and their sums: one CTA per SM above NV = 16, 8 warps of 32 loads each in
 // flight) and skips the empty ones four at a time (SKIP): 222 us at nv = 28,
-// 175 against 270 at 17 .. 24, 130 against 192 at 13 .. 16.
+// 175 against 270 at 17 .. 24, 130 against 192 at 13 .. 16.  At 13 .. 16 vectors
+// two CTAs of 128 registers a thread are kept although pass CA then spills 300 bytes
+// (its 32-vector form 320); over cycles of 16 it takes 96 us on average against
+// 141 with two lanes.
 template <typename T, int NV> constexpr int LANES = sizeof(T) == sizeof(double) || NV <= 16 ? 1 : 2;
 template <typename T, int NV> constexpr int MIN_CTAS = sizeof(T) == sizeof(double) && NV > 16 ? 1 : 2;
 template <typename T> constexpr bool SKIP = sizeof(T) == sizeof(double);

@@ -182,7 +182,7 @@ __device__ __forceinline__ T smag_nu(T ux, T uz, T wx, T wz, T cs2) {
 // coefficient, 14 fluxes, 18 point-wise, 32 flux derivatives, 16 output and
 // norms) and 45 per arm point, against about 255 for the form that rebuilt
 // the products at every tap and formed all derivatives on the whole halo.
-// One F(u) at 1024 x 512, Smagorinsky: 236 -> 142 us; at 128 x 64: 31 -> 6 us.
+// One F(u) at 1024 x 512, Smagorinsky: 236 -> 144 us; at 128 x 64: 31 -> 8 us.
 // ============================================================================
 // The strain magnitude sqrt(2 S:S) from the velocity gradients.
 template <typename T>
@@ -490,7 +490,7 @@ __device__ __forceinline__ void cpa_vec(T* dst, const T* src) {
 // and below) alone.  Phase 3 differentiates the fluxes and writes Jv.
 // The arithmetic is explicitly rounded, so a flux formed in a tile and the same
 // flux formed in a neighbour's arm are bitwise equal and every tile shape gives
-// the same result.  The eddy coefficient of a point in a ghost row is that of
+// the same result for the same step eps.  The eddy coefficient of a point in a ghost row is that of
 // its mirror image.
 //
 // Bound: issue and shared-memory latency.  The form with one point per thread,
@@ -973,12 +973,12 @@ __global__ void pc_setup(Geo G, int sweeps, Ctl* ctl) {
 // pc_sweeps = 2); p is written by the last sweep.  Explicitly rounded, so every
 // tile shape computes the same bits.
 //
-// Bound: latency of the one load phase and issue (23 MB a launch at
-// 1024 x 512, 3.4 us).  One field per CTA with three barriers and the fluxes in
+// Bound: latency of the one load phase and issue (19 MB a launch at
+// 1024 x 512, 2.8 us).  One field per CTA with three barriers and the fluxes in
 // shared memory took 19-20 us there and 7.1-7.8 us at 250 x 119; this form 11.2 and 4.4 us (with
-// the overlap of the launches before it; 12.0 us at 1024 x 512 with the first
-// field's loads hoisted over the loop and 72 registers, three CTAs per SM: 1024
-// threads an SM need 64).
+// the overlap of the launches before it).  1024 threads an SM need 64 registers a
+// thread, at which the 16-byte rows spill 80 bytes (Deardorff 136); 72 registers and
+// three CTAs per SM, with the first field's loads hoisted over the loop, took 12.0 us.
 // ----------------------------------------------------------------------------
 template <int W> struct PcRow { static constexpr int NXT = W == 4 ? 16 : 32; };   // threads along x
 
@@ -1718,9 +1718,10 @@ static cudaError_t launch_jv_t(const Geo& G, const float* u, const float* v, flo
 }
 
 // Rows of 16-byte, 8-byte or single-element vectors as nx allows (u and v are
-// workspace vectors: their planes start multiples of npt elements in); 256 or 128
-// threads a CTA by Geo::tile_jv, 256 for tile_jv = 0 (a step with 256 / 128 at
-// 1024 x 512: 52.9 / 57.1 ms, at 250 x 119: 3.91 / 4.01 ms: a smaller tile has more arms).
+// workspace vectors: their planes start multiples of npt elements in); 256 threads
+// a CTA (a step with 256 / 128 at 1024 x 512: 52.9 / 57.1 ms, at 250 x 119: 3.91 / 4.01
+// ms: a smaller tile has more arms), 128 for the autotuner and jfnk_set_tiles
+// (tile index 2).
 int jv2d_threads(const Geo& G, int tile) { return G.dim == 3 ? 0 : (tile == 2 ? 128 : 256); }
 
 template <int SMAG>
@@ -1791,9 +1792,10 @@ static cudaError_t launch_precond_w(const Geo& G, int sweeps, const float* r, fl
 // Rows of 16-byte, 8-byte or single-element vectors as nx allows (r and z of the
 // batched and per-call paths are workspace vectors: their planes start multiples
 // of npt elements in); 256, 128 or 64 threads a CTA by Geo::tile_pc, by the grid
-// for tile_pc = 0: 256 where that leaves no SM without a CTA, else 128 (a step at
-// 1024 x 512 with 256 / 128 / 64: 52.9 / 53.6 / 55.5 ms, at 250 x 119: 3.83 /
-// 3.81 / 3.90 ms).
+// for tile_pc = 0: 256 where that leaves no SM without a CTA, else 128, so that the
+// CTAs reach more SMs (a step at 1024 x 512 with 256 / 128 / 64: 52.9 / 53.6 / 55.5 ms;
+// at 250 x 119, below the line, 3.83 / 3.81 / 3.90 ms: 256 and 128 differ by less than
+// runs do).  64 is for the autotuner and jfnk_set_tiles.
 int cheb2d_threads(const Geo& G, int tile) {
     constexpr int SMS = 152;
     if (G.dim == 3 || G.pc_schur) return 0;

@@ -367,7 +367,7 @@ template <int CI, int IH, int IW, int HP, int INMODE, int CU>
 struct Stager {
     static constexpr int VPP = CI / 8, N = IH * IW * VPP, NS = (N + CONV_THREADS - 1) / CONV_THREADS;
     int rel[NS];        // source offset from the tile's (elements)
-    int pos[NS];        // (iy - HP) << 16 | (ix - HP) + 8, -1: no slot
+    int pos[NS];        // iy << 16 | ix in the staged tile, -1: no slot
     uint32_t dst[NS];   // byte offset in the staged tile
     unsigned up;        // bit q: slot q reads the upsampled source
 

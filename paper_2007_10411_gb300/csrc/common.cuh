@@ -48,11 +48,13 @@ struct Geo {
     double dd_cm, dd_cM, dd_cl, dd_delta, dd_ah, dd_az;
     // derivative weights with 1/h folded in: D f = w1 (f_{+1} - f_{-1}) + w2 (f_{+2} - f_{-2})
     double wx1, wx2, wy1, wy2, wz1, wz2;
-    // relative difference of 2/3 times 1/h (each rounded) from w1, and of -1/12 times 1/h
-    // from w2 = -w1/8: D f = w (1 + e) (...).  The divergence of a nearly solenoidal flow
-    // is a small part of its terms, so what the rounding of one axis's weight adds counts
-    // in full, and the pressure equation multiplies it by gamma_p pbar.
-    double ex, ey, ez;
+    // D f = w (1 + e) (...): what rounding took from the weights, e the relative difference
+    // of 2/3 times 1/h (each rounded) from w1, and of -1/12 times 1/h from w2 = -w1/8; here
+    // (not in GeoF) that of y and z less that of x, the common factor being harmless
+    // and an operation of the FP64 pipe.  The divergence of a nearly solenoidal flow is a
+    // small part of its terms, so what the rounding of one axis's weight adds against the
+    // others counts in full, and the pressure equation multiplies it by gamma_p pbar.
+    double ey, ez;
     double gth;                       // g / theta0
     double inv_Pr;
     double two_over_dt;

@@ -359,9 +359,8 @@ extern "C" jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_strat* stra
     G.wz1 = 2.0 / 3.0 / dz;
     G.wz2 = -1.0 / 12.0 / dz;
     auto lost = [](double w, double inv_h) { return fma(2.0 / 3.0, inv_h, -w) / w; };
-    G.ex = lost(G.wx1, G.inv_dx);
-    G.ey = lost(G.wy1, G.inv_dy);
-    G.ez = lost(G.wz1, G.inv_dz);
+    G.ey = lost(G.wy1, G.inv_dy) - lost(G.wx1, G.inv_dx);
+    G.ez = lost(G.wz1, G.inv_dz) - lost(G.wx1, G.inv_dx);
     G.gth = strat->g / strat->theta0;
     G.theta0 = strat->theta0;
     G.beta = strat->beta;

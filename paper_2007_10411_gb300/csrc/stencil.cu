@@ -265,7 +265,9 @@ __device__ __forceinline__ void flux_point(const Geo& G, const FluxShape& sh, co
     }
     if (XF && ZF) {
         const T px = wd(P, i, 1, wx1, wx2), pz = wd(P, i, SX, wz1, wz2);
-        const T th0 = GC(theta0), div = rfma(GC(ex), ux, rfma(GC(ez), wz, ux + wz));
+        const T th0 = GC(theta0);
+        T div = rfma(GC(ez), wz, ux + wz);
+        if constexpr (sizeof(T) == sizeof(float)) div = rfma(G.f32.ex, ux, div);
         S[0] = rfma(-hu, ux, rfma(-hw, uz, -rmul(th0, px)));
         S[1] = rfma(-hu, wx, rfma(-hw, wz, rfma(GC(gth), H[i], -rmul(th0, pz))));
         S[2] = rfma(-hu, tx, rfma(-hw, tz, -rmul(GC(beta), W[i])));

@@ -547,12 +547,12 @@ __device__ __forceinline__ void plane_point(const Geo& G, const T* __restrict__ 
             // the small advective terms first: the large linear ones are rounded once
             s = advect<T, KIND>(s, mu, bu, dmx, dbx);
             s = advect<T, KIND>(s, mv, bv, dmy, dby);
-            if (f == 0) { divb = dbx; divm = dmx; dive = GC(ex) * dbx; }
+            if (f == 0) { divb = dbx; divm = dmx; if constexpr (sizeof(T) == sizeof(float)) dive = G.f32.ex * dbx; }
             if (f == 1) { divb += dby; divm += dmy; dive = fma(GC(ey), dby, dive); }
             if (f == 2) s += GC(gth) * B[3 * SP + c];
             if (f == 3) s -= GC(beta) * B[2 * SP + c];
             if (f == 4) {       // pressure equation, x and y parts of the divergence; gradient of p
-                // (what the weights lost, Geo::ex, with the small terms: see pressure_part)
+                // (what the weights lost, Geo::ey, with the small terms: see pressure_part)
                 s = pressure_part<T, KIND>(G, s, KIND == PAIR ? m : b, b, divb, divm, dive);
                 S[0] -= GC(theta0) * dbx;
                 S[1] -= GC(theta0) * dby;

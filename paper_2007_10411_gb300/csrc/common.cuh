@@ -364,7 +364,8 @@ __device__ __forceinline__ void put_eps_norm2(Ctl* ctl, double zn2) {
 // pending partials.  The first four warps add them (a float64 addition takes a
 // sub-partition's pipe for 64 cycles; more warps would queue for it), across the
 // warps in float64, in one fixed order: every block of the launch, whatever its
-// size, obtains bitwise the same value.  Called by all threads of a block of at
+// size, obtains bitwise the same value.  (0.7 us of jv2d's 22.9 at 1024 x 512 against
+// float-float sums across all warps.)  Called by all threads of a block of at
 // least 128.
 __device__ __forceinline__ double2 pending_eps(const Ctl* ctl, const double* part) {
     constexpr int NT = 128;
